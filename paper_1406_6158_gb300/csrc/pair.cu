@@ -24,9 +24,10 @@
 // into zeroed outputs.
 // rsqrtf runs on the CUDA cores: the pair sum is not a dense contraction.
 //
-// FP64 form (the plain form): one warp per group, one sink per lane, plain
-// FP64 differences and 1/sqrt.
+// FP64 form (the plain form): plain FP64 differences; see k_pair_f64.
 #include "hy_internal.cuh"
+
+#include "fp64_rsqrt.cuh"
 
 namespace hy {
 
@@ -132,16 +133,6 @@ __device__ __forceinline__ void near_finish(float w, float dx, float dy, float d
         hay = fmaf(dy, fh, hay);
         haz = fmaf(dz, fh, haz);
     }
-}
-
-// ---- FP64 bodies ----------------------------------------------------------
-__device__ __forceinline__ double dll_K64(double r, double R1, double R2)
-{
-    const double Y = (R2 - r) / (R2 - R1);
-    if (Y >= 1.0) return 1.0;
-    if (Y <= 0.0) return 0.0;
-    const double Y2 = Y * Y;
-    return (Y2 * Y2 * Y2) * (10.0 + Y2 * (-15.0 + 6.0 * Y2));
 }
 
 __device__ __forceinline__ int64_t next_item(unsigned long long *counter, int lane)
@@ -736,97 +727,159 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR ? NEAR_MIN_BLOCKS : 0) k_pa
 }
 
 // ---------------------------------------------------------------------------
-// FP64 kernel: one warp per group, one lane per sink (rounds of 32 sinks),
-// sources staged as double4 in shared memory.
+// FP64 kernel. The FP64 pipe (2 lanes per SM and clock) bounds it, so what
+// counts is that every SM has work and every lane holds a pair. Work unit =
+// (group, slice of at most F64_SINKS sinks), one block of F64_WARPS warps
+// each: a warp's lanes are lpc sinks (a power of two) times 32 / lpc copies,
+// and the unit's sources go round robin to the F64_WARPS x copies lanes of a
+// sink, straight from global memory (a source is 32 B against 8 sinks x 16
+// FP64 instructions of 16 clocks: loads are nowhere near the limit). The
+// partial sums are added in a fixed order (butterfly over the copies, then the
+// warps), and the split depends on the group alone, so a system's forces are
+// the same bit for bit alone and in any batch.
+// Before, one warp per group with sqrt and division: the far launch of a system
+// of 4096 particles took 4.1 ms, its ~100 groups leaving most SMs idle. A soft
+// step of 4 hard sub-steps went from 11.9 to 2.07 ms at N = 4096, one
+// kick-drift-kick step at N = 30011 from 30.3 to 4.8 ms.
 // ---------------------------------------------------------------------------
-template <bool NEAR>
-__global__ void __launch_bounds__(PAIR_THREADS) k_pair_f64(PairArgs a)
+constexpr int F64_SINKS = 8, F64_WARPS = 4;
+
+template <bool NEAR, bool SOFT, bool HARD>
+__global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int slices)
 {
-    __shared__ double4_32a tiles[PAIR_WARPS][TILE];
+    constexpr int NS = (SOFT ? 3 : 0) + (HARD ? 3 : 0);
+    __shared__ double part[F64_WARPS][F64_SINKS][NS];
+    __shared__ int64_t unit;
     if (a.st->code) return;
-    const int lane = threadIdx.x & 31;
-    double4_32a *tile = tiles[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t ng = *a.ngroups;
     unsigned long long inter = 0;
     for (;;) {
-        const int64_t g = next_item(a.counter, lane);
+        __syncthreads();   // the last unit's sums are read
+        if (threadIdx.x == 0) unit = (int64_t)atomicAdd(a.counter, 1ull);
+        __syncthreads();
+        const int64_t g = unit / slices;
         if (g >= ng) break;
-        const uint32_t first = a.gfirst[g];
+        const int slice = (int)(unit - g * slices);
         const int n = (int)a.gcount[g];
-        const SysParams P = a.sp[a.gsys[g]];
-        uint64_t c0, c1, p0, p1;
+        if (slice * F64_SINKS >= n) continue;
+        const uint32_t first = a.gfirst[g];
+        const SysParams &P = a.sp[a.gsys[g]];
+        const double eps2 = P.eps2, R2 = P.R2, R2sq = P.R2sq, invdR = P.invdR;
+        uint64_t c0 = 0, p0;
+        int64_t Lc = 0, L;   // entries: cells [0, Lc), then particles [Lc, L)
         if (!NEAR) {
             c0 = a.off[g];
-            c1 = a.off[g + 1];
+            Lc = (int64_t)(a.off[g + 1] - c0);
             p0 = a.off[ng + g];
-            p1 = a.off[ng + g + 1];
+            L = Lc + (int64_t)(a.off[ng + g + 1] - p0);
         } else {
-            c0 = c1 = 0;
             p0 = a.off[2 * ng + g];
-            p1 = a.off[2 * ng + g + 1];
+            L = (int64_t)(a.off[2 * ng + g + 1] - p0);
         }
-        inter += (unsigned long long)n * ((c1 - c0) + (p1 - p0));
-        for (int r0 = 0; r0 < n; r0 += 32) {
-            const int si = r0 + lane;
-            const double4_32a s = a.pd[first + (si < n ? si : n - 1)];
+        if (slice == 0) inter += (unsigned long long)n * (unsigned long long)L;
+        for (int r0 = slice * F64_SINKS; r0 < n; r0 += slices * F64_SINKS) {   // more than one round: leaves above n_crit
+            const int rem = min(n - r0, F64_SINKS);
+            const int lpc = rem <= 1 ? 1 : 1 << (32 - __clz(rem - 1));   // power of two >= rem
+            const int copies = 32 / lpc, copy = lane / lpc, slot = lane & (lpc - 1);
+            const double4_32a s = a.pd[first + r0 + min(slot, rem - 1)];
             double ax = 0.0, ay = 0.0, az = 0.0, bx = 0.0, by = 0.0, bz = 0.0;
-            for (int part = 0; part < 2; ++part) {
-                const uint64_t q0 = part ? p0 : c0, q1 = part ? p1 : c1;
-                for (uint64_t t0 = q0; t0 < q1; t0 += TILE) {
-                    const int nt = (int)min((uint64_t)TILE, q1 - t0);
-                    for (int e = lane; e < nt; e += 32) {
-                        const uint32_t idx = a.list[t0 + e];
-                        tile[e] = part ? a.pd[idx] : a.nD[idx];
+            const int64_t step = F64_WARPS * copies;
+            auto index = [&](int64_t e) -> uint32_t {
+                return e < L ? (!NEAR && e < Lc ? a.list[c0 + e] : a.list[p0 + (uint64_t)(e - Lc)]) : 0u;
+            };
+            auto source = [&](int64_t e, uint32_t i) -> double4_32a {   // a massless copy of the sink past the end
+                return e < L ? (!NEAR && e < Lc ? a.nD[i] : a.pd[i]) : make_double4_32a(s.x, s.y, s.z, 0.0);
+            };
+            int64_t e = w * copies + copy;
+            // the source of the next pair and the index of the one after it are on their way during a pair
+            uint32_t i1 = index(e + step);
+            double4_32a q1 = source(e, index(e));
+            for (int64_t k = w * copies; k < L; k += step, e += step) {   // k: the same trip count on every lane
+                const double4_32a q = q1;
+                q1 = source(e + step, i1);
+                i1 = index(e + 2 * step);
+                const double dx = __dsub_rn(q.x, s.x), dy = __dsub_rn(q.y, s.y), dz = __dsub_rn(q.z, s.z);
+                if (!NEAR) {
+                    const double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, __fma_rn(dz, dz, eps2)));
+                    const double f = mass_over_r3(q.w, r2);
+                    ax = __fma_rn(f, dx, ax);
+                    ay = __fma_rn(f, dy, ay);
+                    az = __fma_rn(f, dz, az);
+                } else {
+                    const double r2u = __fma_rn(dx, dx, __fma_rn(dy, dy, __dmul_rn(dz, dz)));
+                    // r2u < R2^2, compared as integers (both are >= 0; NaN compares above)
+                    const bool in = e < L && __double_as_longlong(r2u) < __double_as_longlong(R2sq);
+                    const bool any_in = __any_sync(0xffffffffu, in);
+                    if (!SOFT && !any_in) continue;
+                    const double f = mass_over_r3(q.w, __dadd_rn(r2u, eps2));
+                    double K = 0.0;
+                    if (any_in) {   // Eq. (10); 0 outside R2
+                        const double r = sqrt_seeded(r2u);
+                        const double Y = __dmul_rn(__dsub_rn(R2, r), invdR);
+                        const double Y2 = __dmul_rn(Y, Y);
+                        K = __dmul_rn(__dmul_rn(Y2, __dmul_rn(Y2, Y2)),
+                                      __fma_rn(Y2, __fma_rn(Y2, 6.0, -15.0), 10.0));
+                        K = __double2hiint(Y) >= 0x3ff00000 ? 1.0 : K;   // Y >= 1
+                        K = in && __double2hiint(Y) >= 0 ? K : 0.0;      // Y >= 0
                     }
-                    __syncwarp();
-                    for (int j = 0; j < nt; ++j) {
-                        const double4_32a q = tile[j];
-                        const double dx = q.x - s.x, dy = q.y - s.y, dz = q.z - s.z;
-                        const double r2u = dx * dx + dy * dy + dz * dz;
-                        const double r2 = r2u + P.eps2;
-                        const double ri = r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0;
-                        const double f = q.w * ri * ri * ri;
-                        if (!NEAR) {
-                            ax += f * dx;
-                            ay += f * dy;
-                            az += f * dz;
-                        } else {
-                            const double K = r2u < P.R2sq ? dll_K64(sqrt(r2u), P.R1, P.R2) : 0.0;
-                            const double fs = f * (1.0 - K);
-                            ax += fs * dx;
-                            ay += fs * dy;
-                            az += fs * dz;
-                            const double fh = f * K;
-                            bx += fh * dx;
-                            by += fh * dy;
-                            bz += fh * dz;
-                        }
+                    if (SOFT) {
+                        const double fs = any_in ? __dmul_rn(f, __dsub_rn(1.0, K)) : f;
+                        ax = __fma_rn(fs, dx, ax);
+                        ay = __fma_rn(fs, dy, ay);
+                        az = __fma_rn(fs, dz, az);
                     }
-                    __syncwarp();
+                    if (HARD && any_in) {
+                        const double fh = __dmul_rn(f, K);
+                        bx = __fma_rn(fh, dx, bx);
+                        by = __fma_rn(fh, dy, by);
+                        bz = __fma_rn(fh, dz, bz);
+                    }
                 }
             }
-            if (si < n) {
-                const uint32_t i = first + si;
-                if (!NEAR) {
-                    ((double *)a.as[0])[i] = P.G * ax;
-                    ((double *)a.as[1])[i] = P.G * ay;
-                    ((double *)a.as[2])[i] = P.G * az;
+            for (int o = lpc; o < 32; o <<= 1) {
+                if (SOFT) {
+                    ax += __shfl_xor_sync(0xffffffffu, ax, o);
+                    ay += __shfl_xor_sync(0xffffffffu, ay, o);
+                    az += __shfl_xor_sync(0xffffffffu, az, o);
+                }
+                if (HARD) {
+                    bx += __shfl_xor_sync(0xffffffffu, bx, o);
+                    by += __shfl_xor_sync(0xffffffffu, by, o);
+                    bz += __shfl_xor_sync(0xffffffffu, bz, o);
+                }
+            }
+            if (r0 != slice * F64_SINKS) __syncthreads();   // the last round's sums are read
+            if (copy == 0) {
+                double *o = part[w][slot];
+                if (SOFT) {
+                    o[0] = ax;
+                    o[1] = ay;
+                    o[2] = az;
+                }
+                if (HARD) {
+                    o[NS - 3] = bx;
+                    o[NS - 2] = by;
+                    o[NS - 1] = bz;
+                }
+            }
+            __syncthreads();
+            if (threadIdx.x < rem * NS) {
+                const int k = threadIdx.x / NS, d = threadIdx.x - k * NS;
+                double v = part[0][k][d];
+                for (int u = 1; u < F64_WARPS; ++u) v += part[u][k][d];
+                v *= P.G;
+                const uint32_t i = first + r0 + k;
+                if (SOFT && d < 3) {
+                    double *o = (double *)a.as[d];
+                    o[i] = NEAR ? o[i] + v : v;   // near: the far kernel ran first on the same stream
                 } else {
-                    if (a.want_soft) {   // the far kernel ran first on the same stream
-                        ((double *)a.as[0])[i] += P.G * ax;
-                        ((double *)a.as[1])[i] += P.G * ay;
-                        ((double *)a.as[2])[i] += P.G * az;
-                    }
-                    if (a.want_hard) {
-                        ((double *)a.ah[0])[i] = P.G * bx;
-                        ((double *)a.ah[1])[i] = P.G * by;
-                        ((double *)a.ah[2])[i] = P.G * bz;
-                    }
+                    ((double *)a.ah[HARD && SOFT ? d - 3 : d])[i] = v;
                 }
             }
         }
     }
-    if (lane == 0) atomicAdd(NEAR ? a.inter_hard : a.inter_soft, inter);
+    if (threadIdx.x == 0) atomicAdd(NEAR ? a.inter_hard : a.inter_soft, inter);
 }
 
 void fill_args(hybrid_ctx *c, PairArgs &a)
@@ -900,8 +953,14 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
     cudaEvent_t e0 = nullptr;
     prof_begin(c, kind, &e0);
     if (c->p.precision == 0) {
-        if (near) k_pair_f64<true><<<c->nsm * 12, PAIR_THREADS, 0, c->st>>>(a);
-        else k_pair_f64<false><<<c->nsm * 12, PAIR_THREADS, 0, c->st>>>(a);
+        // a unit for each slice of F64_SINKS sinks a group of n_crit can have (32 slices at most: larger groups take
+        // rounds); units past a group's size are passed over
+        const int slices = std::min(32, (c->p.n_crit + F64_SINKS - 1) / F64_SINKS);
+        const int grid = c->nsm * 16;
+        if (!near) k_pair_f64<false, true, false><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
+        else if (a.want_soft && a.want_hard) k_pair_f64<true, true, true><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
+        else if (a.want_soft) k_pair_f64<true, true, false><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
+        else k_pair_f64<true, false, true><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
         c->launches++;
     } else {
         // work items written by the one-pass walk: far ones in wmap, near ones in wnear

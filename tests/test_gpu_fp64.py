@@ -1,0 +1,105 @@
+"""The plain FP64 pair kernel and the energy sums at the edges of their work splits, against the oracle.
+
+Forces within 1e-12 of the sum of term magnitudes (as for every FP64 force); energies within 1e-13 of the oracle's
+(n <= 4000 terms per sum, each within a few 2^-53, against a plain sum).
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1406_6158_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def H():
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1406_6158_gb300 import build, hybrid
+    build.build()
+    hybrid.load()
+    return hybrid
+
+
+def state(n, same=0):
+    st = ics.plummer(n, 31 + n)
+    for k in ("x", "y", "z"):
+        st[k][:same] = 0.25
+    return st
+
+
+# slices of 8 sinks: groups below, at and above one slice, ragged last slices of every size, groups above
+# 32 slices (the cap: rounds), and a leaf of coincident particles larger than n_crit with and without softening
+@pytest.mark.parametrize("n,n_crit,same,eps", [(1, 64, 0, 0.01), (2, 1, 0, 0.01), (700, 1, 0, 0.01), (700, 8, 0, 0.01),
+                                               (701, 9, 0, 0.01), (1500, 64, 0, 0.01), (1500, 300, 0, 0.01),
+                                               (900, 16, 333, 0.01), (900, 16, 333, 0.0)])
+def test_fp64_forces_at_the_splits_edges(H, n, n_crit, same, eps):
+    st = state(n, same)
+    P = H.Params(eps=eps, theta=0.6, R1=0.04, R2=0.08, precision=0, n_crit=n_crit, n_leaf=min(16, n_crit))
+    ctx, s = H.Context(P), H.System(st, precision=0)
+    ctx.hybrid_build_tree(s)
+    ctx.hybrid_hard_force(s)
+    ctx.hybrid_soft_force(s)
+    out = s.numpy()
+    T = oracle.Tree(out["x"], out["y"], out["z"], out["m"],
+                    oracle.Params(eps=eps, theta=0.6, R1=0.04, R2=0.08, n_crit=n_crit, n_leaf=min(16, n_crit)))
+    a_s, a_h, sc_s, sc_h = T.forces()
+    # without softening the oracle has no value (0 / 0) for the coincident particles
+    ok = np.isfinite(sc_s) & np.isfinite(sc_h)
+    assert np.sum(~ok) == (same if eps == 0.0 else 0)
+    floor = 1e-24 * np.max(sc_s[ok])   # a pair at r = R2 to the last bit: K ~ 1e-90 or 0
+
+    def check(o):
+        for d, k in enumerate("xyz"):
+            assert np.all(np.abs(o["a%s_s" % k] - a_s[:, d])[ok] <= 1e-12 * sc_s[ok] + floor)
+            assert np.all(np.abs(o["a%s_h" % k] - a_h[:, d])[ok] <= 1e-12 * sc_h[ok] + floor)
+    check(out)
+    # both forces in one launch (a step's first forces): the combined walk lists the same entries in another order
+    s2, ctx2 = H.System(st, precision=0), H.Context(P)
+    ctx2.hybrid_step(s2, 0)
+    check(s2.numpy())
+
+
+@pytest.mark.parametrize("scale", [-328, -300, 300, 330])
+def test_fp64_forces_scale_with_the_lengths(H, scale):
+    # lengths times 2^scale: forces times 2^(-2 scale) (inside the seed's range, 2^-640 < r^2 < 2^640, bit for
+    # bit; beyond it the fallback's roundings differ, a few 2^-53 per term)
+    f = 2.0 ** scale
+    st = state(800)
+    res = []
+    for g in (1.0, f):
+        P = H.Params(eps=0.01 * g, theta=0.6, R1=0.04 * g, R2=0.08 * g, precision=0)
+        s = H.System(dict(st, x=st["x"] * g, y=st["y"] * g, z=st["z"] * g), precision=0)
+        ctx = H.Context(P)
+        ctx.hybrid_build_tree(s)
+        ctx.hybrid_soft_force(s)
+        ctx.hybrid_hard_force(s)
+        res.append((s.acc("s").cpu().numpy() * g * g, s.acc("h").cpu().numpy() * g * g))
+    for a, b in zip(*res):
+        assert np.all(np.isfinite(a)) and np.all(np.isfinite(b)) and np.any(b != 0.0)
+        tol = 0.0 if abs(scale) <= 300 else 1e-13 * np.max(np.abs(a))
+        assert np.max(np.abs(a - b)) <= tol
+
+
+@pytest.mark.parametrize("n", [1, 2, 63, 64, 65, 255, 256, 257, 320, 1023, 4000])
+def test_energy_at_the_tiles_edges(H, n):
+    st = state(n)
+    T0, W0 = oracle.energy(*[st[k] for k in ("x", "y", "z", "vx", "vy", "vz", "m")], G=0.7, eps=0.02)
+    ctx, s = H.Context(H.Params(G=0.7, eps=0.02)), H.System(st, precision=1)
+    T, W = ctx.hybrid_energy(s)
+    Tn, Wn = H.hybrid_energy_noalloc(*[s.t[k] for k in H.System.FIELDS], 0.7, 0.02)
+    for a, b in ((T, T0), (W, W0), (Tn, T0), (Wn, W0)):
+        assert abs(a - b) <= 1e-13 * abs(b)
+    assert (T, W) == ctx.hybrid_energy(s)
+
+
+def test_energy_beyond_the_seeds_range(H):
+    st = state(300)
+    W0 = H.Context(H.Params(eps=0.0)).hybrid_energy(H.System(st))[1]
+    for scale in (-460, 460):   # r^2 ~ 2^(2 scale): sqrt and division
+        f = 2.0 ** scale
+        s = H.System(dict(st, x=st["x"] * f, y=st["y"] * f, z=st["z"] * f))
+        W = H.Context(H.Params(eps=0.0)).hybrid_energy(s)[1]
+        assert abs(W * f - W0) <= 1e-13 * abs(W0)
