@@ -285,7 +285,9 @@ void launch_kick_seq(hybrid_ctx *c, int n, const int *which, const int *mode, co
                      double dval, bool resplit = false);
 void launch_kick_ext(hybrid_ctx *c, const hybrid_system *s, int which, double h);
 void launch_drift_ext(hybrid_ctx *c, const hybrid_system *s, double dt);
-void launch_energy(hybrid_ctx *c, double *d_out /* 2*S */);
+// kinetic and potential energy of a single system's working state to d_out[0..1]; d_out holds energy_scratch_bytes
+void launch_energy(hybrid_ctx *c, double *d_out);
+size_t energy_scratch_bytes(int nsm);
 
 }  // namespace hy
 

@@ -221,7 +221,7 @@ bool reserve(hybrid_ctx *c)
         ok = ok && ensure(c, c->off_dev, (s + 1) * 8) && ensure(c, c->sp_dev, s * sizeof(SysParams));
         ok = ok && ensure(c, c->boxmin, s * 24) && ensure(c, c->boxmax, s * 24) && ensure(c, c->box, s * sizeof(SysBox));
         ok = ok && ensure(c, c->sysroot, s * 4) && ensure(c, c->io_dev, s * sizeof(SysIO));
-        ok = ok && ensure(c, c->energy_dev, s * 16);
+        ok = ok && ensure(c, c->energy_dev, energy_scratch_bytes(c->nsm));
         if (ok) c->capS = S;
     }
     if (c->nchunks > c->capChunks) {

@@ -6,6 +6,8 @@
 // the FP64 path reproduces a plain CPU evaluation of the same sequence.
 #include "hy_internal.cuh"
 
+#include "energy_pairs.cuh"
+
 namespace hy {
 
 namespace {
@@ -187,68 +189,15 @@ __global__ void __launch_bounds__(256) k_drift_ext(int64_t n, double *x, double 
     }
 }
 
-// Softened energies by direct FP64 summation: one thread per sink, sources of
-// the same system staged through shared memory; per-system sums by atomics.
-constexpr int EN_THREADS = 256;
-__global__ void __launch_bounds__(EN_THREADS) k_energy(const Chunk *__restrict__ chunks, int nchunks, int SUB,
-                                                       const int64_t *__restrict__ off, StatePtrs w,
-                                                       const SysParams *__restrict__ sp, double *out)
+// Softened energies of the (single) system in the working state; see energy_pairs.cuh.
+__global__ void __launch_bounds__(EN_ROW) k_energy(EnergyArgs a, double *part)
 {
-    __shared__ double4_32a tile[EN_THREADS];
-    __shared__ double red[2][EN_THREADS / 32];
-    // SUB = sink tiles of EN_THREADS per radix chunk
-    for (int b = blockIdx.x; b < nchunks * SUB; b += gridDim.x) {
-        const Chunk ch = chunks[b / SUB];
-        const int t0 = (b % SUB) * EN_THREADS;
-        if (t0 >= ch.len) continue;
-        const SysParams P = sp[ch.sys];
-        const int64_t s0 = off[ch.sys], s1 = off[ch.sys + 1];
-        {
-            const int t = t0 + threadIdx.x;
-            const bool ok = t < ch.len;
-            const int64_t i = ch.start + (ok ? t : 0);
-            const double xi = w.x[0][i], yi = w.x[1][i], zi = w.x[2][i], mi = w.x[6][i];
-            double W = 0.0;
-            for (int64_t j0 = s0; j0 < s1; j0 += EN_THREADS) {
-                const int64_t j = j0 + threadIdx.x;
-                __syncthreads();
-                if (j < s1) tile[threadIdx.x] = make_double4_32a(w.x[0][j], w.x[1][j], w.x[2][j], w.x[6][j]);
-                __syncthreads();
-                const int nt = (int)min((int64_t)EN_THREADS, s1 - j0);
-                for (int k = 0; k < nt; ++k) {
-                    if (j0 + k == i) continue;
-                    const double4_32a q = tile[k];
-                    const double dx = q.x - xi, dy = q.y - yi, dz = q.z - zi;
-                    W += q.w / sqrt(dx * dx + dy * dy + dz * dz + P.eps2);
-                }
-            }
-            double T = 0.0, Wi = 0.0;
-            if (ok) {
-                const double v0 = w.x[3][i], v1 = w.x[4][i], v2 = w.x[5][i];
-                T = 0.5 * mi * (v0 * v0 + v1 * v1 + v2 * v2);
-                Wi = -0.5 * P.G * mi * W;
-            }
-            for (int o = 16; o > 0; o >>= 1) {
-                T += __shfl_xor_sync(0xffffffffu, T, o);
-                Wi += __shfl_xor_sync(0xffffffffu, Wi, o);
-            }
-            if ((threadIdx.x & 31) == 0) {
-                red[0][threadIdx.x >> 5] = T;
-                red[1][threadIdx.x >> 5] = Wi;
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                double tT = 0.0, tW = 0.0;
-                for (int k = 0; k < EN_THREADS / 32; ++k) {
-                    tT += red[0][k];
-                    tW += red[1][k];
-                }
-                atomicAdd(&out[2 * ch.sys], tT);
-                atomicAdd(&out[2 * ch.sys + 1], tW);
-            }
-            __syncthreads();
-        }
-    }
+    energy_block(a, part + 2 * (int64_t)blockIdx.x);
+}
+
+__global__ void __launch_bounds__(EN_ROW) k_energy_sum(int nb, const double *part, double *out)
+{
+    energy_total(nb, part, out);
 }
 
 StatePtrs state_ptrs(hybrid_ctx *c)
@@ -338,14 +287,21 @@ void launch_drift_ext(hybrid_ctx *c, const hybrid_system *s, double dt)
     c->launches++;
 }
 
+size_t energy_scratch_bytes(int nsm) { return ((size_t)2 * EN_BLOCKS_PER_SM * nsm + 2) * sizeof(double); }
+
 void launch_energy(hybrid_ctx *c, double *d_out)
 {
-    cudaMemsetAsync(d_out, 0, (size_t)2 * c->S * sizeof(double), c->st);
-    const int sub = c->tile / EN_THREADS;
-    k_energy<<<std::min(c->nchunks * sub, c->nsm * 8), EN_THREADS, 0, c->st>>>(
-        (const Chunk *)c->chunks_dev.p, c->nchunks, sub, (const int64_t *)c->off_dev.p, state_ptrs(c),
-        (const SysParams *)c->sp_dev.p, d_out);
-    c->launches++;
+    const int grid = (int)std::min<int64_t>(energy_items(c->N), (int64_t)c->nsm * EN_BLOCKS_PER_SM);
+    EnergyArgs a;
+    a.n = c->N;
+    const double **xs[7] = {&a.x, &a.y, &a.z, &a.vx, &a.vy, &a.vz, &a.m};
+    for (int f = 0; f < 7; ++f) *xs[f] = (const double *)c->x[f].p;
+    a.G = c->h_sp[0].G;
+    a.eps2 = c->h_sp[0].eps2;
+    double *part = d_out + 2;
+    k_energy<<<grid, EN_ROW, 0, c->st>>>(a, part);
+    k_energy_sum<<<1, EN_ROW, 0, c->st>>>(grid, part, d_out);
+    c->launches += 2;
 }
 
 }  // namespace hy
