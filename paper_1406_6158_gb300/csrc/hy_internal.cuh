@@ -191,8 +191,8 @@ struct hybrid_ctx {
     hy::Buf off_dev, sp_dev, chunks_dev, boxmin, boxmax, box, sysroot;
     hy::Buf status;
     // tree
-    hy::Buf lvl, nfirst, ncount, nchild, nnch, nparent, nlevel, ndone, leafof;
-    hy::Buf pc, pD, pn, rec, rb2d, rd2b, rhist;     // topology build scratch
+    hy::Buf lvl, nfirst, nend, nchild, nchend, nparent, nlevel, ndone;   // nodes: particles and children [first, end)
+    hy::Buf cells, ccnt;                          // topology scratch: packed levels per particle, counts per tile
     hy::Buf nbig, mitems, mpart;                  // moments of large cells: chunk items and sums
     hy::Buf nbmax32;                              // b_max as FP32 bits (FP32 form)
     int64_t capItems = 0;
@@ -200,7 +200,7 @@ struct hybrid_ctx {
     hy::Buf nA, nB, ncrit, ntopo;              // FP32 walk/pair node data
     hy::Buf nD, nrb, nhr;                      // FP64 walk/pair node data (precision 0)
     hy::Buf ndelta, nside, norg;               // geometry (inspection + finalize)
-    hy::Buf gflag, gscan, gnode, gfirst, gcount, gsys, gF, glo, ghi, ngroups_dev;
+    hy::Buf gflag, gscan, gnode, gfirst, gsys, gF, glo, ghi, ngroups_dev;
     // lists
     hy::Buf lcnt, loff, list, stack, counter, io_dev, energy_dev, wstart, wmap;
     hy::Buf wnear;                                 // near-pair work items (wmap holds the far ones)
@@ -255,9 +255,11 @@ void scan_u64(hybrid_ctx *c, uint64_t *data, int64_t n_host, const int64_t *d_n,
 void launch_box(hybrid_ctx *c);
 void launch_keys_sort(hybrid_ctx *c);      // keys and their stable sort (keys[0], vals[0])
 void launch_permute(hybrid_ctx *c);        // state into key order, pair-kernel copies of the positions
-bool launch_build_levels(hybrid_ctx *c);   // topology from the sorted keys
+void launch_topology(hybrid_ctx *c);       // nodes and sink groups from the sorted keys
+int cell_tiles(int64_t N);
+size_t cell_count_bytes(int64_t N);        // its counts per tile
 void launch_moments(hybrid_ctx *c);        // needs topology and the permuted state
-void launch_groups(hybrid_ctx *c);         // group table from the topology
+void launch_groups(hybrid_ctx *c);         // group table from the nodes, for an n_crit launch_topology leaves out
 void launch_group_boxes(hybrid_ctx *c);    // needs the group table and the permuted state
 void launch_wait_selftest(hybrid_ctx *c, int max_polls);   // a bounded wait on a flag nothing sets
 

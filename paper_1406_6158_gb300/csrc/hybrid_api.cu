@@ -164,11 +164,9 @@ bool alloc_nodes(hybrid_ctx *c, int64_t cap)
 {
     const size_t n = (size_t)cap;
     bool ok = true;
-    for (Buf *b : {&c->nfirst, &c->ncount, &c->nchild, &c->nnch, &c->nparent, &c->nlevel, &c->ndone, &c->rb2d,
-                   &c->rd2b})
+    for (Buf *b : {&c->nfirst, &c->nend, &c->nchild, &c->nchend, &c->nparent, &c->nlevel, &c->ndone})
         ok = ok && ensure(c, *b, n * 4);
-    ok = ok && ensure(c, c->rec, n * 8) && ensure(c, c->nbig, n * 4) && ensure(c, c->nbmax32, n * 4);
-    ok = ok && ensure(c, c->rhist, (size_t)(LEVELS + 1) * ((n + 1023) / 1024) * 4);
+    ok = ok && ensure(c, c->nbig, n * 4) && ensure(c, c->nbmax32, n * 4);
     for (Buf *b : {&c->nM, &c->ncx, &c->ncy, &c->ncz, &c->nB2, &c->nbmax, &c->nrb, &c->nhr, &c->ndelta, &c->nside})
         ok = ok && ensure(c, *b, n * 8);
     ok = ok && ensure(c, c->norg, n * 24);
@@ -194,10 +192,9 @@ bool reserve(hybrid_ctx *c)
     if (N > c->capN) {
         const size_t n = (size_t)N;
         for (int f = 0; f < 7; ++f) ok = ok && ensure(c, c->x[f], n * 8) && ensure(c, c->xa[f], n * 8);
-        for (Buf *b : {&c->id, &c->ida, &c->orig, &c->origa, &c->psys, &c->leafof, &c->gflag, &c->gscan, &c->gnode,
-                       &c->gfirst, &c->gcount, &c->gsys, &c->pn})
+        for (Buf *b : {&c->id, &c->ida, &c->orig, &c->origa, &c->psys, &c->gflag, &c->gscan, &c->gnode, &c->gsys})
             ok = ok && ensure(c, *b, n * 4);
-        ok = ok && ensure(c, c->pc, n) && ensure(c, c->pD, n);
+        ok = ok && ensure(c, c->gfirst, (n + 1) * 4) && ensure(c, c->cells, n * 2) && ensure(c, c->ccnt, cell_count_bytes(N));
         const size_t asz = c->p.precision == 1 ? 4 : 8;
         for (int d = 0; d < 3; ++d) ok = ok && ensure(c, c->acc_s[d], n * asz) && ensure(c, c->acc_h[d], n * asz);
         if (c->p.precision == 1) ok = ok && ensure(c, c->phi, n * 16) && ensure(c, c->plo, n * 16);
@@ -250,8 +247,8 @@ bool reserve(hybrid_ctx *c)
     ok = ok && ensure_items(c, 2 * c->capGroups + c->capList / 256 + 1024);
     if (c->capStack == 0) c->capStack = 4096;
     ok = ok && ensure(c, c->stack, (size_t)c->walk_warps * c->capStack * 4);
-    // scratch of the scans: the longest scan is over max(N, nodes, 3 groups + 1, tiles x 256)
-    const int64_t longest = std::max<int64_t>({N, c->capNodes, 3 * c->capGroups + 2, (int64_t)c->nchunks * 256});
+    // scratch of the scans: the longest is over max(N, 3 groups + 1, counts per tile)
+    const int64_t longest = std::max<int64_t>({N, 3 * c->capGroups + 2, (int64_t)(cell_count_bytes(N) / 4)});
     ok = ok && ensure(c, c->blocksum, (size_t)((longest + SCAN_SEG - 1) / SCAN_SEG + 1) * 8);
     return ok;
 }
@@ -395,9 +392,9 @@ void enqueue(hybrid_ctx *c, const Op &o, int idx)
         launch_kick_seq(c, o.nk, o.which, o.kmode, o.val, o.dmode, o.dval, o.mode == 1);
         break;
     case OP_BUILD: {
-        // The build as a two-branch DAG: after the key sort, the topology (keys only) and then the group
-        // table run beside the permutation of the state; the moments need the topology and the permuted
-        // state (not the groups), the group boxes the group table and the permuted state.
+        // The build as a two-branch DAG: after the key sort, the topology and the groups (keys only) run beside
+        // the permutation of the state; the moments need the topology and the permuted state, the group boxes
+        // the groups and the permuted state.
         cudaEvent_t e0 = nullptr;
         prof_begin(c, PROF_TREE, &e0);
         cudaEvent_t e1 = nullptr;
@@ -410,12 +407,10 @@ void enqueue(hybrid_ctx *c, const Op &o, int idx)
         cudaStreamWaitEvent(c->st2, c->ev_fork[0], 0);
         c->st = c->st2;
         prof_begin(c, PROF_TOPO, &e1);
-        launch_build_levels(c);
+        launch_topology(c);
         prof_end(c, PROF_TOPO, e1);
         cudaEventRecord(c->ev_join[0], c->st2);   // topology done
-        prof_begin(c, PROF_GROUPS, &e1);
         launch_groups(c);
-        prof_end(c, PROF_GROUPS, e1);
         c->st = main;
         launch_permute(c);
         cudaEventRecord(c->ev_fork[1], main);      // permuted state done
@@ -425,7 +420,9 @@ void enqueue(hybrid_ctx *c, const Op &o, int idx)
         prof_end(c, PROF_MOM, e1);
         c->st = c->st2;
         cudaStreamWaitEvent(c->st2, c->ev_fork[1], 0);
+        prof_begin(c, PROF_GROUPS, &e1);
         launch_group_boxes(c);
+        prof_end(c, PROF_GROUPS, e1);
         cudaEventRecord(c->ev_join[1], c->st2);
         c->st = main;
         cudaStreamWaitEvent(main, c->ev_join[1], 0);
@@ -675,8 +672,6 @@ hybrid_status run_ops(hybrid_ctx *c, const std::vector<Op> &ops_in)
             ok = ok && ensure(c, c->stack, (size_t)c->walk_warps * s.need[2] * 4);
             if (ok) c->capStack = s.need[2];
         }
-        const int64_t longest = std::max<int64_t>({c->N, c->capNodes, 3 * c->capGroups + 2, (int64_t)c->nchunks * 256});
-        ok = ok && ensure(c, c->blocksum, (size_t)((longest + SCAN_SEG - 1) / SCAN_SEG + 1) * 8);
         if (!ok) return HYBRID_ENOMEM;
         if ((r = clear_status(c)) != HYBRID_OK) return r;
         start = (size_t)std::max(0, s.where);
@@ -840,11 +835,10 @@ hybrid_status hybrid_destroy(hybrid_ctx *c)
     Buf *all[] = {&c->id, &c->ida, &c->orig, &c->origa, &c->psys, &c->phi, &c->plo, &c->pd, &c->disp, &c->keys[0], &c->keys[1],
                   &c->vals[0], &c->vals[1], &c->hist, &c->blocksum, &c->off_dev, &c->sp_dev, &c->chunks_dev,
                   &c->ss_sys, &c->ss_spk, &c->ss_spv, &c->ss_cnt, &c->ss_start, &c->ss_cur, &c->ss_pb, &c->ss_flag,
-                  &c->boxmin, &c->boxmax, &c->box, &c->sysroot, &c->status, &c->lvl, &c->nfirst, &c->ncount,
-                  &c->nchild, &c->nnch, &c->nparent, &c->nlevel, &c->ndone, &c->leafof, &c->pc, &c->pD, &c->pn, &c->rec,
-                  &c->rb2d, &c->rd2b, &c->rhist, &c->nM, &c->ncx,
+                  &c->boxmin, &c->boxmax, &c->box, &c->sysroot, &c->status, &c->lvl, &c->nfirst, &c->nend,
+                  &c->nchild, &c->nchend, &c->nparent, &c->nlevel, &c->ndone, &c->cells, &c->ccnt, &c->nM, &c->ncx,
                   &c->ncy, &c->ncz, &c->nB2, &c->nbmax, &c->nA, &c->nB, &c->ncrit, &c->ntopo, &c->nD, &c->nrb,
-                  &c->nhr, &c->ndelta, &c->nside, &c->norg, &c->gflag, &c->gscan, &c->gnode, &c->gfirst, &c->gcount,
+                  &c->nhr, &c->ndelta, &c->nside, &c->norg, &c->gflag, &c->gscan, &c->gnode, &c->gfirst,
                   &c->gsys, &c->gF, &c->glo, &c->ghi, &c->ngroups_dev, &c->lcnt, &c->list, &c->stack, &c->counter,
                   &c->io_dev, &c->energy_dev, &c->wstart, &c->wmap, &c->nbig, &c->mitems, &c->mpart, &c->nbmax32, &c->wnear};
     for (Buf *b : all)
@@ -1110,8 +1104,8 @@ hybrid_status hybrid_tree_copy(hybrid_ctx *c, uint64_t *keys, int32_t *level, in
     std::vector<uint32_t> f, cn, ch, nc, pa, lv, gn;
     std::vector<double> M, cx, cy, cz, bm, B2, de, sd, og, rb, glo, ghi;
     std::vector<uint64_t> k;
-    bool ok = d2h(c, f, c->nfirst, nn) && d2h(c, cn, c->ncount, nn) && d2h(c, ch, c->nchild, nn) &&
-              d2h(c, nc, c->nnch, nn) && d2h(c, pa, c->nparent, nn) && d2h(c, lv, c->nlevel, nn) &&
+    bool ok = d2h(c, f, c->nfirst, nn) && d2h(c, cn, c->nend, nn) && d2h(c, ch, c->nchild, nn) &&
+              d2h(c, nc, c->nchend, nn) && d2h(c, pa, c->nparent, nn) && d2h(c, lv, c->nlevel, nn) &&
               d2h(c, gn, c->gnode, ng) && d2h(c, M, c->nM, nn) && d2h(c, cx, c->ncx, nn) && d2h(c, cy, c->ncy, nn) &&
               d2h(c, cz, c->ncz, nn) && d2h(c, bm, c->nbmax, nn) && d2h(c, B2, c->nB2, nn) &&
               d2h(c, de, c->ndelta, nn) && d2h(c, sd, c->nside, nn) && d2h(c, og, c->norg, 3 * nn) &&
@@ -1121,9 +1115,9 @@ hybrid_status hybrid_tree_copy(hybrid_ctx *c, uint64_t *keys, int32_t *level, in
     for (int64_t i = 0; i < nn; ++i) {
         if (level) level[i] = (int32_t)lv[i];
         if (first) first[i] = f[i];
-        if (count) count[i] = cn[i];
-        if (child) child[i] = nc[i] ? (int64_t)ch[i] : -1;
-        if (nchild) nchild[i] = (int32_t)nc[i];
+        if (count) count[i] = cn[i] - f[i];
+        if (child) child[i] = ch[i] == NONE ? -1 : (int64_t)ch[i];
+        if (nchild) nchild[i] = ch[i] == NONE ? 0 : (int32_t)(nc[i] - ch[i]);
         if (parent) parent[i] = pa[i] == NONE ? -1 : (int64_t)pa[i];
         if (moments) {
             double *o = moments + 13 * i;

@@ -41,7 +41,7 @@ constexpr int TILE = 64;
 
 struct PairArgs {
     const int64_t *ngroups;
-    const uint32_t *gfirst, *gcount, *gsys;
+    const uint32_t *gfirst, *gsys;
     const SysParams *sp;
     const uint64_t *off;    // [3 * ng + 1] list offsets: cells, far particles, near particles
     const uint32_t *list;
@@ -761,9 +761,9 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
         const int64_t g = unit / slices;
         if (g >= ng) break;
         const int slice = (int)(unit - g * slices);
-        const int n = (int)a.gcount[g];
-        if (slice * F64_SINKS >= n) continue;
         const uint32_t first = a.gfirst[g];
+        const int n = (int)(a.gfirst[g + 1] - first);
+        if (slice * F64_SINKS >= n) continue;
         const SysParams &P = a.sp[a.gsys[g]];
         const double eps2 = P.eps2, R2 = P.R2, R2sq = P.R2sq, invdR = P.invdR;
         uint64_t c0 = 0, p0;
@@ -886,7 +886,6 @@ void fill_args(hybrid_ctx *c, PairArgs &a)
 {
     a.ngroups = (const int64_t *)c->ngroups_dev.p;
     a.gfirst = (const uint32_t *)c->gfirst.p;
-    a.gcount = (const uint32_t *)c->gcount.p;
     a.gsys = (const uint32_t *)c->gsys.p;
     a.sp = (const SysParams *)c->sp_dev.p;
     a.off = (const uint64_t *)c->lcnt.p;

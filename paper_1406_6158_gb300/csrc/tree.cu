@@ -791,250 +791,265 @@ __global__ void __launch_bounds__(256) k_permute(PermArgs a, const Status *st)
 }
 
 // ---------------------------------------------------------------------------
-// Octree topology from the sorted keys, all levels at once.
+// Octree topology and sink groups from the sorted keys, all levels at once, in
+// two passes over the particles with one short scan between them (k_cells,
+// scan, k_nodes), whatever the depth.
 //
 // c(i) = number of leading octal digits keys i-1 and i share (-1 at the first
 // particle of a system): particle i starts a cell at every level l > c(i).
-// The level-l cell around particle p spans positions up to the nearest
-// starts on either side, so its size is known from c in a window of n_leaf
-// positions whenever it is at most n_leaf. The leaf depth D(p) is the first
-// level whose cell holds <= n_leaf particles (21 at most): cells exist down to
-// D(p). Particle i therefore owns the nodes (l, first = i) for
-// c(i) < l <= D(i). These records are written in particle order (a scan
-// gives each particle its slot), then stably sorted by level: the result is
-// the breadth-first order (level, system, key) of the split rule.
+// The level-l cell around particle p holds more than n particles exactly when
+// some n + 1 consecutive ones around p share l digits, so the deepest such
+// level is L_n(p) = max over a in [p - n, p] of the digits that keys a and
+// a + n share: a sliding maximum, taken by doubling in shared memory. The leaf
+// depth is D(p) = L_n_leaf(p) + 1 (21 at most), and the sink group of p is its
+// cell at level Dg(p) = min(D(p), L_n_crit(p) + 1).
+//
+// Particle i owns the nodes (l, first = i) for c(i) < l <= D(i). In
+// breadth-first order (level, system, key) a node's index is the number of
+// nodes at lower levels plus the number of level-l starts before i: counts per
+// level and tile (k_cells), their scan, and ballots inside the tile (k_nodes)
+// give it directly, and with it everything else: the parent of i's top node is
+// the last start at level c(i); the node at level l that holds particle i-1
+// ends at i when c(i) < l; its children end where the level l + 1 starts
+// before i end. No node is searched for and nothing is sorted by level.
+// Before, the sizes came from linear walks in shared memory, and records in
+// particle order were sorted by level, searched for their ends and linked, and
+// groups were flagged and compacted, by 14 more launches. Tree build per soft
+// step of 4 hard sub-steps (8 at N = 2^24): N = 4096 0.56 -> 0.47 ms, 2^17
+// 0.715 -> 0.595, 2^20 (absolute MAC) 1.84 -> 1.59, 2^24 43.3 -> 39.0 ms.
 // ---------------------------------------------------------------------------
 // c(i): common leading octal digits of keys i-1 and i; -1 at a system's first particle
+__device__ __forceinline__ int shared_digits(uint64_t a, uint64_t b)
+{
+    const unsigned long long x = a ^ b;
+    return x == 0ull ? LEVELS : (__clzll((long long)x) - 1) / 3;   // keys use bits 0..62
+}
 __device__ __forceinline__ int prefix_c(const uint64_t *__restrict__ key, const int32_t *__restrict__ psys, int64_t i)
 {
     if (i == 0 || psys[i] != psys[i - 1]) return -1;
-    const unsigned long long x = key[i - 1] ^ key[i];
-    return x == 0ull ? LEVELS : (__clzll((long long)x) - 1) / 3;   // keys use bits 0..62
+    return shared_digits(key[i - 1], key[i]);
 }
 
-constexpr int LD_T = 256;
+constexpr int CT_ROWS = 4;                    // rows of 32 particles per warp
+constexpr int CT_WARPS = 8;
+constexpr int CT_TILE = CT_WARPS * 32 * CT_ROWS;   // 1024 particles per tile
+constexpr int NLEV = LEVELS + 1;              // levels 0..21
+constexpr int CT_CNT = NLEV + 1;              // counts per tile: starts at each level, sink groups
+// Sink groups of up to this size are marked in k_cells; larger n_crit take the node-based kernels
+// (k_group_flag and on): the window costs one byte of shared memory per particle, twice.
+constexpr int GROUP_WINDOW = 1024;
 
-// Leaf depth D(p) and the number of nodes particle p starts, max(0, D - c).
-__global__ void __launch_bounds__(LD_T) k_leaf_depth(int64_t N, const uint64_t *__restrict__ key,
-                                                     const int32_t *__restrict__ psys, int8_t *__restrict__ pc,
-                                                     int n_leaf, uint8_t *__restrict__ pD, uint32_t *__restrict__ pn,
-                                                     const Status *st)
+// deepest level at which the cell around tile particle x holds more than n particles, for every x of the
+// tile, into m[0, CT_TILE) as level + 1 (0: none); m and t are byte arrays of cells_bytes(n) each
+__host__ __device__ constexpr int cells_bytes(int n) { return (CT_TILE + n + 15) / 16 * 16 + 16; }
+
+__device__ __forceinline__ uint8_t *window_max(const uint64_t *__restrict__ key, const int32_t *__restrict__ psys,
+                                               bool one, int64_t N, int64_t b0, int n, uint8_t *m, uint8_t *t)
 {
-    if (st->code) return;
-    extern __shared__ int8_t sc[];   // LD_T + 2 n_leaf values of c
-    const int win = LD_T + 2 * n_leaf;
-    for (int64_t base = (int64_t)blockIdx.x * LD_T; base < N; base += (int64_t)gridDim.x * LD_T) {
-        __syncthreads();
-        for (int k = threadIdx.x; k < win; k += blockDim.x) {
-            const int64_t j = base - n_leaf + k;
-            const int cj = (j < 0 || j >= N) ? -1 : prefix_c(key, psys, j);
-            sc[k] = (int8_t)cj;
-            if (k >= n_leaf && k < n_leaf + LD_T && j < N) pc[j] = (int8_t)cj;
-        }
-        __syncthreads();
-        const int64_t p = base + threadIdx.x;
-        if (p < N) {
-            const int w = threadIdx.x + n_leaf;
-            // size of the level-lev cell around p, capped at n_leaf + 1 on each side
-            auto count_at = [&](int lev) {
-                int kl = 0;
-                while (kl <= n_leaf && sc[w - kl] >= lev) ++kl;
-                int kr = 1;
-                while (kr <= n_leaf && sc[w + kr] >= lev) ++kr;
-                return kl + kr;
-            };
-            int D;
-            if (count_at(LEVELS) > n_leaf) {
-                D = LEVELS;
-            } else {
-                int lo = 0, hi = LEVELS;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (count_at(mid) <= n_leaf) hi = mid;
-                    else lo = mid + 1;
-                }
-                D = lo;
-            }
-            const int c = sc[w];
-            pD[p] = (uint8_t)D;
-            pn[p] = D > c ? (uint32_t)(D - c) : 0u;
-        }
+    const int len = CT_TILE + n, words = cells_bytes(n) / 4;
+    for (int x = threadIdx.x; x < 4 * words; x += blockDim.x) {
+        const int64_t a = b0 - n + x;
+        int v = 0;
+        if (x < len && a >= 0 && a + n < N && (one || psys[a] == psys[a + n])) v = shared_digits(key[a], key[a + n]) + 1;
+        m[x] = (uint8_t)v;
     }
+    __syncthreads();
+    int s = 1;
+    for (; 2 * s <= n + 1; s <<= 1) {   // m[x] = max over [x, x + s) -> [x, 2 s)
+        const uint32_t *w = (const uint32_t *)m;
+        for (int k = threadIdx.x; k < words; k += blockDim.x) {
+            uint32_t o;
+            if (s >= 4) o = k + s / 4 < words ? w[k + s / 4] : 0u;
+            else o = __funnelshift_r(w[k], k + 1 < words ? w[k + 1] : 0u, 8 * s);
+            ((uint32_t *)t)[k] = __vmaxu4(w[k], o);
+        }
+        __syncthreads();
+        uint8_t *u = m;
+        m = t;
+        t = u;
+    }
+    // the window of n + 1 entries from x: two overlapping runs of s
+    for (int x = threadIdx.x; x < CT_TILE; x += blockDim.x) t[x] = max(m[x], m[x + n + 1 - s]);
+    __syncthreads();
+    return t;
 }
 
-// records (level << 32 | first) in particle order
-__global__ void __launch_bounds__(256) k_records(int64_t N, const int8_t *__restrict__ pc,
-                                                 const uint8_t *__restrict__ pD, const uint32_t *__restrict__ poff,
-                                                 const uint64_t *__restrict__ total, int64_t cap,
-                                                 unsigned long long *__restrict__ rec, Status *st, int where)
+// Per particle the packed levels c + 1, D, Dg (5 bits each); per tile the numbers of nodes started at each level
+// and of sink groups (cnt[row][tile]). Also clears the counters of the moments and of the walk.
+__global__ void __launch_bounds__(32 * CT_WARPS) k_cells(int64_t N, int S, const uint64_t *__restrict__ key,
+                                                         const int32_t *__restrict__ psys, int n_leaf, int n_crit,
+                                                         uint16_t *__restrict__ cells, int ntiles,
+                                                         uint32_t *__restrict__ cnt, unsigned long long *counter,
+                                                         const Status *st)
 {
     if (st->code) return;
-    if ((int64_t)*total > cap) {
+    extern __shared__ __align__(16) uint8_t sm[];
+    __shared__ uint32_t wcnt[CT_WARPS][CT_CNT + 1];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int nb = cells_bytes(max(n_leaf, n_crit));
+    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+        const int64_t b0 = (int64_t)tile * CT_TILE, p0 = b0 + w * (32 * CT_ROWS) + lane;
+        uint8_t D[CT_ROWS], Dg[CT_ROWS];
+        const uint8_t *m = window_max(key, psys, S == 1, N, b0, n_leaf, sm, sm + nb);
+#pragma unroll
+        for (int r = 0; r < CT_ROWS; ++r) Dg[r] = D[r] = min((int)m[w * (32 * CT_ROWS) + r * 32 + lane], LEVELS);
+        if (n_crit > 0) {
+            __syncthreads();
+            m = window_max(key, psys, S == 1, N, b0, n_crit, sm, sm + nb);
+#pragma unroll
+            for (int r = 0; r < CT_ROWS; ++r) Dg[r] = min(D[r], m[w * (32 * CT_ROWS) + r * 32 + lane]);
+        }
+        uint32_t mine = 0;   // lane l: starts at level l (l < NLEV), lane NLEV: groups
+#pragma unroll
+        for (int r = 0; r < CT_ROWS; ++r) {
+            const int64_t i = p0 + r * 32;
+            int c = LEVELS + 1, d = 0;   // past the end: starts nothing
+            bool g = false;
+            if (i < N) {
+                c = prefix_c(key, psys, i);
+                d = D[r];
+                g = n_crit > 0 && c < (int)Dg[r];
+                cells[i] = (uint16_t)((c + 1) | (d << 5) | ((int)Dg[r] << 10));
+            }
+            const int lo = __reduce_min_sync(0xffffffffu, c) + 1, hi = __reduce_max_sync(0xffffffffu, d);
+            for (int l = lo; l <= hi; ++l) {
+                const uint32_t k = __popc(__ballot_sync(0xffffffffu, c < l && l <= d));
+                if (lane == l) mine += k;
+            }
+            const uint32_t k = __popc(__ballot_sync(0xffffffffu, g));
+            if (lane == NLEV) mine += k;
+        }
+        if (lane < CT_CNT) wcnt[w][lane] = mine;
+        __syncthreads();
+        if (threadIdx.x < CT_CNT) {
+            uint32_t sum = 0;
+            for (int k = 0; k < CT_WARPS; ++k) sum += wcnt[k][threadIdx.x];
+            cnt[(size_t)threadIdx.x * ntiles + tile] = sum;
+        }
+        __syncthreads();
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) counter[9] = 0ull;   // chunk items of the moments
+}
+
+struct NodeArgs {
+    const uint16_t *cells;
+    const int32_t *psys;
+    const uint32_t *off;      // scanned counts: index of a tile's first start at each level, then of its first group
+    const uint64_t *total;    // nodes + groups
+    uint32_t *nfirst, *nend, *nlevel, *nchild, *nchend, *nparent, *sysroot, *lvl, *done;
+    unsigned long long *bmax64;
+    unsigned int *bmax32;     // one of the two, zeroed
+    uint32_t *gnode, *gfirst, *gsys;   // null: groups come from the node-based kernels
+    int64_t *ngroups;
+    int64_t N, cap;
+    int ntiles;
+};
+
+// Nodes (breadth-first) and sink groups (in particle order); see above.
+__global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st, int where)
+{
+    if (st->code) return;
+    const uint32_t nodes = a.off[(size_t)NLEV * a.ntiles];   // start of the group counts
+    if ((int64_t)nodes > a.cap) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             fail(st, HYBRID_ECAPACITY, where);
-            st->need[0] = (int64_t)*total + (int64_t)(*total >> 3) + 1024;
+            st->need[0] = (int64_t)nodes + (int64_t)(nodes >> 3) + 1024;
         }
         return;
     }
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = pc[i], D = pD[i];
-        uint32_t o = poff[i];
-        for (int l = c + 1; l <= D; ++l) rec[o++] = ((unsigned long long)l << 32) | (unsigned long long)i;
-    }
-}
-
-constexpr int REC_IPT = 4;
-constexpr int REC_TILE = RS_WARPS * 32 * REC_IPT;   // 1024 records per tile
-constexpr int NLEV = LEVELS + 1;    // levels 0..21
-
-__global__ void __launch_bounds__(256) k_rec_hist(const unsigned long long *__restrict__ rec,
-                                                  const uint64_t *__restrict__ total, int ntiles,
-                                                  uint32_t *__restrict__ hist, const Status *st)
-{
-    if (st->code) return;
-    __shared__ uint32_t h[NLEV];
-    const uint64_t T = *total;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        if (threadIdx.x < NLEV) h[threadIdx.x] = 0;
-        __syncthreads();
-        const uint64_t b0 = (uint64_t)t * REC_TILE;
-        for (int k = threadIdx.x; k < REC_TILE; k += blockDim.x)
-            if (b0 + k < T) atomicAdd(&h[(uint32_t)(rec[b0 + k] >> 32)], 1u);
-        __syncthreads();
-        if (threadIdx.x < NLEV) hist[(size_t)threadIdx.x * ntiles + t] = h[threadIdx.x];
-        __syncthreads();
-    }
-}
-
-// stable scatter by level; also the level starts lvl[0..23]
-__global__ void __launch_bounds__(256) k_rec_scatter(const unsigned long long *__restrict__ rec,
-                                                     const uint64_t *__restrict__ total, int ntiles,
-                                                     const uint32_t *__restrict__ hoff, uint32_t *__restrict__ bfs2dfs,
-                                                     uint32_t *__restrict__ dfs2bfs, uint32_t *__restrict__ lvl,
-                                                     const Status *st)
-{
-    if (st->code) return;
-    __shared__ uint32_t whist[RS_WARPS][NLEV];
-    __shared__ uint32_t base[NLEV];
+    __shared__ uint32_t wcnt[CT_WARPS][CT_CNT + 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned ltmask = (1u << lane) - 1u;
-    const uint64_t T = *total;
-    if (blockIdx.x == 0 && threadIdx.x <= NLEV + 1)
-        lvl[threadIdx.x] = threadIdx.x < NLEV ? hoff[(size_t)threadIdx.x * ntiles] : (uint32_t)T;
-    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
-        const uint64_t b0 = (uint64_t)t * REC_TILE;
-        if (b0 >= T) break;
-        for (int k = threadIdx.x; k < RS_WARPS * NLEV; k += blockDim.x) (&whist[0][0])[k] = 0;
-        if (threadIdx.x < NLEV) base[threadIdx.x] = hoff[(size_t)threadIdx.x * ntiles + t];
-        __syncthreads();
-        uint32_t lv[REC_IPT], r[REC_IPT];
-        const int wbase = w * 32 * REC_IPT;
-#pragma unroll
-        for (int it = 0; it < REC_IPT; ++it) {
-            const uint64_t li = b0 + wbase + it * 32 + lane;
-            const bool ok = li < T;
-            const uint32_t d = ok ? (uint32_t)(rec[li] >> 32) : 32u;
-            const unsigned peers = __match_any_sync(0xffffffffu, d);
-            const uint32_t before = ok ? whist[w][d] : 0u;
-            __syncwarp();
-            if (ok && (peers & ltmask) == 0u) whist[w][d] = before + (uint32_t)__popc(peers);
-            __syncwarp();
-            r[it] = before + (uint32_t)__popc(peers & ltmask);
-            lv[it] = d;
+    const unsigned lt = (1u << lane) - 1u;
+    if (blockIdx.x == 0) {
+        if (threadIdx.x <= NLEV + 1) a.lvl[threadIdx.x] = threadIdx.x < NLEV ? a.off[(size_t)threadIdx.x * a.ntiles] : nodes;
+        if (threadIdx.x == 0 && a.gnode) {
+            const uint64_t ng = *a.total - nodes;
+            *a.ngroups = (int64_t)ng;
+            a.gfirst[ng] = (uint32_t)a.N;
         }
-        __syncthreads();
-        if (threadIdx.x < NLEV) {
-            uint32_t run = 0;
-            for (int ww = 0; ww < RS_WARPS; ++ww) {
-                const uint32_t cnt = whist[ww][threadIdx.x];
-                whist[ww][threadIdx.x] = run;
-                run += cnt;
-            }
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < REC_IPT; ++it) {
-            const uint64_t li = b0 + wbase + it * 32 + lane;
-            if (li < T) {
-                const uint32_t dst = base[lv[it]] + whist[w][lv[it]] + r[it];
-                bfs2dfs[dst] = (uint32_t)li;
-                dfs2bfs[li] = dst;
-            }
-        }
-        __syncthreads();
     }
-}
-
-// per node: level, first, count (end of the key-prefix run, exponential then
-// binary search), first child, parent of the roots, system roots
-__global__ void __launch_bounds__(256) k_nodes_a(const uint64_t *__restrict__ total,
-                                                 const uint32_t *__restrict__ bfs2dfs,
-                                                 const uint32_t *__restrict__ dfs2bfs,
-                                                 const unsigned long long *__restrict__ rec,
-                                                 const uint8_t *__restrict__ pD, const uint64_t *__restrict__ key,
-                                                 const int32_t *__restrict__ psys, const int64_t *__restrict__ off,
-                                                 uint32_t *nfirst, uint32_t *ncount, uint32_t *nlevel, uint32_t *nchild,
-                                                 uint32_t *nparent, uint32_t *sysroot, const Status *st)
-{
-    if (st->code) return;
-    const uint64_t T = *total;
-    for (uint64_t b = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; b < T; b += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t r = bfs2dfs[b];
-        const unsigned long long R = rec[r];
-        const int lev = (int)(R >> 32);
-        const uint32_t f = (uint32_t)R;
-        const int s = psys[f];
-        const uint32_t send = (uint32_t)off[s + 1];
-        uint32_t end;
-        if (lev == 0) {
-            end = send;
-            nparent[b] = NONE;
-            sysroot[s] = (uint32_t)b;
-        } else {
-            const int sh = 3 * (LEVELS - lev);
-            const uint64_t pre = key[f] >> sh;
-            uint32_t step = 1, lo = f;   // key[lo] has the prefix
-            while (f + step < send && (key[f + step] >> sh) == pre) {
-                lo = f + step;
-                step <<= 1;
+    for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+        const int64_t p0 = (int64_t)tile * CT_TILE + w * (32 * CT_ROWS) + lane;
+        int c[CT_ROWS], d[CT_ROWS], dp[CT_ROWS], dg[CT_ROWS];   // dp: D of the particle before
+        uint32_t mine = 0;
+#pragma unroll
+        for (int r = 0; r < CT_ROWS; ++r) {
+            const int64_t i = p0 + r * 32;
+            c[r] = LEVELS + 1;
+            d[r] = dp[r] = dg[r] = 0;
+            if (i < a.N) {
+                const int k = a.cells[i];
+                c[r] = (k & 31) - 1;
+                d[r] = (k >> 5) & 31;
+                dg[r] = k >> 10;
             }
-            uint32_t hi = min(f + step, send);   // first index known not to have it (or the end)
-            while (hi - lo > 1) {
-                const uint32_t mid = lo + ((hi - lo) >> 1);
-                if ((key[mid] >> sh) == pre) lo = mid;
-                else hi = mid;
-            }
-            end = hi;
+            if (i > 0 && i <= a.N) dp[r] = (a.cells[i - 1] >> 5) & 31;
+            if (i == a.N) c[r] = -1;   // the end of the batch ends every cell around the last particle
         }
-        nfirst[b] = f;
-        ncount[b] = end - f;
-        nlevel[b] = (uint32_t)lev;
-        nchild[b] = (lev < (int)pD[f]) ? dfs2bfs[r + 1] : NONE;
-    }
-}
-
-// children: the level l+1 nodes that start inside the parent's range
-__global__ void __launch_bounds__(256) k_nodes_b(const uint64_t *__restrict__ total, const uint32_t *__restrict__ lvl,
-                                                 const uint32_t *__restrict__ nfirst,
-                                                 const uint32_t *__restrict__ ncount,
-                                                 const uint32_t *__restrict__ nlevel,
-                                                 const uint32_t *__restrict__ nchild, uint32_t *nnch,
-                                                 uint32_t *nparent, const Status *st)
-{
-    if (st->code) return;
-    const uint64_t T = *total;
-    for (uint64_t b = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; b < T; b += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t ch = nchild[b];
-        uint32_t k = 0;
-        if (ch != NONE) {
-            const uint32_t end = nfirst[b] + ncount[b];
-            const uint32_t lend = lvl[nlevel[b] + 2];
-            while (k < 8 && ch + k < lend && nfirst[ch + k] < end) {
-                nparent[ch + k] = (uint32_t)b;
-                ++k;
+#pragma unroll
+        for (int r = 0; r < CT_ROWS; ++r) {
+            const bool real = p0 + r * 32 < a.N;
+            const int lo = __reduce_min_sync(0xffffffffu, real ? c[r] : LEVELS + 1) + 1;
+            const int hi = __reduce_max_sync(0xffffffffu, d[r]);
+            for (int l = lo; l <= hi; ++l) {
+                const uint32_t k = __popc(__ballot_sync(0xffffffffu, real && c[r] < l && l <= d[r]));
+                if (lane == l) mine += k;
             }
+            const uint32_t k = __popc(__ballot_sync(0xffffffffu, real && a.gnode && c[r] < dg[r]));
+            if (lane == NLEV) mine += k;
         }
-        nnch[b] = k;
+        if (lane < CT_CNT) wcnt[w][lane] = mine;
+        __syncthreads();
+        uint32_t base = 0;   // lane l: index of this warp's first start at level l; lane NLEV: of its first group
+        if (lane < CT_CNT) {
+            base = a.off[(size_t)lane * a.ntiles + tile] - (lane == NLEV ? nodes : 0u);
+            for (int k = 0; k < w; ++k) base += wcnt[k][lane];
+        }
+        __syncthreads();
+#pragma unroll
+        for (int r = 0; r < CT_ROWS; ++r) {
+            const int64_t i = p0 + r * 32;
+            const bool real = i < a.N, here = i <= a.N;
+            const unsigned gm = __ballot_sync(0xffffffffu, real && a.gnode && c[r] < dg[r]);
+            const uint32_t g = __shfl_sync(0xffffffffu, base, NLEV) + __popc(gm & lt);
+            const int sys = real ? a.psys[i] : 0;
+            // levels: from the parent's (c) to one past the deepest node started or closed here
+            const int lo = max(__reduce_min_sync(0xffffffffu, here ? c[r] : LEVELS + 1), 0);
+            const int hi = __reduce_max_sync(0xffffffffu, max(d[r], dp[r])) + 1;
+            uint32_t up = NONE;     // the node one level up: the parent of the next start
+            uint32_t last = NONE;   // the node at level l - 1 that ends at i
+            for (int l = lo; l <= hi; ++l) {
+                const bool start = real && c[r] < l && l <= d[r];
+                const unsigned m = __ballot_sync(0xffffffffu, start);
+                const uint32_t x = __shfl_sync(0xffffffffu, base, l) + __popc(m & lt);   // starts before i at this level
+                if (lane == l) base += __popc(m);
+                if (last != NONE) a.nchend[last] = x;
+                last = NONE;
+                if (here && c[r] < l && l <= dp[r] && i > 0) {   // the cell of particle i - 1 ends
+                    last = x - 1;
+                    a.nend[last] = (uint32_t)i;
+                }
+                if (l == c[r]) up = x - 1;
+                if (start) {
+                    a.nfirst[x] = (uint32_t)i;
+                    a.nlevel[x] = (uint32_t)l;
+                    a.nparent[x] = up;
+                    if (l > c[r] + 1) a.nchild[up] = x;
+                    if (l == d[r]) a.nchild[x] = NONE;
+                    a.done[x] = 0u;
+                    if (a.bmax64) a.bmax64[x] = 0ull;
+                    else a.bmax32[x] = 0u;
+                    if (l == 0) a.sysroot[sys] = x;
+                    if (l == dg[r] && ((gm >> lane) & 1u)) {
+                        a.gnode[g] = x;
+                        a.gfirst[g] = (uint32_t)i;
+                        a.gsys[g] = (uint32_t)sys;
+                    }
+                    up = x;
+                }
+            }
+            if (lane == NLEV) base += __popc(gm);
+        }
     }
 }
 
@@ -1049,7 +1064,7 @@ __global__ void __launch_bounds__(256) k_nodes_b(const uint64_t *__restrict__ to
 // chunks of BM_CH particles with one atomic max per chunk.
 // ---------------------------------------------------------------------------
 struct MomArgs {
-    const uint32_t *lvl, *nfirst, *ncount, *nnch, *nchild, *nparent, *nlevel;
+    const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nparent, *nlevel;   // a node's particles and children: [first, end)
     const double *x, *y, *z, *m;
     const uint64_t *key;
     const int32_t *psys;
@@ -1248,7 +1263,7 @@ __device__ __forceinline__ double warp_sum_d(double v)
 // small cell's, by G lanes (a warp or an aligned group of 8 with mask gm).
 __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, int lane)
 {
-    const uint32_t ch0 = a.nchild[c], k = a.nnch[c];
+    const uint32_t ch0 = a.nchild[c], k = a.nchend[c] - ch0;
     const uint32_t f = a.nfirst[c];
     const SysBox &b = a.box[a.psys[f]];
     const bool on = (uint32_t)lane < k;
@@ -1286,7 +1301,7 @@ __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, int lane)
 template <int G>
 __device__ void mom_combine_f32(const MomArgs &a, uint32_t c, int lane, unsigned gm)
 {
-    const uint32_t ch0 = a.nchild[c], k = a.nnch[c];
+    const uint32_t ch0 = a.nchild[c], k = a.nchend[c] - ch0;
     const uint32_t f = a.nfirst[c];
     const SysBox &b = a.box[a.psys[f]];
     const bool on = (uint32_t)lane < k;
@@ -1341,7 +1356,7 @@ __device__ void mom_climb(const MomArgs &a, uint32_t c, int lane, unsigned gm)
 {
     for (;;) {
         const uint32_t p = a.nparent[c];
-        if (p == NONE || a.ncount[p] <= MOM_CH) return;
+        if (p == NONE || a.nend[p] - a.nfirst[p] <= MOM_CH) return;
         __syncwarp(gm);
         unsigned int old = 0;
         if (lane == 0) {   // release: c's moments (stored by this lane) before the count; acquire: the others' after
@@ -1349,7 +1364,7 @@ __device__ void mom_climb(const MomArgs &a, uint32_t c, int lane, unsigned gm)
             old = cnt.fetch_add(1u, cuda::memory_order_acq_rel);
         }
         old = __shfl_sync(gm, old, 0, G);
-        if (old + 1u != a.nnch[p]) return;
+        if (old + 1u != a.nchend[p] - a.nchild[p]) return;
         __syncwarp(gm);
         if (F64) mom_combine_f64(a, p, lane);
         else mom_combine_f32<G>(a, p, lane, gm);
@@ -1373,8 +1388,8 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (F64) {   // one warp per cell
         for (uint32_t c = warp; c < total; c += nw) {
-            const uint32_t f = a.nfirst[c], n = a.ncount[c];
-            if (n <= MOM_CH || a.nnch[c] == 0) {
+            const uint32_t f = a.nfirst[c], n = a.nend[c] - f;
+            if (n <= MOM_CH || a.nchild[c] == NONE) {
                 const double o0 = a.x[f], o1 = a.y[f], o2 = a.z[f];
                 const MomSums r = mom_range(a, f, n, o0, o1, o2, lane);
                 if (lane == 0) mom_store(a, c, r, o0, o1, o2);
@@ -1409,8 +1424,8 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
         for (uint32_t q = warp; q < nq; q += nw) {
             const uint32_t c = 4 * q + sub;
             if (c >= total) continue;
-            const uint32_t f = a.nfirst[c], n = a.ncount[c];
-            if (n <= MOM_CH || a.nnch[c] == 0) {
+            const uint32_t f = a.nfirst[c], n = a.nend[c] - f;
+            if (n <= MOM_CH || a.nchild[c] == NONE) {
                 const MomSumsF r = mom_range_f32<8>(a.phi, a.plo, f, n, f, sl, gm);
                 const float iM = r.M > 0.0f ? 1.0f / r.M : 0.0f;
                 const float e0 = r.sx * iM, e1 = r.sy * iM, e2 = r.sz * iM;
@@ -1448,7 +1463,7 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
     for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < T; w += nw) {
         const uint32_t c = items[w];
         const uint32_t k = w - bigbase[c];
-        const uint32_t f = a.nfirst[c], n = a.ncount[c];
+        const uint32_t f = a.nfirst[c], n = a.nend[c] - f;
         const uint32_t f0 = f + k * BM_CH, n0 = min(BM_CH, f + n - f0);
         if (F64) {
             const double c0 = a.cx[c], c1 = a.cy[c], c2 = a.cz[c];
@@ -1479,7 +1494,7 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
 
 // Per node: geometry, delta, MAC radius, walk criteria and packed topology.
 struct FinArgs {
-    const uint32_t *lvl, *nfirst, *ncount, *nnch, *nchild, *nlevel;
+    const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nlevel;
     const uint64_t *key;
     const int32_t *psys;
     const SysBox *box;
@@ -1568,8 +1583,8 @@ __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
             hr = hrf;
             delta = df;
         }
-        const uint32_t k = a.nnch[c];
-        a.topo[c] = make_uint4(k ? a.nchild[c] : NONE, k, f, a.ncount[c]);
+        const uint32_t ch = a.nchild[c];
+        a.topo[c] = make_uint4(ch, ch == NONE ? 0u : a.nchend[c] - ch, f, a.nend[c] - f);
         a.rb[c] = rb;
         a.hr[c] = hr;
         a.delta[c] = delta;
@@ -1579,21 +1594,22 @@ __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
 
 // ---------------------------------------------------------------------------
 // Sink groups: first cells (from the root) with count <= n_crit, or leaves.
-// Marked at their first particle, compacted in particle order.
+// Marked at their first particle, compacted in particle order. Only for n_crit
+// above GROUP_WINDOW (k_nodes makes the others).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_group_flag(const uint32_t *__restrict__ lvl,
                                                     const uint32_t *__restrict__ nfirst,
-                                                    const uint32_t *__restrict__ ncount,
-                                                    const uint32_t *__restrict__ nnch,
+                                                    const uint32_t *__restrict__ nend,
+                                                    const uint32_t *__restrict__ nchild,
                                                     const uint32_t *__restrict__ nparent, int n_crit,
                                                     uint32_t *__restrict__ gflag, const Status *st)
 {
     if (st->code) return;
     const uint32_t total = lvl[LEVELS + 1];
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
-        const bool stop = ncount[c] <= (uint32_t)n_crit || nnch[c] == 0;
+        const bool stop = nend[c] - nfirst[c] <= (uint32_t)n_crit || nchild[c] == NONE;
         const uint32_t p = nparent[c];
-        const bool parent_goes_on = (p == NONE) || (ncount[p] > (uint32_t)n_crit);
+        const bool parent_goes_on = (p == NONE) || (nend[p] - nfirst[p] > (uint32_t)n_crit);
         if (stop && parent_goes_on) gflag[nfirst[c]] = c;
     }
 }
@@ -1608,20 +1624,20 @@ __global__ void __launch_bounds__(256) k_group_mark(int64_t N, const uint32_t *_
 
 __global__ void __launch_bounds__(256) k_group_compact(int64_t N, const uint32_t *__restrict__ gflag,
                                                        const uint32_t *__restrict__ gscan,
-                                                       const uint32_t *__restrict__ ncount,
                                                        const int32_t *__restrict__ psys, uint32_t *gnode,
-                                                       uint32_t *gfirst, uint32_t *gcount, uint32_t *gsys,
-                                                       const uint64_t *total, int64_t *ngroups, const Status *st)
+                                                       uint32_t *gfirst, uint32_t *gsys, const uint64_t *total, int64_t *ngroups, const Status *st)
 {
     if (st->code) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ngroups = (int64_t)*total;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *ngroups = (int64_t)*total;
+        gfirst[*total] = (uint32_t)N;
+    }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t c = gflag[i];
         if (c != NONE) {
             const uint32_t g = gscan[i];
             gnode[g] = c;
             gfirst[g] = (uint32_t)i;
-            gcount[g] = ncount[c];
             gsys[g] = (uint32_t)psys[i];
         }
     }
@@ -1630,8 +1646,7 @@ __global__ void __launch_bounds__(256) k_group_compact(int64_t N, const uint32_t
 // One warp per group: box of the members (FP64, exact min/max), its centre
 // as an FP32 hi/lo pair and its half extents rounded up.
 __global__ void __launch_bounds__(256) k_group_box(const int64_t *__restrict__ ngroups,
-                                                   const uint32_t *__restrict__ gfirst,
-                                                   const uint32_t *__restrict__ gcount, const double *__restrict__ x,
+                                                   const uint32_t *__restrict__ gfirst, const double *__restrict__ x,
                                                    const double *__restrict__ y, const double *__restrict__ z,
                                                    const int32_t *__restrict__ psys, const SysBox *__restrict__ box,
                                                    double *glo, double *ghi, GroupF *gF, const Status *st)
@@ -1649,7 +1664,7 @@ __global__ void __launch_bounds__(256) k_group_box(const int64_t *__restrict__ n
         unsigned long long mine[6] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull};
         for (int k = 0; k < gn; ++k) {
             const int64_t g = g0 + k;
-            const uint32_t f = gfirst[g], n = gcount[g];
+            const uint32_t f = gfirst[g], n = gfirst[g + 1] - f;
             // exact min/max through the order-preserving integer images (no FP64 pipe work)
             unsigned long long u[6] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull};
             for (uint32_t i = f + lane; i < f + n; i += 32) {
@@ -1807,52 +1822,61 @@ void launch_permute(hybrid_ctx *c)
     c->swaps ^= 1;
 }
 
-bool launch_build_levels(hybrid_ctx *c)
+// sink groups marked with the cells (k_cells, k_nodes) or, for a large n_crit, from the nodes afterwards
+static bool groups_in_nodes(const hybrid_ctx *c) { return c->p.n_crit <= GROUP_WINDOW; }
+
+void launch_topology(hybrid_ctx *c)
 {
     Status *st = status_dev(c);
     const int64_t N = c->N;
-    const int gridN = grid_for(c, N, 256, 8);
-    int8_t *pc = (int8_t *)c->pc.p;
-    uint8_t *pD = (uint8_t *)c->pD.p;
-    uint32_t *pn = (uint32_t *)c->pn.p;
+    const bool groups = groups_in_nodes(c);
+    const int n_crit = groups ? c->p.n_crit : 0;
     const uint64_t *keys = (const uint64_t *)c->keys[0].p;
+    const int32_t *psys = (const int32_t *)c->psys.p;
     uint64_t *d_tot = (uint64_t *)((char *)c->lvl.p + 256);
-    const size_t shm = (size_t)(LD_T + 2 * c->p.n_leaf);
-    k_leaf_depth<<<grid_for(c, N, LD_T, 8), LD_T, shm, c->st>>>(N, keys, (const int32_t *)c->psys.p, pc,
-                                                                c->p.n_leaf, pD, pn, st);
-    scan_u32(c, pn, N, nullptr, N, d_tot);
-    unsigned long long *rec = (unsigned long long *)c->rec.p;
-    k_records<<<gridN, 256, 0, c->st>>>(N, pc, pD, pn, d_tot, c->capNodes, rec, st, c->op);
-    const int ntiles = (int)((c->capNodes + REC_TILE - 1) / REC_TILE);
-    uint32_t *rh = (uint32_t *)c->rhist.p;
-    k_rec_hist<<<std::min(ntiles, c->nsm * 4), 256, 0, c->st>>>(rec, d_tot, ntiles, rh, st);
-    scan_u32(c, rh, (int64_t)NLEV * ntiles, nullptr, (int64_t)NLEV * ntiles, nullptr);
-    uint32_t *b2d = (uint32_t *)c->rb2d.p, *d2b = (uint32_t *)c->rd2b.p;
-    uint32_t *lvl = (uint32_t *)c->lvl.p;
-    k_rec_scatter<<<std::min(ntiles, c->nsm * 4), 256, 0, c->st>>>(rec, d_tot, ntiles, rh, b2d, d2b, lvl, st);
-    const int gridT = grid_for(c, c->capNodes, 256, 8);
-    k_nodes_a<<<gridT, 256, 0, c->st>>>(d_tot, b2d, d2b, rec, pD, keys, (const int32_t *)c->psys.p,
-                                        (const int64_t *)c->off_dev.p, (uint32_t *)c->nfirst.p, (uint32_t *)c->ncount.p,
-                                        (uint32_t *)c->nlevel.p, (uint32_t *)c->nchild.p, (uint32_t *)c->nparent.p,
-                                        (uint32_t *)c->sysroot.p, st);
-    k_nodes_b<<<gridT, 256, 0, c->st>>>(d_tot, lvl, (const uint32_t *)c->nfirst.p, (const uint32_t *)c->ncount.p,
-                                        (const uint32_t *)c->nlevel.p, (const uint32_t *)c->nchild.p,
-                                        (uint32_t *)c->nnch.p, (uint32_t *)c->nparent.p, st);
-    c->launches += 7;
-    return true;
+    uint32_t *cnt = (uint32_t *)c->ccnt.p;
+    uint16_t *cells = (uint16_t *)c->cells.p;
+    const int ntiles = cell_tiles(N);
+    const int grid = std::min(ntiles, c->nsm * 8);
+    k_cells<<<grid, 32 * CT_WARPS, 2 * (size_t)cells_bytes(std::max(c->p.n_leaf, n_crit)), c->st>>>(
+        N, c->S, keys, psys, c->p.n_leaf, n_crit, cells, ntiles, cnt, (unsigned long long *)c->counter.p, st);
+    scan_u32(c, cnt, (int64_t)CT_CNT * ntiles, nullptr, (int64_t)CT_CNT * ntiles, d_tot);
+    NodeArgs a;
+    a.cells = cells;
+    a.psys = psys;
+    a.off = cnt;
+    a.total = d_tot;
+    a.nfirst = (uint32_t *)c->nfirst.p;
+    a.nend = (uint32_t *)c->nend.p;
+    a.nlevel = (uint32_t *)c->nlevel.p;
+    a.nchild = (uint32_t *)c->nchild.p;
+    a.nchend = (uint32_t *)c->nchend.p;
+    a.nparent = (uint32_t *)c->nparent.p;
+    a.sysroot = (uint32_t *)c->sysroot.p;
+    a.lvl = (uint32_t *)c->lvl.p;
+    a.done = (uint32_t *)c->ndone.p;
+    a.bmax64 = c->p.precision == 0 ? (unsigned long long *)c->nbmax.p : nullptr;
+    a.bmax32 = (unsigned int *)c->nbmax32.p;
+    a.gnode = groups ? (uint32_t *)c->gnode.p : nullptr;
+    a.gfirst = (uint32_t *)c->gfirst.p;
+    a.gsys = (uint32_t *)c->gsys.p;
+    a.ngroups = (int64_t *)c->ngroups_dev.p;
+    a.N = N;
+    a.cap = c->capNodes;
+    a.ntiles = ntiles;
+    k_nodes<<<grid, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
+    c->launches += 2;
 }
 
 void launch_moments(hybrid_ctx *c)
 {
     Status *st = status_dev(c);
     const int grid = grid_for(c, c->capNodes, 256, 8);
-    if (c->p.precision == 0) cudaMemsetAsync(c->nbmax.p, 0, (size_t)c->capNodes * sizeof(unsigned long long), c->st);
-    else cudaMemsetAsync(c->nbmax32.p, 0, (size_t)c->capNodes * sizeof(unsigned int), c->st);
     MomArgs a;
     a.lvl = (const uint32_t *)c->lvl.p;
     a.nfirst = (const uint32_t *)c->nfirst.p;
-    a.ncount = (const uint32_t *)c->ncount.p;
-    a.nnch = (const uint32_t *)c->nnch.p;
+    a.nend = (const uint32_t *)c->nend.p;
+    a.nchend = (const uint32_t *)c->nchend.p;
     a.nchild = (const uint32_t *)c->nchild.p;
     a.nparent = (const uint32_t *)c->nparent.p;
     a.nlevel = (const uint32_t *)c->nlevel.p;
@@ -1876,8 +1900,6 @@ void launch_moments(hybrid_ctx *c)
     a.phi = (const float4 *)c->phi.p;
     a.plo = (const float4 *)c->plo.p;
     unsigned long long *nitems = (unsigned long long *)c->counter.p + 9;
-    cudaMemsetAsync(nitems, 0, sizeof(unsigned long long), c->st);
-    cudaMemsetAsync(c->ndone.p, 0, (size_t)c->capNodes * sizeof(uint32_t), c->st);
     const int gridw = grid_for(c, c->capNodes * 32, 256, 16);
     uint32_t *bigbase = (uint32_t *)c->nbig.p, *items = (uint32_t *)c->mitems.p;
     if (c->p.precision == 0) {
@@ -1891,8 +1913,8 @@ void launch_moments(hybrid_ctx *c)
     FinArgs f;
     f.lvl = a.lvl;
     f.nfirst = a.nfirst;
-    f.ncount = a.ncount;
-    f.nnch = a.nnch;
+    f.nend = a.nend;
+    f.nchend = a.nchend;
     f.nchild = a.nchild;
     f.nlevel = a.nlevel;
     f.key = a.key;
@@ -1923,19 +1945,19 @@ void launch_moments(hybrid_ctx *c)
 
 void launch_groups(hybrid_ctx *c)
 {
+    if (groups_in_nodes(c)) return;
     Status *st = status_dev(c);
     const int64_t N = c->N;
     cudaMemsetAsync(c->gflag.p, 0xff, (size_t)N * sizeof(uint32_t), c->st);
     k_group_flag<<<grid_for(c, c->capNodes, 256), 256, 0, c->st>>>(
-        (const uint32_t *)c->lvl.p, (const uint32_t *)c->nfirst.p, (const uint32_t *)c->ncount.p,
-        (const uint32_t *)c->nnch.p, (const uint32_t *)c->nparent.p, c->p.n_crit, (uint32_t *)c->gflag.p, st);
+        (const uint32_t *)c->lvl.p, (const uint32_t *)c->nfirst.p, (const uint32_t *)c->nend.p,
+        (const uint32_t *)c->nchild.p, (const uint32_t *)c->nparent.p, c->p.n_crit, (uint32_t *)c->gflag.p, st);
     k_group_mark<<<grid_for(c, N, 256), 256, 0, c->st>>>(N, (const uint32_t *)c->gflag.p, (uint32_t *)c->gscan.p, st);
     uint64_t *d_tot = (uint64_t *)((char *)c->lvl.p + 64 * sizeof(uint32_t) + 64 + 8);
     scan_u32(c, (uint32_t *)c->gscan.p, N, nullptr, N, d_tot);
     k_group_compact<<<grid_for(c, N, 256), 256, 0, c->st>>>(
-        N, (const uint32_t *)c->gflag.p, (const uint32_t *)c->gscan.p, (const uint32_t *)c->ncount.p,
-        (const int32_t *)c->psys.p, (uint32_t *)c->gnode.p, (uint32_t *)c->gfirst.p, (uint32_t *)c->gcount.p,
-        (uint32_t *)c->gsys.p, d_tot, (int64_t *)c->ngroups_dev.p, st);
+        N, (const uint32_t *)c->gflag.p, (const uint32_t *)c->gscan.p, (const int32_t *)c->psys.p,
+        (uint32_t *)c->gnode.p, (uint32_t *)c->gfirst.p, (uint32_t *)c->gsys.p, d_tot, (int64_t *)c->ngroups_dev.p, st);
     c->launches += 3;
 }
 
@@ -1944,14 +1966,20 @@ void launch_group_boxes(hybrid_ctx *c)
     Status *st = status_dev(c);
     const int64_t N = c->N;
     k_group_box<<<grid_for(c, N * 32 / 16, 256), 256, 0, c->st>>>(
-        (const int64_t *)c->ngroups_dev.p, (const uint32_t *)c->gfirst.p, (const uint32_t *)c->gcount.p,
-        (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p, (const int32_t *)c->psys.p,
+        (const int64_t *)c->ngroups_dev.p, (const uint32_t *)c->gfirst.p, (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p, (const int32_t *)c->psys.p,
         (const SysBox *)c->box.p, (double *)c->glo.p, (double *)c->ghi.p, (GroupF *)c->gF.p, st);
     c->launches += 1;
 }
 
+int cell_tiles(int64_t N) { return (int)(N / CT_TILE) + 1; }   // N + 1 positions: the end of the batch is one
+
+size_t cell_count_bytes(int64_t N) { return (size_t)CT_CNT * cell_tiles(N) * sizeof(uint32_t); }
+
 cudaError_t init_tree_kernels()
 {
+    // leaves of up to 24448 particles, as far as their window fits in shared memory
+    cudaError_t e = cudaFuncSetAttribute(k_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * cells_bytes(24448));
+    if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(k_ss_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_CAP * 12);
 }
 

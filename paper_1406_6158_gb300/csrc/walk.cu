@@ -56,7 +56,7 @@ struct WalkArgs {
     Status *st;
     int where;
     // one-pass form
-    const uint32_t *gfirst, *gcount;
+    const uint32_t *gfirst;
     unsigned long long *list_cursor;     // next free list entry
     unsigned long long *item_count;      // [0] far items, [1] near items
     WorkItem *items_far, *items_near;
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
         const uint32_t s = a.gsys[g];
         const bool has_hard = a.sp[s].has_hard != 0;
         const bool wh0 = want_hard && has_hard;
-        const uint32_t gfirst = a.gfirst[g], gn = a.gcount[g];
+        const uint32_t gfirst = a.gfirst[g], gn = a.gfirst[g + 1] - gfirst;
         const GroupF G = a.gF[g];
         const float cx = G.c_hi.x, cy = G.c_hi.y, cz = G.c_hi.z, hx = G.c_hi.w;
         const float lx = G.c_lo.x, ly = G.c_lo.y, lz = G.c_lo.z, hy = G.c_lo.w, hz = G.hz_root.x;
@@ -531,7 +531,6 @@ void launch_walk(hybrid_ctx *c, int mode)
     a.st = st;
     a.where = c->op;
     a.gfirst = (const uint32_t *)c->gfirst.p;
-    a.gcount = (const uint32_t *)c->gcount.p;
     a.list_cursor = (unsigned long long *)c->counter.p + 10;
     a.item_count = (unsigned long long *)c->counter.p + 11;
     a.items_far = (WorkItem *)c->wmap.p;

@@ -1,0 +1,51 @@
+"""Nodes and sink groups at the edges of the topology kernels' tiles and windows, bit for bit against the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1406_6158_gb300 import ics
+from test_gpu_parity import H, check_tree, oparams  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+torch = pytest.importorskip("torch")
+
+
+def tree_of(H, st, **kw):
+    P = H.Params(eps=0.01, theta=0.6, R1=0.04, R2=0.08, **kw)
+    ctx, s = H.Context(P), H.System(st, precision=P.precision)
+    ctx.hybrid_build_tree(s)
+    T = oracle.Tree(st["x"], st["y"], st["z"], st["m"], oparams(P))
+    assert np.array_equal(s.numpy()["id"], T.perm)
+    return T, ctx.tree(s.n)
+
+
+# tiles of 1024 particles (the end of the batch is a position of its own), windows of n_leaf and n_crit, groups
+# from the cells (n_crit <= 1024) and from the nodes (above)
+@pytest.mark.parametrize("n", [1, 2, 1023, 1024, 1025, 2048, 5000])
+@pytest.mark.parametrize("n_leaf,n_crit", [(1, 1), (16, 64), (16, 5), (3, 256), (40, 1024), (16, 1025), (7, 100000)])
+def test_tiles_and_windows(H, n, n_leaf, n_crit):  # noqa: F811
+    check_tree(*tree_of(H, ics.plummer(n, 77 + n), n_leaf=n_leaf, n_crit=n_crit, precision=1), 1)
+
+
+@pytest.mark.parametrize("n_leaf,n_crit", [(16, 64), (300, 500), (2000, 64)])
+def test_coincident_particles_across_tiles(H, n_leaf, n_crit):  # noqa: F811
+    st = ics.plummer(4000, 5)
+    for k in "xyz":
+        st[k][500:1900] = 0.125      # 1400 particles in one cell of the finest level
+        st[k][3000:3010] = -0.5
+    check_tree(*tree_of(H, st, n_leaf=n_leaf, n_crit=n_crit, precision=0), 0)
+
+
+def test_batch_boundaries(H):  # noqa: F811
+    # systems that end inside, at and past a tile's end: each must get the tree it has alone
+    sizes = [1024, 1, 1023, 3000, 2, 40]
+    P = H.Params(eps=0.01, theta=0.6, R1=0.04, R2=0.08, precision=0)
+    states = [ics.plummer(n, 200 + n) for n in sizes]
+    systems = [H.System(st, precision=0) for st in states]
+    H.Context(P).hybrid_step_batched(systems, 0)
+    for st, s in zip(states, systems):
+        alone = H.System(st, precision=0)
+        H.Context(P).hybrid_step(alone, 0)
+        a, b = alone.numpy(), s.numpy()
+        for k in a:
+            assert np.array_equal(a[k], b[k]), k
