@@ -66,13 +66,14 @@ constexpr int32_t ST_SKIN = 100;
 constexpr int32_t ST_SORT = 101;
 
 // Sample sort of the keys (the usual path once the state is close to key
-// order): per system, nb buckets of about SS_BUCKET keys split by keys taken
-// at regular positions; a bucket of at most SS_CAP keys (twice the target:
-// the splitters are the last build's quantiles, and only the particles that
-// crossed a coarse cell boundary since move between buckets) is sorted in one
-// block.
-constexpr int SS_BUCKET = 2048;
-constexpr int SS_CAP = 4096;
+// order): per system, nb buckets of about SS_BUCKET keys split by the last
+// build's keys at every SS_BUCKET-th position; a bucket of at most SS_CAP keys
+// (over twice the target: only the particles that crossed a coarse cell boundary
+// since move between buckets) is sorted by one warp: 8 keys a lane for up to
+// 256 keys, which a bucket of 224 seldom outgrows, else 16.
+constexpr int SS_BUCKET = 224;
+constexpr int SS_CAP = 512;
+constexpr int SS_SUM_MAX = 4096;   // buckets up to which the sorting blocks add up the counts themselves
 struct SSys {
     int32_t nb;      // buckets of the system
     int32_t bbase;   // index of its first bucket
@@ -168,7 +169,7 @@ struct hybrid_ctx {
     // with the radix sort after a bucket overflowed
     std::vector<hy::SSys> h_ss;
     int nbk = 0;
-    bool ss_ok = false, sort_fallback = false;
+    bool sort_fallback = false;
     int64_t sort_fallbacks = 0;
     bool tree_valid = false, have_soft = false, have_hard = false;
     // reused neighbour lists (skin > 0): the lists of the last walk still hold for the working state of the
@@ -186,7 +187,7 @@ struct hybrid_ctx {
     hy::Buf phi, plo, pd;                  // float4 hi/lo (precision 1), double4_32a (precision 0)
     hy::Buf disp;                          // float: bound of the distance moved since the last build (skin > 0)
     hy::Buf keys[2], vals[2], hist, blocksum;
-    hy::Buf ss_sys, ss_spk, ss_spv, ss_cnt, ss_start, ss_cur, ss_pb, ss_flag;   // sample sort
+    hy::Buf ss_sys, ss_cnt, ss_rk, ss_rv, ss_flag;   // sample sort: counts and regions of the buckets
     int64_t capBk = 0;
     hy::Buf off_dev, sp_dev, chunks_dev, boxmin, boxmax, box, sysroot;
     hy::Buf status;
@@ -274,7 +275,7 @@ void launch_pair_far(hybrid_ctx *c);
 void launch_pair_near(hybrid_ctx *c, int mode);
 // shared-memory attributes of the far kernels (once per device, before any launch or capture)
 cudaError_t init_pair_kernels();
-// shared-memory attribute of the sample sort's splitter kernel
+// shared-memory attribute of the topology's window kernel
 cudaError_t init_tree_kernels();
 
 // ---- integrator and io (integrate.cu) ----

@@ -225,13 +225,12 @@ bool reserve(hybrid_ctx *c)
         ok = ok && ensure(c, c->chunks_dev, (size_t)c->nchunks * sizeof(Chunk));
         if (ok) c->capChunks = c->nchunks;
     }
-    // sample sort: a system table, splitters and bucket counts, starts and cursors, each key's bucket
-    ok = ok && ensure(c, c->ss_sys, (size_t)S * sizeof(SSys)) && ensure(c, c->ss_flag, 256) &&
-         ensure(c, c->ss_pb, (size_t)std::max<int64_t>(N, 1) * 4);
+    // sample sort: a system table, bucket counts and regions
+    ok = ok && ensure(c, c->ss_sys, (size_t)S * sizeof(SSys)) && ensure(c, c->ss_flag, 256);
     if (c->nbk > c->capBk) {
         const size_t nb = (size_t)c->nbk;
-        ok = ok && ensure(c, c->ss_spk, nb * 8) && ensure(c, c->ss_spv, nb * 4) && ensure(c, c->ss_cnt, nb * 4) &&
-             ensure(c, c->ss_start, nb * 4) && ensure(c, c->ss_cur, nb * 4);
+        ok = ok && ensure(c, c->ss_cnt, (nb + 1) * 4) && ensure(c, c->ss_rk, nb * SS_CAP * 8) &&
+             ensure(c, c->ss_rv, nb * SS_CAP * 4);
         if (ok) c->capBk = c->nbk;
     }
     // radix sort scratch: 64 tickets, digit counts [S][8][256], look-back words [8][chunks][256]
@@ -247,8 +246,8 @@ bool reserve(hybrid_ctx *c)
     ok = ok && ensure_items(c, 2 * c->capGroups + c->capList / 256 + 1024);
     if (c->capStack == 0) c->capStack = 4096;
     ok = ok && ensure(c, c->stack, (size_t)c->walk_warps * c->capStack * 4);
-    // scratch of the scans: the longest is over max(N, 3 groups + 1, counts per tile)
-    const int64_t longest = std::max<int64_t>({N, 3 * c->capGroups + 2, (int64_t)(cell_count_bytes(N) / 4)});
+    // scratch of the scans: the longest is over max(N, 3 groups + 1, counts per tile, buckets + 1)
+    const int64_t longest = std::max<int64_t>({N, 3 * c->capGroups + 2, (int64_t)(cell_count_bytes(N) / 4), (int64_t)c->nbk + 1});
     ok = ok && ensure(c, c->blocksum, (size_t)((longest + SCAN_SEG - 1) / SCAN_SEG + 1) * 8);
     return ok;
 }
@@ -324,16 +323,13 @@ hybrid_status setup_batch(hybrid_ctx *c, const hybrid_system *sys, int S, bool n
         }
     }
     c->nchunks = (int)c->h_chunks.size();
-    // sample sort layout: about SS_BUCKET keys per bucket, half that on batches of at most 2^20 particles (more
-    // blocks for the bucket sort when the whole batch is a few tens of buckets)
+    // sample sort layout: about SS_BUCKET keys per bucket
     c->h_ss.resize(S);
     c->nbk = 0;
-    c->ss_ok = true;
-    const int64_t bucket = c->N <= ((int64_t)1 << 20) ? SS_BUCKET / 2 : SS_BUCKET;
     for (int s = 0; s < S; ++s) {
         const int64_t n = c->h_off[s + 1] - c->h_off[s];
         SSys &y = c->h_ss[s];
-        y.nb = (int32_t)((n + bucket - 1) / bucket);
+        y.nb = (int32_t)((n + SS_BUCKET - 1) / SS_BUCKET);
         y.bbase = c->nbk;
         c->nbk += y.nb;
     }
@@ -499,7 +495,6 @@ uint64_t ops_signature(const hybrid_ctx *c, const std::vector<Op> &ops)
     mix((uint64_t)c->nchunks);
     mix((uint64_t)c->ipt);
     mix((uint64_t)c->nbk);
-    mix((uint64_t)c->ss_ok);
     mix((uint64_t)c->prof);
     for (const Op &o : ops) {
         mix((uint64_t)o.kind);
@@ -834,7 +829,7 @@ hybrid_status hybrid_destroy(hybrid_ctx *c)
     else cudaDeviceSynchronize();
     Buf *all[] = {&c->id, &c->ida, &c->orig, &c->origa, &c->psys, &c->phi, &c->plo, &c->pd, &c->disp, &c->keys[0], &c->keys[1],
                   &c->vals[0], &c->vals[1], &c->hist, &c->blocksum, &c->off_dev, &c->sp_dev, &c->chunks_dev,
-                  &c->ss_sys, &c->ss_spk, &c->ss_spv, &c->ss_cnt, &c->ss_start, &c->ss_cur, &c->ss_pb, &c->ss_flag,
+                  &c->ss_sys, &c->ss_cnt, &c->ss_rk, &c->ss_rv, &c->ss_flag,
                   &c->boxmin, &c->boxmax, &c->box, &c->sysroot, &c->status, &c->lvl, &c->nfirst, &c->nend,
                   &c->nchild, &c->nchend, &c->nparent, &c->nlevel, &c->ndone, &c->cells, &c->ccnt, &c->nM, &c->ncx,
                   &c->ncy, &c->ncz, &c->nB2, &c->nbmax, &c->nA, &c->nB, &c->ncrit, &c->ntopo, &c->nD, &c->nrb,

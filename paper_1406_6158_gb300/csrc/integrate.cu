@@ -41,8 +41,15 @@ __device__ __forceinline__ int sys_of(const int64_t *__restrict__ off, int S, in
 }
 
 __global__ void __launch_bounds__(256) k_copy_in(int64_t N, int S, const int64_t *__restrict__ off,
-                                                 const SysIO *__restrict__ io, StatePtrs w, int prec, int with_acc)
+                                                 const SysIO *__restrict__ io, StatePtrs w, int prec, int with_acc,
+                                                 unsigned long long *bmin, unsigned long long *bmax, uint32_t *ss_flag)
 {
+    // a new state: empty root boxes and no verdict on the sample sort's splitters yet
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * S; k += gridDim.x * blockDim.x) {
+        bmin[k] = ~0ull;
+        bmax[k] = 0ull;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) ss_flag[1] = 0u;
     for (int64_t gi = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; gi < N; gi += (int64_t)gridDim.x * blockDim.x) {
         const int s = sys_of(off, S, gi);
         const SysIO &y = io[s];
@@ -228,7 +235,9 @@ static int grid_n(hybrid_ctx *c, int64_t n)
 void launch_copy_in(hybrid_ctx *c, const SysIO *d_io, bool with_acc)
 {
     k_copy_in<<<grid_n(c, c->N), 256, 0, c->st>>>(c->N, c->S, (const int64_t *)c->off_dev.p, d_io, state_ptrs(c),
-                                                   c->p.precision, with_acc ? 1 : 0);
+                                                   c->p.precision, with_acc ? 1 : 0,
+                                                   (unsigned long long *)c->boxmin.p, (unsigned long long *)c->boxmax.p,
+                                                   (uint32_t *)c->ss_flag.p);
     c->launches++;
 }
 

@@ -41,10 +41,33 @@ __device__ __forceinline__ double unord_dbl(unsigned long long u)
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) k_box(const double *__restrict__ x, const double *__restrict__ y,
                                              const double *__restrict__ z, const Chunk *__restrict__ chunks,
-                                             int nchunks, unsigned long long *bmin, unsigned long long *bmax,
-                                             const Status *st)
+                                             int nchunks, unsigned long long *bmin, unsigned long long *bmax, int nbk,
+                                             int S, const int64_t *__restrict__ off, const SSys *__restrict__ ss,
+                                             const uint64_t *__restrict__ key, uint32_t *__restrict__ cnt,
+                                             uint32_t *__restrict__ flag)
 {
-    (void)st;   // the sort always runs: later kernels rely on a consistent permutation
+    // the sort always runs, whatever the status: later kernels rely on a consistent permutation
+    // sample sort (nbk buckets, 0 for the radix sort): bucket counts cleared, and whether the splitters (the
+    // last build's keys at every SS_BUCKET-th position) are in order
+    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
+    if (gtid == 0) flag[0] = 0u;
+    for (int b = gtid; b < nbk; b += gridDim.x * blockDim.x) {
+        cnt[b] = 0u;
+        int s = 0;
+        if (S > 1) {   // system of bucket b
+            int hi = S;
+            while (hi - s > 1) {
+                const int mid = (s + hi) >> 1;
+                if (ss[mid].bbase <= b) s = mid;
+                else hi = mid;
+            }
+        }
+        const SSys y = ss[s];
+        const int j = b - y.bbase;
+        const uint64_t *k = key + off[s] + (int64_t)j * SS_BUCKET;
+        if (j >= 1 && j + 1 < y.nb && k[SS_BUCKET] < k[0]) flag[1] = 1u;
+    }
+    if (gtid == 0) cnt[nbk] = 0u;
     // min/max of the order-preserving integer images: exact, and no FP64 pipe work
     __shared__ unsigned long long sh[6][8];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -385,229 +408,41 @@ __global__ void __launch_bounds__(256) k_onesweep(const uint64_t *__restrict__ k
 // Sample sort of the keys, for a state that is close to key order (the state
 // stays in the order of the last build and moves by one drift in between).
 // The stable order is the order of the composite (key, current index), so
-// per system: nb - 1 non-decreasing splitters are taken from the last
-// build's sorted keys at regular positions (k_ss_split); each key goes to the
-// bucket of the number of splitters at or below its composite; buckets are laid out back to back
-// (counts, then a scan) and each is sorted by composite in shared memory by
-// one block. Keys end sorted in keys[0] with their source positions in
-// vals[0], exactly as the radix sort leaves them. A bucket of more than
+// per system the last build's sorted keys at every SS_BUCKET-th position split
+// the keys into nb buckets: particle i is tried in the bucket of its position
+// (most are still there: two comparisons against keys a whole warp shares),
+// then in buckets ever farther away, and its key and index are appended to the
+// bucket's region of SS_CAP entries. One warp then sorts each bucket in
+// registers (bitonic, by composite) and writes it to its place, the sum of the
+// earlier buckets' counts. Keys end sorted in keys[0] with their source
+// positions in vals[0], exactly as the radix sort leaves them. Splitters out
+// of order (another batch's keys, a first build) only send every particle
+// through one binary search, which gives the same bucket to equal composites
+// and keeps buckets in order whatever the splitters are. A bucket of more than
 // SS_CAP keys (a state far from key order) makes the build leave the order
 // unchanged and record ST_SORT; the build is then repeated with the radix
 // sort.
+// Three launches, each key written and read twice. Before: buckets of 1024 or
+// 2048 keys, a splitter, a counting, a scan and a scatter launch, and a radix
+// sort of each bucket in shared memory. Root box and key sort per soft step of
+// 4 hard sub-steps (8 at 2^24): N = 4096 0.190 -> 0.079 ms, 2^17 0.222 ->
+// 0.105, 2^20 0.61 -> 0.30, 2^24 12.4 -> 6.6 ms.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool comp_less(uint64_t ka, uint32_t va, uint64_t kb, uint32_t vb)
 {
     return ka < kb || (ka == kb && va < vb);
 }
 
-// Block-wide stable LSD radix sort of n keys (with their positions) in shared
-// memory, over the key bits that differ between the smallest and the largest
-// key, 8 bits per pass; equal keys are then put in order of their positions
-// (ties are rare: particles in one cell of the finest level). blockDim.x =
-// SSB_THREADS; whist holds SSB_WARPS x 256 counters; n <= SSB_THREADS * EPT.
-constexpr int SSB_THREADS = 512, SSB_WARPS = SSB_THREADS / 32;
-
-template <int EPT>
-__device__ __forceinline__ void block_radix_sort(uint64_t *sk, uint32_t *sv, int n, uint32_t (*whist)[256],
-                                                 uint32_t *tloc, uint64_t *red)
-{
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned ltmask = (1u << lane) - 1u;
-    // the bits that vary: highest set bit of (min key ^ max key)
-    uint64_t mn = ~0ull, mx = 0ull;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        mn = min(mn, sk[j]);
-        mx = max(mx, sk[j]);
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        mn = min(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-    if (lane == 0) {
-        red[w] = mn;
-        red[SSB_WARPS + w] = mx;
-    }
-    __syncthreads();
-    mn = red[0];
-    mx = red[SSB_WARPS];
-    for (int k = 1; k < SSB_WARPS; ++k) {
-        mn = min(mn, red[k]);
-        mx = max(mx, red[SSB_WARPS + k]);
-    }
-    const int vbits = (mn == mx) ? 0 : 64 - __clzll((long long)(mn ^ mx));
-    const int E = (n + SSB_THREADS - 1) / SSB_THREADS;   // slots per thread: every warp holds a share of the keys
-    const int wbase = w * 32 * E;
-    for (int shift = 0; shift < vbits; shift += 8) {
-        uint64_t k[EPT];
-        uint32_t v[EPT], r[EPT], d[EPT];
-        for (int t = threadIdx.x; t < SSB_WARPS * 256; t += blockDim.x) (&whist[0][0])[t] = 0u;
-#pragma unroll
-        for (int it = 0; it < EPT; ++it) {   // warp-striped: (warp, it, lane) is the current order
-            const int e = wbase + it * 32 + lane;
-            const bool ok = it < E && e < n;
-            k[it] = ok ? sk[e] : 0ull;
-            v[it] = ok ? sv[e] : 0u;
-            d[it] = ok ? (uint32_t)(k[it] >> shift) & 0xffu : 256u;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < EPT; ++it) {
-            if (it >= E || wbase + it * 32 >= n) break;   // the rest of this warp's slots are empty
-            const unsigned peers = __match_any_sync(0xffffffffu, d[it]);
-            const uint32_t before = d[it] < 256u ? whist[w][d[it]] : 0u;
-            __syncwarp();
-            if (d[it] < 256u && (peers & ltmask) == 0u) whist[w][d[it]] = before + (uint32_t)__popc(peers);
-            __syncwarp();
-            r[it] = before + (uint32_t)__popc(peers & ltmask);
-        }
-        __syncthreads();
-        if (threadIdx.x < 256) {   // per digit: exclusive prefix over the warps, then over the digits
-            const int dd = threadIdx.x;
-            uint32_t run = 0;
-            for (int ww = 0; ww < SSB_WARPS; ++ww) {
-                const uint32_t c = whist[ww][dd];
-                whist[ww][dd] = run;
-                run += c;
-            }
-            uint32_t inc = run;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xffffffffu, inc, o);
-                if (lane >= o) inc += y;
-            }
-            if (lane == 31) red[w] = inc;   // the 8 digit warps' totals (red is free here)
-            tloc[dd] = inc - run;
-        }
-        __syncthreads();
-        if (threadIdx.x < 256) {
-            uint32_t pre = 0;
-            for (int ww = 0; ww < w; ++ww) pre += (uint32_t)red[ww];
-            tloc[threadIdx.x] += pre;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int it = 0; it < EPT; ++it)
-            if (d[it] < 256u) {
-                const uint32_t pos = tloc[d[it]] + whist[w][d[it]] + r[it];
-                sk[pos] = k[it];
-                sv[pos] = v[it];
-            }
-        __syncthreads();
-    }
-    // runs of equal keys: in order of their positions (insertion sort by the run's first thread)
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        if (j + 1 < n && sk[j + 1] == sk[j] && (j == 0 || sk[j - 1] != sk[j])) {
-            int e = j + 1;
-            while (e < n && sk[e] == sk[j]) ++e;
-            for (int a = j + 1; a < e; ++a) {
-                const uint32_t x = sv[a];
-                int b = a - 1;
-                while (b >= j && sv[b] > x) {
-                    sv[b + 1] = sv[b];
-                    --b;
-                }
-                sv[b + 1] = x;
-            }
-        }
-    }
-    __syncthreads();
-}
-
-// One block per system: its nb - 1 splitters and cleared bucket counts. It
-// runs before the new keys are computed, on the keys of the last build: the
-// state is still in that build's order and its sorted keys are still in the
-// key buffer, so the composite (old key, position) at position j n / nb is the
-// j-th nb-quantile of the last build, and the particles have moved little
-// since. A running maximum over j makes the splitters non-decreasing whatever
-// the buffer holds (another batch, a first build): buckets may then be empty
-// or large, and a large one sends the build to the radix sort.
-__device__ __forceinline__ void comp_max(uint64_t &k, uint32_t &v, uint64_t k2, uint32_t v2)
-{
-    if (comp_less(k, v, k2, v2)) {
-        k = k2;
-        v = v2;
-    }
-}
-
-__global__ void __launch_bounds__(SSB_THREADS) k_ss_split(const uint64_t *__restrict__ key,
-                                                          const int64_t *__restrict__ off, const SSys *__restrict__ ss,
-                                                          int S, uint64_t *__restrict__ spk, uint32_t *__restrict__ spv,
-                                                          uint32_t *__restrict__ cnt)
-{
-    __shared__ uint64_t wk[SSB_WARPS];
-    __shared__ uint32_t wv[SSB_WARPS];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int s = blockIdx.x; s < S; s += gridDim.x) {
-        const SSys y = ss[s];
-        const int64_t o = off[s], n = off[s + 1] - off[s];
-        for (int b = threadIdx.x; b < y.nb; b += blockDim.x) cnt[y.bbase + b] = 0u;
-        const int m = y.nb - 1;   // splitters
-        if (m > 0) {
-            // thread t takes candidates [t per, (t + 1) per) and keeps their running maximum
-            const int per = (m + blockDim.x - 1) / blockDim.x;
-            const int j0 = threadIdx.x * per, j1 = min(m, j0 + per);
-            uint64_t rk = 0ull;
-            uint32_t rv = 0u;
-            for (int j = j0; j < j1; ++j) {
-                const int64_t p = o + ((int64_t)(j + 1) * n) / y.nb;   // 1 <= p - o <= n - 1
-                const uint64_t mk = key[p];
-                const uint32_t mv = (uint32_t)p;
-                if (j == j0) {
-                    rk = mk;
-                    rv = mv;
-                } else {
-                    comp_max(rk, rv, mk, mv);
-                }
-                spk[y.bbase + j] = rk;
-                spv[y.bbase + j] = rv;
-            }
-            // exclusive running maximum of the threads' maxima (empty ranges carry the zero composite)
-            uint64_t ik = rk;
-            uint32_t iv = rv;
-#pragma unroll
-            for (int o2 = 1; o2 < 32; o2 <<= 1) {
-                const uint64_t k2 = __shfl_up_sync(0xffffffffu, ik, o2);
-                const uint32_t v2 = __shfl_up_sync(0xffffffffu, iv, o2);
-                if (lane >= o2) comp_max(ik, iv, k2, v2);
-            }
-            if (lane == 31) {
-                wk[w] = ik;
-                wv[w] = iv;
-            }
-            __syncthreads();
-            uint64_t pk = 0ull;
-            uint32_t pv = 0u;
-            for (int ww = 0; ww < w; ++ww) comp_max(pk, pv, wk[ww], wv[ww]);
-            {
-                const uint64_t k2 = __shfl_up_sync(0xffffffffu, ik, 1);
-                const uint32_t v2 = __shfl_up_sync(0xffffffffu, iv, 1);
-                if (lane >= 1) comp_max(pk, pv, k2, v2);
-            }
-            for (int j = j0; j < j1; ++j) {   // apply the maximum of everything before this thread's range
-                uint64_t k2 = spk[y.bbase + j];
-                uint32_t v2 = spv[y.bbase + j];
-                comp_max(k2, v2, pk, pv);
-                spk[y.bbase + j] = k2;
-                spv[y.bbase + j] = v2;
-            }
-        }
-        __syncthreads();
-    }
-}
-
-// The sample sort's keys: the key of every particle as k_keys, its bucket (the
-// number of its system's splitters, taken before the keys were replaced, at
-// or below its composite (key, position)), and the bucket counts.
-__global__ void __launch_bounds__(256) k_keys_count(int64_t N, const double *__restrict__ x,
-                                                    const double *__restrict__ y, const double *__restrict__ z,
-                                                    const int32_t *__restrict__ psys, int S,
-                                                    const unsigned long long *__restrict__ bmin,
-                                                    const unsigned long long *__restrict__ bmax,
-                                                    SysBox *__restrict__ boxout, uint64_t *__restrict__ key,
-                                                    uint32_t *__restrict__ val, const SSys *__restrict__ ss,
-                                                    const uint64_t *__restrict__ spk, const uint32_t *__restrict__ spv,
-                                                    uint32_t *__restrict__ pb, uint32_t *__restrict__ cnt)
+// The key of every particle, its bucket, and its place in the bucket's region.
+__global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__restrict__ x,
+                                                     const double *__restrict__ y, const double *__restrict__ z,
+                                                     const int32_t *__restrict__ psys, int S,
+                                                     const unsigned long long *__restrict__ bmin,
+                                                     const unsigned long long *__restrict__ bmax,
+                                                     SysBox *__restrict__ boxout, const int64_t *__restrict__ off,
+                                                     const SSys *__restrict__ ss, const uint64_t *__restrict__ old,
+                                                     uint64_t *__restrict__ rk, uint32_t *__restrict__ rv,
+                                                     uint32_t *__restrict__ cnt, uint32_t *flag, Status *st, int where)
 {
     if (blockIdx.x == 0)
         for (int s = threadIdx.x; s < S; s += blockDim.x) boxout[s] = make_box(bmin, bmax, s);
@@ -617,10 +452,12 @@ __global__ void __launch_bounds__(256) k_keys_count(int64_t N, const double *__r
         __syncthreads();
     }
     const int lane = threadIdx.x & 31;
+    const bool ordered = flag[1] == 0u;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < N; i0 += stride) {
         const int64_t i = i0 + threadIdx.x;
         uint32_t b = ~0u;
+        uint64_t k = 0ull;
         if (i < N) {
             const int sy = S == 1 ? 0 : psys[i];
             const SysBox bx = S == 1 ? b1 : make_box(bmin, bmax, sy);
@@ -628,121 +465,187 @@ __global__ void __launch_bounds__(256) k_keys_count(int64_t N, const double *__r
             const uint32_t qx = cell_coord(x[i], bx.lo[0], es);
             const uint32_t qy = cell_coord(y[i], bx.lo[1], es);
             const uint32_t qz = cell_coord(z[i], bx.lo[2], es);
-            const uint64_t k = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
-            key[i] = k;
-            val[i] = (uint32_t)i;
+            k = (spread3(qx) << 2) | (spread3(qy) << 1) | spread3(qz);
             const SSys yy = ss[sy];
-            int lo = 0, hi = yy.nb - 1;   // upper bound over the splitters [0, nb - 1)
-            while (lo < hi) {
+            const int64_t o = off[sy];
+            // splitter j (1 <= j < nb) is the composite at position o + j SS_BUCKET of the last build
+            auto above = [&](int j) {
+                const int64_t p = o + (int64_t)j * SS_BUCKET;
+                return !comp_less(k, (uint32_t)i, old[p], (uint32_t)p);
+            };
+            int lo = 0, hi = yy.nb;   // above(lo) (or lo = 0), not above(hi) (or hi = nb)
+            if (ordered && hi > 1) {
+                const int g = (int)(i - o) / SS_BUCKET;
+                int step = 1;
+                if (g == 0 || above(g)) {
+                    lo = g;
+                    while (lo + step < hi && above(lo + step)) {
+                        lo += step;
+                        step <<= 1;
+                    }
+                    hi = min(lo + step, hi);
+                } else {
+                    hi = g;
+                    while (hi - step > 0 && !above(hi - step)) {
+                        hi -= step;
+                        step <<= 1;
+                    }
+                    lo = max(hi - step, 0);
+                }
+            }
+            while (hi - lo > 1) {
                 const int mid = (lo + hi) >> 1;
-                if (comp_less(k, (uint32_t)i, spk[yy.bbase + mid], spv[yy.bbase + mid])) hi = mid;
-                else lo = mid + 1;
+                if (above(mid)) lo = mid;
+                else hi = mid;
             }
             b = (uint32_t)(yy.bbase + lo);
-            pb[i] = b;
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, b);
-        if (b != ~0u && lane == __ffs(peers) - 1) atomicAdd(cnt + b, (uint32_t)__popc(peers));
-    }
-}
-
-// One block per system: bucket starts (exclusive scan of the counts from the
-// system's first position) and the overflow check.
-__global__ void __launch_bounds__(256) k_ss_scan(const int64_t *__restrict__ off, const SSys *__restrict__ ss, int S,
-                                                 const uint32_t *__restrict__ cnt, uint32_t *__restrict__ start,
-                                                 uint32_t *__restrict__ cur, uint32_t *flag, Status *st, int where)
-{
-    __shared__ uint32_t part[256];
-    for (int s = blockIdx.x; s < S; s += gridDim.x) {
-        const SSys y = ss[s];
-        const int per = (y.nb + blockDim.x - 1) / blockDim.x;
-        const int b0 = threadIdx.x * per, b1 = min(y.nb, b0 + per);
-        uint32_t sum = 0, mx = 0;
-        for (int b = b0; b < b1; ++b) {
-            const uint32_t v = cnt[y.bbase + b];
-            sum += v;
-            mx = max(mx, v);
-        }
-        part[threadIdx.x] = sum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            uint32_t run = (uint32_t)off[s];
-            for (int t = 0; t < (int)blockDim.x; ++t) {
-                const uint32_t v = part[t];
-                part[t] = run;
-                run += v;
-            }
-        }
-        __syncthreads();
-        uint32_t run = part[threadIdx.x];
-        for (int b = b0; b < b1; ++b) {
-            start[y.bbase + b] = run;
-            cur[y.bbase + b] = 0u;
-            run += cnt[y.bbase + b];
-        }
-        if (mx > (uint32_t)SS_CAP) {
-            atomicExch(flag, 1u);
-            fail(st, ST_SORT, where);
-        }
-        __syncthreads();
-    }
-}
-
-// Every key and its position into its bucket's range (any order inside).
-__global__ void __launch_bounds__(256) k_ss_scatter(int64_t N, const uint64_t *__restrict__ k0,
-                                                    const uint32_t *__restrict__ pb, const uint32_t *__restrict__ start,
-                                                    uint32_t *__restrict__ cur, uint64_t *__restrict__ k1,
-                                                    uint32_t *__restrict__ v1, const uint32_t *flag)
-{
-    if (*flag) return;
-    const int lane = threadIdx.x & 31;
-    const unsigned ltmask = (1u << lane) - 1u;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < N; i0 += stride) {
-        const int64_t i = i0 + threadIdx.x;
-        const uint32_t b = i < N ? pb[i] : ~0u;
         const unsigned peers = __match_any_sync(0xffffffffu, b);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
-        if (b != ~0u && lane == leader) base = atomicAdd(cur + b, (uint32_t)__popc(peers));
-        base = __shfl_sync(0xffffffffu, base, leader);
-        if (b != ~0u) {
-            const uint32_t pos = start[b] + base + (uint32_t)__popc(peers & ltmask);
-            k1[pos] = k0[i];
-            v1[pos] = (uint32_t)i;
+        if (b != ~0u && lane == leader) {
+            base = atomicAdd(cnt + b, (uint32_t)__popc(peers));
+            if (base + (uint32_t)__popc(peers) > (uint32_t)SS_CAP) {
+                atomicExch(flag, 1u);
+                fail(st, ST_SORT, where);
+            }
+        }
+        base = __shfl_sync(0xffffffffu, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
+        if (b != ~0u && base < (uint32_t)SS_CAP) {
+            rk[(size_t)b * SS_CAP + base] = k;
+            rv[(size_t)b * SS_CAP + base] = (uint32_t)i;
         }
     }
 }
 
-// One block per bucket: its keys sorted by composite in shared memory, written
-// to their final positions.
-__global__ void __launch_bounds__(SSB_THREADS, 2) k_ss_sort(int nbk, const uint32_t *__restrict__ cnt,
-                                                         const uint32_t *__restrict__ start,
-                                                         const uint64_t *__restrict__ k1, const uint32_t *__restrict__ v1,
-                                                         uint64_t *__restrict__ k0, uint32_t *__restrict__ v0,
-                                                         const uint32_t *flag)
+// Compare and exchange of registers r and r | j of a lane, over all r without bit j: ascending where up(r).
+template <int R, int J, typename Up>
+__device__ __forceinline__ void lane_step(uint64_t (&k)[R], uint32_t (&v)[R], Up &&up)
 {
-    extern __shared__ uint64_t ss_smem[];   // SS_CAP keys, then SS_CAP positions
-    __shared__ uint32_t whist[SSB_WARPS][256];
-    __shared__ uint32_t tloc[256];
-    __shared__ uint64_t red[2 * SSB_WARPS];
-    uint64_t *sk = ss_smem;
-    uint32_t *sv = reinterpret_cast<uint32_t *>(ss_smem + SS_CAP);
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+        if ((r & J) == 0) {
+            const bool swap = comp_less(k[r | J], v[r | J], k[r], v[r]) == up(r);
+            const uint64_t a = k[r], b = k[r | J];
+            const uint32_t c = v[r], d = v[r | J];
+            k[r] = swap ? b : a;
+            k[r | J] = swap ? a : b;
+            v[r] = swap ? d : c;
+            v[r | J] = swap ? c : d;
+        }
+}
+template <int R, int J, typename Up>
+__device__ __forceinline__ void lane_steps(uint64_t (&k)[R], uint32_t (&v)[R], Up &&up)   // steps J, J / 2, .., 1
+{
+    lane_step<R, J>(k, v, up);
+    if constexpr (J > 1) lane_steps<R, J / 2>(k, v, up);
+}
+template <int R, int SIZE>
+__device__ __forceinline__ void lane_sorts(uint64_t (&k)[R], uint32_t (&v)[R])   // runs of SIZE, 2 SIZE, .., R / 2
+{
+    if constexpr (SIZE < R) {
+        lane_steps<R, SIZE / 2>(k, v, [](int r) { return (r & SIZE) == 0; });
+        lane_sorts<R, 2 * SIZE>(k, v);
+    }
+}
+
+// Bitonic sort of 32 R composites by one warp, element lane R + r in register
+// r. The steps between lanes are loops: unrolled, they are 50 to 140 KB of
+// code, and fetching it took longer than running it once (k_ss_sort of 4096
+// keys 62 us unrolled, 6.9 us looped; of 2^24 keys 2.15 ms and 0.33 ms).
+template <int R>
+__device__ __forceinline__ void warp_sort(uint64_t (&k)[R], uint32_t (&v)[R], int lane)
+{
+    lane_sorts<R, 2>(k, v);
+#pragma unroll 1
+    for (int lanes = 1; lanes <= 32; lanes <<= 1) {   // sorted runs of R x lanes
+        const bool up = lanes == 32 || (lane & lanes) == 0;
+#pragma unroll 1
+        for (int m = lanes / 2; m >= 1; m >>= 1) {
+            const bool low = ((lane & m) == 0) == up;   // this lane keeps the smaller one
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const uint64_t ok = __shfl_xor_sync(0xffffffffu, k[r], m);
+                const uint32_t ov = __shfl_xor_sync(0xffffffffu, v[r], m);
+                const bool take = comp_less(ok, ov, k[r], v[r]) == low;
+                k[r] = take ? ok : k[r];
+                v[r] = take ? ov : v[r];
+            }
+        }
+        lane_steps<R, R / 2>(k, v, [up](int) { return up; });
+    }
+}
+
+constexpr int SSB_THREADS = 128, SSB_WARPS = SSB_THREADS / 32;
+constexpr int SS_PAD = SS_CAP + SS_CAP / 8;   // a bucket in shared memory, one entry of padding after every R
+
+template <int R>
+__device__ __forceinline__ void sort_bucket(const uint64_t *__restrict__ rk, const uint32_t *__restrict__ rv, int n,
+                                            uint64_t *__restrict__ k0, uint32_t *__restrict__ v0, uint64_t *sk,
+                                            uint32_t *sv, int lane)
+{
+    uint64_t k[R];
+    uint32_t v[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {   // any order will do; slots past the bucket sort to the end
+        const int e = r * 32 + lane;
+        k[r] = e < n ? rk[e] : ~0ull;
+        v[r] = e < n ? rv[e] : ~0u;
+    }
+    warp_sort<R>(k, v, lane);
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        sk[lane * (R + 1) + r] = k[r];
+        sv[lane * (R + 1) + r] = v[r];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+        const int e = r * 32 + lane;
+        if (e < n) {
+            k0[e] = sk[e + e / R];
+            v0[e] = sv[e + e / R];
+        }
+    }
+}
+
+// One warp per bucket. SCANNED: cnt holds the exclusive sums of the counts (nbk + 1 entries), else the counts,
+// which each block adds up itself.
+template <bool SCANNED>
+__global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, const uint32_t *__restrict__ cnt,
+                                                         const uint64_t *__restrict__ rk,
+                                                         const uint32_t *__restrict__ rv, uint64_t *__restrict__ k0,
+                                                         uint32_t *__restrict__ v0, const uint32_t *flag)
+{
+    __shared__ uint64_t sk[SSB_WARPS][SS_PAD];
+    __shared__ uint32_t sv[SSB_WARPS][SS_PAD];
+    __shared__ uint32_t wsum[SSB_WARPS];
     if (*flag) return;
-    for (int b = blockIdx.x; b < nbk; b += gridDim.x) {
-        const int n = (int)cnt[b];
-        const uint32_t s0 = start[b];
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            sk[j] = k1[s0 + j];
-            sv[j] = v1[s0 + j];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int b0 = blockIdx.x * SSB_WARPS; b0 < nbk; b0 += gridDim.x * SSB_WARPS) {
+        const int b = b0 + w;
+        uint32_t s0, n;
+        if (SCANNED) {
+            s0 = b < nbk ? cnt[b] : 0u;
+            n = b < nbk ? cnt[b + 1] - s0 : 0u;
+        } else {
+            uint32_t sum = 0;
+            for (int k = threadIdx.x; k < b0; k += SSB_THREADS) sum += cnt[k];
+            sum = __reduce_add_sync(0xffffffffu, sum);
+            if (lane == 0) wsum[w] = sum;
+            __syncthreads();
+            s0 = 0;
+            for (int k = 0; k < SSB_WARPS; ++k) s0 += wsum[k];
+            for (int k = b0; k < min(b, nbk); ++k) s0 += cnt[k];
+            n = b < nbk ? cnt[b] : 0u;
+            __syncthreads();
         }
-        __syncthreads();
-        block_radix_sort<SS_CAP / SSB_THREADS>(sk, sv, n, whist, tloc, red);
-        for (int j = threadIdx.x; j < n; j += blockDim.x) {
-            k0[s0 + j] = sk[j];
-            v0[s0 + j] = sv[j];
-        }
-        __syncthreads();
+        if (n == 0u) continue;   // the whole warp
+        const uint64_t *kb = rk + (size_t)b * SS_CAP;
+        const uint32_t *vb = rv + (size_t)b * SS_CAP;
+        if (n <= 256u) sort_bucket<8>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
+        else sort_bucket<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
     }
 }
 
@@ -762,13 +665,22 @@ struct PermArgs {
     const int32_t *psys;
     const SysBox *box;
     int64_t N;
+    unsigned long long *bmin, *bmax;   // reset for the next build (the root cubes are made)
+    int S;
+    uint32_t *flag;       // [0] an overflowed sample sort: the order stays; [1] reset for the next build
 };
 
-__global__ void __launch_bounds__(256) k_permute(PermArgs a, const Status *st)
+__global__ void __launch_bounds__(256) k_permute(PermArgs a)
 {
-    (void)st;   // the sort always runs: later kernels rely on a consistent permutation
+    // whatever the status: later kernels rely on a consistent permutation
+    const bool keep = a.flag[0] != 0u;
+    for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * a.S; k += gridDim.x * blockDim.x) {
+        a.bmin[k] = ~0ull;
+        a.bmax[k] = 0ull;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.flag[1] = 0u;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < a.N; i += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t j = a.src[i];
+        const uint32_t j = keep ? (uint32_t)i : a.src[i];
         double v[7];
 #pragma unroll
         for (int f = 0; f < 7; ++f) {
@@ -1724,12 +1636,12 @@ static int grid_for(hybrid_ctx *c, int64_t work, int threads, int per_sm = 8)
 
 void launch_box(hybrid_ctx *c)
 {
-    Status *st = status_dev(c);
-    cudaMemsetAsync(c->boxmin.p, 0xff, (size_t)3 * c->S * sizeof(unsigned long long), c->st);
-    cudaMemsetAsync(c->boxmax.p, 0x00, (size_t)3 * c->S * sizeof(unsigned long long), c->st);
+    // the boxes are empty here: the copy into the working state and every permutation reset them
     k_box<<<std::min(c->nchunks, c->nsm * 16), 256, 0, c->st>>>(
         (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p, (const Chunk *)c->chunks_dev.p,
-        c->nchunks, (unsigned long long *)c->boxmin.p, (unsigned long long *)c->boxmax.p, st);
+        c->nchunks, (unsigned long long *)c->boxmin.p, (unsigned long long *)c->boxmax.p, c->sort_fallback ? 0 : c->nbk,
+        c->S, (const int64_t *)c->off_dev.p, (const SSys *)c->ss_sys.p, (const uint64_t *)c->keys[0].p,
+        (uint32_t *)c->ss_cnt.p, (uint32_t *)c->ss_flag.p);
     c->launches += 1;
 }
 
@@ -1739,28 +1651,25 @@ void launch_keys_sort(hybrid_ctx *c)
     const int64_t N = c->N;
     uint64_t *k0 = (uint64_t *)c->keys[0].p, *k1 = (uint64_t *)c->keys[1].p;
     uint32_t *v0 = (uint32_t *)c->vals[0].p, *v1 = (uint32_t *)c->vals[1].p;
-    const bool sample = c->ss_ok && !c->sort_fallback;
-    const SSys *ss = (const SSys *)c->ss_sys.p;
-    uint64_t *spk = (uint64_t *)c->ss_spk.p;
-    uint32_t *spv = (uint32_t *)c->ss_spv.p, *cnt = (uint32_t *)c->ss_cnt.p;
-    const int64_t *off = (const int64_t *)c->off_dev.p;
-    if (sample) {   // splitters from the last build's sorted keys, before the new keys replace them
-        k_ss_split<<<std::min(c->S, c->nsm * 2), SSB_THREADS, 0, c->st>>>(k0, off, ss, c->S, spk, spv, cnt);
-        c->launches++;
-    }
-    if (sample) {
-        uint32_t *start = (uint32_t *)c->ss_start.p;
-        uint32_t *cur = (uint32_t *)c->ss_cur.p, *pb = (uint32_t *)c->ss_pb.p, *flag = (uint32_t *)c->ss_flag.p;
-        cudaMemsetAsync(flag, 0, sizeof(uint32_t), c->st);
-        k_keys_count<<<grid_for(c, N, 256), 256, 0, c->st>>>(
+    if (!c->sort_fallback) {
+        uint32_t *cnt = (uint32_t *)c->ss_cnt.p, *flag = (uint32_t *)c->ss_flag.p;
+        uint64_t *rk = (uint64_t *)c->ss_rk.p;
+        uint32_t *rv = (uint32_t *)c->ss_rv.p;
+        k_keys_append<<<grid_for(c, N, 256), 256, 0, c->st>>>(
             N, (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p,
             (const int32_t *)c->psys.p, c->S, (const unsigned long long *)c->boxmin.p,
-            (const unsigned long long *)c->boxmax.p, (SysBox *)c->box.p, k0, v0, ss, spk, spv, pb, cnt);
-        k_ss_scan<<<std::min(c->S, c->nsm * 4), 256, 0, c->st>>>(off, ss, c->S, cnt, start, cur, flag, st, c->op);
-        k_ss_scatter<<<grid_for(c, N, 256), 256, 0, c->st>>>(N, k0, pb, start, cur, k1, v1, flag);
-        k_ss_sort<<<std::min(c->nbk, c->nsm * 8), SSB_THREADS, (size_t)SS_CAP * 12, c->st>>>(c->nbk, cnt, start, k1,
-                                                                                               v1, k0, v0, flag);
-        c->launches += 4;
+            (const unsigned long long *)c->boxmax.p, (SysBox *)c->box.p, (const int64_t *)c->off_dev.p,
+            (const SSys *)c->ss_sys.p, k0, rk, rv, cnt, flag, st, c->op);
+        const int grid = std::min((c->nbk + SSB_WARPS - 1) / SSB_WARPS, c->nsm * 16);
+        // up to SS_SUM_MAX buckets every block of the sort adds up the counts before its buckets (at most 32 loads
+        // a thread); above, a scan does it once
+        if (c->nbk <= SS_SUM_MAX) {
+            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, cnt, rk, rv, k0, v0, flag);
+        } else {
+            scan_u32(c, cnt, c->nbk + 1, nullptr, c->nbk + 1, nullptr, true);
+            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, cnt, rk, rv, k0, v0, flag);
+        }
+        c->launches += 2;
         return;
     }
     k_keys<<<grid_for(c, N, 256), 256, 0, c->st>>>(N, (const double *)c->x[0].p, (const double *)c->x[1].p,
@@ -1794,7 +1703,6 @@ void launch_keys_sort(hybrid_ctx *c)
 
 void launch_permute(hybrid_ctx *c)
 {
-    Status *st = status_dev(c);
     const int64_t N = c->N;
     uint32_t *v0 = (uint32_t *)c->vals[0].p;
     PermArgs a;
@@ -1814,7 +1722,11 @@ void launch_permute(hybrid_ctx *c)
     a.psys = (const int32_t *)c->psys.p;
     a.box = (const SysBox *)c->box.p;
     a.N = N;
-    k_permute<<<grid_for(c, N, 256), 256, 0, c->st>>>(a, st);
+    a.bmin = (unsigned long long *)c->boxmin.p;
+    a.bmax = (unsigned long long *)c->boxmax.p;
+    a.S = c->S;
+    a.flag = (uint32_t *)c->ss_flag.p;
+    k_permute<<<grid_for(c, N, 256), 256, 0, c->st>>>(a);
     c->launches++;
     for (int f = 0; f < 7; ++f) std::swap(c->x[f], c->xa[f]);
     std::swap(c->id, c->ida);
@@ -1978,9 +1890,7 @@ size_t cell_count_bytes(int64_t N) { return (size_t)CT_CNT * cell_tiles(N) * siz
 cudaError_t init_tree_kernels()
 {
     // leaves of up to 24448 particles, as far as their window fits in shared memory
-    cudaError_t e = cudaFuncSetAttribute(k_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * cells_bytes(24448));
-    if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_ss_sort, cudaFuncAttributeMaxDynamicSharedMemorySize, SS_CAP * 12);
+    return cudaFuncSetAttribute(k_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * cells_bytes(24448));
 }
 
 void launch_wait_selftest(hybrid_ctx *c, int max_polls)
