@@ -59,8 +59,8 @@ typedef enum {
  *          coordinates relative to each sink group (state stays FP64)
  * mac      0: opening angle theta; 1: absolute MAC with a_err (Eq. 5-6)
  * threads_per_group: lanes that share one copy of a sink group in the FP32
- *          pair kernels; each lane then keeps ceil(n_crit / threads_per_group)
- *          sinks in registers (1, 2, 4 or 8; 4 at most in the near kernel).
+ *          far pair kernel; each lane then keeps ceil(n_crit /
+ *          threads_per_group) sinks in registers (1, 2, 4 or 8).
  *          0 = built-in default.
  * tile_depth: shared-memory staging depth of the FP32 far pair kernel: source
  *          gathers run tile_depth - 1 tiles of 64 list entries ahead of their

@@ -4,18 +4,20 @@
 //   cells and far particles: K = 0 for every pair (the walk's R2 + b_max
 //     test), so they only add F to the soft force ("far" kernel);
 //   near particles: the only pairs where K can be non-zero; one pass adds
-//     F (1 - K) to the soft force and F K to the hard force ("near" kernel).
+//     F (1 - K) to the soft force and F K to the hard force ("near" kernel,
+//     k_near).
 //
 // FP32 form. Work item = (group, run of at most item_len consecutive entries
 // of one of the group's lists), written by the walk and pulled from a global
-// counter. One warp per work item: sources are staged, 64 at a time, into the
+// counter. Near kernel: one block per work item, see k_near. Far kernel: one
+// warp per work item; sources are staged, 64 at a time, into the
 // warp's shared-memory tile relative to the group's reference point (the hi
 // part of its first sink: on the hi grid, so hi - c is exact), as {x, y, z, m}
-// or, for far sources, in the expanded form of body_exp2; the gathers run
+// or in the expanded form of body_exp2; the gathers run
 // ahead of their use (see the staging ring). A group of n sinks uses
 // lpc = ceil(n / KS) lanes per copy with KS sinks per lane in registers, and
 // copies = 32 / lpc copies of the group split the sources (source j goes to
-// copy j mod copies) and are added at the end. In the far kernel, when that
+// copy j mod copies) and are added at the end. When that
 // leaves many lanes idle (e.g. 72 sinks, KS = 4: 18 lanes, one copy), the
 // sinks are taken in rounds whose lanes per copy are a power of two (64
 // sinks on 2 copies of 16 lanes, then 8 sinks on 16 copies of 2 lanes):
@@ -36,7 +38,7 @@ namespace {
 constexpr int PAIR_THREADS = 128;
 constexpr int FAR_SPLIT_PCT = 75;   // far kernel: a round below this fill of its sink slots is split (see below)
 constexpr int PAIR_WARPS = PAIR_THREADS / 32;
-constexpr int NEAR_MIN_BLOCKS = 4;  // near kernels: resident blocks of PAIR_THREADS per SM (see k_pair_f32)
+constexpr int NEAR_MIN_BLOCKS = 8;  // near kernel: resident blocks of PAIR_THREADS per SM (64 registers, see k_near)
 constexpr int TILE = 64;
 
 struct PairArgs {
@@ -62,23 +64,6 @@ struct HardC {
 };
 
 // ---- FP32 bodies ----------------------------------------------------------
-// weight 1 (cells, far particles). GUARD: r^2 + eps^2 may be 0 (eps = 0 and a
-// self pair, only possible without a hard part).
-template <bool GUARD>
-__device__ __forceinline__ void body_far(const float4 q, float sx, float sy, float sz, float eps2, float &ax, float &ay,
-                                         float &az)
-{
-    const float dx = q.x - sx, dy = q.y - sy, dz = q.z - sz;
-    const float r2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-    float ri = rsqrtf(r2);
-    if (GUARD) ri = r2 > 0.0f ? ri : 0.0f;
-    const float mr = q.w * ri;
-    const float f = mr * (ri * ri);
-    ax = fmaf(dx, f, ax);
-    ay = fmaf(dy, f, ay);
-    az = fmaf(dz, f, az);
-}
-
 // Eq. (10) with Y from D = R2^2 - r^2: Y = D / ((R2 + r)(R2 - R1)), clamped
 // to [0, 1]; K = Y^6 (10 + Y^2 (-15 + 6 Y^2)), exactly 1 at Y = 1 and 0 at Y = 0.
 // D is rebuilt in double-float arithmetic from the grid-aligned hi parts
@@ -103,38 +88,6 @@ __device__ __forceinline__ float dll_K_precise(float r2u, float hx, float hy, fl
     return (Y2 * Y2 * Y2) * fmaf(Y2, fmaf(6.0f, Y2, -15.0f), 10.0f);
 }
 
-// near particle: soft += F (1 - K), hard += F K. (dx, dy, dz) = source - sink
-// and r2u = |.|^2 are computed by the caller; hh/ll are the source's raw hi
-// and lo parts and (shx, ..), (slx, ..) the sink's: hi differences are exact.
-template <bool SOFT, bool HARD>
-__device__ __forceinline__ void near_finish(float w, float dx, float dy, float dz, float r2u, const float4 &hh,
-                                            const float4 &ll, float shx, float shy, float shz, float slx, float sly,
-                                            float slz, const HardC &H, float &sax, float &say, float &saz, float &hax,
-                                            float &hay, float &haz)
-{
-    const bool inside = r2u < H.R2sq;
-    if (!SOFT && !inside) return;
-    const float r2 = r2u + H.eps2;
-    const float ri = r2 > 0.0f ? rsqrtf(r2) : 0.0f;
-    const float f = w * ri * (ri * ri);
-    float K = 0.0f;
-    if (inside)
-        K = dll_K_precise(r2u, __fsub_rn(hh.x, shx), __fsub_rn(hh.y, shy), __fsub_rn(hh.z, shz),
-                          __fsub_rn(ll.x, slx), __fsub_rn(ll.y, sly), __fsub_rn(ll.z, slz), H);
-    if (SOFT) {
-        const float fs = f * (1.0f - K);
-        sax = fmaf(dx, fs, sax);
-        say = fmaf(dy, fs, say);
-        saz = fmaf(dz, fs, saz);
-    }
-    if (HARD) {
-        const float fh = f * K;
-        hax = fmaf(dx, fh, hax);
-        hay = fmaf(dy, fh, hay);
-        haz = fmaf(dz, fh, haz);
-    }
-}
-
 __device__ __forceinline__ int64_t next_item(unsigned long long *counter, int lane)
 {
     unsigned long long g = 0;
@@ -148,23 +101,20 @@ __device__ __forceinline__ int64_t next_item(unsigned long long *counter, int la
 constexpr uint32_t MULTI = ITEM_MULTI;
 
 // Raw sources (hi, lo float4 pairs of cells or particles) are gathered into a
-// ring of NST shared-memory stages (the staging depth, 2 to 4; the near
-// kernel uses 3) with 16-byte cp.async copies issued NST - 1 tiles ahead,
+// ring of NST shared-memory stages (the staging depth, 2 to 4) with 16-byte cp.async copies issued NST - 1 tiles ahead,
 // from list indices loaded one tile before that; only the rebasing to the
 // group's reference point (one pass per staged entry, by the lane that copied
 // it) stands between a landed stage and its use.
 constexpr int PER = TILE / 32;
 
-// Rebased sources: the near kernel keeps {x, y, z, m} in tile[0, TILE); the
-// far kernel keeps each source twice over, {x, x, y, y} {z, z, m, m}, for the
-// packed two-sink arithmetic, or in the expanded form of exp_tile, two float4
-// per entry, in tile[0, 2 PADT): entries from nt up to PADT = TILE + 32 are
-// zero-mass sources (all zero in either form).
+// Rebased sources of the far kernel: each source twice over, {x, x, y, y} {z, z,
+// m, m}, for the packed two-sink arithmetic, or in the expanded form of
+// exp_tile, two float4 per entry, in tile[0, 2 PADT): entries from nt up to
+// PADT = TILE + 32 are zero-mass sources (all zero in either form).
 constexpr int PADT = TILE + 32;
-static_assert(2 * PADT >= 3 * TILE, "the near filter keeps three float4 rows of TILE entries");
-template <int NST>
+template <int NST, int TILE4>
 struct WarpStage {
-    float4 tile[2 * PADT];
+    float4 tile[TILE4];
     float4 rh[NST][TILE];     // raw hi parts (cells: nA, particles: phi)
     float4 rl[NST][TILE];     // raw lo parts (cells: nB, particles: plo)
 };
@@ -212,26 +162,11 @@ struct ItemSrc {
     }
 };
 
-// Runs the staging pipeline over the item's entries and calls
-// body(stage, nt) once per tile, after the tile has been rebased into S.tile.
-// Box of a warp's sinks (group-relative FP32) for the near filter.
-struct SinkBox {
-    float lo[3], hi[3], R2sq;
-};
-
-// Staging modes: FAR_PACKED writes every source twice over for the packed far
-// sweep and calls body(stage, nt); FAR_EXP writes the expanded form of
-// exp_tile and calls body(stage, nt). NEAR_FILTER keeps a source for the near
-// body only when its distance to the sinks' box is below R2 (computed like the
-// pair distance, so no pair with r < R2 is dropped): kept sources go to
-// tile[0, n_in) with their rebased hi part at tile[TILE + j] and raw lo part at
-// tile[2 TILE + j]; the others (K = 0 for every sink) to tile[TILE - n_out,
-// TILE); then body(n_in, n_out).
-enum { FAR_PACKED = 0, NEAR_FILTER = 1, FAR_EXP = 2 };
-
-template <int SMODE, int NST, typename Stage, typename Body>
-__device__ __forceinline__ void pipeline(const PairArgs &a, const ItemSrc &src, Stage &S, int lane,
-                                         float crx, float cry, float crz, const SinkBox &sb, Body &&body)
+// Runs the staging pipeline over the item's entries and calls body(stage, nt)
+// once per tile: the tile's nt raw entries have landed in rh / rl[stage], entry
+// e from lane e % 32, which alone may read it before a __syncwarp.
+template <int NST, typename Stage, typename Body>
+__device__ __forceinline__ void pipeline(const PairArgs &a, const ItemSrc &src, Stage &S, int lane, Body &&body)
 {
     static_assert(NST >= 2 && NST <= 4, "staging depth");
     const uint32_t ne = src.e1 - src.e0;
@@ -250,68 +185,33 @@ __device__ __forceinline__ void pipeline(const PairArgs &a, const ItemSrc &src, 
         src.issue<NST>(a, S, t + NST - 1, lane, i0);   // no copies past the end, but one group per tile
         if (t + NST < ntile) src.load_idx(a, t + NST, lane, i0);
         cp_wait<NST - 1>();                       // this lane's copies of tile t have landed
-        const int st = t % NST;
-        const int nt = (int)min((uint32_t)TILE, ne - (uint32_t)(t * TILE));
-        if (SMODE == FAR_PACKED || SMODE == FAR_EXP) {
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {   // entries past nt become zero-mass sources
-                const int el = u * 32 + lane;
-                float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-                if (el < nt) {
-                    const float4 h = S.rh[st][el], l = S.rl[st][el];
-                    v = make_float4((h.x - crx) + l.x, (h.y - cry) + l.y, (h.z - crz) + l.z, h.w);
-                }
-                if (SMODE == FAR_PACKED) {
-                    S.tile[2 * el] = make_float4(v.x, v.x, v.y, v.y);
-                    S.tile[2 * el + 1] = make_float4(v.z, v.z, v.w, v.w);
-                } else {
-                    const float c = fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z));
-                    S.tile[2 * el] = make_float4(-2.0f * v.x, -2.0f * v.y, -2.0f * v.z, c);
-                    S.tile[2 * el + 1] = make_float4(v.w * v.x, v.w * v.y, v.w * v.z, v.w);
-                }
-            }
-            __syncwarp();
-            body(st, nt);
-        } else {
-            float4 v[PER], vh[PER], vl[PER];
-            bool keep[PER], out[PER];
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {
-                const int el = u * 32 + lane;
-                keep[u] = out[u] = false;
-                if (el < nt) {
-                    const float4 h = S.rh[st][el], l = S.rl[st][el];
-                    vh[u] = make_float4(h.x - crx, h.y - cry, h.z - crz, 0.0f);
-                    vl[u] = l;
-                    v[u] = make_float4(vh[u].x + l.x, vh[u].y + l.y, vh[u].z + l.z, h.w);
-                    const float gx = fmaxf(fmaxf(sb.lo[0] - v[u].x, v[u].x - sb.hi[0]), 0.0f);
-                    const float gy = fmaxf(fmaxf(sb.lo[1] - v[u].y, v[u].y - sb.hi[1]), 0.0f);
-                    const float gz = fmaxf(fmaxf(sb.lo[2] - v[u].z, v[u].z - sb.hi[2]), 0.0f);
-                    keep[u] = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < sb.R2sq;
-                    out[u] = !keep[u];
-                }
-            }
-            const unsigned ltm = (1u << lane) - 1u;
-            const unsigned k0 = __ballot_sync(0xffffffffu, keep[0]), k1 = __ballot_sync(0xffffffffu, keep[1]);
-            const unsigned o0 = __ballot_sync(0xffffffffu, out[0]), o1 = __ballot_sync(0xffffffffu, out[1]);
-            const int n_in = __popc(k0) + __popc(k1), n_out = __popc(o0) + __popc(o1);
-#pragma unroll
-            for (int u = 0; u < PER; ++u) {   // order kept within each part
-                if (keep[u]) {
-                    const int j = u == 0 ? __popc(k0 & ltm) : __popc(k0) + __popc(k1 & ltm);
-                    S.tile[j] = v[u];
-                    S.tile[TILE + j] = vh[u];
-                    S.tile[2 * TILE + j] = vl[u];
-                } else if (out[u]) {
-                    const int j = u == 0 ? __popc(o0 & ltm) : __popc(o0) + __popc(o1 & ltm);
-                    S.tile[TILE - n_out + j] = v[u];
-                }
-            }
-            __syncwarp();
-            body(n_in, n_out);
-        }
+        body(t % NST, (int)min((uint32_t)TILE, ne - (uint32_t)(t * TILE)));
         __syncwarp();
     }
+}
+
+// The far kernel's tile from a stage: every source twice over, or expanded (EXP).
+template <bool EXP, typename Stage>
+__device__ __forceinline__ void stage_far(Stage &S, int st, int nt, int lane, float crx, float cry, float crz)
+{
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {   // entries past nt become zero-mass sources
+        const int el = u * 32 + lane;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (el < nt) {
+            const float4 h = S.rh[st][el], l = S.rl[st][el];
+            v = make_float4((h.x - crx) + l.x, (h.y - cry) + l.y, (h.z - crz) + l.z, h.w);
+        }
+        if (!EXP) {
+            S.tile[2 * el] = make_float4(v.x, v.x, v.y, v.y);
+            S.tile[2 * el + 1] = make_float4(v.z, v.z, v.w, v.w);
+        } else {
+            const float c = fmaf(v.x, v.x, fmaf(v.y, v.y, v.z * v.z));
+            S.tile[2 * el] = make_float4(-2.0f * v.x, -2.0f * v.y, -2.0f * v.z, c);
+            S.tile[2 * el + 1] = make_float4(v.w * v.x, v.w * v.y, v.w * v.z, v.w);
+        }
+    }
+    __syncwarp();
 }
 
 // sums of the copies into copy 0: a butterfly over the copies when they fill the warp (lpc a power of
@@ -384,8 +284,9 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
     return d;
 }
 
-// the body of body_far for two sinks (S*) against one source given twice
-// over (X2 = {x, x}, ..): the same roundings per lane
+// Weight 1 (cells, far particles): two sinks (S*) against one source given
+// twice over (X2 = {x, x}, ..). GUARD: r^2 + eps^2 may be 0 (eps = 0 and a self
+// pair, only possible without a hard part).
 template <bool GUARD>
 __device__ __forceinline__ void body_far2(uint64_t X2, uint64_t Y2, uint64_t Z2, uint64_t M2, uint64_t SX, uint64_t SY,
                                           uint64_t SZ, uint64_t E2, uint64_t &AX, uint64_t &AY, uint64_t &AZ)
@@ -437,7 +338,7 @@ __device__ __forceinline__ void far_tile(const Stage &S, int nt, int copy, int c
 // sum_j m_j r_j^-3 (s_j - k) = sum_j r_j^-3 (m_j s_j) - k sum_j r_j^-3 m_j, so
 // a source stages {-2s, |s|^2, m s, m} and a pair costs the sum c + Q, three
 // fma for r^2, rsqrt, two mul for r^-3 and four fma: 10 FP32 lane operations
-// against 12 for body_far. The rounding of r^2 is at most about
+// against 12 for body_far2. The rounding of r^2 is at most about
 // 4 u (|s| + |k|)^2 <= 4 u (r + 2 |k|)^2 (u = 2^-24). With a hard part the walk
 // takes a cell only beyond R2 + b_max (and beyond its opening radius) and a far
 // particle only beyond R2 of the sinks' box, so r >= R2, and with every sink
@@ -490,15 +391,35 @@ __device__ __forceinline__ void exp_tile(const Stage &S, int nt, int copy, int c
     }
 }
 
-// NEAR = false: cells + far particles -> soft. NEAR = true: near particles ->
-// soft (1 - K) and/or hard (K), by SOFT/HARD.
-// The near kernels wait on the latency of their loads (work items, sinks, list
-// entries): they are held to 4 blocks of 128 threads per SM (at most 128
-// registers), one block more than they would use freely.
-template <int KS, bool NEAR, bool SOFT, bool HARD, int NST>
-__global__ void __launch_bounds__(PAIR_THREADS, NEAR ? NEAR_MIN_BLOCKS : 0) k_pair_f32(PairArgs a)
+// Sums of a round to the outputs, by copy 0: one item of a group stores, several add.
+template <int KS>
+__device__ __forceinline__ void put_sums(void *const *acc, bool add, float Gf, uint32_t first, int n, int r0, int lpc,
+                                         int slot, const float (&x)[KS], const float (&y)[KS], const float (&z)[KS])
 {
-    using Stage = WarpStage<NST>;
+    float *ox = (float *)acc[0], *oy = (float *)acc[1], *oz = (float *)acc[2];
+#pragma unroll
+    for (int kk = 0; kk < KS; ++kk) {
+        const int si = r0 + kk * lpc + slot;
+        if (si < n) {
+            const uint32_t i = first + si;
+            if (!add) {
+                ox[i] = Gf * x[kk];
+                oy[i] = Gf * y[kk];
+                oz[i] = Gf * z[kk];
+            } else {
+                atomicAdd(ox + i, Gf * x[kk]);
+                atomicAdd(oy + i, Gf * y[kk]);
+                atomicAdd(oz + i, Gf * z[kk]);
+            }
+        }
+    }
+}
+
+// Cells and far particles -> soft accelerations.
+template <int KS, int NST>
+__global__ void __launch_bounds__(PAIR_THREADS, 0) k_far(PairArgs a)
+{
+    using Stage = WarpStage<NST, 2 * PADT>;
     __shared__ Stage stages[PAIR_WARPS];
     if (a.st->code) return;
     const int lane = threadIdx.x & 31;
@@ -509,17 +430,9 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR ? NEAR_MIN_BLOCKS : 0) k_pa
     int64_t w = next_item(a.counter, lane);
     while (w < W) {
         const int64_t wn = next_item(a.counter, lane);   // the next item's number arrives while this one runs
-        // the near kernel takes its items from the last written to the first, which shortens the end of its
-        // launch (fewer SMs idle while the last items run: 0.353 -> 0.338 ms per soft step at N = 2^17; the same
-        // at 2^24); the far kernel is faster in the walk's order
-        const WorkItem d = a.items[NEAR ? W - 1 - w : w];
+        const WorkItem d = a.items[w];
         const SysParams &P = a.sp[d.sys];
-        HardC H;
-        H.eps2 = P.eps2f;
-        H.R2 = P.R2f;
-        H.R2sq = P.R2sqf;
-        H.R2sqlo = P.R2sqlo;
-        H.invdR = P.invdRf;
+        const float eps2 = P.eps2f;
         const ItemSrc src = {d.cbase, d.pbase, d.Lc, d.e0, d.e1};
         const uint32_t first = d.first;
         const int n = (int)(d.n & ~MULTI);
@@ -530,200 +443,388 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR ? NEAR_MIN_BLOCKS : 0) k_pa
         for (int r0 = 0, per_round = 0; r0 < n; r0 += per_round) {
             const int rem = n - r0;
             int lpc = rem <= 32 * KS ? (rem + KS - 1) / KS : 32;
-            // far kernel: when the copies would leave many sink slots idle (rem * copies below
-            // FAR_SPLIT_PCT % of 32 KS), this round takes a power of two of lanes per copy, which keeps
-            // every slot busy, and leaves the other sinks to the next round
-            if (!NEAR && rem * (32 / lpc) * 100 < FAR_SPLIT_PCT * 32 * KS) lpc = 1 << (31 - __clz(lpc));
+            // when the copies would leave many sink slots idle (rem * copies below FAR_SPLIT_PCT % of 32 KS), this
+            // round takes a power of two of lanes per copy, which keeps every slot busy, and leaves the other sinks
+            // to the next round
+            if (rem * (32 / lpc) * 100 < FAR_SPLIT_PCT * 32 * KS) lpc = 1 << (31 - __clz(lpc));
             const int copies = 32 / lpc;
             const int copy = lane / lpc, slot = lane - copy * lpc;
-            const bool active = copy < copies;
             per_round = lpc * KS;
-            float sx[KS], sy[KS], sz[KS], ax[KS], ay[KS], az[KS], bx[KS], by[KS], bz[KS];
-            float shx[KS], shy[KS], shz[KS], slx[KS], sly[KS], slz[KS];
+            float sx[KS], sy[KS], sz[KS], ax[KS], ay[KS], az[KS];
 #pragma unroll
             for (int kk = 0; kk < KS; ++kk) {
                 int si = r0 + kk * lpc + slot;
                 si = si < n ? si : n - 1;
                 const float4 h = a.phi[first + si], l = a.plo[first + si];
-                shx[kk] = h.x - crx;   // rebased hi (exact): differences with the staged sources' are exact
-                shy[kk] = h.y - cry;
-                shz[kk] = h.z - crz;
-                slx[kk] = l.x;
-                sly[kk] = l.y;
-                slz[kk] = l.z;
                 sx[kk] = (h.x - crx) + l.x;
                 sy[kk] = (h.y - cry) + l.y;
                 sz[kk] = (h.z - crz) + l.z;
-                ax[kk] = ay[kk] = az[kk] = 0.0f;
-                bx[kk] = by[kk] = bz[kk] = 0.0f;
             }
-            if (!NEAR) {
-                constexpr int KP = (KS + 1) / 2;
-                uint64_t SX[KP], SY[KP], SZ[KP], AX[KP], AY[KP], AZ[KP];
+            constexpr int KP = (KS + 1) / 2;
+            uint64_t SX[KP], SY[KP], SZ[KP], AX[KP], AY[KP], AZ[KP];
+#pragma unroll
+            for (int p = 0; p < KP; ++p) {
+                const int k1 = 2 * p + 1 < KS ? 2 * p + 1 : 2 * p;
+                SX[p] = pk2(sx[2 * p], sx[k1]);
+                SY[p] = pk2(sy[2 * p], sy[k1]);
+                SZ[p] = pk2(sz[2 * p], sz[k1]);
+                AX[p] = AY[p] = AZ[p] = 0ull;
+            }
+            const uint64_t E2 = pk2(eps2, eps2);
+            // the expanded form only with a hard part (then every far source is at least R2 from the sinks'
+            // box; without one, cells and particles can sit next to the sinks) and for sinks within 64 R2
+            // of the reference point: the rounding of r^2 stays below 4 u (1 + 2 * 64)^2 ~ 4e-3 of r^2
+            float k2 = 0.0f;
+#pragma unroll
+            for (int kk = 0; kk < KS; ++kk) k2 = fmaxf(k2, fmaf(sx[kk], sx[kk], fmaf(sy[kk], sy[kk], sz[kk] * sz[kk])));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
+            if (eps2 > 0.0f && P.has_hard && k2 <= 4096.0f * P.R2sqf) {
+                uint64_t Q[KP], FM[KP];
 #pragma unroll
                 for (int p = 0; p < KP; ++p) {
                     const int k1 = 2 * p + 1 < KS ? 2 * p + 1 : 2 * p;
-                    SX[p] = pk2(sx[2 * p], sx[k1]);
-                    SY[p] = pk2(sy[2 * p], sy[k1]);
-                    SZ[p] = pk2(sz[2 * p], sz[k1]);
-                    AX[p] = AY[p] = AZ[p] = 0ull;
+                    Q[p] = pk2(fmaf(sx[2 * p], sx[2 * p], fmaf(sy[2 * p], sy[2 * p], fmaf(sz[2 * p], sz[2 * p], eps2))),
+                               fmaf(sx[k1], sx[k1], fmaf(sy[k1], sy[k1], fmaf(sz[k1], sz[k1], eps2))));
+                    FM[p] = 0ull;
                 }
-                const uint64_t E2 = pk2(H.eps2, H.eps2);
-                // the expanded form only with a hard part (then every far source is at least R2 from the sinks'
-                // box; without one, cells and particles can sit next to the sinks) and for sinks within 64 R2
-                // of the reference point: the rounding of r^2 stays below 4 u (1 + 2 * 64)^2 ~ 4e-3 of r^2
-                float k2 = 0.0f;
+                pipeline<NST>(a, src, S, lane, [&](int st, int nt) {
+                    stage_far<true>(S, st, nt, lane, crx, cry, crz);
+                    exp_tile<KP>(S, nt, copy, copies, SX, SY, SZ, Q, AX, AY, AZ, FM);
+                });
 #pragma unroll
-                for (int kk = 0; kk < KS; ++kk) k2 = fmaxf(k2, fmaf(sx[kk], sx[kk], fmaf(sy[kk], sy[kk], sz[kk] * sz[kk])));
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) k2 = fmaxf(k2, __shfl_xor_sync(0xffffffffu, k2, o));
-                if (H.eps2 > 0.0f && P.has_hard && k2 <= 4096.0f * H.R2sq) {
-                    uint64_t Q[KP], FM[KP];
-#pragma unroll
-                    for (int p = 0; p < KP; ++p) {
-                        const int k1 = 2 * p + 1 < KS ? 2 * p + 1 : 2 * p;
-                        Q[p] = pk2(fmaf(sx[2 * p], sx[2 * p], fmaf(sy[2 * p], sy[2 * p], fmaf(sz[2 * p], sz[2 * p], H.eps2))),
-                                   fmaf(sx[k1], sx[k1], fmaf(sy[k1], sy[k1], fmaf(sz[k1], sz[k1], H.eps2))));
-                        FM[p] = 0ull;
-                    }
-                    pipeline<FAR_EXP, NST>(a, src, S, lane, crx, cry, crz, SinkBox(), [&](int, int nt) {
-                        exp_tile<KP>(S, nt, copy, copies, SX, SY, SZ, Q, AX, AY, AZ, FM);
-                    });
-#pragma unroll
-                    for (int p = 0; p < KP; ++p) {   // A - k FM
-                        const int k1 = 2 * p + 1 < KS ? 2 * p + 1 : 2 * p;
-                        AX[p] = fma2(pk2(-sx[2 * p], -sx[k1]), FM[p], AX[p]);
-                        AY[p] = fma2(pk2(-sy[2 * p], -sy[k1]), FM[p], AY[p]);
-                        AZ[p] = fma2(pk2(-sz[2 * p], -sz[k1]), FM[p], AZ[p]);
-                    }
-                } else {
-                    if (H.eps2 > 0.0f)
-                        pipeline<FAR_PACKED, NST>(a, src, S, lane, crx, cry, crz, SinkBox(), [&](int, int nt) {
-                            far_tile<KP, false>(S, nt, copy, copies, E2, SX, SY, SZ, AX, AY, AZ);
-                        });
-                    else   // eps = 0 without a hard part: a sink meets itself in its far particles
-                        pipeline<FAR_PACKED, NST>(a, src, S, lane, crx, cry, crz, SinkBox(), [&](int, int nt) {
-                            far_tile<KP, true>(S, nt, copy, copies, E2, SX, SY, SZ, AX, AY, AZ);
-                        });
+                for (int p = 0; p < KP; ++p) {   // A - k FM
+                    const int k1 = 2 * p + 1 < KS ? 2 * p + 1 : 2 * p;
+                    AX[p] = fma2(pk2(-sx[2 * p], -sx[k1]), FM[p], AX[p]);
+                    AY[p] = fma2(pk2(-sy[2 * p], -sy[k1]), FM[p], AY[p]);
+                    AZ[p] = fma2(pk2(-sz[2 * p], -sz[k1]), FM[p], AZ[p]);
                 }
-#pragma unroll
-                for (int p = 0; p < KP; ++p) {
-                    float t0, t1;
-                    upk2(AX[p], t0, t1);
-                    ax[2 * p] = t0;
-                    if (2 * p + 1 < KS) ax[2 * p + 1] = t1;
-                    upk2(AY[p], t0, t1);
-                    ay[2 * p] = t0;
-                    if (2 * p + 1 < KS) ay[2 * p + 1] = t1;
-                    upk2(AZ[p], t0, t1);
-                    az[2 * p] = t0;
-                    if (2 * p + 1 < KS) az[2 * p + 1] = t1;
-                }
-            } else {
-                // the box of this round's sinks: sources farther than R2 from it have K = 0 for every sink
-                SinkBox sb;
-                sb.R2sq = H.R2sq;
-                {
-                    float lo0 = sx[0], lo1 = sy[0], lo2 = sz[0], hi0 = sx[0], hi1 = sy[0], hi2 = sz[0];
-#pragma unroll
-                    for (int k = 1; k < KS; ++k) {
-                        lo0 = fminf(lo0, sx[k]);
-                        lo1 = fminf(lo1, sy[k]);
-                        lo2 = fminf(lo2, sz[k]);
-                        hi0 = fmaxf(hi0, sx[k]);
-                        hi1 = fmaxf(hi1, sy[k]);
-                        hi2 = fmaxf(hi2, sz[k]);
-                    }
-#pragma unroll
-                    for (int o = 16; o > 0; o >>= 1) {
-                        lo0 = fminf(lo0, __shfl_xor_sync(0xffffffffu, lo0, o));
-                        lo1 = fminf(lo1, __shfl_xor_sync(0xffffffffu, lo1, o));
-                        lo2 = fminf(lo2, __shfl_xor_sync(0xffffffffu, lo2, o));
-                        hi0 = fmaxf(hi0, __shfl_xor_sync(0xffffffffu, hi0, o));
-                        hi1 = fmaxf(hi1, __shfl_xor_sync(0xffffffffu, hi1, o));
-                        hi2 = fmaxf(hi2, __shfl_xor_sync(0xffffffffu, hi2, o));
-                    }
-                    sb.lo[0] = lo0;
-                    sb.lo[1] = lo1;
-                    sb.lo[2] = lo2;
-                    sb.hi[0] = hi0;
-                    sb.hi[1] = hi1;
-                    sb.hi[2] = hi2;
-                }
-                pipeline<NEAR_FILTER, NST>(a, src, S, lane, crx, cry, crz, sb, [&](int n_in, int n_out) {
-                    if (!active) return;
-                    for (int j = copy; j < n_in; j += copies) {   // sources within R2 of the box
-                        const float4 q = S.tile[j];
-                        float dx[KS], dy[KS], dz[KS], r2u[KS];
-                        bool any_in = false;
-#pragma unroll
-                        for (int k = 0; k < KS; ++k) {
-                            dx[k] = q.x - sx[k];
-                            dy[k] = q.y - sy[k];
-                            dz[k] = q.z - sz[k];
-                            r2u[k] = fmaf(dx[k], dx[k], fmaf(dy[k], dy[k], dz[k] * dz[k]));
-                            any_in |= r2u[k] < H.R2sq;
-                        }
-                        float4 hh = make_float4(0.0f, 0.0f, 0.0f, 0.0f), ll = hh;
-                        if (any_in) {
-                            hh = S.tile[TILE + j];
-                            ll = S.tile[2 * TILE + j];
-                        }
-#pragma unroll
-                        for (int k = 0; k < KS; ++k)
-                            near_finish<SOFT, HARD>(q.w, dx[k], dy[k], dz[k], r2u[k], hh, ll, shx[k], shy[k], shz[k],
-                                                    slx[k], sly[k], slz[k], H, ax[k], ay[k], az[k], bx[k], by[k],
-                                                    bz[k]);
-                    }
-                    if (SOFT)   // the rest: K = 0 for every sink, weight 1 on the soft force
-                        for (int j = TILE - n_out + copy; j < TILE; j += copies) {
-                            const float4 q = S.tile[j];
-#pragma unroll
-                            for (int k = 0; k < KS; ++k) body_far<false>(q, sx[k], sy[k], sz[k], H.eps2, ax[k], ay[k], az[k]);
-                        }
+            } else if (eps2 > 0.0f) {
+                pipeline<NST>(a, src, S, lane, [&](int st, int nt) {
+                    stage_far<false>(S, st, nt, lane, crx, cry, crz);
+                    far_tile<KP, false>(S, nt, copy, copies, E2, SX, SY, SZ, AX, AY, AZ);
+                });
+            } else {   // eps = 0 without a hard part: a sink meets itself in its far particles
+                pipeline<NST>(a, src, S, lane, [&](int st, int nt) {
+                    stage_far<false>(S, st, nt, lane, crx, cry, crz);
+                    far_tile<KP, true>(S, nt, copy, copies, E2, SX, SY, SZ, AX, AY, AZ);
                 });
             }
-            if (SOFT) reduce_copies<KS>(lane, copy, copies, lpc, ax, ay, az);
-            if (HARD) reduce_copies<KS>(lane, copy, copies, lpc, bx, by, bz);
-            if (copy == 0) {
-                const float Gf = P.Gf;
 #pragma unroll
-                for (int kk = 0; kk < KS; ++kk) {
-                    const int si = r0 + kk * lpc + slot;
-                    if (si < n) {
-                        const uint32_t i = first + si;
-                        if (SOFT) {
-                            float *ox = (float *)a.as[0], *oy = (float *)a.as[1], *oz = (float *)a.as[2];
-                            if (!NEAR && !multi) {
-                                ox[i] = Gf * ax[kk];
-                                oy[i] = Gf * ay[kk];
-                                oz[i] = Gf * az[kk];
-                            } else {   // several items, or the near part added to the far part
-                                atomicAdd(ox + i, Gf * ax[kk]);
-                                atomicAdd(oy + i, Gf * ay[kk]);
-                                atomicAdd(oz + i, Gf * az[kk]);
-                            }
-                        }
-                        if (HARD) {
-                            float *ox = (float *)a.ah[0], *oy = (float *)a.ah[1], *oz = (float *)a.ah[2];
-                            if (!multi) {
-                                ox[i] = Gf * bx[kk];
-                                oy[i] = Gf * by[kk];
-                                oz[i] = Gf * bz[kk];
-                            } else {
-                                atomicAdd(ox + i, Gf * bx[kk]);
-                                atomicAdd(oy + i, Gf * by[kk]);
-                                atomicAdd(oz + i, Gf * bz[kk]);
-                            }
-                        }
-                    }
-                }
+            for (int p = 0; p < KP; ++p) {
+                float t0, t1;
+                upk2(AX[p], t0, t1);
+                ax[2 * p] = t0;
+                if (2 * p + 1 < KS) ax[2 * p + 1] = t1;
+                upk2(AY[p], t0, t1);
+                ay[2 * p] = t0;
+                if (2 * p + 1 < KS) ay[2 * p + 1] = t1;
+                upk2(AZ[p], t0, t1);
+                az[2 * p] = t0;
+                if (2 * p + 1 < KS) az[2 * p + 1] = t1;
             }
+            reduce_copies<KS>(lane, copy, copies, lpc, ax, ay, az);
+            if (copy == 0) put_sums<KS>(a.as, multi, P.Gf, first, n, r0, lpc, slot, ax, ay, az);
         }
         w = wn;
     }
     cp_wait<0>();   // nothing may stay in flight into shared memory at exit
-    if (lane == 0) atomicAdd(NEAR ? a.inter_hard : a.inter_soft, inter);
+    if (lane == 0) atomicAdd(a.inter_soft, inter);
+}
+
+// ---------------------------------------------------------------------------
+// Near particles -> F (1 - K) into the soft and F K into the hard accelerations.
+//
+// Few near pairs lie within R2 (1.4 % at N = 2^24), but only they need K, some
+// 60 instructions, so each tile of sources takes two steps. The distance step
+// touches every pair that has to be touched, two sources per instruction and
+// without branches, and marks the pairs within R2 in a bit mask per lane; the K
+// step then walks the masks, every lane with its own next pair, so a warp runs
+// as many K evaluations as its fullest lane has, not one for every source that
+// some lane is close to.
+//  - HARD alone: pairs beyond R2 contribute nothing, so a warp first packs
+//    together the sources within R2 of the box of its sinks (computed with the
+//    pair distance's roundings: none is missed).
+//  - SOFT: every pair adds F at weight 1 unless it is marked.
+//
+// One block per work item: its warps take blocks of at most 32 consecutive
+// sinks (compact in key order), one sink per lane, and share the tiles of
+// NEAR_TILE sources, one gathered by each thread while the last tile is worked
+// on; with one or two blocks of sinks the warps split the sources. One sink a
+// lane keeps the kernel at 64 registers, 32 warps per SM: with 4 sinks a lane
+// (124 registers, 16 warps) it was bound by latency at 38-50 % of the issue
+// slots, whatever the instruction count; 6 blocks per SM are slower too (2^24
+// 39.1 against 35.7 ms). Near time per step against the form before (one warp
+// per item, 4 sinks a lane, a divergent K for every source within R2 of some
+// lane): N = 2^12 0.139 -> 0.071 ms, 2^17 0.337 -> 0.256, 2^20 (absolute MAC)
+// 1.60 -> 1.09, 2^24 40.2 -> 35.2 ms.
+// ---------------------------------------------------------------------------
+constexpr int NEAR_TILE = PAIR_THREADS;
+constexpr float FAR_AWAY = 1e18f;   // padding sources: far beyond any R2, r^2 still finite
+
+struct NearTile {
+    float4 hi[NEAR_TILE];   // rebased hi parts and mass (differences with the sinks' hi parts are exact)
+    float4 lo[NEAR_TILE];
+};
+
+// the sources a distance step runs over, two by two
+struct NearPacked {
+    float x[NEAR_TILE + 2], y[NEAR_TILE + 2], z[NEAR_TILE + 2];
+    uint8_t j[NEAR_TILE];   // their entries in the tile
+};
+
+struct NearSink {
+    float hx, hy, hz, lx, ly, lz;   // rebased hi parts and lo parts
+};
+
+// One marked pair per lane (on: whether this lane has one), entry j of the tile: r^2 and K as the FP32 form defines them.
+template <bool SOFT, bool HARD>
+__device__ __forceinline__ void near_pair(const NearTile &T, int j, bool on, const NearSink &s, const HardC &H, float &sax,
+                                          float &say, float &saz, float &hax, float &hay, float &haz)
+{
+    const float4 h = T.hi[j], l = T.lo[j];
+    const float dx = (h.x + l.x) - (s.hx + s.lx), dy = (h.y + l.y) - (s.hy + s.ly), dz = (h.z + l.z) - (s.hz + s.lz);
+    const float r2u = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+    const float r2 = r2u + H.eps2;
+    const float ri = r2 > 0.0f ? rsqrtf(r2) : 0.0f;
+    const float f = on ? h.w * ri * (ri * ri) : 0.0f;
+    float K = dll_K_precise(r2u, __fsub_rn(h.x, s.hx), __fsub_rn(h.y, s.hy), __fsub_rn(h.z, s.hz), __fsub_rn(l.x, s.lx),
+                            __fsub_rn(l.y, s.ly), __fsub_rn(l.z, s.lz), H);
+    if (SOFT) {
+        K = r2u < H.R2sq ? K : 0.0f;   // the mark of the soft form is a little generous
+        const float fs = f * (1.0f - K);
+        sax = fmaf(dx, fs, sax);
+        say = fmaf(dy, fs, say);
+        saz = fmaf(dz, fs, saz);
+    }
+    if (HARD) {
+        const float fh = f * K;
+        hax = fmaf(dx, fh, hax);
+        hay = fmaf(dy, fh, hay);
+        haz = fmaf(dz, fh, haz);
+    }
+}
+
+// order-preserving integer image of a float (and back)
+__device__ __forceinline__ int ord_f(float v)
+{
+    const int i = __float_as_int(v);
+    return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float unord_f(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
+
+template <bool SOFT, bool HARD>
+__global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs a)
+{
+    __shared__ NearTile tiles[2];
+    __shared__ __align__(16) float packed_mem[SOFT ? 2 * 4 * NEAR_TILE : PAIR_WARPS * (sizeof(NearPacked) + 3) / 4];
+    __shared__ int64_t sh_item;
+    if (a.st->code) return;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned ltm = (1u << lane) - 1u;
+    const int64_t W = (int64_t)*a.nwork;
+    unsigned long long inter = 0;
+    unsigned long long next = 0;
+    if (threadIdx.x == 0) next = atomicAdd(a.counter, 1ull);
+    for (;;) {
+        __syncthreads();   // the last item's tiles are used
+        if (threadIdx.x == 0) {
+            sh_item = (int64_t)next;
+            next = atomicAdd(a.counter, 1ull);   // arrives while this item runs
+        }
+        __syncthreads();
+        const int64_t it = sh_item;
+        if (it >= W) break;
+        // items from the last written to the first, which shortens the end of the launch
+        const WorkItem d = a.items[W - 1 - it];
+        const SysParams &P = a.sp[d.sys];
+        HardC H;
+        H.eps2 = P.eps2f;
+        H.R2 = P.R2f;
+        H.R2sq = P.R2sqf;
+        H.R2sqlo = P.R2sqlo;
+        H.invdR = P.invdRf;
+        const uint32_t *list = a.list + d.pbase;   // entries [e0, e1): particles
+        const int ne = (int)(d.e1 - d.e0);
+        const int n = (int)(d.n & ~MULTI);
+        const bool multi = (d.n & MULTI) != 0;
+        const float4 cref = a.phi[d.first];
+        inter += (unsigned long long)n * (unsigned long long)ne;
+        const int nblk = (n + 31) / 32, per = (n + nblk - 1) / nblk;   // blocks of at most 32 sinks, about equal
+        const int ntile = (ne + NEAR_TILE - 1) / NEAR_TILE;
+        for (int b0 = 0; b0 < nblk; b0 += PAIR_WARPS) {
+            const int here = min(nblk - b0, PAIR_WARPS);
+            const int splits = here == 1 ? 4 : (here == 2 ? 2 : 1);   // warps per block of sinks, each a part of every tile
+            const int blk = b0 + w / splits, part = w - (w / splits) * splits;
+            const bool busy = blk < nblk;
+            const int s0 = blk * per, sn = busy ? min(per, n - s0) : 0;
+            NearSink s = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+            if (busy) {
+                const uint32_t i = d.first + s0 + min(lane, sn - 1);
+                const float4 h = a.phi[i], l = a.plo[i];
+                s = NearSink{h.x - cref.x, h.y - cref.y, h.z - cref.z, l.x, l.y, l.z};
+            }
+            const float sx = s.hx + s.lx, sy = s.hy + s.ly, sz = s.hz + s.lz;
+            const uint64_t SX = pk2(sx, sx), SY = pk2(sy, sy), SZ = pk2(sz, sz);
+            float lo[3], hi[3];
+            if (!SOFT) {   // the box of the warp's sinks
+                lo[0] = unord_f(__reduce_min_sync(0xffffffffu, ord_f(sx)));
+                lo[1] = unord_f(__reduce_min_sync(0xffffffffu, ord_f(sy)));
+                lo[2] = unord_f(__reduce_min_sync(0xffffffffu, ord_f(sz)));
+                hi[0] = unord_f(__reduce_max_sync(0xffffffffu, ord_f(sx)));
+                hi[1] = unord_f(__reduce_max_sync(0xffffffffu, ord_f(sy)));
+                hi[2] = unord_f(__reduce_max_sync(0xffffffffu, ord_f(sz)));
+            }
+            float ax = 0.0f, ay = 0.0f, az = 0.0f, bx = 0.0f, by = 0.0f, bz = 0.0f;
+            uint64_t AX = 0ull, AY = 0ull, AZ = 0ull;
+            const uint64_t E2 = pk2(H.eps2, H.eps2);
+            // this thread's source of a tile; past the end a far-away massless one
+            auto index = [&](int t) -> uint32_t {
+                const int e = t * NEAR_TILE + (int)threadIdx.x;
+                return e < ne ? list[d.e0 + (uint32_t)e] : NONE;
+            };
+            float4 gh = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.0f), gl = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            auto gather = [&](uint32_t i) {
+                if (i != NONE) {
+                    gh = a.phi[i];
+                    gl = a.plo[i];
+                } else {
+                    gh = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.0f);
+                }
+            };
+            uint32_t i1 = index(0);
+            gather(i1);
+            i1 = ntile > 1 ? index(1) : NONE;
+            for (int t = 0; t < ntile; ++t) {
+                // double-buffered: a tile is written again only after a barrier that follows its use
+                NearTile &T = tiles[t & 1];
+                const float4 h = make_float4(gh.x - cref.x, gh.y - cref.y, gh.z - cref.z, gh.w);
+                T.hi[threadIdx.x] = h;
+                T.lo[threadIdx.x] = gl;
+                if (SOFT) {   // source pairs {x x' y y'} {z z' m m'}
+                    float *q = packed_mem + (t & 1) * 4 * NEAR_TILE + (threadIdx.x >> 1) * 8 + (threadIdx.x & 1);
+                    q[0] = h.x + gl.x;
+                    q[2] = h.y + gl.y;
+                    q[4] = h.z + gl.z;
+                    q[6] = h.w;
+                }
+                if (t + 1 < ntile) {   // the next tile's sources, and the indices of the one after
+                    gather(i1);
+                    i1 = t + 2 < ntile ? index(t + 2) : NONE;
+                }
+                __syncthreads();
+                if (!busy) continue;
+                const int nt = min(NEAR_TILE, ne - t * NEAR_TILE);
+                if constexpr (SOFT) {
+                    const float near2 = (H.R2sq + H.eps2) * 1.000001f;   // marks every pair within R2, a few beyond
+                    const int q0 = part * (NEAR_TILE / 2 / splits), q1 = min((nt + 1) / 2, q0 + NEAR_TILE / 2 / splits);
+                    const float4 *pk = (const float4 *)(packed_mem + (t & 1) * 4 * NEAR_TILE);
+                    for (int m0 = q0; m0 < q1; m0 += 16) {   // 16 source pairs: one mask word
+                        uint32_t mark = 0u, bit = 1u;
+                        const int m1 = min(q1, m0 + 16);
+#pragma unroll 2
+                        for (int m = m0; m < m1; ++m, bit <<= 2) {
+                            const float4 u = pk[2 * m], v = pk[2 * m + 1];
+                            const uint64_t dx = sub2(pk2(u.x, u.y), SX), dy = sub2(pk2(u.z, u.w), SY), dz = sub2(pk2(v.x, v.y), SZ);
+                            const uint64_t r2 = fma2(dx, dx, fma2(dy, dy, fma2(dz, dz, E2)));
+                            float ra, rb, fa, fb;
+                            upk2(r2, ra, rb);
+                            const uint64_t ri = pk2(rsqrtf(ra), rsqrtf(rb));
+                            upk2(mul2(mul2(pk2(v.z, v.w), ri), mul2(ri, ri)), fa, fb);
+                            const bool ia = ra < near2, ib = rb < near2;
+                            const uint64_t f = pk2(ia ? 0.0f : fa, ib ? 0.0f : fb);
+                            mark |= ia ? bit : 0u;
+                            mark |= ib ? 2u * bit : 0u;
+                            AX = fma2(dx, f, AX);
+                            AY = fma2(dy, f, AY);
+                            AZ = fma2(dz, f, AZ);
+                        }
+                        while (__any_sync(0xffffffffu, mark != 0u)) {
+                            const bool on = mark != 0u;
+                            const int j = on ? 2 * m0 + __ffs(mark) - 1 : 0;
+                            near_pair<SOFT, HARD>(T, j, on, s, H, ax, ay, az, bx, by, bz);
+                            mark &= mark - 1u;
+                        }
+                    }
+                } else {
+                    NearPacked &p = *(NearPacked *)((char *)packed_mem + w * ((sizeof(NearPacked) + 3) / 4 * 4));
+                    int nin = 0;
+#pragma unroll
+                    for (int u = 0; u < NEAR_TILE / 32; ++u) {
+                        const int el = u * 32 + lane;
+                        if (u / (4 / splits) != part) continue;   // this warp's part of the tile
+                        if (u * 32 >= nt) break;
+                        const float4 qh = T.hi[el], ql = T.lo[el];
+                        const float x = qh.x + ql.x, y = qh.y + ql.y, z = qh.z + ql.z;
+                        const float gx = fmaxf(fmaxf(lo[0] - x, x - hi[0]), 0.0f);
+                        const float gy = fmaxf(fmaxf(lo[1] - y, y - hi[1]), 0.0f);
+                        const float gz = fmaxf(fmaxf(lo[2] - z, z - hi[2]), 0.0f);
+                        const bool keep = fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < H.R2sq;
+                        const unsigned km = __ballot_sync(0xffffffffu, keep);
+                        if (keep) {
+                            const int q = nin + __popc(km & ltm);
+                            p.x[q] = x;
+                            p.y[q] = y;
+                            p.z[q] = z;
+                            p.j[q] = (uint8_t)el;
+                        }
+                        nin += __popc(km);
+                    }
+                    if (nin == 0) continue;
+                    if (lane == 0) p.x[nin] = FAR_AWAY;   // the last pair's other half, if any
+                    __syncwarp();
+                    const int rounds = (nin + 1) / 2;
+                    for (int m0 = 0; m0 < rounds; m0 += 16) {   // 16 source pairs: one mask word
+                        uint32_t mark = 0u, bit = 1u;
+                        const int m1 = min(rounds, m0 + 16);
+#pragma unroll 4
+                        for (int m = m0; m < m1; ++m, bit <<= 2) {
+                            const float2 x = *(const float2 *)&p.x[2 * m], y = *(const float2 *)&p.y[2 * m],
+                                         z = *(const float2 *)&p.z[2 * m];
+                            const uint64_t dx = sub2(pk2(x.x, x.y), SX), dy = sub2(pk2(y.x, y.y), SY), dz = sub2(pk2(z.x, z.y), SZ);
+                            float ra, rb;
+                            upk2(fma2(dx, dx, fma2(dy, dy, mul2(dz, dz))), ra, rb);
+                            mark |= ra < H.R2sq ? bit : 0u;
+                            mark |= rb < H.R2sq ? 2u * bit : 0u;
+                        }
+                        while (__any_sync(0xffffffffu, mark != 0u)) {
+                            const bool on = mark != 0u;
+                            const int j = on ? p.j[2 * m0 + __ffs(mark) - 1] : 0;
+                            near_pair<SOFT, HARD>(T, j, on, s, H, ax, ay, az, bx, by, bz);
+                            mark &= mark - 1u;
+                        }
+                    }
+                    __syncwarp();   // the packed sources are used
+                }
+            }
+            if (busy && lane < sn) {
+                const uint32_t i = d.first + s0 + lane;
+                const float Gf = P.Gf;
+                if (SOFT) {   // the near part is added to the far part
+                    float t0, t1;
+                    upk2(AX, t0, t1);
+                    atomicAdd((float *)a.as[0] + i, Gf * (ax + (t0 + t1)));
+                    upk2(AY, t0, t1);
+                    atomicAdd((float *)a.as[1] + i, Gf * (ay + (t0 + t1)));
+                    upk2(AZ, t0, t1);
+                    atomicAdd((float *)a.as[2] + i, Gf * (az + (t0 + t1)));
+                }
+                if (HARD) {
+                    if (!multi && splits == 1) {
+                        ((float *)a.ah[0])[i] = Gf * bx;
+                        ((float *)a.ah[1])[i] = Gf * by;
+                        ((float *)a.ah[2])[i] = Gf * bz;
+                    } else {
+                        atomicAdd((float *)a.ah[0] + i, Gf * bx);
+                        atomicAdd((float *)a.ah[1] + i, Gf * by);
+                        atomicAdd((float *)a.ah[2] + i, Gf * bz);
+                    }
+                }
+            }
+            if (b0 + PAIR_WARPS < nblk) __syncthreads();   // the next blocks of sinks write tile 0 again
+        }
+    }
+    if (threadIdx.x == 0) atomicAdd(a.inter_hard, inter);
 }
 
 // ---------------------------------------------------------------------------
@@ -910,30 +1011,22 @@ void fill_args(hybrid_ctx *c, PairArgs &a)
     a.want_soft = a.want_hard = 0;
 }
 
-// staging depth: tile_depth (2, 3 or 4; 0 = 3) for the far kernel, 3 for the near kernel
-template <int KS, bool NEAR, bool SOFT, bool HARD>
-void go_f32(hybrid_ctx *c, const PairArgs &a)
+// Far kernel: sinks per lane KS = ceil(n_crit / threads_per_group): 1, 2, 4 or
+// 8; the default is 4 (one shared-memory read feeds 4 interactions). Staging
+// depth: tile_depth (2, 3 or 4; 0 = 3).
+int sinks_per_lane(const hybrid_ctx *c)
 {
-    const int depth = NEAR || c->p.tile_depth == 0 ? 3 : c->p.tile_depth;
-    if (!NEAR && depth == 2) k_pair_f32<KS, NEAR, SOFT, HARD, 2><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
-    else if (!NEAR && depth == 4) k_pair_f32<KS, NEAR, SOFT, HARD, 4><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
-    else k_pair_f32<KS, NEAR, SOFT, HARD, 3><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
+    const int ks = c->p.threads_per_group > 0 ? (c->p.n_crit + c->p.threads_per_group - 1) / c->p.threads_per_group : 4;
+    return ks <= 1 ? 1 : (ks <= 2 ? 2 : (ks <= 4 ? 4 : 8));
 }
 
-// Sinks per lane KS = ceil(n_crit / threads_per_group): 1, 2, 4 or (far
-// kernel only) 8; the default is 4 (one shared-memory read feeds 4
-// interactions; the far kernel runs them as packed sink pairs).
-template <bool NEAR, bool SOFT, bool HARD>
-void go_ks(hybrid_ctx *c, const PairArgs &a)
+template <int KS>
+void go_far(hybrid_ctx *c, const PairArgs &a)
 {
-    int ks;
-    if (c->p.threads_per_group > 0) ks = (c->p.n_crit + c->p.threads_per_group - 1) / c->p.threads_per_group;
-    else ks = 4;
-    ks = ks <= 1 ? 1 : (ks <= 2 ? 2 : (ks <= 4 || NEAR ? 4 : 8));   // 8 sinks per lane: far kernel only
-    if (ks == 1) go_f32<1, NEAR, SOFT, HARD>(c, a);
-    else if (ks == 2) go_f32<2, NEAR, SOFT, HARD>(c, a);
-    else if (ks == 4) go_f32<4, NEAR, SOFT, HARD>(c, a);
-    else if constexpr (!NEAR) go_f32<8, NEAR, SOFT, HARD>(c, a);
+    const int depth = c->p.tile_depth == 0 ? 3 : c->p.tile_depth;
+    if (depth == 2) k_far<KS, 2><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
+    else if (depth == 4) k_far<KS, 4><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
+    else k_far<KS, 3><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
 }
 
 // near = false: cells and far particles (soft); near = true: near particles
@@ -969,10 +1062,18 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
             for (int d = 0; d < 3; ++d) cudaMemsetAsync(c->acc_s[d].p, 0, (size_t)c->N * sizeof(float), c->st);
         if (near && a.want_hard)
             for (int d = 0; d < 3; ++d) cudaMemsetAsync(c->acc_h[d].p, 0, (size_t)c->N * sizeof(float), c->st);
-        if (!near) go_ks<false, true, false>(c, a);
-        else if (a.want_soft && a.want_hard) go_ks<true, true, true>(c, a);
-        else if (a.want_soft) go_ks<true, true, false>(c, a);
-        else go_ks<true, false, true>(c, a);
+        if (!near) {
+            const int ks = sinks_per_lane(c);
+            if (ks == 1) go_far<1>(c, a);
+            else if (ks == 2) go_far<2>(c, a);
+            else if (ks == 4) go_far<4>(c, a);
+            else go_far<8>(c, a);
+        } else {
+            const int grid = c->nsm * NEAR_MIN_BLOCKS;
+            if (a.want_soft && a.want_hard) k_near<true, true><<<grid, PAIR_THREADS, 0, c->st>>>(a);
+            else if (a.want_soft) k_near<true, false><<<grid, PAIR_THREADS, 0, c->st>>>(a);
+            else k_near<false, true><<<grid, PAIR_THREADS, 0, c->st>>>(a);
+        }
         c->launches += 1;
     }
     prof_end(c, kind, e0);
@@ -983,10 +1084,10 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
 void launch_pair_far(hybrid_ctx *c) { launch_pairs(c, false, 1); }
 
 namespace {
-template <int KS, bool NEAR, bool SOFT, bool HARD, int NST>
-cudaError_t prefer_shared()
+template <typename K>
+cudaError_t prefer_shared(K *kernel)
 {
-    return cudaFuncSetAttribute(k_pair_f32<KS, NEAR, SOFT, HARD, NST>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                 (int)cudaSharedmemCarveoutMaxShared);
 }
 }  // namespace
@@ -997,17 +1098,12 @@ cudaError_t prefer_shared()
 cudaError_t init_pair_kernels()
 {
     cudaError_t e = cudaSuccess;
-    for (cudaError_t r : {prefer_shared<1, false, true, false, 2>(), prefer_shared<1, false, true, false, 3>(),
-                          prefer_shared<1, false, true, false, 4>(), prefer_shared<2, false, true, false, 2>(),
-                          prefer_shared<2, false, true, false, 3>(), prefer_shared<2, false, true, false, 4>(),
-                          prefer_shared<4, false, true, false, 2>(), prefer_shared<4, false, true, false, 3>(),
-                          prefer_shared<4, false, true, false, 4>(), prefer_shared<8, false, true, false, 2>(),
-                          prefer_shared<8, false, true, false, 3>(), prefer_shared<8, false, true, false, 4>(),
-                          prefer_shared<1, true, true, true, 3>(), prefer_shared<2, true, true, true, 3>(),
-                          prefer_shared<4, true, true, true, 3>(), prefer_shared<1, true, true, false, 3>(),
-                          prefer_shared<2, true, true, false, 3>(), prefer_shared<4, true, true, false, 3>(),
-                          prefer_shared<1, true, false, true, 3>(), prefer_shared<2, true, false, true, 3>(),
-                          prefer_shared<4, true, false, true, 3>()})
+    for (cudaError_t r : {prefer_shared(k_far<1, 2>), prefer_shared(k_far<1, 3>), prefer_shared(k_far<1, 4>),
+                          prefer_shared(k_far<2, 2>), prefer_shared(k_far<2, 3>), prefer_shared(k_far<2, 4>),
+                          prefer_shared(k_far<4, 2>), prefer_shared(k_far<4, 3>), prefer_shared(k_far<4, 4>),
+                          prefer_shared(k_far<8, 2>), prefer_shared(k_far<8, 3>), prefer_shared(k_far<8, 4>),
+                          prefer_shared(k_near<true, true>), prefer_shared(k_near<true, false>),
+                          prefer_shared(k_near<false, true>)})
         if (e == cudaSuccess) e = r;
     return e;
 }

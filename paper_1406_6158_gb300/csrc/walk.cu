@@ -536,12 +536,13 @@ void launch_walk(hybrid_ctx *c, int mode)
     a.items_far = (WorkItem *)c->wmap.p;
     a.items_near = (WorkItem *)c->wnear.p;
     a.cap_items = c->capWork;
-    // near items: the near kernel's time per tile is mostly latency, so short items spread a small job over more
-    // warps; on large jobs every warp has items anyway and longer ones save the per-item set-up. Far items: on a
-    // small job short items even out the warps' ends; on a large job long ones hide the set-up of each item (its
-    // descriptor, sinks and first gathers) behind more tiles
+    // Far items: on a small job short items even out the warps' ends; on a large job long ones hide the set-up of
+    // each item (its descriptor, sinks and first gathers) behind more tiles.
     const bool small_job = c->N <= (int64_t)1 << 20;
-    a.lch_near = small_job ? LCH_NEAR_SMALL : LCH_NEAR;
+    // Near items (one block each, tiles of 128 sources): as long as there are enough of them for every resident block.
+    // Near time per step with 64, 128, 256 entries: N = 2^12 0.071, 0.077, 0.083 ms; 2^17 0.292, 0.256, 0.266;
+    // 2^20 1.51, 1.17, 1.09; with 512 and 1024: 2^24 35.6, 35.2.
+    a.lch_near = c->N <= 1 << 15 ? 64 : (c->N <= 1 << 18 ? 128 : (c->N <= 1 << 20 ? 256 : 1024));
     a.lch_far = small_job ? LCH_FAR_SMALL : LCH_FAR;
     const int grid = c->walk_warps * 32 / WALK_THREADS;
     cudaEvent_t e0 = nullptr;
