@@ -207,6 +207,10 @@ struct hybrid_ctx {
     hy::Buf wnear;                                 // near-pair work items (wmap holds the far ones)
     int64_t capWork = 0;                           // work items per kind
     int last_walk_mode = 0;
+    // within an op sequence: the counters of the next walk are zero (a build cleared them); the counters and sums of
+    // the pair kernels are clear for these forces (bit 0 soft, 1 hard: the walk cleared them)
+    bool walk_clean = false;
+    int pairs_clean = 0;
 
     // profiling
     int prof = 0;                          // 0 off, 1 pair kernels, 2 every stage

@@ -380,6 +380,13 @@ struct Op {
     double dval = 0.0;
 };
 
+// Nothing is known to be clear at the start of a sequence (or of a resumed one).
+void begin_sequence(hybrid_ctx *c)
+{
+    c->walk_clean = false;
+    c->pairs_clean = 0;
+}
+
 void enqueue(hybrid_ctx *c, const Op &o, int idx)
 {
     c->op = idx;
@@ -539,6 +546,7 @@ bool launch_as_graph(hybrid_ctx *c, const std::vector<Op> &ops, std::vector<std:
     c->capturing = true;
     cudaError_t e = cudaStreamBeginCapture(c->st, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
+        begin_sequence(c);
         for (size_t i = 0; i < ops.size(); ++i) enqueue(c, ops[i], (int)i);
         e = cudaStreamEndCapture(c->st, &graph);
     }
@@ -596,8 +604,10 @@ hybrid_status run_ops(hybrid_ctx *c, const std::vector<Op> &ops_in)
     } sort_mode{c};
     for (int attempt = 0; attempt < 12; ++attempt) {
         std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> *gev = nullptr;
-        if (!(attempt == 0 && !skin_recovered && !c->sort_fallback && launch_as_graph(c, ops, &gev)))
+        if (!(attempt == 0 && !skin_recovered && !c->sort_fallback && launch_as_graph(c, ops, &gev))) {
+            begin_sequence(c);
             for (size_t i = start; i < ops.size(); ++i) enqueue(c, ops[i], (int)i);
+        }
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return cuda_fail(c, le, "kernel launch");
         Status s;

@@ -1002,7 +1002,7 @@ void fill_args(hybrid_ctx *c, PairArgs &a)
         a.ah[d] = c->acc_h[d].p;
     }
     unsigned long long *ctr = (unsigned long long *)c->counter.p;
-    a.counter = ctr + 2;
+    a.counter = ctr + 2;   // + 1 for the near kernels
     a.inter_soft = ctr + 6;
     a.inter_hard = ctr + 7;
     a.st = status_dev(c);
@@ -1029,6 +1029,19 @@ void go_far(hybrid_ctx *c, const PairArgs &a)
     else k_far<KS, 3><<<c->nsm * 16, PAIR_THREADS, 0, c->st>>>(a);
 }
 
+// Counters and FP32 sums of the next far (soft sums) or near (hard sums) launch to zero.
+__global__ void __launch_bounds__(256) k_clear_pairs(PairArgs a, bool near, int bits, int64_t N, int prec)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        *a.counter = 0ull;
+        *(near ? a.inter_hard : a.inter_soft) = 0ull;
+    }
+    void *const *acc = near ? a.ah : a.as;
+    if (prec == 1 && (!near || (bits & 2)))
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x)
+            for (int d = 0; d < 3; ++d) ((float *)acc[d])[i] = 0.0f;
+}
+
 // near = false: cells and far particles (soft); near = true: near particles
 // (soft and/or hard per mode bits)
 void launch_pairs(hybrid_ctx *c, bool near, int mode)
@@ -1037,10 +1050,17 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
     fill_args(c, a);
     a.want_soft = mode & 1;
     a.want_hard = (mode >> 1) & 1;
-    Status *st = status_dev(c);
-    unsigned long long *ctr = (unsigned long long *)c->counter.p;
-    cudaMemsetAsync(ctr + 2, 0, sizeof(unsigned long long), c->st);
-    cudaMemsetAsync(ctr + (near ? 7 : 6), 0, sizeof(unsigned long long), c->st);
+    if (near) a.counter += 1;
+    // the walk clears the counters and sums of the pair kernels after it; a near launch without a walk of its own
+    // (reused lists) clears them here
+    const int bits = near ? mode & 3 : 1;
+    const bool clean = (c->pairs_clean & bits) == bits;
+    c->pairs_clean &= near ? 0 : ~0;
+    if (!clean) {
+        k_clear_pairs<<<(int)std::min<int64_t>((c->N + 255) / 256, (int64_t)c->nsm * 8), 256, 0, c->st>>>(
+            a, near, bits, c->N, c->p.precision);
+        c->launches++;
+    }
     const int kind = near ? PROF_HARD : PROF_SOFT;
     cudaEvent_t e0 = nullptr;
     prof_begin(c, kind, &e0);
@@ -1058,10 +1078,6 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
         // work items written by the one-pass walk: far ones in wmap, near ones in wnear
         a.items = (const WorkItem *)(near ? c->wnear.p : c->wmap.p);
         a.nwork = (const uint64_t *)c->counter.p + (near ? 12 : 11);
-        if (!near)
-            for (int d = 0; d < 3; ++d) cudaMemsetAsync(c->acc_s[d].p, 0, (size_t)c->N * sizeof(float), c->st);
-        if (near && a.want_hard)
-            for (int d = 0; d < 3; ++d) cudaMemsetAsync(c->acc_h[d].p, 0, (size_t)c->N * sizeof(float), c->st);
         if (!near) {
             const int ks = sinks_per_lane(c);
             if (ks == 1) go_far<1>(c, a);

@@ -840,7 +840,11 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_cells(int64_t N, int S, const
         }
         __syncthreads();
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) counter[9] = 0ull;   // chunk items of the moments
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        counter[9] = 0ull;                                       // chunk items of the moments
+        counter[0] = counter[1] = 0ull;                          // the walk's groups,
+        counter[10] = counter[11] = counter[12] = 0ull;          // list cursor and items
+    }
 }
 
 struct NodeArgs {
@@ -1778,6 +1782,7 @@ void launch_topology(hybrid_ctx *c)
     a.ntiles = ntiles;
     k_nodes<<<grid, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
     c->launches += 2;
+    c->walk_clean = true;
 }
 
 void launch_moments(hybrid_ctx *c)

@@ -55,6 +55,9 @@ struct WalkArgs {
     int mode;
     Status *st;
     int where;
+    unsigned long long *queue;   // [0], [1]: next far / near item or unit of the pair kernels, zeroed here with
+    unsigned long long *pairs;   // [0], [1]: the pair counts
+    float *acc_s[3], *acc_h[3];  // FP32 form: the accelerations this walk's pair kernels add to, zeroed here
     // one-pass form
     const uint32_t *gfirst;
     unsigned long long *list_cursor;     // next free list entry
@@ -104,11 +107,22 @@ __device__ __forceinline__ double dist_box_f64(double p0, double p1, double p2, 
     return sqrt(s);
 }
 
+// What the pair kernels after this walk count from (the far counts only when the soft force follows).
+__device__ __forceinline__ void clear_pair_counters(const WalkArgs &a)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        a.queue[0] = a.queue[1] = 0ull;
+        if (a.mode & 1) a.pairs[0] = 0ull;
+        a.pairs[1] = 0ull;
+    }
+}
+
 template <bool F64, bool FILL>
 __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
 {
     Status *st = a.st;
     if (st->code) return;
+    if (FILL) clear_pair_counters(a);
     const int lane = threadIdx.x & 31;
     const unsigned ltmask = (1u << lane) - 1u;
     const int64_t ng = *a.ngroups;
@@ -302,6 +316,7 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
 {
     Status *st = a.st;
     if (st->code) return;
+    clear_pair_counters(a);
     const int lane = threadIdx.x & 31;
     const int64_t ng = *a.ngroups;
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -324,6 +339,12 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
         const GroupF G = a.gF[g];
         const float cx = G.c_hi.x, cy = G.c_hi.y, cz = G.c_hi.z, hx = G.c_hi.w;
         const float lx = G.c_lo.x, ly = G.c_lo.y, lz = G.c_lo.z, hy = G.c_lo.w, hz = G.hz_root.x;
+        for (uint32_t i = gfirst + lane; i < gfirst + gn; i += 32)
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                if (want_soft) a.acc_s[d][i] = 0.0f;
+                if (want_hard) a.acc_h[d][i] = 0.0f;
+            }
         my_start = my_cur;
         my_len = 0;
         uint32_t early_far = 0, early_near = 0;   // items already emitted for this group
@@ -531,6 +552,12 @@ void launch_walk(hybrid_ctx *c, int mode)
     a.st = st;
     a.where = c->op;
     a.gfirst = (const uint32_t *)c->gfirst.p;
+    a.queue = (unsigned long long *)c->counter.p + 2;
+    a.pairs = (unsigned long long *)c->counter.p + 6;
+    for (int d = 0; d < 3; ++d) {
+        a.acc_s[d] = (float *)c->acc_s[d].p;
+        a.acc_h[d] = (float *)c->acc_h[d].p;
+    }
     a.list_cursor = (unsigned long long *)c->counter.p + 10;
     a.item_count = (unsigned long long *)c->counter.p + 11;
     a.items_far = (WorkItem *)c->wmap.p;
@@ -547,9 +574,14 @@ void launch_walk(hybrid_ctx *c, int mode)
     const int grid = c->walk_warps * 32 / WALK_THREADS;
     cudaEvent_t e0 = nullptr;
     prof_begin(c, PROF_WALK, &e0);
-    if (c->p.precision == 1) {   // one pass: the group counter, the list cursor and the item counts start at 0
-        cudaMemsetAsync(c->counter.p, 0, sizeof(unsigned long long), c->st);
+    // the group counters, the list cursor and the item counts start at 0: the build before this walk zeroed them
+    if (!c->walk_clean) {
+        cudaMemsetAsync(c->counter.p, 0, 2 * sizeof(unsigned long long), c->st);
         cudaMemsetAsync((unsigned long long *)c->counter.p + 10, 0, 3 * sizeof(unsigned long long), c->st);
+    }
+    c->walk_clean = false;
+    c->pairs_clean = mode;
+    if (c->p.precision == 1) {   // one pass
         a.counter = (unsigned long long *)c->counter.p;
         if (small_job) k_walk1<6><<<grid, WALK_THREADS, 0, c->st>>>(a);
         else k_walk1<8><<<grid, WALK_THREADS, 0, c->st>>>(a);
@@ -559,7 +591,6 @@ void launch_walk(hybrid_ctx *c, int mode)
         return;
     }
     // count pass
-    cudaMemsetAsync(c->counter.p, 0, 2 * sizeof(unsigned long long), c->st);
     a.counter = (unsigned long long *)c->counter.p;
     k_walk<true, false><<<grid, WALK_THREADS, 0, c->st>>>(a);
     scan_u64(c, (uint64_t *)c->lcnt.p, 0, d_n3, 3 * c->capGroups, d_total);
