@@ -264,6 +264,7 @@ void launch_topology(hybrid_ctx *c);       // nodes and sink groups from the sor
 int cell_tiles(int64_t N);
 size_t cell_count_bytes(int64_t N);        // its counts per tile
 void launch_moments(hybrid_ctx *c);        // needs topology and the permuted state
+void launch_inspect(hybrid_ctx *c);        // FP32 form: the moments and geometry hybrid_tree_copy reports
 void launch_groups(hybrid_ctx *c);         // group table from the nodes, for an n_crit launch_topology leaves out
 void launch_group_boxes(hybrid_ctx *c);    // needs the group table and the permuted state
 void launch_wait_selftest(hybrid_ctx *c, int max_polls);   // a bounded wait on a flag nothing sets

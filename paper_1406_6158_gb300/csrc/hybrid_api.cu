@@ -1106,6 +1106,7 @@ hybrid_status hybrid_tree_copy(hybrid_ctx *c, uint64_t *keys, int32_t *level, in
     int64_t nn = 0, ng = 0;
     hybrid_status r = hybrid_tree_info(c, &nn, &ng);
     if (r != HYBRID_OK) return r;
+    launch_inspect(c);
     std::vector<uint32_t> f, cn, ch, nc, pa, lv, gn;
     std::vector<double> M, cx, cy, cz, bm, B2, de, sd, og, rb, glo, ghi;
     std::vector<uint64_t> k;

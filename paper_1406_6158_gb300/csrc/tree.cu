@@ -1413,6 +1413,7 @@ struct FinArgs {
     const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nlevel;
     const uint64_t *key;
     const int32_t *psys;
+    int S;
     const SysBox *box;
     const SysParams *sp;
     double *M, *cx, *cy, *cz, *B2;
@@ -1425,21 +1426,53 @@ struct FinArgs {
     double *rb, *hr, *delta, *side, *org;
 };
 
-__device__ __forceinline__ void prefix_q(uint64_t key, uint32_t lev, uint32_t q[3])
+// every third bit of a key, from bit 0 (the inverse of spread3)
+__device__ __forceinline__ uint32_t compact3(uint64_t x)
 {
-    q[0] = q[1] = q[2] = 0;
-    for (uint32_t l = 1; l <= lev; ++l) {
-        const uint32_t d = digit_at(key, (int)l);
-        q[0] = (q[0] << 1) | ((d >> 2) & 1u);
-        q[1] = (q[1] << 1) | ((d >> 1) & 1u);
-        q[2] = (q[2] << 1) | (d & 1u);
-    }
+    x &= 0x1249249249249249ull;
+    x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
+    x = (x | (x >> 4)) & 0x100f00f00f00f00full;
+    x = (x | (x >> 8)) & 0x1f0000ff0000ffull;
+    x = (x | (x >> 16)) & 0x1f00000000ffffull;
+    x = (x | (x >> 32)) & 0x1fffffull;
+    return (uint32_t)x;
 }
 
-// Per node: geometry, delta, MAC radius, walk criteria and packed topology.
-// F64: from the FP64 moments. FP32 form: delta, r_b and the criteria in FP32
-// from the hi/lo centre of mass (cell centres are exact in FP32 on the hi
-// grid), then the FP64 copies of the moments for inspection.
+// integer cell coordinates of a key's level-lev cell
+__device__ __forceinline__ void prefix_q(uint64_t key, uint32_t lev, uint32_t q[3])
+{
+    q[0] = compact3(key >> 2) >> (LEVELS - lev);
+    q[1] = compact3(key >> 1) >> (LEVELS - lev);
+    q[2] = compact3(key) >> (LEVELS - lev);
+}
+
+struct CritF {
+    float rb, hr, delta;
+};
+
+// FP32 form: delta, r_b and the Eq. (15) radius from the hi/lo centre of mass (cell centres are exact in FP32 on the
+// hi grid)
+__device__ __forceinline__ CritF crit_f32(const FinArgs &a, uint32_t c, uint32_t lev, const uint32_t q[3],
+                                          const SysParams &P, const SysBox &bx)
+{
+    const float sdf = ldexpf((float)bx.L, -(int)lev);
+    const float4 A = a.nA[c], B = a.nB[c];
+    // cell centre relative to the root corner: (q + 1/2) side, exact in FP32
+    const float e0 = (A.x - ((float)q[0] + 0.5f) * sdf) + B.x;
+    const float e1 = (A.y - ((float)q[1] + 0.5f) * sdf) + B.y;
+    const float e2 = (A.z - ((float)q[2] + 0.5f) * sdf) + B.z;
+    CritF r;
+    r.delta = sqrtf(e0 * e0 + e1 * e1 + e2 * e2);
+    const float bm = __uint_as_float(a.bmax32[c]);
+    if (P.mac == 1) r.rb = 0.5f * bm + sqrtf(0.25f * bm * bm + sqrtf(3.0f * B.w / (float)P.a_err));
+    else r.rb = (P.theta > 0.0) ? sdf / (float)P.theta + r.delta : INFINITY;
+    r.hr = P.R2f + P.skinf + bm;
+    return r;
+}
+
+// F64: criteria from the FP64 moments, and what hybrid_tree_copy reports. FP32 form: the walk's records only
+// (k_inspect makes the reports when they are asked for: 170 bytes and a dozen FP64 operations a node that no
+// force needs).
 template <bool F64>
 __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
 {
@@ -1447,63 +1480,64 @@ __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
     const uint32_t total = a.lvl[LEVELS + 1];
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
         const uint32_t f = a.nfirst[c];
-        const int s = a.psys[f];
+        const int s = a.S == 1 ? 0 : a.psys[f];
         const SysParams &P = a.sp[s];
         const SysBox &bx = a.box[s];
         const uint32_t lev = a.nlevel[c];
         uint32_t q[3];
         prefix_q(a.key[f], lev, q);
-        const double sd = ldexp(bx.L, -(int)lev);
-        double rb, hr, delta;
         if (F64) {
-            double o[3];
+            const double sd = ldexp(bx.L, -(int)lev);
+            double o[3], rb;
             for (int k = 0; k < 3; ++k) o[k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
             const double ctr0 = o[0] + 0.5 * sd, ctr1 = o[1] + 0.5 * sd, ctr2 = o[2] + 0.5 * sd;
             const double e0 = a.cx[c] - ctr0, e1 = a.cy[c] - ctr1, e2 = a.cz[c] - ctr2;
-            delta = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
+            const double delta = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
             const double bm = __longlong_as_double((long long)a.bmax[c]);
             if (P.mac == 1) rb = 0.5 * bm + sqrt(0.25 * bm * bm + sqrt(3.0 * a.B2[c] / P.a_err));
             else rb = (P.theta > 0.0) ? sd / P.theta + delta : INFINITY;
-            hr = P.R2 + P.skin + bm;   // Eq. (15) radius (plus the skin of reused lists)
+            const double hr = P.R2 + P.skin + bm;   // Eq. (15) radius (plus the skin of reused lists)
             const double sacc = fmax(rb, hr);
             a.crit[c] = make_float2((float)(sacc * sacc), P.has_hard ? (float)(hr * hr) : -1.0f);
             a.nD[c] = make_double4_32a(a.cx[c], a.cy[c], a.cz[c], a.M[c]);
             for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = o[k];
+            a.rb[c] = rb;
+            a.hr[c] = hr;
+            a.delta[c] = delta;
+            a.side[c] = sd;
         } else {
-            const float sdf = ldexpf((float)bx.L, -(int)lev);
-            const float4 A = a.nA[c], B = a.nB[c];
-            // cell centre relative to the root corner: (q + 1/2) side, exact in FP32
-            const float e0 = (A.x - ((float)q[0] + 0.5f) * sdf) + B.x;
-            const float e1 = (A.y - ((float)q[1] + 0.5f) * sdf) + B.y;
-            const float e2 = (A.z - ((float)q[2] + 0.5f) * sdf) + B.z;
-            const float df = sqrtf(e0 * e0 + e1 * e1 + e2 * e2);
-            const float bm = __uint_as_float(a.bmax32[c]);
-            float rbf;
-            if (P.mac == 1) rbf = 0.5f * bm + sqrtf(0.25f * bm * bm + sqrtf(3.0f * B.w / (float)P.a_err));
-            else rbf = (P.theta > 0.0) ? sdf / (float)P.theta + df : INFINITY;
-            const float hrf = P.R2f + P.skinf + bm;
-            const float sacc = fmaxf(rbf, hrf);
-            a.crit[c] = make_float2(sacc * sacc, P.has_hard ? hrf * hrf : -1.0f);
-            // FP64 copies (all lanes busy): moments, b_max, geometry
-            const double c0 = bx.lo[0] + ((double)A.x + (double)B.x), c1 = bx.lo[1] + ((double)A.y + (double)B.y),
-                         c2 = bx.lo[2] + ((double)A.z + (double)B.z);
-            a.M[c] = (double)A.w;
-            a.cx[c] = c0;
-            a.cy[c] = c1;
-            a.cz[c] = c2;
-            a.B2[c] = (double)B.w;
-            a.bmax[c] = (unsigned long long)__double_as_longlong((double)bm);
-            a.nD[c] = make_double4_32a(c0, c1, c2, (double)A.w);
-            for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
-            rb = rbf;
-            hr = hrf;
-            delta = df;
+            const CritF r = crit_f32(a, c, lev, q, P, bx);
+            const float sacc = fmaxf(r.rb, r.hr);
+            a.crit[c] = make_float2(sacc * sacc, P.has_hard ? r.hr * r.hr : -1.0f);
         }
         const uint32_t ch = a.nchild[c];
         a.topo[c] = make_uint4(ch, ch == NONE ? 0u : a.nchend[c] - ch, f, a.nend[c] - f);
-        a.rb[c] = rb;
-        a.hr[c] = hr;
-        a.delta[c] = delta;
+    }
+}
+
+// FP32 form: the FP64 copies of the moments and the geometry that hybrid_tree_copy reports.
+__global__ void __launch_bounds__(256) k_inspect(FinArgs a)
+{
+    const uint32_t total = a.lvl[LEVELS + 1];
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
+        const uint32_t f = a.nfirst[c];
+        const int s = a.psys[f];
+        const SysBox &bx = a.box[s];
+        const uint32_t lev = a.nlevel[c];
+        uint32_t q[3];
+        prefix_q(a.key[f], lev, q);
+        const CritF r = crit_f32(a, c, lev, q, a.sp[s], bx);
+        const float4 A = a.nA[c], B = a.nB[c];
+        a.M[c] = (double)A.w;
+        a.cx[c] = bx.lo[0] + ((double)A.x + (double)B.x);
+        a.cy[c] = bx.lo[1] + ((double)A.y + (double)B.y);
+        a.cz[c] = bx.lo[2] + ((double)A.z + (double)B.z);
+        a.B2[c] = (double)B.w;
+        a.bmax[c] = (unsigned long long)__double_as_longlong((double)__uint_as_float(a.bmax32[c]));
+        const double sd = ldexp(bx.L, -(int)lev);
+        for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
+        a.rb[c] = r.rb;
+        a.delta[c] = r.delta;
         a.side[c] = sd;
     }
 }
@@ -1785,6 +1819,40 @@ void launch_topology(hybrid_ctx *c)
     c->walk_clean = true;
 }
 
+static FinArgs fin_args(hybrid_ctx *c)
+{
+    FinArgs f;
+    f.lvl = (const uint32_t *)c->lvl.p;
+    f.nfirst = (const uint32_t *)c->nfirst.p;
+    f.nend = (const uint32_t *)c->nend.p;
+    f.nchend = (const uint32_t *)c->nchend.p;
+    f.nchild = (const uint32_t *)c->nchild.p;
+    f.nlevel = (const uint32_t *)c->nlevel.p;
+    f.key = (const uint64_t *)c->keys[0].p;
+    f.psys = (const int32_t *)c->psys.p;
+    f.S = c->S;
+    f.box = (const SysBox *)c->box.p;
+    f.sp = (const SysParams *)c->sp_dev.p;
+    f.M = (double *)c->nM.p;
+    f.cx = (double *)c->ncx.p;
+    f.cy = (double *)c->ncy.p;
+    f.cz = (double *)c->ncz.p;
+    f.B2 = (double *)c->nB2.p;
+    f.bmax = (unsigned long long *)c->nbmax.p;
+    f.bmax32 = (const unsigned int *)c->nbmax32.p;
+    f.nA = (const float4 *)c->nA.p;
+    f.nB = (const float4 *)c->nB.p;
+    f.crit = (float2 *)c->ncrit.p;
+    f.topo = (uint4 *)c->ntopo.p;
+    f.nD = (double4_32a *)c->nD.p;
+    f.rb = (double *)c->nrb.p;
+    f.hr = (double *)c->nhr.p;
+    f.delta = (double *)c->ndelta.p;
+    f.side = (double *)c->nside.p;
+    f.org = (double *)c->norg.p;
+    return f;
+}
+
 void launch_moments(hybrid_ctx *c)
 {
     Status *st = status_dev(c);
@@ -1827,37 +1895,17 @@ void launch_moments(hybrid_ctx *c)
         k_bmax_big<false><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, st);
     }
     c->launches += 2;
-    FinArgs f;
-    f.lvl = a.lvl;
-    f.nfirst = a.nfirst;
-    f.nend = a.nend;
-    f.nchend = a.nchend;
-    f.nchild = a.nchild;
-    f.nlevel = a.nlevel;
-    f.key = a.key;
-    f.psys = a.psys;
-    f.box = a.box;
-    f.sp = (const SysParams *)c->sp_dev.p;
-    f.M = (double *)c->nM.p;
-    f.cx = (double *)c->ncx.p;
-    f.cy = (double *)c->ncy.p;
-    f.cz = (double *)c->ncz.p;
-    f.B2 = (double *)c->nB2.p;
-    f.bmax = (unsigned long long *)c->nbmax.p;
-    f.bmax32 = (const unsigned int *)c->nbmax32.p;
-    f.nA = (const float4 *)c->nA.p;
-    f.nB = (const float4 *)c->nB.p;
-    f.crit = (float2 *)c->ncrit.p;
-    f.topo = (uint4 *)c->ntopo.p;
-    f.nD = (double4_32a *)c->nD.p;
-    f.rb = (double *)c->nrb.p;
-    f.hr = (double *)c->nhr.p;
-    f.delta = (double *)c->ndelta.p;
-    f.side = (double *)c->nside.p;
-    f.org = (double *)c->norg.p;
+    const FinArgs f = fin_args(c);
     if (c->p.precision == 0) k_finalize<true><<<grid, 256, 0, c->st>>>(f, st);
     else k_finalize<false><<<grid, 256, 0, c->st>>>(f, st);
-    c->launches += 3;
+    c->launches += 1;
+}
+
+void launch_inspect(hybrid_ctx *c)
+{
+    if (c->p.precision == 0) return;
+    k_inspect<<<grid_for(c, c->capNodes, 256, 8), 256, 0, c->st>>>(fin_args(c));
+    c->launches += 1;
 }
 
 void launch_groups(hybrid_ctx *c)
