@@ -984,6 +984,7 @@ struct MomArgs {
     const double *x, *y, *z, *m;
     const uint64_t *key;
     const int32_t *psys;
+    int S;
     const SysBox *box;
     double *M, *cx, *cy, *cz, *B2;
     float4 *nA, *nB;
@@ -1085,7 +1086,7 @@ __device__ __forceinline__ MomSumsF mom_range_f32(const float4 *__restrict__ phi
 __device__ __forceinline__ void mom_store_f32(const MomArgs &a, uint32_t c, uint32_t f, float M, float e0, float e1,
                                               float e2, float B2)
 {
-    const SysBox &b = a.box[a.psys[f]];
+    const SysBox &b = a.box[a.S == 1 ? 0 : a.psys[f]];
     const float4 h = a.phi[f], l = a.plo[f];
     const float t0 = l.x + e0, t1 = l.y + e1, t2 = l.z + e2;
     const float g0 = rintf(t0 * b.inv_uf) * b.uf, g1 = rintf(t1 * b.inv_uf) * b.uf, g2 = rintf(t2 * b.inv_uf) * b.uf;
@@ -1177,11 +1178,10 @@ __device__ __forceinline__ double warp_sum_d(double v)
 // FP64 form in FP64 (a whole warp). FP32 form in FP32 on offsets from the
 // first child's hi/lo centre of mass (hi differences exact), stored like a
 // small cell's, by G lanes (a warp or an aligned group of 8 with mask gm).
-__device__ void mom_combine_f64(const MomArgs &a, uint32_t c, int lane)
+// f: the cell's first particle; [ch0, ch0 + k): its children.
+__device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32_t ch0, uint32_t k, int lane)
 {
-    const uint32_t ch0 = a.nchild[c], k = a.nchend[c] - ch0;
-    const uint32_t f = a.nfirst[c];
-    const SysBox &b = a.box[a.psys[f]];
+    const SysBox &b = a.box[a.S == 1 ? 0 : a.psys[f]];
     const bool on = (uint32_t)lane < k;
     double M = 0.0, x = 0.0, y = 0.0, z = 0.0, B2 = 0.0;
     if (on) {
@@ -1215,11 +1215,10 @@ __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, int lane)
 }
 
 template <int G>
-__device__ void mom_combine_f32(const MomArgs &a, uint32_t c, int lane, unsigned gm)
+__device__ void mom_combine_f32(const MomArgs &a, uint32_t c, uint32_t f, uint32_t ch0, uint32_t k, int lane,
+                                unsigned gm)
 {
-    const uint32_t ch0 = a.nchild[c], k = a.nchend[c] - ch0;
-    const uint32_t f = a.nfirst[c];
-    const SysBox &b = a.box[a.psys[f]];
+    const SysBox &b = a.box[a.S == 1 ? 0 : a.psys[f]];
     const bool on = (uint32_t)lane < k;
     float4 A = make_float4(0.0f, 0.0f, 0.0f, 0.0f), B = A;
     if (on) {
@@ -1264,27 +1263,30 @@ __device__ void mom_combine_f32(const MomArgs &a, uint32_t c, int lane, unsigned
     }
 }
 
-// After cell c is final: if its parent is a larger cell and c is the last of
-// its children to finish, combine the parent, and so on upwards. G lanes (a
-// warp, or an aligned group of 8 with mask gm; lane = lane within the group).
+// After cell c (with parent p) is final: if its parent is a larger cell and c is
+// the last of its children to finish, combine the parent, and so on upwards. G
+// lanes (a warp, or an aligned group of 8 with mask gm; lane = lane within the
+// group). This chain of levels is what k_mom_small's time on a small system is
+// made of, so a level costs three waits: the parent's record (all fields at
+// once), the count, the children's moments.
 template <bool F64, int G>
-__device__ void mom_climb(const MomArgs &a, uint32_t c, int lane, unsigned gm)
+__device__ void mom_climb(const MomArgs &a, uint32_t p, int lane, unsigned gm)
 {
-    for (;;) {
-        const uint32_t p = a.nparent[c];
-        if (p == NONE || a.nend[p] - a.nfirst[p] <= MOM_CH) return;
+    while (p != NONE) {
+        const uint32_t f = a.nfirst[p], e = a.nend[p], ch0 = a.nchild[p], k = a.nchend[p] - ch0, up = a.nparent[p];
+        if (e - f <= MOM_CH) return;
         __syncwarp(gm);
         unsigned int old = 0;
-        if (lane == 0) {   // release: c's moments (stored by this lane) before the count; acquire: the others' after
+        if (lane == 0) {   // release: the child's moments (stored by this lane) before the count; acquire: the others' after
             cuda::atomic_ref<unsigned int, cuda::thread_scope_device> cnt(a.done[p]);
             old = cnt.fetch_add(1u, cuda::memory_order_acq_rel);
         }
         old = __shfl_sync(gm, old, 0, G);
-        if (old + 1u != a.nchend[p] - a.nchild[p]) return;
+        if (old + 1u != k) return;
         __syncwarp(gm);
-        if (F64) mom_combine_f64(a, p, lane);
-        else mom_combine_f32<G>(a, p, lane, gm);
-        c = p;
+        if (F64) mom_combine_f64(a, p, f, ch0, k, lane);
+        else mom_combine_f32<G>(a, p, f, ch0, k, lane, gm);
+        p = up;
     }
 }
 
@@ -1304,7 +1306,7 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (F64) {   // one warp per cell
         for (uint32_t c = warp; c < total; c += nw) {
-            const uint32_t f = a.nfirst[c], n = a.nend[c] - f;
+            const uint32_t f = a.nfirst[c], n = a.nend[c] - f, up = a.nparent[c];
             if (n <= MOM_CH || a.nchild[c] == NONE) {
                 const double o0 = a.x[f], o1 = a.y[f], o2 = a.z[f];
                 const MomSums r = mom_range(a, f, n, o0, o1, o2, lane);
@@ -1321,7 +1323,7 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
                 if (lane == 0) a.bmax64[c] = (unsigned long long)__double_as_longlong(dm);
-                mom_climb<true, 32>(a, c, lane, 0xffffffffu);
+                mom_climb<true, 32>(a, up, lane, 0xffffffffu);
             } else if (lane == 0) {
                 const uint32_t nch = (n + BM_CH - 1) / BM_CH;
                 const unsigned long long base = atomicAdd(nitems, (unsigned long long)nch);
@@ -1340,7 +1342,7 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
         for (uint32_t q = warp; q < nq; q += nw) {
             const uint32_t c = 4 * q + sub;
             if (c >= total) continue;
-            const uint32_t f = a.nfirst[c], n = a.nend[c] - f;
+            const uint32_t f = a.nfirst[c], n = a.nend[c] - f, up = a.nparent[c];
             if (n <= MOM_CH || a.nchild[c] == NONE) {
                 const MomSumsF r = mom_range_f32<8>(a.phi, a.plo, f, n, f, sl, gm);
                 const float iM = r.M > 0.0f ? 1.0f / r.M : 0.0f;
@@ -1351,7 +1353,7 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
                     mom_store_f32(a, c, f, r.M, e0, e1, e2, B2);
                     a.bmax32[c] = __float_as_uint(bm);
                 }
-                mom_climb<false, 8>(a, c, sl, gm);
+                mom_climb<false, 8>(a, up, sl, gm);
             } else if (sl == 0) {
                 const uint32_t nch = (n + BM_CH - 1) / BM_CH;
                 const unsigned long long base = atomicAdd(nitems, (unsigned long long)nch);
@@ -1871,6 +1873,7 @@ void launch_moments(hybrid_ctx *c)
     a.m = (const double *)c->x[6].p;
     a.key = (const uint64_t *)c->keys[0].p;
     a.psys = (const int32_t *)c->psys.p;
+    a.S = c->S;
     a.box = (const SysBox *)c->box.p;
     a.M = (double *)c->nM.p;
     a.cx = (double *)c->ncx.p;
