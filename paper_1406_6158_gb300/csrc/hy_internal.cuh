@@ -114,10 +114,10 @@ constexpr int LCH_FAR = 2048, LCH_FAR_SMALL = 256;
 // Entries per work item of a group of n sinks: lch for n >= 64, longer runs
 // (up to 8 lch) for smaller groups, so that items cost about the same
 // n x entries and a small group pays the per-item set-up less often.
-__host__ __device__ __forceinline__ uint64_t item_len(uint32_t n, int lch)
+__host__ __device__ __forceinline__ uint32_t item_len(uint32_t n, int lch)
 {
     const uint32_t f = n >= 64 ? 1u : (64u / (n > 0 ? n : 1u) < 8u ? 64u / (n > 0 ? n : 1u) : 8u);
-    return (uint64_t)lch * f;
+    return (uint32_t)lch * f;
 }
 
 struct GroupF {
