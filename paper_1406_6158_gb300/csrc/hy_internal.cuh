@@ -6,6 +6,7 @@
 
 #include <algorithm>
 #include <cstdint>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -46,12 +47,77 @@ struct SysBox {
     float uf, inv_uf;   // u and 1/u in FP32 (powers of two: exact)
 };
 
+// FP32 nearest to v, with integer operations where v is a normal FP32 number (a conversion from FP64 takes the FP64
+// pipe, 2 lanes per SM and clock).
+__host__ __device__ __forceinline__ float narrow_bits(uint64_t bits, bool &done)
+{
+    const int E = (int)(bits >> 52) & 0x7ff;
+    done = (unsigned)(E - 897) <= 252u;   // 2^-126 .. below 2^127: rounding up cannot overflow
+    const uint64_t t = (bits & 0x7fffffffffffffffull) - (896ull << 52);
+    const uint32_t f = (uint32_t)((t + 0x0fffffffull + ((t >> 29) & 1ull)) >> 29) | (uint32_t)((bits >> 63) << 31);
+    float r;
+    memcpy(&r, &f, 4);
+    return r;
+}
+__device__ __forceinline__ float narrow(double v)
+{
+    bool done;
+    const float r = narrow_bits((uint64_t)__double_as_longlong(v), done);
+    return done ? r : (float)v;
+}
+
+// The split below of d (its bits) on the grid of step 2^eu with integer operations: k = d / 2^eu rounded to the
+// nearest integer (ties to even) and the FP32 nearest to d - k 2^eu. False outside 2^-74 <= |d| < 2^30 2^eu.
+__host__ __device__ __forceinline__ bool split_bits(uint64_t bits, int eu, int32_t &k, float &rest)
+{
+    const int E = (int)(bits >> 52) & 0x7ff;
+    const int sh = eu + 1075 - E;                  // |d| = M 2^(E - 1075), the grid step is 2^sh units of M
+    if (E < 949 || E > 1150 || sh < 23) return false;
+    const bool neg = (bits >> 63) != 0;
+    const uint64_t M = (bits & ((1ull << 52) - 1ull)) | (1ull << 52);
+    uint32_t q = 0;
+    int64_t r = (int64_t)M;
+    if (sh <= 54) {
+        const uint64_t half = 1ull << (sh - 1), rem = M & ((half << 1) - 1ull);
+        q = (uint32_t)(M >> sh);
+        q += (rem > half || (rem == half && (q & 1u))) ? 1u : 0u;
+        r = (int64_t)(M - ((uint64_t)q << sh));
+    }
+    k = neg ? -(int32_t)q : (int32_t)q;
+    const bool rneg = (r < 0) != neg;
+    const uint64_t a = (uint64_t)(r < 0 ? -r : r);
+    uint32_t f = 0;
+    if (a) {
+        // the top 32 bits with the rest folded into the last one, rounded once to FP32, then the exponent
+#ifdef __CUDA_ARCH__
+        const int lz = __clzll((long long)a);
+#else
+        const int lz = __builtin_clzll(a);
+#endif
+        const uint64_t t = a << lz;
+        const float v = (float)((uint32_t)(t >> 32) | ((uint32_t)t ? 1u : 0u));
+        memcpy(&f, &v, 4);
+        f += (uint32_t)(32 - lz + E - 1075) << 23;
+        f |= rneg ? 0x80000000u : 0u;
+    }
+    memcpy(&rest, &f, 4);
+    return true;
+}
+
 // FP32 hi/lo copy of a coordinate relative to the root corner: hi = the
 // nearest multiple of u (at most 2^20 steps: exact in FP32), lo = the rest
-// (exact in FP64, then rounded to FP32, |lo| <= u/2).
+// (exact, then rounded to FP32, |lo| <= u/2). One FP64 instruction; with the
+// rounding and the conversions in FP64 (nine) the permutation of the state
+// was bound by the FP64 pipe.
 __device__ __forceinline__ void grid_split(double x, double lo0, const SysBox &b, float &h, float &l)
 {
     const double xp = __dsub_rn(x, lo0);
+    const int eu = (int)(((uint64_t)__double_as_longlong(b.u) >> 52) & 0x7ffu) - 1023;
+    int32_t k;
+    if ((unsigned)(eu + 126) <= 220u && split_bits((uint64_t)__double_as_longlong(xp), eu, k, l)) {
+        h = (float)k * b.uf;
+        return;
+    }
     const double hh = __dmul_rn(rint(__dmul_rn(xp, b.inv_u)), b.u);
     h = (float)hh;
     l = (float)__dsub_rn(xp, hh);

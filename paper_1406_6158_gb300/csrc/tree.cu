@@ -670,7 +670,11 @@ struct PermArgs {
     uint32_t *flag;       // [0] an overflowed sample sort: the order stays; [1] reset for the next build
 };
 
-__global__ void __launch_bounds__(256) k_permute(PermArgs a)
+// MINB blocks per SM: 8 (32 registers) for batches above 2^18 particles, where the gathers' bandwidth counts (2^24:
+// tree build 30.1 -> 28.7 ms per soft step against 64 registers, 2^20 1.172 -> 1.138); below, a thread's loads all go
+// out at once with 64 (2^12 and 2^17 2 and 1 % of the step faster).
+template <int MINB>
+__global__ void __launch_bounds__(256, MINB) k_permute(PermArgs a)
 {
     // whatever the status: later kernels rely on a consistent permutation
     const bool keep = a.flag[0] != 0u;
@@ -694,7 +698,7 @@ __global__ void __launch_bounds__(256) k_permute(PermArgs a)
             float h[3], l[3];
 #pragma unroll
             for (int d = 0; d < 3; ++d) grid_split(v[d], b.lo[d], b, h[d], l[d]);
-            a.phi[i] = make_float4(h[0], h[1], h[2], (float)v[6]);
+            a.phi[i] = make_float4(h[0], h[1], h[2], narrow(v[6]));
             a.plo[i] = make_float4(l[0], l[1], l[2], 0.0f);
         }
         if (a.pd) a.pd[i] = make_double4_32a(v[0], v[1], v[2], v[6]);
@@ -1766,7 +1770,8 @@ void launch_permute(hybrid_ctx *c)
     a.bmax = (unsigned long long *)c->boxmax.p;
     a.S = c->S;
     a.flag = (uint32_t *)c->ss_flag.p;
-    k_permute<<<grid_for(c, N, 256), 256, 0, c->st>>>(a);
+    if (N <= 1 << 18) k_permute<4><<<grid_for(c, N, 256), 256, 0, c->st>>>(a);
+    else k_permute<8><<<grid_for(c, N, 256), 256, 0, c->st>>>(a);
     c->launches++;
     for (int f = 0; f < 7; ++f) std::swap(c->x[f], c->xa[f]);
     std::swap(c->id, c->ida);
