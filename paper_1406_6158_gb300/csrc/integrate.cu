@@ -124,46 +124,69 @@ __device__ __forceinline__ double widen(double f) { return f; }
 
 // The step sizes of each kind are per-system constants (SysParams), so a
 // particle's update is the three products and sums per vector and nothing else.
+// Every array a particle needs is loaded before the first kick: at small sizes
+// the launch lasts as long as its chain of loads.
 template <typename A>
 __global__ void __launch_bounds__(256) k_kick_drift(int64_t N, StatePtrs w, const SysParams *__restrict__ sp,
-                                                    KickSpec ks, Status *st)
+                                                    KickSpec ks, int S, Status *st)
 {
     if (st->code) return;
+    bool soft = false, hard = false;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        soft = soft || (k < ks.n && ks.which[k] == 0);
+        hard = hard || (k < ks.n && ks.which[k] != 0);
+    }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const SysParams &P = sp[w.psys[i]];
-        double v0 = w.x[3][i], v1 = w.x[4][i], v2 = w.x[5][i];
-        for (int k = 0; k < ks.n; ++k) {
-            const double h = ks.mode[k] == 1 ? P.h_soft : ks.mode[k] == 2 ? P.h_hard : ks.val[k];
-            void *const *acc = ks.which[k] ? w.ah : w.as;
-            const double a0 = widen(((const A *)acc[0])[i]);
-            const double a1 = widen(((const A *)acc[1])[i]);
-            const double a2 = widen(((const A *)acc[2])[i]);
-            v0 = __dadd_rn(v0, __dmul_rn(h, a0));
-            v1 = __dadd_rn(v1, __dmul_rn(h, a1));
-            v2 = __dadd_rn(v2, __dmul_rn(h, a2));
+        const SysParams &P = sp[S == 1 ? 0 : w.psys[i]];
+        double v0 = w.x[3][i], v1 = w.x[4][i], v2 = w.x[5][i], x0 = 0.0, x1 = 0.0, x2 = 0.0;
+        A s0 = 0, s1 = 0, s2 = 0, h0 = 0, h1 = 0, h2 = 0;
+        if (soft) {
+            s0 = ((const A *)w.as[0])[i];
+            s1 = ((const A *)w.as[1])[i];
+            s2 = ((const A *)w.as[2])[i];
         }
+        if (hard) {
+            h0 = ((const A *)w.ah[0])[i];
+            h1 = ((const A *)w.ah[1])[i];
+            h2 = ((const A *)w.ah[2])[i];
+        }
+        if (ks.dmode >= 0) {
+            x0 = w.x[0][i];
+            x1 = w.x[1][i];
+            x2 = w.x[2][i];
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < ks.n) {
+                const double h = ks.mode[k] == 1 ? P.h_soft : ks.mode[k] == 2 ? P.h_hard : ks.val[k];
+                const bool hd = ks.which[k] != 0;
+                v0 = __dadd_rn(v0, __dmul_rn(h, widen(hd ? h0 : s0)));
+                v1 = __dadd_rn(v1, __dmul_rn(h, widen(hd ? h1 : s1)));
+                v2 = __dadd_rn(v2, __dmul_rn(h, widen(hd ? h2 : s2)));
+            }
         w.x[3][i] = v0;
         w.x[4][i] = v1;
         w.x[5][i] = v2;
         if (ks.dmode >= 0) {
             const double dt = ks.dmode == 0 ? ks.dval : P.dt_hard;
-            const double x0 = __dadd_rn(w.x[0][i], __dmul_rn(dt, v0));
-            const double x1 = __dadd_rn(w.x[1][i], __dmul_rn(dt, v1));
-            const double x2 = __dadd_rn(w.x[2][i], __dmul_rn(dt, v2));
+            x0 = __dadd_rn(x0, __dmul_rn(dt, v0));
+            x1 = __dadd_rn(x1, __dmul_rn(dt, v1));
+            x2 = __dadd_rn(x2, __dmul_rn(dt, v2));
             w.x[0][i] = x0;
             w.x[1][i] = x1;
             w.x[2][i] = x2;
             if (ks.resplit) {
                 // the pair kernels' copy of the moved positions, and the distance of this drift (from the old
                 // and new hi/lo copies: hi differences are exact) added to the bound since the last build
-                const SysBox &b = w.box[w.psys[i]];
-                float h0, h1, h2, l0, l1, l2;
-                grid_split(x0, b.lo[0], b, h0, l0);
-                grid_split(x1, b.lo[1], b, h1, l1);
-                grid_split(x2, b.lo[2], b, h2, l2);
+                const SysBox &b = w.box[S == 1 ? 0 : w.psys[i]];
+                float g0, g1, g2, l0, l1, l2;
+                grid_split(x0, b.lo[0], b, g0, l0);
+                grid_split(x1, b.lo[1], b, g1, l1);
+                grid_split(x2, b.lo[2], b, g2, l2);
                 const float4 oh = w.phi[i], ol = w.plo[i];
-                const float d0 = (h0 - oh.x) + (l0 - ol.x), d1 = (h1 - oh.y) + (l1 - ol.y), d2 = (h2 - oh.z) + (l2 - ol.z);
-                w.phi[i] = make_float4(h0, h1, h2, oh.w);
+                const float d0 = (g0 - oh.x) + (l0 - ol.x), d1 = (g1 - oh.y) + (l1 - ol.y), d2 = (g2 - oh.z) + (l2 - ol.z);
+                w.phi[i] = make_float4(g0, g1, g2, oh.w);
                 w.plo[i] = make_float4(l0, l1, l2, 0.0f);
                 // rounded up by a few units in the last place: a bound, not an estimate
                 const float moved = w.disp[i] + sqrtf(d0 * d0 + d1 * d1 + d2 * d2) * 1.000001f + 1e-30f;
@@ -268,10 +291,10 @@ void launch_kick_seq(hybrid_ctx *c, int n, const int *which, const int *mode, co
     prof_begin(c, PROF_INTEG, &e0);
     if (c->p.precision == 1)
         k_kick_drift<float><<<grid, 256, 0, c->st>>>(N, state_ptrs(c), (const SysParams *)c->sp_dev.p, ks,
-                                                      status_dev(c));
+                                                      c->S, status_dev(c));
     else
         k_kick_drift<double><<<grid, 256, 0, c->st>>>(N, state_ptrs(c), (const SysParams *)c->sp_dev.p, ks,
-                                                       status_dev(c));
+                                                       c->S, status_dev(c));
     prof_end(c, PROF_INTEG, e0);
     c->launches++;
 }
