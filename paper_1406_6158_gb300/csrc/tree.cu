@@ -39,12 +39,40 @@ __device__ __forceinline__ double unord_dbl(unsigned long long u)
 // Root cube: per-axis minimum lo; side L = smallest power of two >= the
 // largest extent (1 when all particles coincide); scale = 2^21 / L.
 // ---------------------------------------------------------------------------
+__device__ __forceinline__ SysBox make_box(const unsigned long long *bmin, const unsigned long long *bmax, int s)   // values other blocks made
+{
+    double lo[3], ext = 0.0;
+    for (int d = 0; d < 3; ++d) {
+        lo[d] = unord_dbl(__ldcg(bmin + 3 * s + d));
+        const double e = __dsub_rn(unord_dbl(__ldcg(bmax + 3 * s + d)), lo[d]);
+        if (e > ext) ext = e;
+    }
+    double L = 1.0;
+    if (ext > 0.0) {
+        int e2;
+        const double f = frexp(ext, &e2);
+        L = (f == 0.5) ? ext : ldexp(1.0, e2);
+    }
+    SysBox b;
+    b.lo[0] = lo[0];
+    b.lo[1] = lo[1];
+    b.lo[2] = lo[2];
+    b.L = L;
+    b.scale = ldexp(1.0, LEVELS) / L;   // ratio of powers of two: exact
+    b.u = ldexp(L, -20);
+    b.inv_u = ldexp(1.0, 20) / L;
+    b.uf = (float)b.u;
+    b.inv_uf = (float)b.inv_u;
+    return b;
+}
+
+// The last block to finish (a ticket, no waiting) makes the cubes.
 __global__ void __launch_bounds__(256) k_box(const double *__restrict__ x, const double *__restrict__ y,
                                              const double *__restrict__ z, const Chunk *__restrict__ chunks,
                                              int nchunks, unsigned long long *bmin, unsigned long long *bmax, int nbk,
                                              int S, const int64_t *__restrict__ off, const SSys *__restrict__ ss,
                                              const uint64_t *__restrict__ key, uint32_t *__restrict__ cnt,
-                                             uint32_t *__restrict__ flag)
+                                             uint32_t *__restrict__ flag, unsigned *ticket, SysBox *__restrict__ boxout)
 {
     // the sort always runs, whatever the status: later kernels rely on a consistent permutation
     // sample sort (nbk buckets, 0 for the radix sort): bucket counts cleared, and whether the splitters (the
@@ -103,33 +131,15 @@ __global__ void __launch_bounds__(256) k_box(const double *__restrict__ x, const
         }
         __syncthreads();
     }
-}
-
-__device__ __forceinline__ SysBox make_box(const unsigned long long *bmin, const unsigned long long *bmax, int s)
-{
-    double lo[3], ext = 0.0;
-    for (int d = 0; d < 3; ++d) {
-        lo[d] = unord_dbl(bmin[3 * s + d]);
-        const double e = __dsub_rn(unord_dbl(bmax[3 * s + d]), lo[d]);
-        if (e > ext) ext = e;
-    }
-    double L = 1.0;
-    if (ext > 0.0) {
-        int e2;
-        const double f = frexp(ext, &e2);
-        L = (f == 0.5) ? ext : ldexp(1.0, e2);
-    }
-    SysBox b;
-    b.lo[0] = lo[0];
-    b.lo[1] = lo[1];
-    b.lo[2] = lo[2];
-    b.L = L;
-    b.scale = ldexp(1.0, LEVELS) / L;   // ratio of powers of two: exact
-    b.u = ldexp(L, -20);
-    b.inv_u = ldexp(1.0, 20) / L;
-    b.uf = (float)b.u;
-    b.inv_uf = (float)b.inv_u;
-    return b;
+    __shared__ bool last;
+    __threadfence();   // this block's bounds are visible before its ticket
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    for (int s = threadIdx.x; s < S; s += blockDim.x) boxout[s] = make_box(bmin, bmax, s);
+    if (threadIdx.x == 0) *ticket = 0u;
 }
 
 // ---------------------------------------------------------------------------
@@ -172,23 +182,14 @@ __device__ __forceinline__ int pow2_exponent(double scale)
     return (int)(((unsigned long long)__double_as_longlong(scale) >> 52) & 0x7ffu) - 1023;
 }
 
-// Also finishes the root cubes (from the atomic min/max) and stores them.
 __global__ void __launch_bounds__(256) k_keys(int64_t N, const double *__restrict__ x, const double *__restrict__ y,
                                               const double *__restrict__ z, const int32_t *__restrict__ psys, int S,
-                                              const unsigned long long *__restrict__ bmin,
-                                              const unsigned long long *__restrict__ bmax, SysBox *__restrict__ boxout,
-                                              uint64_t *__restrict__ key, uint32_t *__restrict__ val, const Status *st)
+                                              const SysBox *__restrict__ box, uint64_t *__restrict__ key,
+                                              uint32_t *__restrict__ val)
 {
-    if (blockIdx.x == 0)
-        for (int s = threadIdx.x; s < S; s += blockDim.x) boxout[s] = make_box(bmin, bmax, s);
-    __shared__ SysBox b1;   // single-system batches: the cube computed once per block
-    if (S == 1) {
-        if (threadIdx.x == 0) b1 = make_box(bmin, bmax, 0);
-        __syncthreads();
-    }
-    (void)st;   // the sort always runs: later kernels rely on a consistent permutation
+    // the sort always runs, whatever the status: later kernels rely on a consistent permutation
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
-        const SysBox b = S == 1 ? b1 : make_box(bmin, bmax, psys[i]);
+        const SysBox &b = box[S == 1 ? 0 : psys[i]];
         const int es = pow2_exponent(b.scale);
         const uint32_t qx = cell_coord(x[i], b.lo[0], es);
         const uint32_t qy = cell_coord(y[i], b.lo[1], es);
@@ -437,20 +438,11 @@ __device__ __forceinline__ bool comp_less(uint64_t ka, uint32_t va, uint64_t kb,
 __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__restrict__ x,
                                                      const double *__restrict__ y, const double *__restrict__ z,
                                                      const int32_t *__restrict__ psys, int S,
-                                                     const unsigned long long *__restrict__ bmin,
-                                                     const unsigned long long *__restrict__ bmax,
-                                                     SysBox *__restrict__ boxout, const int64_t *__restrict__ off,
+                                                     const SysBox *__restrict__ box, const int64_t *__restrict__ off,
                                                      const SSys *__restrict__ ss, const uint64_t *__restrict__ old,
                                                      uint64_t *__restrict__ rk, uint32_t *__restrict__ rv,
                                                      uint32_t *__restrict__ cnt, uint32_t *flag, Status *st, int where)
 {
-    if (blockIdx.x == 0)
-        for (int s = threadIdx.x; s < S; s += blockDim.x) boxout[s] = make_box(bmin, bmax, s);
-    __shared__ SysBox b1;   // single-system batches: the cube computed once per block
-    if (S == 1) {
-        if (threadIdx.x == 0) b1 = make_box(bmin, bmax, 0);
-        __syncthreads();
-    }
     const int lane = threadIdx.x & 31;
     const bool ordered = flag[1] == 0u;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -460,7 +452,7 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
         uint64_t k = 0ull;
         if (i < N) {
             const int sy = S == 1 ? 0 : psys[i];
-            const SysBox bx = S == 1 ? b1 : make_box(bmin, bmax, sy);
+            const SysBox &bx = box[sy];
             const int es = pow2_exponent(bx.scale);
             const uint32_t qx = cell_coord(x[i], bx.lo[0], es);
             const uint32_t qy = cell_coord(y[i], bx.lo[1], es);
@@ -1685,7 +1677,8 @@ void launch_box(hybrid_ctx *c)
         (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p, (const Chunk *)c->chunks_dev.p,
         c->nchunks, (unsigned long long *)c->boxmin.p, (unsigned long long *)c->boxmax.p, c->sort_fallback ? 0 : c->nbk,
         c->S, (const int64_t *)c->off_dev.p, (const SSys *)c->ss_sys.p, (const uint64_t *)c->keys[0].p,
-        (uint32_t *)c->ss_cnt.p, (uint32_t *)c->ss_flag.p);
+        (uint32_t *)c->ss_cnt.p, (uint32_t *)c->ss_flag.p, (unsigned *)((unsigned long long *)c->counter.p + 14),
+        (SysBox *)c->box.p);
     c->launches += 1;
 }
 
@@ -1701,8 +1694,7 @@ void launch_keys_sort(hybrid_ctx *c)
         uint32_t *rv = (uint32_t *)c->ss_rv.p;
         k_keys_append<<<grid_for(c, N, 256), 256, 0, c->st>>>(
             N, (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p,
-            (const int32_t *)c->psys.p, c->S, (const unsigned long long *)c->boxmin.p,
-            (const unsigned long long *)c->boxmax.p, (SysBox *)c->box.p, (const int64_t *)c->off_dev.p,
+            (const int32_t *)c->psys.p, c->S, (const SysBox *)c->box.p, (const int64_t *)c->off_dev.p,
             (const SSys *)c->ss_sys.p, k0, rk, rv, cnt, flag, st, c->op);
         const int grid = std::min((c->nbk + SSB_WARPS - 1) / SSB_WARPS, c->nsm * 16);
         // up to SS_SUM_MAX buckets every block of the sort adds up the counts before its buckets (at most 32 loads
@@ -1718,9 +1710,7 @@ void launch_keys_sort(hybrid_ctx *c)
     }
     k_keys<<<grid_for(c, N, 256), 256, 0, c->st>>>(N, (const double *)c->x[0].p, (const double *)c->x[1].p,
                                                     (const double *)c->x[2].p, (const int32_t *)c->psys.p, c->S,
-                                                    (const unsigned long long *)c->boxmin.p,
-                                                    (const unsigned long long *)c->boxmax.p, (SysBox *)c->box.p, k0, v0,
-                                                    st);
+                                                    (const SysBox *)c->box.p, k0, v0);
     c->launches++;
     uint32_t *rs = (uint32_t *)c->hist.p;
     uint32_t *counts = rs + RS_HDR, *look = counts + (size_t)2048 * c->S;
