@@ -32,6 +32,7 @@ struct SysParams {
     double skin;                      // Verlet skin of reused neighbour lists (0: rebuild every hard step)
     float Gf, eps2f, R2f, R2sqf, invdRf, R2sqlo;   // R2sqf + R2sqlo = R2^2 to ~2^-48
     float skinf, half_skinf;       // skin and skin / 2 in FP32
+    float thetaf, a_errf;
     int32_t mac, has_hard;
 };
 
@@ -260,7 +261,7 @@ struct hybrid_ctx {
     // tree
     hy::Buf lvl, nfirst, nend, nchild, nchend, nparent, nlevel, ndone;   // nodes: particles and children [first, end)
     hy::Buf cells, ccnt;                          // topology scratch: packed levels per particle, counts per tile
-    hy::Buf nbig, mitems, mpart;                  // moments of large cells: chunk items and sums
+    hy::Buf nbig, mitems;                         // b_max of large cells: the cells (FP64 form: their chunks)
     hy::Buf nbmax32;                              // b_max as FP32 bits (FP32 form)
     int64_t capItems = 0;
     hy::Buf nM, ncx, ncy, ncz, nB2, nbmax;     // FP64 moments

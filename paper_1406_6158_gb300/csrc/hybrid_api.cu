@@ -140,6 +140,8 @@ SysParams make_sp(const hybrid_params &p)
     s.skin = p.R2 > 0.0 ? p.skin : 0.0;
     s.skinf = (float)s.skin;
     s.half_skinf = (float)(0.5 * s.skin);
+    s.thetaf = (float)p.theta;
+    s.a_errf = (float)p.a_err;
     s.has_hard = p.R2 > 0.0 ? 1 : 0;
     s.R2sq = s.has_hard ? p.R2 * p.R2 : 0.0;
     s.invdR = s.has_hard ? 1.0 / (p.R2 - p.R1) : 0.0;
@@ -206,7 +208,7 @@ bool reserve(hybrid_ctx *c)
         ok = ok && ensure(c, c->lcnt, (3 * n + 2) * 8) && ensure(c, c->wstart, (n + 2) * 4);
         // chunks of 128 particles of the large cells: at most 2 N / 128 per level
         const size_t items = 44 * n / 128 + 4096;
-        ok = ok && ensure(c, c->mitems, items * 4) && ensure(c, c->mpart, items * 40);
+        ok = ok && ensure(c, c->mitems, items * 4);
         if (ok) c->capItems = (int64_t)items;
         if (ok) {
             c->capN = N;
@@ -845,7 +847,7 @@ hybrid_status hybrid_destroy(hybrid_ctx *c)
                   &c->ncy, &c->ncz, &c->nB2, &c->nbmax, &c->nA, &c->nB, &c->ncrit, &c->ntopo, &c->nD, &c->nrb,
                   &c->nhr, &c->ndelta, &c->nside, &c->norg, &c->gflag, &c->gscan, &c->gnode, &c->gfirst,
                   &c->gsys, &c->gF, &c->glo, &c->ghi, &c->ngroups_dev, &c->lcnt, &c->list, &c->stack, &c->counter,
-                  &c->io_dev, &c->energy_dev, &c->wstart, &c->wmap, &c->nbig, &c->mitems, &c->mpart, &c->nbmax32, &c->wnear};
+                  &c->io_dev, &c->energy_dev, &c->wstart, &c->wmap, &c->nbig, &c->mitems, &c->nbmax32, &c->wnear};
     for (Buf *b : all)
         if (b->p) cudaFree(b->p);
     for (int f = 0; f < 7; ++f) {

@@ -849,8 +849,8 @@ struct NodeArgs {
     const uint32_t *off;      // scanned counts: index of a tile's first start at each level, then of its first group
     const uint64_t *total;    // nodes + groups
     uint32_t *nfirst, *nend, *nlevel, *nchild, *nchend, *nparent, *sysroot, *lvl, *done;
-    unsigned long long *bmax64;
-    unsigned int *bmax32;     // one of the two, zeroed
+    unsigned long long *bmax64;   // zeroed for the chunks' maxima, FP64 or FP32 form
+    unsigned int *bmax32;         // (null: b_max by search)
     uint32_t *gnode, *gfirst, *gsys;   // null: groups come from the node-based kernels
     int64_t *ngroups;
     int64_t N, cap;
@@ -950,7 +950,7 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st,
                     if (l == d[r]) a.nchild[x] = NONE;
                     a.done[x] = 0u;
                     if (a.bmax64) a.bmax64[x] = 0ull;
-                    else a.bmax32[x] = 0u;
+                    if (a.bmax32) a.bmax32[x] = 0u;
                     if (l == 0) a.sysroot[sys] = x;
                     if (l == dg[r] && ((gm >> lane) & 1u)) {
                         a.gnode[g] = x;
@@ -972,8 +972,8 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st,
 // (counted with an atomic; no wait anywhere): M = sum M_j, COM = sum M_j
 // COM_j / M, B2 = sum_j [B2_j + M_j |COM_j - COM|^2] (parallel axis, no
 // cancellation), in a fixed order. b_max of a larger cell is the largest
-// distance of its particles to its centre of mass, taken afterwards over
-// chunks of BM_CH particles with one atomic max per chunk.
+// distance of its particles to its centre of mass, taken afterwards (k_bmax_big or
+// k_finish).
 // ---------------------------------------------------------------------------
 struct MomArgs {
     const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nparent, *nlevel;   // a node's particles and children: [first, end)
@@ -988,6 +988,7 @@ struct MomArgs {
     const float4 *phi, *plo;
     unsigned long long *bmax64;   // FP64 form: b_max as FP64 bits
     unsigned int *bmax32;         // FP32 form: b_max as FP32 bits
+    bool search;                  // FP32 form: b_max of the larger cells by search (k_finish), else by chunks (k_bmax_big)
 };
 
 __device__ __forceinline__ uint32_t digit_at(uint64_t key, int lev)
@@ -1217,9 +1218,11 @@ __device__ void mom_combine_f32(const MomArgs &a, uint32_t c, uint32_t f, uint32
     const SysBox &b = a.box[a.S == 1 ? 0 : a.psys[f]];
     const bool on = (uint32_t)lane < k;
     float4 A = make_float4(0.0f, 0.0f, 0.0f, 0.0f), B = A;
+    float rad = 0.0f;   // the child's particles lie within this of its centre of mass
     if (on) {
         A = __ldcg(a.nA + ch0 + lane);
         B = __ldcg(a.nB + ch0 + lane);
+        if (a.search) rad = __uint_as_float(__ldcg(a.bmax32 + ch0 + lane));
     }
     const float hx = __shfl_sync(gm, A.x, 0, G), hy = __shfl_sync(gm, A.y, 0, G),
                 hz = __shfl_sync(gm, A.z, 0, G);
@@ -1249,6 +1252,13 @@ __device__ void mom_combine_f32(const MomArgs &a, uint32_t c, uint32_t f, uint32
         e0 = (float)((o[0] + 0.5 * sd - b.lo[0]) - ((double)hx + (double)lx));
         e1 = (float)((o[1] + 0.5 * sd - b.lo[1]) - ((double)hy + (double)ly));
         e2 = (float)((o[2] + 0.5 * sd - b.lo[2]) - ((double)hz + (double)lz));
+    }
+    if (a.search) {   // and this cell's particles within this of its own: a bound, which k_finish replaces by b_max
+        const float qx = dx - e0, qy = dy - e1, qz = dz - e2;
+        rad = on ? (sqrtf(qx * qx + qy * qy + qz * qz) + rad) * 1.00001f : 0.0f;
+#pragma unroll
+        for (int o = G / 2; o > 0; o >>= 1) rad = fmaxf(rad, __shfl_xor_sync(gm, rad, o, G));
+        if (lane == 0) a.bmax32[c] = __float_as_uint(rad);
     }
     if (lane == 0) {
         const float t0 = lx + e0, t1 = ly + e1, t2 = lz + e2;
@@ -1286,11 +1296,89 @@ __device__ void mom_climb(const MomArgs &a, uint32_t p, int lane, unsigned gm)
     }
 }
 
+// Per node: geometry, delta, MAC radius, walk criteria and packed topology.
+struct FinArgs {
+    const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nlevel;
+    const uint64_t *key;
+    const int32_t *psys;
+    int S;
+    const SysBox *box;
+    const SysParams *sp;
+    double *M, *cx, *cy, *cz, *B2;
+    unsigned long long *bmax;
+    unsigned int *bmax32;
+    const float4 *nA, *nB;
+    float2 *crit;
+    uint4 *topo;
+    double4_32a *nD;
+    double *rb, *hr, *delta, *side, *org;
+};
+
+// every third bit of a key, from bit 0 (the inverse of spread3)
+__device__ __forceinline__ uint32_t compact3(uint64_t x)
+{
+    x &= 0x1249249249249249ull;
+    x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
+    x = (x | (x >> 4)) & 0x100f00f00f00f00full;
+    x = (x | (x >> 8)) & 0x1f0000ff0000ffull;
+    x = (x | (x >> 16)) & 0x1f00000000ffffull;
+    x = (x | (x >> 32)) & 0x1fffffull;
+    return (uint32_t)x;
+}
+
+// integer cell coordinates of a key's level-lev cell
+__device__ __forceinline__ void prefix_q(uint64_t key, uint32_t lev, uint32_t q[3])
+{
+    q[0] = compact3(key >> 2) >> (LEVELS - lev);
+    q[1] = compact3(key >> 1) >> (LEVELS - lev);
+    q[2] = compact3(key) >> (LEVELS - lev);
+}
+
+struct CritF {
+    float rb, hr, delta;
+};
+
+// FP32 form: delta, r_b and the Eq. (15) radius from the hi/lo centre of mass (cell centres are exact in FP32 on the
+// hi grid)
+__device__ __forceinline__ CritF crit_f32(const float4 &A, const float4 &B, float bm, uint32_t lev, const uint32_t q[3],
+                                          const SysParams &P, const SysBox &bx)
+{
+    // no FP64 instruction here (conversions count): the FP64 pipe has 2 lanes per SM
+    const float sdf = bx.uf * __int_as_float((127 + 20 - (int)lev) << 23);   // L 2^-lev: exact
+    // cell centre relative to the root corner: (q + 1/2) side, exact in FP32
+    const float e0 = (A.x - ((float)q[0] + 0.5f) * sdf) + B.x;
+    const float e1 = (A.y - ((float)q[1] + 0.5f) * sdf) + B.y;
+    const float e2 = (A.z - ((float)q[2] + 0.5f) * sdf) + B.z;
+    CritF r;
+    r.delta = sqrtf(e0 * e0 + e1 * e1 + e2 * e2);
+    if (P.mac == 1) r.rb = 0.5f * bm + sqrtf(0.25f * bm * bm + sqrtf(3.0f * B.w / P.a_errf));
+    else r.rb = (P.thetaf > 0.0f) ? sdf / P.thetaf + r.delta : INFINITY;
+    r.hr = P.R2f + P.skinf + bm;
+    return r;
+}
+
+// FP32 form: what the walk reads of cell c (particles [f, e), centre of mass A, B, b_max bm)
+__device__ __forceinline__ void finish_f32(const FinArgs &a, uint32_t c, uint32_t f, uint32_t e, const float4 &A,
+                                           const float4 &B, float bm)
+{
+    const int s = a.S == 1 ? 0 : a.psys[f];
+    const SysParams &P = a.sp[s];
+    const uint32_t lev = a.nlevel[c], ch = a.nchild[c];
+    uint32_t q[3];
+    prefix_q(a.key[f], lev, q);
+    const CritF r = crit_f32(A, B, bm, lev, q, P, a.box[s]);
+    const float sacc = fmaxf(r.rb, r.hr);
+    a.crit[c] = make_float2(sacc * sacc, P.has_hard ? r.hr * r.hr : -1.0f);
+    a.topo[c] = make_uint4(ch, ch == NONE ? 0u : a.nchend[c] - ch, f, e - f);
+    a.bmax32[c] = __float_as_uint(bm);
+}
+
 constexpr uint32_t BM_CH = 256;
 
 // every cell of at most MOM_CH particles, and every leaf (a leaf holds more
 // only when its particles share one level-21 cell): moments and b_max from its
-// particles, then the climb; larger cells get their b_max chunk items
+// particles, then the climb; the larger cells are listed for their b_max, in
+// chunks of BM_CH particles (once each where b_max is searched for)
 template <bool F64>
 __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long *nitems, uint32_t *bigbase,
                                                    uint32_t *items, uint32_t cap_items, Status *st, int where)
@@ -1350,21 +1438,23 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
                     a.bmax32[c] = __float_as_uint(bm);
                 }
                 mom_climb<false, 8>(a, up, sl, gm);
-            } else if (sl == 0) {
-                const uint32_t nch = (n + BM_CH - 1) / BM_CH;
-                const unsigned long long base = atomicAdd(nitems, (unsigned long long)nch);
+            } else {
+                const uint32_t nch = a.search ? 1u : (n + BM_CH - 1) / BM_CH;
+                unsigned long long base = 0;
+                if (sl == 0) base = atomicAdd(nitems, (unsigned long long)nch);
+                base = __shfl_sync(gm, base, 0, 8);
                 if (base + nch > cap_items) {
-                    fail(st, HYBRID_ECAPACITY, where);
+                    if (sl == 0) fail(st, HYBRID_ECAPACITY, where);
                     continue;
                 }
-                bigbase[c] = (uint32_t)base;
-                for (uint32_t k = 0; k < nch; ++k) items[base + k] = c;
+                if (sl == 0) bigbase[c] = (uint32_t)base;
+                for (uint32_t k = sl; k < nch; k += 8) items[base + k] = c;
             }
         }
     }
 }
 
-// b_max of the larger cells: one warp per chunk of BM_CH particles, one atomic
+// b_max of the larger cells, one warp per chunk of BM_CH particles, one atomic
 // max per chunk (non-negative floats order as their bit patterns)
 template <bool F64>
 __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long long *nitems,
@@ -1392,6 +1482,7 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
         } else {
             const float4 A = a.nA[c], B = a.nB[c];
             float dm = 0.0f;
+#pragma unroll 4
             for (uint32_t i = f0 + lane; i < f0 + n0; i += 32) {
                 const float4 h = a.phi[i], l = a.plo[i];
                 const float d0 = (h.x - A.x) + (l.x - B.x);
@@ -1399,79 +1490,139 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
                 const float d2 = (h.z - A.z) + (l.z - B.z);
                 dm = fmaxf(dm, d0 * d0 + d1 * d1 + d2 * d2);
             }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dm = fmaxf(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+            dm = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(dm)));
             if (lane == 0) atomicMax(a.bmax32 + c, __float_as_uint(sqrtf(dm)));
         }
     }
 }
 
-// Per node: geometry, delta, MAC radius, walk criteria and packed topology.
-struct FinArgs {
-    const uint32_t *lvl, *nfirst, *nend, *nchend, *nchild, *nlevel;
-    const uint64_t *key;
-    const int32_t *psys;
-    int S;
-    const SysBox *box;
-    const SysParams *sp;
-    double *M, *cx, *cy, *cz, *B2;
-    unsigned long long *bmax;
-    const unsigned int *bmax32;
-    const float4 *nA, *nB;
-    float2 *crit;
-    uint4 *topo;
-    double4_32a *nD;
-    double *rb, *hr, *delta, *side, *org;
-};
+// FP32 form: what the walk reads of every cell; with SEARCH, before that, b_max
+// of the larger ones: the distance of the particle farthest from the centre of
+// mass, one warp per cell; up to BIG_ALL particles by taking all of them, above
+// by a search of the cell's subtree. A node's particles lie within r of its
+// centre of mass, at d from the cell's (r = b_max up to MOM_CH particles, above
+// the bound that its combine made of its children's, or by now its own b_max).
+// It can hold the farthest particle only if d + r reaches the best distance so
+// far; and it holds one at d - r at least (and at r - d, where r is b_max).
+// Leaves left over are measured particle by particle, so the value is that of
+// taking every particle (the bounds carry 1e-5 of slack for their rounding).
+// Taking every particle (k_bmax_big) reads the state once per level of larger
+// cells, a search about 50 nodes and 5 leaves, in a few steps that wait for one
+// another: searching is for batches above 2^20 particles (moments per soft
+// step: 2^24 13.6 -> 12.0 ms, 512 systems of 12.9 M particles 5.9 -> 4.7; below
+// it loses: 2^17 0.177 -> 0.186, 2^20 0.465 -> 0.49). The other cells are
+// finished meanwhile, one per thread: on one lane in eight, with their moments,
+// the same work took longer.
+constexpr int BIG_THREADS = 128, BIG_STACK = 1024, BIG_QUEUE = 512;
+constexpr uint32_t BIG_ALL = 512;
+constexpr int BIG_SLACK = 160;   // stack entries kept for a descent one node at a time: 7 more per level, 21 levels
 
-// every third bit of a key, from bit 0 (the inverse of spread3)
-__device__ __forceinline__ uint32_t compact3(uint64_t x)
+template <bool SEARCH>
+__global__ void __launch_bounds__(BIG_THREADS) k_finish(MomArgs a, FinArgs fa, const unsigned long long *nitems,
+                                                        const uint32_t *items, const Status *st)
 {
-    x &= 0x1249249249249249ull;
-    x = (x | (x >> 2)) & 0x10c30c30c30c30c3ull;
-    x = (x | (x >> 4)) & 0x100f00f00f00f00full;
-    x = (x | (x >> 8)) & 0x1f0000ff0000ffull;
-    x = (x | (x >> 16)) & 0x1f00000000ffffull;
-    x = (x | (x >> 32)) & 0x1fffffull;
-    return (uint32_t)x;
+    __shared__ uint32_t stacks[SEARCH ? BIG_THREADS / 32 : 1][SEARCH ? BIG_STACK : 1];
+    __shared__ uint32_t queues[SEARCH ? BIG_THREADS / 32 : 1][SEARCH ? BIG_QUEUE : 1];   // particles to measure
+    if (st->code) return;
+    const uint32_t T = SEARCH ? (uint32_t)*nitems : 0u;
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    uint32_t *stk = stacks[SEARCH ? threadIdx.x >> 5 : 0], *que = queues[SEARCH ? threadIdx.x >> 5 : 0];
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; SEARCH && w < T; w += nw) {
+        const uint32_t c = items[w];
+        const uint32_t f = a.nfirst[c], e = a.nend[c], ch0 = a.nchild[c];
+        int sp = (int)(a.nchend[c] - ch0);
+        const float4 A = a.nA[c], B = a.nB[c];
+        float far = 0.0f, best2 = 0.0f;   // some particle is at least this far; this lane's farthest one, squared
+        auto measure = [&](uint32_t i) {
+            const float4 h = a.phi[i], l = a.plo[i];
+            const float d0 = (h.x - A.x) + (l.x - B.x);
+            const float d1 = (h.y - A.y) + (l.y - B.y);
+            const float d2 = (h.z - A.z) + (l.z - B.z);
+            best2 = fmaxf(best2, d0 * d0 + d1 * d1 + d2 * d2);
+        };
+        if (e - f <= BIG_ALL) {
+#pragma unroll 4
+            for (uint32_t i = f + lane; i < e; i += 32) measure(i);
+            sp = 0;
+        }
+        if (lane < sp) stk[lane] = ch0 + lane;
+        __syncwarp();
+        while (sp > 0) {
+            const int take = min(sp, max(1, min(32, (BIG_STACK - BIG_SLACK - sp) / 7)));
+            const bool on = lane < take;
+            uint32_t first = 0, count = 0, ch = NONE, k = 0;
+            float least = 0.0f, reach = -1.0f;
+            if (on) {
+                const uint32_t q = stk[sp - take + lane];
+                first = a.nfirst[q];
+                count = a.nend[q] - first;
+                ch = a.nchild[q];
+                k = ch == NONE ? 0u : a.nchend[q] - ch;
+                const float4 qa = a.nA[q], qb = a.nB[q];
+                const float r = __uint_as_float(a.bmax32[q]);
+                const float dx = (qa.x - A.x) + (qb.x - B.x), dy = (qa.y - A.y) + (qb.y - B.y), dz = (qa.z - A.z) + (qb.z - B.z);
+                const float d = sqrtf(dx * dx + dy * dy + dz * dz);
+                least = fmaxf(d - r, count <= MOM_CH || ch == NONE ? r - d : 0.0f);
+                reach = (d + r) * 1.00001f;
+            }
+            sp -= take;
+            // distances are >= 0: they order as integers
+            far = fmaxf(far, 0.99999f * __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(least))));
+            const bool alive = on && reach >= far;
+            const uint32_t np = alive && k == 0u ? count : 0u;
+            if (__any_sync(0xffffffffu, np > 0u)) {
+                if (__all_sync(0xffffffffu, np <= (uint32_t)(BIG_QUEUE / 32))) {   // all leaves' particles together
+                    uint32_t ex = 0, tot = 0;
+#pragma unroll
+                    for (int b = 0; b < 5; ++b) {
+                        const unsigned m = __ballot_sync(0xffffffffu, (np >> b) & 1u);
+                        ex += (uint32_t)__popc(m & lt) << b;
+                        tot += (uint32_t)__popc(m) << b;
+                    }
+                    for (uint32_t j = 0; j < np; ++j) que[ex + j] = first + j;
+                    __syncwarp();
+                    for (uint32_t i = lane; i < tot; i += 32) measure(que[i]);
+                    __syncwarp();
+                } else {
+                    unsigned leaves = __ballot_sync(0xffffffffu, np > 0u);
+                    do {
+                        const int src = __ffs(leaves) - 1;
+                        leaves &= leaves - 1u;
+                        const uint32_t p0 = __shfl_sync(0xffffffffu, first, src), p1 = p0 + __shfl_sync(0xffffffffu, np, src);
+                        for (uint32_t i = p0 + lane; i < p1; i += 32) measure(i);
+                    } while (leaves);
+                }
+                far = fmaxf(far, 0.99999f * sqrtf(__uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best2)))));
+            }
+            const uint32_t push = alive && reach >= far ? k : 0u;
+            uint32_t ex = 0, tot = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const unsigned m = __ballot_sync(0xffffffffu, (push >> b) & 1u);
+                ex += (uint32_t)__popc(m & lt) << b;
+                tot += (uint32_t)__popc(m) << b;
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < 8; ++j)
+                if (j < push) stk[sp + ex + j] = ch + j;
+            sp += (int)tot;
+            __syncwarp();
+        }
+        best2 = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(best2)));
+        if (lane == 0) finish_f32(fa, c, f, e, A, B, sqrtf(best2));
+    }
+    const uint32_t total = a.lvl[LEVELS + 1];
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < total; c += gridDim.x * blockDim.x) {
+        const uint32_t f = a.nfirst[c], e = a.nend[c];
+        if (!SEARCH || e - f <= MOM_CH || a.nchild[c] == NONE) finish_f32(fa, c, f, e, a.nA[c], a.nB[c], __uint_as_float(a.bmax32[c]));
+    }
 }
 
-// integer cell coordinates of a key's level-lev cell
-__device__ __forceinline__ void prefix_q(uint64_t key, uint32_t lev, uint32_t q[3])
-{
-    q[0] = compact3(key >> 2) >> (LEVELS - lev);
-    q[1] = compact3(key >> 1) >> (LEVELS - lev);
-    q[2] = compact3(key) >> (LEVELS - lev);
-}
-
-struct CritF {
-    float rb, hr, delta;
-};
-
-// FP32 form: delta, r_b and the Eq. (15) radius from the hi/lo centre of mass (cell centres are exact in FP32 on the
-// hi grid)
-__device__ __forceinline__ CritF crit_f32(const FinArgs &a, uint32_t c, uint32_t lev, const uint32_t q[3],
-                                          const SysParams &P, const SysBox &bx)
-{
-    const float sdf = ldexpf((float)bx.L, -(int)lev);
-    const float4 A = a.nA[c], B = a.nB[c];
-    // cell centre relative to the root corner: (q + 1/2) side, exact in FP32
-    const float e0 = (A.x - ((float)q[0] + 0.5f) * sdf) + B.x;
-    const float e1 = (A.y - ((float)q[1] + 0.5f) * sdf) + B.y;
-    const float e2 = (A.z - ((float)q[2] + 0.5f) * sdf) + B.z;
-    CritF r;
-    r.delta = sqrtf(e0 * e0 + e1 * e1 + e2 * e2);
-    const float bm = __uint_as_float(a.bmax32[c]);
-    if (P.mac == 1) r.rb = 0.5f * bm + sqrtf(0.25f * bm * bm + sqrtf(3.0f * B.w / (float)P.a_err));
-    else r.rb = (P.theta > 0.0) ? sdf / (float)P.theta + r.delta : INFINITY;
-    r.hr = P.R2f + P.skinf + bm;
-    return r;
-}
-
-// F64: criteria from the FP64 moments, and what hybrid_tree_copy reports. FP32 form: the walk's records only
-// (k_inspect makes the reports when they are asked for: 170 bytes and a dozen FP64 operations a node that no
-// force needs).
-template <bool F64>
+// FP64 form: criteria from the FP64 moments, and what hybrid_tree_copy reports. (The FP32 form finishes a cell with its
+// moments, and k_inspect makes the reports when they are asked for: 170 bytes and a dozen FP64 operations a node that
+// no force needs.)
 __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
 {
     if (st->code) return;
@@ -1484,30 +1635,24 @@ __global__ void __launch_bounds__(256) k_finalize(FinArgs a, const Status *st)
         const uint32_t lev = a.nlevel[c];
         uint32_t q[3];
         prefix_q(a.key[f], lev, q);
-        if (F64) {
-            const double sd = ldexp(bx.L, -(int)lev);
-            double o[3], rb;
-            for (int k = 0; k < 3; ++k) o[k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
-            const double ctr0 = o[0] + 0.5 * sd, ctr1 = o[1] + 0.5 * sd, ctr2 = o[2] + 0.5 * sd;
-            const double e0 = a.cx[c] - ctr0, e1 = a.cy[c] - ctr1, e2 = a.cz[c] - ctr2;
-            const double delta = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
-            const double bm = __longlong_as_double((long long)a.bmax[c]);
-            if (P.mac == 1) rb = 0.5 * bm + sqrt(0.25 * bm * bm + sqrt(3.0 * a.B2[c] / P.a_err));
-            else rb = (P.theta > 0.0) ? sd / P.theta + delta : INFINITY;
-            const double hr = P.R2 + P.skin + bm;   // Eq. (15) radius (plus the skin of reused lists)
-            const double sacc = fmax(rb, hr);
-            a.crit[c] = make_float2((float)(sacc * sacc), P.has_hard ? (float)(hr * hr) : -1.0f);
-            a.nD[c] = make_double4_32a(a.cx[c], a.cy[c], a.cz[c], a.M[c]);
-            for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = o[k];
-            a.rb[c] = rb;
-            a.hr[c] = hr;
-            a.delta[c] = delta;
-            a.side[c] = sd;
-        } else {
-            const CritF r = crit_f32(a, c, lev, q, P, bx);
-            const float sacc = fmaxf(r.rb, r.hr);
-            a.crit[c] = make_float2(sacc * sacc, P.has_hard ? r.hr * r.hr : -1.0f);
-        }
+        const double sd = ldexp(bx.L, -(int)lev);
+        double o[3], rb;
+        for (int k = 0; k < 3; ++k) o[k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
+        const double ctr0 = o[0] + 0.5 * sd, ctr1 = o[1] + 0.5 * sd, ctr2 = o[2] + 0.5 * sd;
+        const double e0 = a.cx[c] - ctr0, e1 = a.cy[c] - ctr1, e2 = a.cz[c] - ctr2;
+        const double delta = sqrt(e0 * e0 + e1 * e1 + e2 * e2);
+        const double bm = __longlong_as_double((long long)a.bmax[c]);
+        if (P.mac == 1) rb = 0.5 * bm + sqrt(0.25 * bm * bm + sqrt(3.0 * a.B2[c] / P.a_err));
+        else rb = (P.theta > 0.0) ? sd / P.theta + delta : INFINITY;
+        const double hr = P.R2 + P.skin + bm;   // Eq. (15) radius (plus the skin of reused lists)
+        const double sacc = fmax(rb, hr);
+        a.crit[c] = make_float2((float)(sacc * sacc), P.has_hard ? (float)(hr * hr) : -1.0f);
+        a.nD[c] = make_double4_32a(a.cx[c], a.cy[c], a.cz[c], a.M[c]);
+        for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = o[k];
+        a.rb[c] = rb;
+        a.hr[c] = hr;
+        a.delta[c] = delta;
+        a.side[c] = sd;
         const uint32_t ch = a.nchild[c];
         a.topo[c] = make_uint4(ch, ch == NONE ? 0u : a.nchend[c] - ch, f, a.nend[c] - f);
     }
@@ -1524,14 +1669,15 @@ __global__ void __launch_bounds__(256) k_inspect(FinArgs a)
         const uint32_t lev = a.nlevel[c];
         uint32_t q[3];
         prefix_q(a.key[f], lev, q);
-        const CritF r = crit_f32(a, c, lev, q, a.sp[s], bx);
         const float4 A = a.nA[c], B = a.nB[c];
+        const float bm = __uint_as_float(a.bmax32[c]);
+        const CritF r = crit_f32(A, B, bm, lev, q, a.sp[s], bx);
         a.M[c] = (double)A.w;
         a.cx[c] = bx.lo[0] + ((double)A.x + (double)B.x);
         a.cy[c] = bx.lo[1] + ((double)A.y + (double)B.y);
         a.cz[c] = bx.lo[2] + ((double)A.z + (double)B.z);
         a.B2[c] = (double)B.w;
-        a.bmax[c] = (unsigned long long)__double_as_longlong((double)__uint_as_float(a.bmax32[c]));
+        a.bmax[c] = (unsigned long long)__double_as_longlong((double)bm);
         const double sd = ldexp(bx.L, -(int)lev);
         for (int k = 0; k < 3; ++k) a.org[3 * (size_t)c + k] = __dadd_rn(bx.lo[k], __dmul_rn((double)q[k], sd));
         a.rb[c] = r.rb;
@@ -1769,6 +1915,9 @@ void launch_permute(hybrid_ctx *c)
     c->swaps ^= 1;
 }
 
+// FP32 form: b_max of the larger cells by search instead of taking every particle (see k_finish)
+static bool bmax_by_search(const hybrid_ctx *c) { return c->p.precision == 1 && c->N > (int64_t)1 << 20; }
+
 // sink groups marked with the cells (k_cells, k_nodes) or, for a large n_crit, from the nodes afterwards
 static bool groups_in_nodes(const hybrid_ctx *c) { return c->p.n_crit <= GROUP_WINDOW; }
 
@@ -1803,7 +1952,7 @@ void launch_topology(hybrid_ctx *c)
     a.lvl = (uint32_t *)c->lvl.p;
     a.done = (uint32_t *)c->ndone.p;
     a.bmax64 = c->p.precision == 0 ? (unsigned long long *)c->nbmax.p : nullptr;
-    a.bmax32 = (unsigned int *)c->nbmax32.p;
+    a.bmax32 = c->p.precision == 0 || bmax_by_search(c) ? nullptr : (unsigned int *)c->nbmax32.p;
     a.gnode = groups ? (uint32_t *)c->gnode.p : nullptr;
     a.gfirst = (uint32_t *)c->gfirst.p;
     a.gsys = (uint32_t *)c->gsys.p;
@@ -1836,7 +1985,7 @@ static FinArgs fin_args(hybrid_ctx *c)
     f.cz = (double *)c->ncz.p;
     f.B2 = (double *)c->nB2.p;
     f.bmax = (unsigned long long *)c->nbmax.p;
-    f.bmax32 = (const unsigned int *)c->nbmax32.p;
+    f.bmax32 = (unsigned int *)c->nbmax32.p;
     f.nA = (const float4 *)c->nA.p;
     f.nB = (const float4 *)c->nB.p;
     f.crit = (float2 *)c->ncrit.p;
@@ -1853,7 +2002,6 @@ static FinArgs fin_args(hybrid_ctx *c)
 void launch_moments(hybrid_ctx *c)
 {
     Status *st = status_dev(c);
-    const int grid = grid_for(c, c->capNodes, 256, 8);
     MomArgs a;
     a.lvl = (const uint32_t *)c->lvl.p;
     a.nfirst = (const uint32_t *)c->nfirst.p;
@@ -1880,23 +2028,30 @@ void launch_moments(hybrid_ctx *c)
     a.done = (uint32_t *)c->ndone.p;
     a.bmax64 = (unsigned long long *)c->nbmax.p;
     a.bmax32 = (unsigned int *)c->nbmax32.p;
+    a.search = bmax_by_search(c);
     a.phi = (const float4 *)c->phi.p;
     a.plo = (const float4 *)c->plo.p;
     unsigned long long *nitems = (unsigned long long *)c->counter.p + 9;
     const int gridw = grid_for(c, c->capNodes * 32, 256, 16);
     uint32_t *bigbase = (uint32_t *)c->nbig.p, *items = (uint32_t *)c->mitems.p;
+    const FinArgs f = fin_args(c);
     if (c->p.precision == 0) {
         k_mom_small<true><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, (uint32_t)c->capItems, st, c->op);
         k_bmax_big<true><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, st);
+        k_finalize<<<grid_for(c, c->capNodes, 256, 8), 256, 0, c->st>>>(f, st);
+        c->launches += 3;
     } else {
         k_mom_small<false><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, (uint32_t)c->capItems, st, c->op);
-        k_bmax_big<false><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, st);
+        const int gridf = grid_for(c, c->capNodes, BIG_THREADS, 16);
+        if (a.search) {
+            k_finish<true><<<gridf, BIG_THREADS, 0, c->st>>>(a, f, nitems, items, st);
+        } else {
+            k_bmax_big<false><<<gridw, 256, 0, c->st>>>(a, nitems, bigbase, items, st);
+            k_finish<false><<<gridf, BIG_THREADS, 0, c->st>>>(a, f, nitems, items, st);
+            c->launches += 1;
+        }
+        c->launches += 2;
     }
-    c->launches += 2;
-    const FinArgs f = fin_args(c);
-    if (c->p.precision == 0) k_finalize<true><<<grid, 256, 0, c->st>>>(f, st);
-    else k_finalize<false><<<grid, 256, 0, c->st>>>(f, st);
-    c->launches += 1;
 }
 
 void launch_inspect(hybrid_ctx *c)

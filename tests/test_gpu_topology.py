@@ -49,3 +49,17 @@ def test_batch_boundaries(H):  # noqa: F811
         a, b = alone.numpy(), s.numpy()
         for k in a:
             assert np.array_equal(a[k], b[k]), k
+
+
+def test_search_for_the_farthest_particle(H):  # noqa: F811
+    # above 2^20 particles b_max of the larger cells is searched for: uneven clumps, coincident particles, a lattice
+    # (many particles at the same distance) and outliers, against the oracle's largest distance
+    n = (1 << 20) + 3000
+    st = ics.plummer(n, 12)
+    rng = np.random.default_rng(5)
+    for k, d in enumerate("xyz"):
+        st[d][:400000] = 0.3 + 0.01 * rng.standard_normal(400000)
+        st[d][400000:402000] = 0.75
+        st[d][402000:410000] = (np.arange(8000) // 20 ** k % 20) / 16.0 - 3.0
+    st["x"][500000] = 60.0
+    check_tree(*tree_of(H, st, n_leaf=16, n_crit=256, precision=1), 1)
