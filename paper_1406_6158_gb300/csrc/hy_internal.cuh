@@ -328,8 +328,7 @@ void launch_box(hybrid_ctx *c);
 void launch_keys_sort(hybrid_ctx *c);      // keys and their stable sort (keys[0], vals[0])
 void launch_permute(hybrid_ctx *c);        // state into key order, pair-kernel copies of the positions
 void launch_topology(hybrid_ctx *c);       // nodes and sink groups from the sorted keys
-int cell_tiles(int64_t N);
-size_t cell_count_bytes(int64_t N);        // its counts per tile
+size_t cell_count_bytes(int64_t N);        // its counts per tile, for up to N particles
 void launch_moments(hybrid_ctx *c);        // needs topology and the permuted state
 void launch_inspect(hybrid_ctx *c);        // FP32 form: the moments and geometry hybrid_tree_copy reports
 void launch_groups(hybrid_ctx *c);         // group table from the nodes, for an n_crit launch_topology leaves out

@@ -738,9 +738,12 @@ __device__ __forceinline__ int prefix_c(const uint64_t *__restrict__ key, const 
     return shared_digits(key[i - 1], key[i]);
 }
 
-constexpr int CT_ROWS = 4;                    // rows of 32 particles per warp
+// Tiles of CT_WARPS warps with ROWS rows of 32 particles each: 256, 512 or 1024 particles. Small systems take small
+// tiles (more blocks, shorter ones), as long as the counts of all tiles are few enough for every block of k_nodes to
+// add up by itself.
 constexpr int CT_WARPS = 8;
-constexpr int CT_TILE = CT_WARPS * 32 * CT_ROWS;   // 1024 particles per tile
+constexpr int CT_MAX = CT_WARPS * 32 * 4;
+constexpr int CT_SUM_MAX = 320;               // tiles up to which k_nodes adds up the counts; above, a scan does it
 constexpr int NLEV = LEVELS + 1;              // levels 0..21
 constexpr int CT_CNT = NLEV + 1;              // counts per tile: starts at each level, sink groups
 // Sink groups of up to this size are marked in k_cells; larger n_crit take the node-based kernels
@@ -748,13 +751,13 @@ constexpr int CT_CNT = NLEV + 1;              // counts per tile: starts at each
 constexpr int GROUP_WINDOW = 1024;
 
 // deepest level at which the cell around tile particle x holds more than n particles, for every x of the
-// tile, into m[0, CT_TILE) as level + 1 (0: none); m and t are byte arrays of cells_bytes(n) each
-__host__ __device__ constexpr int cells_bytes(int n) { return (CT_TILE + n + 15) / 16 * 16 + 16; }
+// tile (of len0), into m[0, len0) as level + 1 (0: none); m and t are byte arrays of cells_bytes(n) each
+__host__ __device__ constexpr int cells_bytes(int n) { return (CT_MAX + n + 15) / 16 * 16 + 16; }
 
 __device__ __forceinline__ uint8_t *window_max(const uint64_t *__restrict__ key, const int32_t *__restrict__ psys,
-                                               bool one, int64_t N, int64_t b0, int n, uint8_t *m, uint8_t *t)
+                                               bool one, int64_t N, int64_t b0, int len0, int n, uint8_t *m, uint8_t *t)
 {
-    const int len = CT_TILE + n, words = cells_bytes(n) / 4;
+    const int len = len0 + n, words = (len + 3) / 4 + 1;
     for (int x = threadIdx.x; x < 4 * words; x += blockDim.x) {
         const int64_t a = b0 - n + x;
         int v = 0;
@@ -777,13 +780,14 @@ __device__ __forceinline__ uint8_t *window_max(const uint64_t *__restrict__ key,
         t = u;
     }
     // the window of n + 1 entries from x: two overlapping runs of s
-    for (int x = threadIdx.x; x < CT_TILE; x += blockDim.x) t[x] = max(m[x], m[x + n + 1 - s]);
+    for (int x = threadIdx.x; x < len0; x += blockDim.x) t[x] = max(m[x], m[x + n + 1 - s]);
     __syncthreads();
     return t;
 }
 
 // Per particle the packed levels c + 1, D, Dg (5 bits each); per tile the numbers of nodes started at each level
 // and of sink groups (cnt[row][tile]). Also clears the counters of the moments and of the walk.
+template <int ROWS>
 __global__ void __launch_bounds__(32 * CT_WARPS) k_cells(int64_t N, int S, const uint64_t *__restrict__ key,
                                                          const int32_t *__restrict__ psys, int n_leaf, int n_crit,
                                                          uint16_t *__restrict__ cells, int ntiles,
@@ -796,20 +800,21 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_cells(int64_t N, int S, const
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int nb = cells_bytes(max(n_leaf, n_crit));
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const int64_t b0 = (int64_t)tile * CT_TILE, p0 = b0 + w * (32 * CT_ROWS) + lane;
-        uint8_t D[CT_ROWS], Dg[CT_ROWS];
-        const uint8_t *m = window_max(key, psys, S == 1, N, b0, n_leaf, sm, sm + nb);
+        constexpr int TILE_P = CT_WARPS * 32 * ROWS;
+        const int64_t b0 = (int64_t)tile * TILE_P, p0 = b0 + w * (32 * ROWS) + lane;
+        uint8_t D[ROWS], Dg[ROWS];
+        const uint8_t *m = window_max(key, psys, S == 1, N, b0, TILE_P, n_leaf, sm, sm + nb);
 #pragma unroll
-        for (int r = 0; r < CT_ROWS; ++r) Dg[r] = D[r] = min((int)m[w * (32 * CT_ROWS) + r * 32 + lane], LEVELS);
+        for (int r = 0; r < ROWS; ++r) Dg[r] = D[r] = min((int)m[w * (32 * ROWS) + r * 32 + lane], LEVELS);
         if (n_crit > 0) {
             __syncthreads();
-            m = window_max(key, psys, S == 1, N, b0, n_crit, sm, sm + nb);
+            m = window_max(key, psys, S == 1, N, b0, TILE_P, n_crit, sm, sm + nb);
 #pragma unroll
-            for (int r = 0; r < CT_ROWS; ++r) Dg[r] = min(D[r], m[w * (32 * CT_ROWS) + r * 32 + lane]);
+            for (int r = 0; r < ROWS; ++r) Dg[r] = min(D[r], m[w * (32 * ROWS) + r * 32 + lane]);
         }
         uint32_t mine = 0;   // lane l: starts at level l (l < NLEV), lane NLEV: groups
 #pragma unroll
-        for (int r = 0; r < CT_ROWS; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const int64_t i = p0 + r * 32;
             int c = LEVELS + 1, d = 0;   // past the end: starts nothing
             bool g = false;
@@ -858,10 +863,46 @@ struct NodeArgs {
 };
 
 // Nodes (breadth-first) and sink groups (in particle order); see above.
+template <int ROWS, bool SCANNED>
 __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st, int where)
 {
     if (st->code) return;
-    const uint32_t nodes = a.off[(size_t)NLEV * a.ntiles];   // start of the group counts
+    __shared__ uint32_t wcnt[CT_WARPS][CT_CNT + 1];
+    __shared__ uint32_t before[CT_CNT], start[CT_CNT + 1];   // counts of the earlier tiles; first index of a row
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const unsigned lt = (1u << lane) - 1u;
+    if (SCANNED) {
+        if (threadIdx.x < CT_CNT) start[threadIdx.x] = a.off[(size_t)threadIdx.x * a.ntiles];
+        if (threadIdx.x == 0) start[CT_CNT] = (uint32_t)*a.total;
+        __syncthreads();
+    } else {   // one tile per block
+        for (int r = w; r < CT_CNT; r += CT_WARPS) {
+            const uint32_t *row = a.off + (size_t)r * a.ntiles;
+            uint32_t mine = 0, all = 0;
+            for (int t = lane; t < a.ntiles; t += 32) {
+                const uint32_t v = row[t];
+                all += v;
+                mine += t < (int)blockIdx.x ? v : 0u;
+            }
+            mine = __reduce_add_sync(0xffffffffu, mine);
+            all = __reduce_add_sync(0xffffffffu, all);
+            if (lane == 0) {
+                before[r] = mine;
+                wcnt[0][r] = all;
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            uint32_t run = 0;
+            for (int r = 0; r < CT_CNT; ++r) {
+                start[r] = run;
+                run += wcnt[0][r];
+            }
+            start[CT_CNT] = run;
+        }
+        __syncthreads();
+    }
+    const uint32_t nodes = start[NLEV];   // start of the groups
     if ((int64_t)nodes > a.cap) {
         if (blockIdx.x == 0 && threadIdx.x == 0) {
             fail(st, HYBRID_ECAPACITY, where);
@@ -869,23 +910,20 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st,
         }
         return;
     }
-    __shared__ uint32_t wcnt[CT_WARPS][CT_CNT + 1];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const unsigned lt = (1u << lane) - 1u;
     if (blockIdx.x == 0) {
-        if (threadIdx.x <= NLEV + 1) a.lvl[threadIdx.x] = threadIdx.x < NLEV ? a.off[(size_t)threadIdx.x * a.ntiles] : nodes;
+        if (threadIdx.x <= NLEV + 1) a.lvl[threadIdx.x] = threadIdx.x < NLEV ? start[threadIdx.x] : nodes;
         if (threadIdx.x == 0 && a.gnode) {
-            const uint64_t ng = *a.total - nodes;
+            const uint64_t ng = start[CT_CNT] - nodes;
             *a.ngroups = (int64_t)ng;
             a.gfirst[ng] = (uint32_t)a.N;
         }
     }
     for (int tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
-        const int64_t p0 = (int64_t)tile * CT_TILE + w * (32 * CT_ROWS) + lane;
-        int c[CT_ROWS], d[CT_ROWS], dp[CT_ROWS], dg[CT_ROWS];   // dp: D of the particle before
+        const int64_t p0 = (int64_t)tile * (CT_WARPS * 32 * ROWS) + w * (32 * ROWS) + lane;
+        int c[ROWS], d[ROWS], dp[ROWS], dg[ROWS];   // dp: D of the particle before
         uint32_t mine = 0;
 #pragma unroll
-        for (int r = 0; r < CT_ROWS; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const int64_t i = p0 + r * 32;
             c[r] = LEVELS + 1;
             d[r] = dp[r] = dg[r] = 0;
@@ -899,7 +937,7 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st,
             if (i == a.N) c[r] = -1;   // the end of the batch ends every cell around the last particle
         }
 #pragma unroll
-        for (int r = 0; r < CT_ROWS; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const bool real = p0 + r * 32 < a.N;
             const int lo = __reduce_min_sync(0xffffffffu, real ? c[r] : LEVELS + 1) + 1;
             const int hi = __reduce_max_sync(0xffffffffu, d[r]);
@@ -914,12 +952,12 @@ __global__ void __launch_bounds__(32 * CT_WARPS) k_nodes(NodeArgs a, Status *st,
         __syncthreads();
         uint32_t base = 0;   // lane l: index of this warp's first start at level l; lane NLEV: of its first group
         if (lane < CT_CNT) {
-            base = a.off[(size_t)lane * a.ntiles + tile] - (lane == NLEV ? nodes : 0u);
+            base = (SCANNED ? a.off[(size_t)lane * a.ntiles + tile] : start[lane] + before[lane]) - (lane == NLEV ? nodes : 0u);
             for (int k = 0; k < w; ++k) base += wcnt[k][lane];
         }
         __syncthreads();
 #pragma unroll
-        for (int r = 0; r < CT_ROWS; ++r) {
+        for (int r = 0; r < ROWS; ++r) {
             const int64_t i = p0 + r * 32;
             const bool real = i < a.N, here = i <= a.N;
             const unsigned gm = __ballot_sync(0xffffffffu, real && a.gnode && c[r] < dg[r]);
@@ -1915,6 +1953,19 @@ void launch_permute(hybrid_ctx *c)
     c->swaps ^= 1;
 }
 
+// rows of the topology's tiles, and tiles of N + 1 positions (the end of the batch is one)
+static int cell_rows(int64_t N)
+{
+    return N / (CT_MAX / 4) < CT_SUM_MAX ? 1 : (N / (CT_MAX / 2) < CT_SUM_MAX ? 2 : 4);
+}
+static int cell_tiles(int64_t N) { return (int)(N / (CT_WARPS * 32 * cell_rows(N))) + 1; }
+
+// counts of every batch of up to N particles
+size_t cell_count_bytes(int64_t N)
+{
+    return (size_t)CT_CNT * (std::max<int64_t>(CT_SUM_MAX, N / CT_MAX) + 1) * sizeof(uint32_t);
+}
+
 // FP32 form: b_max of the larger cells by search instead of taking every particle (see k_finish)
 static bool bmax_by_search(const hybrid_ctx *c) { return c->p.precision == 1 && c->N > (int64_t)1 << 20; }
 
@@ -1932,11 +1983,13 @@ void launch_topology(hybrid_ctx *c)
     uint64_t *d_tot = (uint64_t *)((char *)c->lvl.p + 256);
     uint32_t *cnt = (uint32_t *)c->ccnt.p;
     uint16_t *cells = (uint16_t *)c->cells.p;
-    const int ntiles = cell_tiles(N);
+    const int rows = cell_rows(N), ntiles = cell_tiles(N);
     const int grid = std::min(ntiles, c->nsm * 8);
-    k_cells<<<grid, 32 * CT_WARPS, 2 * (size_t)cells_bytes(std::max(c->p.n_leaf, n_crit)), c->st>>>(
-        N, c->S, keys, psys, c->p.n_leaf, n_crit, cells, ntiles, cnt, (unsigned long long *)c->counter.p, st);
-    scan_u32(c, cnt, (int64_t)CT_CNT * ntiles, nullptr, (int64_t)CT_CNT * ntiles, d_tot);
+    const size_t sh = 2 * (size_t)cells_bytes(std::max(c->p.n_leaf, n_crit));
+    auto *kc = rows == 1 ? k_cells<1> : (rows == 2 ? k_cells<2> : k_cells<4>);
+    kc<<<grid, 32 * CT_WARPS, sh, c->st>>>(N, c->S, keys, psys, c->p.n_leaf, n_crit, cells, ntiles, cnt,
+                                           (unsigned long long *)c->counter.p, st);
+    if (ntiles > CT_SUM_MAX) scan_u32(c, cnt, (int64_t)CT_CNT * ntiles, nullptr, (int64_t)CT_CNT * ntiles, d_tot);
     NodeArgs a;
     a.cells = cells;
     a.psys = psys;
@@ -1960,7 +2013,10 @@ void launch_topology(hybrid_ctx *c)
     a.N = N;
     a.cap = c->capNodes;
     a.ntiles = ntiles;
-    k_nodes<<<grid, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
+    if (ntiles > CT_SUM_MAX) k_nodes<4, true><<<grid, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
+    else if (rows == 1) k_nodes<1, false><<<ntiles, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
+    else if (rows == 2) k_nodes<2, false><<<ntiles, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
+    else k_nodes<4, false><<<ntiles, 32 * CT_WARPS, 0, c->st>>>(a, st, c->op);
     c->launches += 2;
     c->walk_clean = true;
 }
@@ -2089,14 +2145,14 @@ void launch_group_boxes(hybrid_ctx *c)
     c->launches += 1;
 }
 
-int cell_tiles(int64_t N) { return (int)(N / CT_TILE) + 1; }   // N + 1 positions: the end of the batch is one
-
-size_t cell_count_bytes(int64_t N) { return (size_t)CT_CNT * cell_tiles(N) * sizeof(uint32_t); }
-
 cudaError_t init_tree_kernels()
 {
     // leaves of up to 24448 particles, as far as their window fits in shared memory
-    return cudaFuncSetAttribute(k_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * cells_bytes(24448));
+    for (auto *k : {k_cells<1>, k_cells<2>, k_cells<4>}) {
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * cells_bytes(24448));
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 void launch_wait_selftest(hybrid_ctx *c, int max_polls)
