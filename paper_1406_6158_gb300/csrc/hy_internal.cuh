@@ -276,7 +276,8 @@ struct hybrid_ctx {
     int last_walk_mode = 0;
     // within an op sequence: the counters of the next walk are zero (a build cleared them); the counters and sums of
     // the pair kernels are clear for these forces (bit 0 soft, 1 hard: the walk cleared them)
-    bool walk_clean = false;
+    // the drift before the next build made its root cubes (launch_kick_seq with box)
+    bool walk_clean = false, box_done = false;
     int pairs_clean = 0;
 
     // profiling
@@ -355,8 +356,9 @@ void launch_copy_out(hybrid_ctx *c, const SysIO *d_io, bool state, bool acc_s, b
 // Applies n <= 4 kicks v <- v + h a_which in order (which 0 soft, 1 hard;
 // mode 0: h = val, 1: h = dt_soft/2, 2: h = (dt_soft/n_hard)/2, per system),
 // then a drift x <- x + dt v (dmode -1: none, 0: dt = dval, 2: dt_soft/n_hard).
+// box: a build follows; the drift of a single system makes its root cube too.
 void launch_kick_seq(hybrid_ctx *c, int n, const int *which, const int *mode, const double *val, int dmode,
-                     double dval, bool resplit = false);
+                     double dval, bool resplit = false, bool box = false);
 void launch_kick_ext(hybrid_ctx *c, const hybrid_system *s, int which, double h);
 void launch_drift_ext(hybrid_ctx *c, const hybrid_system *s, double dt);
 // kinetic and potential energy of a single system's working state to d_out[0..1]; d_out holds energy_scratch_bytes

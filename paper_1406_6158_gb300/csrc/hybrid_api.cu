@@ -386,6 +386,7 @@ struct Op {
 void begin_sequence(hybrid_ctx *c)
 {
     c->walk_clean = false;
+    c->box_done = false;
     c->pairs_clean = 0;
 }
 
@@ -393,8 +394,8 @@ void enqueue(hybrid_ctx *c, const Op &o, int idx)
 {
     c->op = idx;
     switch (o.kind) {
-    case OP_KICKS:   // mode 1: the drift of a hard step that reuses the neighbour lists
-        launch_kick_seq(c, o.nk, o.which, o.kmode, o.val, o.dmode, o.dval, o.mode == 1);
+    case OP_KICKS:   // mode 1: the drift of a hard step that reuses the neighbour lists; 2: a build follows
+        launch_kick_seq(c, o.nk, o.which, o.kmode, o.val, o.dmode, o.dval, o.mode == 1, o.mode == 2);
         break;
     case OP_BUILD: {
         // The build as a two-branch DAG: after the key sort, the topology and the groups (keys only) run beside
@@ -744,6 +745,7 @@ std::vector<Op> step_ops(const hybrid_ctx *c, int n_steps, bool valid, bool list
                 ops.push_back(kd);
                 ops.push_back(simple(OP_PAIR_NEAR, 2));
             } else {
+                kd.mode = 2;
                 ops.push_back(kd);
                 ops.push_back(simple(OP_BUILD));
                 ops.push_back(simple(OP_WALK, k == nh ? 3 : 2));

@@ -8,6 +8,7 @@
 // All systems of a batch are processed by the same launches; every node,
 // particle range and radix tile stays inside one system.
 #include "hy_internal.cuh"
+#include "root_box.cuh"
 
 #include <cuda/atomic>
 #include <cstdio>
@@ -24,122 +25,23 @@ __device__ __forceinline__ void fail(Status *st, int code, int where)
     if (atomicCAS(&st->code, 0, code) == 0) st->where = where;
 }
 
-// order-preserving map of doubles to unsigned integers (for atomic min/max)
-__device__ __forceinline__ unsigned long long ord_dbl(double v)
-{
-    unsigned long long u = (unsigned long long)__double_as_longlong(v);
-    return (u >> 63) ? ~u : (u | 0x8000000000000000ull);
-}
-__device__ __forceinline__ double unord_dbl(unsigned long long u)
-{
-    return __longlong_as_double((long long)((u >> 63) ? (u & 0x7fffffffffffffffull) : ~u));
-}
-
-// ---------------------------------------------------------------------------
-// Root cube: per-axis minimum lo; side L = smallest power of two >= the
-// largest extent (1 when all particles coincide); scale = 2^21 / L.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ SysBox make_box(const unsigned long long *bmin, const unsigned long long *bmax, int s)   // values other blocks made
-{
-    double lo[3], ext = 0.0;
-    for (int d = 0; d < 3; ++d) {
-        lo[d] = unord_dbl(__ldcg(bmin + 3 * s + d));
-        const double e = __dsub_rn(unord_dbl(__ldcg(bmax + 3 * s + d)), lo[d]);
-        if (e > ext) ext = e;
-    }
-    double L = 1.0;
-    if (ext > 0.0) {
-        int e2;
-        const double f = frexp(ext, &e2);
-        L = (f == 0.5) ? ext : ldexp(1.0, e2);
-    }
-    SysBox b;
-    b.lo[0] = lo[0];
-    b.lo[1] = lo[1];
-    b.lo[2] = lo[2];
-    b.L = L;
-    b.scale = ldexp(1.0, LEVELS) / L;   // ratio of powers of two: exact
-    b.u = ldexp(L, -20);
-    b.inv_u = ldexp(1.0, 20) / L;
-    b.uf = (float)b.u;
-    b.inv_uf = (float)b.inv_u;
-    return b;
-}
-
-// The last block to finish (a ticket, no waiting) makes the cubes.
+// Root cubes and the sample sort's start (see root_box.cuh) of a state that no drift of this sequence has moved.
 __global__ void __launch_bounds__(256) k_box(const double *__restrict__ x, const double *__restrict__ y,
                                              const double *__restrict__ z, const Chunk *__restrict__ chunks,
-                                             int nchunks, unsigned long long *bmin, unsigned long long *bmax, int nbk,
-                                             int S, const int64_t *__restrict__ off, const SSys *__restrict__ ss,
-                                             const uint64_t *__restrict__ key, uint32_t *__restrict__ cnt,
-                                             uint32_t *__restrict__ flag, unsigned *ticket, SysBox *__restrict__ boxout)
+                                             int nchunks, BoxArgs b)
 {
     // the sort always runs, whatever the status: later kernels rely on a consistent permutation
-    // sample sort (nbk buckets, 0 for the radix sort): bucket counts cleared, and whether the splitters (the
-    // last build's keys at every SS_BUCKET-th position) are in order
-    const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (gtid == 0) flag[0] = 0u;
-    for (int b = gtid; b < nbk; b += gridDim.x * blockDim.x) {
-        cnt[b] = 0u;
-        int s = 0;
-        if (S > 1) {   // system of bucket b
-            int hi = S;
-            while (hi - s > 1) {
-                const int mid = (s + hi) >> 1;
-                if (ss[mid].bbase <= b) s = mid;
-                else hi = mid;
-            }
-        }
-        const SSys y = ss[s];
-        const int j = b - y.bbase;
-        const uint64_t *k = key + off[s] + (int64_t)j * SS_BUCKET;
-        if (j >= 1 && j + 1 < y.nb && k[SS_BUCKET] < k[0]) flag[1] = 1u;
-    }
-    if (gtid == 0) cnt[nbk] = 0u;
-    // min/max of the order-preserving integer images: exact, and no FP64 pipe work
-    __shared__ unsigned long long sh[6][8];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    begin_sort(b);
     for (int c = blockIdx.x; c < nchunks; c += gridDim.x) {
         const Chunk ch = chunks[c];
-        unsigned long long v[6] = {~0ull, ~0ull, ~0ull, 0ull, 0ull, 0ull};
+        Bounds v;
         for (int i = threadIdx.x; i < ch.len; i += blockDim.x) {
             const int64_t k = ch.start + i;
-            const unsigned long long p0 = ord_dbl(x[k]), p1 = ord_dbl(y[k]), p2 = ord_dbl(z[k]);
-            v[0] = min(v[0], p0);
-            v[1] = min(v[1], p1);
-            v[2] = min(v[2], p2);
-            v[3] = max(v[3], p0);
-            v[4] = max(v[4], p1);
-            v[5] = max(v[5], p2);
+            v.add(x[k], y[k], z[k]);
         }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int j = 0; j < 3; ++j) v[j] = min(v[j], __shfl_xor_sync(0xffffffffu, v[j], o));
-#pragma unroll
-            for (int j = 3; j < 6; ++j) v[j] = max(v[j], __shfl_xor_sync(0xffffffffu, v[j], o));
-        }
-        if (lane == 0)
-            for (int j = 0; j < 6; ++j) sh[j][w] = v[j];
-        __syncthreads();
-        if (threadIdx.x < 6) {
-            const int j = threadIdx.x;
-            unsigned long long r = sh[j][0];
-            for (int k = 1; k < 8; ++k) r = (j < 3) ? min(r, sh[j][k]) : max(r, sh[j][k]);
-            if (j < 3) atomicMin(&bmin[3 * ch.sys + j], r);
-            else atomicMax(&bmax[3 * ch.sys + j - 3], r);
-        }
-        __syncthreads();
+        v.reduce_block(b, ch.sys);
     }
-    __shared__ bool last;
-    __threadfence();   // this block's bounds are visible before its ticket
-    __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    for (int s = threadIdx.x; s < S; s += blockDim.x) boxout[s] = make_box(bmin, bmax, s);
-    if (threadIdx.x == 0) *ticket = 0u;
+    finish_boxes(b);
 }
 
 // ---------------------------------------------------------------------------
@@ -1856,13 +1758,14 @@ static int grid_for(hybrid_ctx *c, int64_t work, int threads, int per_sm = 8)
 
 void launch_box(hybrid_ctx *c)
 {
+    if (c->box_done) {   // by the drift before this build
+        c->box_done = false;
+        return;
+    }
     // the boxes are empty here: the copy into the working state and every permutation reset them
     k_box<<<std::min(c->nchunks, c->nsm * 16), 256, 0, c->st>>>(
         (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p, (const Chunk *)c->chunks_dev.p,
-        c->nchunks, (unsigned long long *)c->boxmin.p, (unsigned long long *)c->boxmax.p, c->sort_fallback ? 0 : c->nbk,
-        c->S, (const int64_t *)c->off_dev.p, (const SSys *)c->ss_sys.p, (const uint64_t *)c->keys[0].p,
-        (uint32_t *)c->ss_cnt.p, (uint32_t *)c->ss_flag.p, (unsigned *)((unsigned long long *)c->counter.p + 14),
-        (SysBox *)c->box.p);
+        c->nchunks, box_args(c));
     c->launches += 1;
 }
 
