@@ -595,7 +595,9 @@ bool launch_as_graph(hybrid_ctx *c, const std::vector<Op> &ops, std::vector<std:
 
 Op simple(int kind, int mode = 0);
 
-hybrid_status run_ops(hybrid_ctx *c, const std::vector<Op> &ops_in)
+// Runs the sequence and, when copy_out is set, copies state and accelerations to the caller's arrays after it (the
+// kernel does nothing while a failure is recorded; after a recovery it runs again), then waits for all of it once.
+hybrid_status run_ops(hybrid_ctx *c, const std::vector<Op> &ops_in, bool copy_out = false)
 {
     std::vector<Op> ops = ops_in;
     size_t start = 0;
@@ -611,6 +613,7 @@ hybrid_status run_ops(hybrid_ctx *c, const std::vector<Op> &ops_in)
             begin_sequence(c);
             for (size_t i = start; i < ops.size(); ++i) enqueue(c, ops[i], (int)i);
         }
+        if (copy_out) launch_copy_out(c, (const SysIO *)c->io_dev.p, true, true, true);
         cudaError_t le = cudaGetLastError();
         if (le != cudaSuccess) return cuda_fail(c, le, "kernel launch");
         Status s;
@@ -963,13 +966,10 @@ hybrid_status hybrid_step_batched(hybrid_ctx *c, hybrid_system *sys, int n_sys, 
     const bool lists_ok = valid && c->lists_fresh && c->lists_sig == sig;
     c->lists_fresh = false;
     launch_copy_in(c, (const SysIO *)c->io_dev.p, valid);
-    r = run_ops(c, step_ops(c, n_soft_steps, valid, lists_ok));
+    r = run_ops(c, step_ops(c, n_soft_steps, valid, lists_ok), true);
     if (r != HYBRID_OK) return r;
     c->lists_fresh = c->p.skin > 0.0;
     c->lists_sig = sig;
-    launch_copy_out(c, (const SysIO *)c->io_dev.p, true, true, true);
-    Status s;
-    if ((r = read_status(c, &s)) != HYBRID_OK) return r;
     for (int k = 0; k < n_sys; ++k) sys[k].forces_valid = 1;
     c->tree_valid = (n_sys == 1);
     c->have_soft = c->have_hard = true;
