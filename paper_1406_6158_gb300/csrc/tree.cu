@@ -1104,10 +1104,11 @@ __device__ __forceinline__ void mom_store(const MomArgs &a, uint32_t c, const Mo
     store_com(a, c, r.M, c0, c1, c2, B2);
 }
 
-__device__ __forceinline__ double warp_sum_d(double v)
+// sum over the lanes of an aligned group of 8 (the children of a cell)
+__device__ __forceinline__ double sum8_d(double v)
 {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
 
@@ -1132,15 +1133,15 @@ __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32
     const double rx = __shfl_sync(0xffffffffu, x, 0), ry = __shfl_sync(0xffffffffu, y, 0),
                  rz = __shfl_sync(0xffffffffu, z, 0);
     const double dx = x - rx, dy = y - ry, dz = z - rz;
-    const double Mt = warp_sum_d(M);
+    const double Mt = __shfl_sync(0xffffffffu, sum8_d(M), 0);   // the same in all lanes: the branch below has full-warp sums
     double c0, c1, c2, B2t = 0.0;
     if (Mt > 0.0) {
-        const double ex = warp_sum_d(M * dx) / Mt, ey = warp_sum_d(M * dy) / Mt, ez = warp_sum_d(M * dz) / Mt;
+        const double ex = sum8_d(M * dx) / Mt, ey = sum8_d(M * dy) / Mt, ez = sum8_d(M * dz) / Mt;
         c0 = rx + ex;
         c1 = ry + ey;
         c2 = rz + ez;
         const double qx = dx - ex, qy = dy - ey, qz = dz - ez;
-        B2t = warp_sum_d(on ? B2 + M * (qx * qx + qy * qy + qz * qz) : 0.0);
+        B2t = sum8_d(on ? B2 + M * (qx * qx + qy * qy + qz * qz) : 0.0);
     } else {   // massless cell: its geometric centre
         double o[3], sd;
         cell_geom(b, a.key[f], a.nlevel[c], o, &sd);
@@ -1315,6 +1316,21 @@ __device__ __forceinline__ void finish_f32(const FinArgs &a, uint32_t c, uint32_
 
 constexpr uint32_t BM_CH = 256;
 
+// largest distance of particles [f, e) to (c0, c1, c2): the largest square, compared as an integer (squares are not
+// negative; a NaN would win), and one square root at the end (it is monotone)
+__device__ __forceinline__ double farthest_f64(const MomArgs &a, uint32_t f, uint32_t e, double c0, double c1, double c2,
+                                               int lane)
+{
+    long long m = 0;
+    for (uint32_t i = f + lane; i < e; i += 32) {
+        const double d0 = a.x[i] - c0, d1 = a.y[i] - c1, d2 = a.z[i] - c2;
+        m = max(m, __double_as_longlong(d0 * d0 + d1 * d1 + d2 * d2));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    return sqrt(__longlong_as_double(m));
+}
+
 // every cell of at most MOM_CH particles, and every leaf (a leaf holds more
 // only when its particles share one level-21 cell): moments and b_max from its
 // particles, then the climb; the larger cells are listed for their b_max, in
@@ -1339,15 +1355,9 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
                 const double c0 = __shfl_sync(0xffffffffu, lane == 0 ? a.cx[c] : 0.0, 0);
                 const double c1 = __shfl_sync(0xffffffffu, lane == 0 ? a.cy[c] : 0.0, 0);
                 const double c2 = __shfl_sync(0xffffffffu, lane == 0 ? a.cz[c] : 0.0, 0);
-                double dm = 0.0;
-                for (uint32_t i = f + lane; i < f + n; i += 32) {
-                    const double d0 = a.x[i] - c0, d1 = a.y[i] - c1, d2 = a.z[i] - c2;
-                    dm = fmax(dm, sqrt(d0 * d0 + d1 * d1 + d2 * d2));
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+                mom_climb<true, 32>(a, up, lane, 0xffffffffu);   // others wait for this
+                const double dm = farthest_f64(a, f, f + n, c0, c1, c2, lane);
                 if (lane == 0) a.bmax64[c] = (unsigned long long)__double_as_longlong(dm);
-                mom_climb<true, 32>(a, up, lane, 0xffffffffu);
             } else if (lane == 0) {
                 const uint32_t nch = (n + BM_CH - 1) / BM_CH;
                 const unsigned long long base = atomicAdd(nitems, (unsigned long long)nch);
@@ -1411,13 +1421,7 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
         const uint32_t f0 = f + k * BM_CH, n0 = min(BM_CH, f + n - f0);
         if (F64) {
             const double c0 = a.cx[c], c1 = a.cy[c], c2 = a.cz[c];
-            double dm = 0.0;
-            for (uint32_t i = f0 + lane; i < f0 + n0; i += 32) {
-                const double d0 = a.x[i] - c0, d1 = a.y[i] - c1, d2 = a.z[i] - c2;
-                dm = fmax(dm, sqrt(d0 * d0 + d1 * d1 + d2 * d2));
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) dm = fmax(dm, __shfl_xor_sync(0xffffffffu, dm, o));
+            const double dm = farthest_f64(a, f0, f0 + n0, c0, c1, c2, lane);
             if (lane == 0) atomicMax(a.bmax64 + c, (unsigned long long)__double_as_longlong(dm));
         } else {
             const float4 A = a.nA[c], B = a.nB[c];

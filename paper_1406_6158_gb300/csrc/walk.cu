@@ -90,21 +90,27 @@ __device__ __forceinline__ uint32_t warp_excl_scan(uint32_t v, uint32_t &total)
     return inc - v;
 }
 
-// distance from p to the box [lo, hi], per axis max(lo - p, 0, p - hi)
-__device__ __forceinline__ double dist_box_f64(double p0, double p1, double p2, const double *lo, const double *hi)
+// square of the distance from p to the box [lo, hi], per axis max(lo - p, 0, p - hi) (signs from the bits: a
+// comparison of doubles takes the FP64 pipe, 2 lanes per SM and clock)
+__device__ __forceinline__ double dist2_box_f64(double p0, double p1, double p2, const double *lo, const double *hi)
 {
     const double p[3] = {p0, p1, p2};
     double s = 0.0;
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
-        double g = 0.0;
-        const double a = lo[d] - p[d];
-        const double b = p[d] - hi[d];
-        if (a > g) g = a;
-        if (b > g) g = b;
+        const double a = lo[d] - p[d], b = p[d] - hi[d];
+        const double g = __double2hiint(a) > 0 ? a : (__double2hiint(b) > 0 ? b : 0.0);
         s += g * g;
     }
-    return sqrt(s);
+    return s;
+}
+
+// whether a distance reaches a radius, from the FP32 nearest to their squares: 1 yes, 0 no, -1 within FP32's rounding
+// (or out of its range)
+__device__ __forceinline__ int reaches(float d2, float r2)
+{
+    if (!(d2 > 1e-30f && r2 > 1e-30f && r2 < 1e30f)) return -1;
+    return d2 > r2 * 1.000001f ? 1 : (d2 < r2 * 0.999999f ? 0 : -1);
 }
 
 // What the pair kernels after this walk count from (the far counts only when the soft force follows).
@@ -117,14 +123,16 @@ __device__ __forceinline__ void clear_pair_counters(const WalkArgs &a)
     }
 }
 
-template <bool F64, bool FILL>
+// FP64 form: count pass, then fill pass, the same walk twice. Tests are decided in FP32 wherever its rounding allows,
+// and the emission is k_walk1's.
+template <bool FILL>
 __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
 {
     Status *st = a.st;
     if (st->code) return;
     if (FILL) clear_pair_counters(a);
     const int lane = threadIdx.x & 31;
-    const unsigned ltmask = (1u << lane) - 1u;
+    const unsigned lt = (1u << lane) - 1u;
     const int64_t ng = *a.ngroups;
     if (!FILL && blockIdx.x == 0 && threadIdx.x == 0) *a.d_n3 = 3 * ng;
     if (FILL) {
@@ -139,7 +147,9 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
         if (blockIdx.x == 0 && threadIdx.x == 0) a.cnt[3 * ng] = total;
     }
     const int64_t gw = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    uint32_t *stk = a.stack + gw * a.cap_stack;
+    uint32_t *stk = a.stack + gw * a.cap_stack;   // overflow part of the stack (older entries)
+    __shared__ uint32_t sstk_all[WALK_THREADS / 32][WALK_SSTK];
+    uint32_t *sstk = sstk_all[threadIdx.x >> 5];  // top part of the stack
     const bool want_soft = a.mode & 1, want_hard = (a.mode >> 1) & 1;
 
     for (;;) {
@@ -150,25 +160,11 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
         const uint32_t s = a.gsys[g];
         const bool has_hard = a.sp[s].has_hard != 0;
         const bool wh0 = want_hard && has_hard;
-        float cx = 0, cy = 0, cz = 0, lx = 0, ly = 0, lz = 0, hx = 0, hy = 0, hz = 0;
-        double blo[3] = {0, 0, 0}, bhi[3] = {0, 0, 0};
-        if (F64) {
+        double blo[3], bhi[3];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) {
-                blo[d] = a.glo[3 * g + d];
-                bhi[d] = a.ghi[3 * g + d];
-            }
-        } else {
-            const GroupF G = a.gF[g];
-            cx = G.c_hi.x;
-            cy = G.c_hi.y;
-            cz = G.c_hi.z;
-            hx = G.c_hi.w;
-            lx = G.c_lo.x;
-            ly = G.c_lo.y;
-            lz = G.c_lo.z;
-            hy = G.c_lo.w;
-            hz = G.hz_root.x;
+        for (int d = 0; d < 3; ++d) {
+            blo[d] = a.glo[3 * g + d];
+            bhi[d] = a.ghi[3 * g + d];
         }
         uint64_t nc = 0, np = 0, nh = 0, oc = 0, op = 0, oh = 0;
         if (FILL) {
@@ -176,17 +172,48 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
             op = a.cnt[ng + g];
             oh = a.cnt[2 * ng + g];
         }
-        int64_t sp = 0;
+        int sp = 0;        // entries in the shared-memory part
+        int64_t gp = 0;    // entries in the global part
         if (want_soft || wh0) {
-            if (lane == 0) stk[0] = a.sysroot[s] | ((uint32_t)want_soft << 30) | ((uint32_t)wh0 << 31);
+            if (lane == 0) sstk[0] = a.sysroot[s] | ((uint32_t)want_soft << 30) | ((uint32_t)wh0 << 31);
             sp = 1;
         }
         __syncwarp();
         bool overflow = false;
-        while (sp > 0) {
-            const int take = (int)(sp < 32 ? sp : 32);
+        // the particles of the lanes' leaves, [first, first + k) each (k = 0: none), counted or written from dst
+        auto leaves = [&](uint64_t dst, uint32_t first, uint32_t k) -> uint32_t {
+            if (!FILL) return __reduce_add_sync(0xffffffffu, k);
+            uint32_t tot, ex;
+            if (__all_sync(0xffffffffu, k < 32u)) {
+                ex = tot = 0u;
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    const unsigned b = __ballot_sync(0xffffffffu, (k >> q) & 1u);
+                    ex += (uint32_t)__popc(b & lt) << q;
+                    tot += (uint32_t)__popc(b) << q;
+                }
+            } else {
+                ex = warp_excl_scan(k, tot);
+            }
+            uint32_t *to = a.list + dst + ex;
+            const uint32_t most = __reduce_max_sync(0xffffffffu, k);
+            for (uint32_t j = 0; j < most; j += 4)
+#pragma unroll
+                for (uint32_t q = 0; q < 4; ++q)
+                    if (j + q < k) to[j + q] = first + j + q;
+            return tot;
+        };
+        while (sp > 0 || gp > 0) {
+            if (sp == 0) {   // refill the shared part from the top of the global part
+                const int m = (int)(gp < WALK_SSTK / 2 ? gp : WALK_SSTK / 2);
+                for (int j = lane; j < m; j += 32) sstk[j] = stk[gp - m + j];
+                gp -= m;
+                sp = m;
+                __syncwarp();
+            }
+            const int take = sp < 32 ? sp : 32;
             uint32_t e = 0;
-            if (lane < take) e = stk[sp - take + lane];
+            if (lane < take) e = sstk[sp - take + lane];
             sp -= take;
             __syncwarp();
             const bool valid = lane < take;
@@ -196,21 +223,17 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
             uint4 T = make_uint4(NONE, 0, 0, 0);
             if (valid) {
                 T = a.topo[c];
-                if (F64) {
-                    const double4_32a D = a.nD[c];
-                    const double d = dist_box_f64(D.x, D.y, D.z, blo, bhi);
-                    const double hr = a.hr[c];
-                    accept = (d >= a.rb[c]) && (d >= hr);
-                    near = has_hard && (d < hr);
-                } else {
-                    const float4 A = a.nA[c], B = a.nB[c];
-                    const float2 cr = a.crit[c];
-                    const float rx = fmaxf(fabsf((A.x - cx) + (B.x - lx)) - hx, 0.0f);
-                    const float ry = fmaxf(fabsf((A.y - cy) + (B.y - ly)) - hy, 0.0f);
-                    const float rz = fmaxf(fabsf((A.z - cz) + (B.z - lz)) - hz, 0.0f);
-                    const float d2 = rx * rx + ry * ry + rz * rz;
-                    accept = d2 >= cr.x;
-                    near = has_hard && (d2 < cr.y);
+                const double4_32a D = a.nD[c];
+                const float2 cr = a.crit[c];   // max(r_b, R2 + b_max)^2 and (R2 + b_max)^2
+                const double d2 = dist2_box_f64(D.x, D.y, D.z, blo, bhi);
+                const float d2f = narrow(d2);
+                const int far_enough = reaches(d2f, cr.x), beyond = has_hard ? reaches(d2f, cr.y) : 1;
+                accept = far_enough > 0;
+                near = beyond == 0;
+                if (far_enough < 0 || beyond < 0) {
+                    const double d = sqrt(d2), hr = a.hr[c];
+                    if (far_enough < 0) accept = d >= a.rb[c] && d >= hr;
+                    if (beyond < 0) near = d < hr;
                 }
             }
             const bool leaf = (T.y == 0);
@@ -222,44 +245,34 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
             const bool open = valid && !leaf && (open_s || open_h);
             // taken cells
             const unsigned bm = __ballot_sync(0xffffffffu, take_cell);
-            if (FILL && take_cell) a.list[oc + nc + __popc(bm & ltmask)] = c;
+            if (FILL && take_cell) a.list[oc + nc + __popc(bm & lt)] = c;
             nc += (uint64_t)__popc(bm);
-            // soft particles
-            {
-                uint32_t tot;
-                const uint32_t k = soft_leaf ? T.w : 0u;
-                const uint32_t ex = warp_excl_scan(k, tot);
-                if (FILL && soft_leaf) {
-                    uint32_t *dst = a.list + op + np + ex;
-                    for (uint32_t j = 0; j < k; ++j) dst[j] = T.z + j;
-                }
-                np += tot;
-            }
-            // hard particles
-            {
-                uint32_t tot;
-                const uint32_t k = hard_leaf ? T.w : 0u;
-                const uint32_t ex = warp_excl_scan(k, tot);
-                if (FILL && hard_leaf) {
-                    uint32_t *dst = a.list + oh + nh + ex;
-                    for (uint32_t j = 0; j < k; ++j) dst[j] = T.z + j;
-                }
-                nh += tot;
-            }
-            // children of opened cells
-            {
-                uint32_t tot;
+            if (__any_sync(0xffffffffu, soft_leaf)) np += leaves(op + np, T.z, soft_leaf ? T.w : 0u);
+            if (__any_sync(0xffffffffu, hard_leaf)) nh += leaves(oh + nh, T.z, hard_leaf ? T.w : 0u);
+            if (__any_sync(0xffffffffu, open)) {   // children of opened cells (at most 8 each)
+                const uint32_t fl = ((uint32_t)open_s << 30) | ((uint32_t)open_h << 31);
                 const uint32_t k = open ? T.y : 0u;
-                const uint32_t ex = warp_excl_scan(k, tot);
-                if (sp + (int64_t)tot > a.cap_stack) {
-                    overflow = true;
-                    break;
+                uint32_t ex = 0, sum = 0;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned b = __ballot_sync(0xffffffffu, (k >> q) & 1u);
+                    ex += (uint32_t)__popc(b & lt) << q;
+                    sum += (uint32_t)__popc(b) << q;
                 }
-                if (open) {
-                    const uint32_t fl = ((uint32_t)open_s << 30) | ((uint32_t)open_h << 31);
-                    for (uint32_t j = 0; j < k; ++j) stk[sp + ex + j] = (T.x + j) | fl;
+                if (sp + (int)sum > WALK_SSTK) {   // move the shared part under the global part
+                    if (gp + sp > a.cap_stack) {
+                        overflow = true;
+                        break;
+                    }
+                    for (int j = lane; j < sp; j += 32) stk[gp + j] = sstk[j];
+                    gp += sp;
+                    sp = 0;
+                    __syncwarp();
                 }
-                sp += tot;
+#pragma unroll
+                for (uint32_t j = 0; j < 8; ++j)
+                    if (j < k) sstk[sp + ex + j] = (T.x + j) | fl;
+                sp += (int)sum;
             }
             __syncwarp();
         }
@@ -605,11 +618,11 @@ void launch_walk(hybrid_ctx *c, int mode)
     }
     // count pass
     a.counter = (unsigned long long *)c->counter.p;
-    k_walk<true, false><<<grid, WALK_THREADS, 0, c->st>>>(a);
+    k_walk<false><<<grid, WALK_THREADS, 0, c->st>>>(a);
     scan_u64(c, (uint64_t *)c->lcnt.p, 0, d_n3, 3 * c->capGroups, d_total);
     // fill pass
     a.counter = (unsigned long long *)c->counter.p + 1;
-    k_walk<true, true><<<grid, WALK_THREADS, 0, c->st>>>(a);
+    k_walk<true><<<grid, WALK_THREADS, 0, c->st>>>(a);
     prof_end(c, PROF_WALK, e0);
     c->launches += 2;
     c->last_walk_mode = mode;

@@ -62,6 +62,24 @@ def test_fp64_forces_at_the_splits_edges(H, n, n_crit, same, eps):
     check(s2.numpy())
 
 
+# the FP64 walk: every cell opened (more pending cells than the shared part of a warp's stack holds), none, leaves of
+# 1 particle and leaves of 32 and more (offsets by ballots and by scan)
+@pytest.mark.parametrize("n,theta,n_leaf,same", [(6000, 0.0, 1, 0), (3000, 1e-3, 16, 0), (2500, 0.6, 31, 0),
+                                                 (2500, 0.6, 64, 0), (2500, 5.0, 1, 0), (1500, 0.6, 16, 40)])
+def test_fp64_walk_at_its_edges(H, n, theta, n_leaf, same):
+    st = state(n, same)
+    kw = dict(eps=0.01, theta=theta, R1=0.04, R2=0.08, n_crit=64, n_leaf=n_leaf)
+    ctx, s = H.Context(H.Params(precision=0, **kw)), H.System(st, precision=0)
+    ctx.hybrid_step(s, 0)
+    o = s.numpy()
+    T = oracle.Tree(o["x"], o["y"], o["z"], o["m"], oracle.Params(**kw))
+    a_s, a_h, sc_s, sc_h = T.forces()
+    floor = 1e-24 * np.max(sc_s)
+    for d, k in enumerate("xyz"):
+        assert np.all(np.abs(o["a%s_s" % k] - a_s[:, d]) <= 1e-12 * sc_s + floor)
+        assert np.all(np.abs(o["a%s_h" % k] - a_h[:, d]) <= 1e-12 * sc_h + floor)
+
+
 @pytest.mark.parametrize("scale", [-328, -300, 300, 330])
 def test_fp64_forces_scale_with_the_lengths(H, scale):
     # lengths times 2^scale: forces times 2^(-2 scale) (inside the seed's range, 2^-640 < r^2 < 2^640, bit for
