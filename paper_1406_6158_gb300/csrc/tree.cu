@@ -959,13 +959,6 @@ __device__ __forceinline__ void store_com(const MomArgs &a, uint32_t c, double M
     a.cy[c] = c1;
     a.cz[c] = c2;
     a.B2[c] = B2;
-    const SysBox b = a.box[a.psys[a.nfirst[c]]];
-    float h[3], l[3];
-    grid_split(c0, b.lo[0], b, h[0], l[0]);
-    grid_split(c1, b.lo[1], b, h[1], l[1]);
-    grid_split(c2, b.lo[2], b, h[2], l[2]);
-    a.nA[c] = make_float4(h[0], h[1], h[2], (float)M);
-    a.nB[c] = make_float4(l[0], l[1], l[2], 0.0f);
 }
 
 // Moments straight from each cell's particle range, with no wait on the
@@ -1058,12 +1051,13 @@ __device__ __forceinline__ void mom_b2_f32(const float4 *__restrict__ phi, const
     bmax = sqrtf(d2max);
 }
 
+template <int G>
 __device__ __forceinline__ MomSums mom_range(const MomArgs &a, uint32_t f, uint32_t n, double o0, double o1, double o2,
-                                             int lane)
+                                             int sl, unsigned gm)
 {
     MomSums r = {0.0, 0.0, 0.0, 0.0, 0.0};
-#pragma unroll 4
-    for (uint32_t i = f + lane; i < f + n; i += 32) {
+#pragma unroll 2
+    for (uint32_t i = f + sl; i < f + n; i += G) {
         const double mi = a.m[i];
         const double d0 = a.x[i] - o0, d1 = a.y[i] - o1, d2 = a.z[i] - o2;
         r.M += mi;
@@ -1073,12 +1067,12 @@ __device__ __forceinline__ MomSums mom_range(const MomArgs &a, uint32_t f, uint3
         r.Q += mi * (d0 * d0 + d1 * d1 + d2 * d2);
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {   // fixed butterfly: the same order every run
-        r.M += __shfl_xor_sync(0xffffffffu, r.M, o);
-        r.sx += __shfl_xor_sync(0xffffffffu, r.sx, o);
-        r.sy += __shfl_xor_sync(0xffffffffu, r.sy, o);
-        r.sz += __shfl_xor_sync(0xffffffffu, r.sz, o);
-        r.Q += __shfl_xor_sync(0xffffffffu, r.Q, o);
+    for (int o = G / 2; o > 0; o >>= 1) {   // fixed butterfly: the same order every run
+        r.M += __shfl_xor_sync(gm, r.M, o, G);
+        r.sx += __shfl_xor_sync(gm, r.sx, o, G);
+        r.sy += __shfl_xor_sync(gm, r.sy, o, G);
+        r.sz += __shfl_xor_sync(gm, r.sz, o, G);
+        r.Q += __shfl_xor_sync(gm, r.Q, o, G);
     }
     return r;
 }
@@ -1104,20 +1098,23 @@ __device__ __forceinline__ void mom_store(const MomArgs &a, uint32_t c, const Mo
     store_com(a, c, r.M, c0, c1, c2, B2);
 }
 
-// sum over the lanes of an aligned group of 8 (the children of a cell)
-__device__ __forceinline__ double sum8_d(double v)
+// sum over the first 8 of G lanes (the children of a cell), in all of them
+template <int G>
+__device__ __forceinline__ double sum8_d(double v, unsigned gm)
 {
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
+    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(gm, v, o, G);
+    return G > 8 ? __shfl_sync(gm, v, 0, G) : v;
 }
 
 // A larger cell from its (at most 8) children, one per lane, in a fixed order.
-// FP64 form in FP64 (a whole warp). FP32 form in FP32 on offsets from the
-// first child's hi/lo centre of mass (hi differences exact), stored like a
-// small cell's, by G lanes (a warp or an aligned group of 8 with mask gm).
+// FP64 form in FP64. FP32 form in FP32 on offsets from the first child's hi/lo
+// centre of mass (hi differences exact), stored like a small cell's. By G lanes
+// (a warp or an aligned group of 8 with mask gm).
 // f: the cell's first particle; [ch0, ch0 + k): its children.
-__device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32_t ch0, uint32_t k, int lane)
+template <int G>
+__device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32_t ch0, uint32_t k, int lane,
+                                unsigned gm)
 {
     const SysBox &b = a.box[a.S == 1 ? 0 : a.psys[f]];
     const bool on = (uint32_t)lane < k;
@@ -1130,18 +1127,17 @@ __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32
         z = __ldcg(a.cz + j);
         B2 = __ldcg(a.B2 + j);
     }
-    const double rx = __shfl_sync(0xffffffffu, x, 0), ry = __shfl_sync(0xffffffffu, y, 0),
-                 rz = __shfl_sync(0xffffffffu, z, 0);
+    const double rx = __shfl_sync(gm, x, 0, G), ry = __shfl_sync(gm, y, 0, G), rz = __shfl_sync(gm, z, 0, G);
     const double dx = x - rx, dy = y - ry, dz = z - rz;
-    const double Mt = __shfl_sync(0xffffffffu, sum8_d(M), 0);   // the same in all lanes: the branch below has full-warp sums
+    const double Mt = sum8_d<G>(M, gm);   // the same in all lanes: the branch below has sums over them
     double c0, c1, c2, B2t = 0.0;
     if (Mt > 0.0) {
-        const double ex = sum8_d(M * dx) / Mt, ey = sum8_d(M * dy) / Mt, ez = sum8_d(M * dz) / Mt;
+        const double ex = sum8_d<G>(M * dx, gm) / Mt, ey = sum8_d<G>(M * dy, gm) / Mt, ez = sum8_d<G>(M * dz, gm) / Mt;
         c0 = rx + ex;
         c1 = ry + ey;
         c2 = rz + ez;
         const double qx = dx - ex, qy = dy - ey, qz = dz - ez;
-        B2t = sum8_d(on ? B2 + M * (qx * qx + qy * qy + qz * qz) : 0.0);
+        B2t = sum8_d<G>(on ? B2 + M * (qx * qx + qy * qy + qz * qz) : 0.0, gm);
     } else {   // massless cell: its geometric centre
         double o[3], sd;
         cell_geom(b, a.key[f], a.nlevel[c], o, &sd);
@@ -1231,7 +1227,7 @@ __device__ void mom_climb(const MomArgs &a, uint32_t p, int lane, unsigned gm)
         old = __shfl_sync(gm, old, 0, G);
         if (old + 1u != k) return;
         __syncwarp(gm);
-        if (F64) mom_combine_f64(a, p, f, ch0, k, lane);
+        if (F64) mom_combine_f64<G>(a, p, f, ch0, k, lane, gm);
         else mom_combine_f32<G>(a, p, f, ch0, k, lane, gm);
         p = up;
     }
@@ -1318,17 +1314,40 @@ constexpr uint32_t BM_CH = 256;
 
 // largest distance of particles [f, e) to (c0, c1, c2): the largest square, compared as an integer (squares are not
 // negative; a NaN would win), and one square root at the end (it is monotone)
+template <int G>
 __device__ __forceinline__ double farthest_f64(const MomArgs &a, uint32_t f, uint32_t e, double c0, double c1, double c2,
-                                               int lane)
+                                               int sl, unsigned gm)
 {
     long long m = 0;
-    for (uint32_t i = f + lane; i < e; i += 32) {
+    for (uint32_t i = f + sl; i < e; i += G) {
         const double d0 = a.x[i] - c0, d1 = a.y[i] - c1, d2 = a.z[i] - c2;
         m = max(m, __double_as_longlong(d0 * d0 + d1 * d1 + d2 * d2));
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    for (int o = G / 2; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(gm, m, o, G));
     return sqrt(__longlong_as_double(m));
+}
+
+// FP64 form: moments of a cell from its particles, the climb, and b_max, by G lanes
+template <int G>
+__device__ __forceinline__ void mom_cell_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32_t n, uint32_t up, int sl,
+                                             unsigned gm)
+{
+    const double o0 = a.x[f], o1 = a.y[f], o2 = a.z[f];
+    const MomSums r = mom_range<G>(a, f, n, o0, o1, o2, sl, gm);
+    double c0 = 0.0, c1 = 0.0, c2 = 0.0;
+    if (sl == 0) {
+        mom_store(a, c, r, o0, o1, o2);
+        c0 = a.cx[c];
+        c1 = a.cy[c];
+        c2 = a.cz[c];
+    }
+    c0 = __shfl_sync(gm, c0, 0, G);
+    c1 = __shfl_sync(gm, c1, 0, G);
+    c2 = __shfl_sync(gm, c2, 0, G);
+    mom_climb<true, G>(a, up, sl, gm);   // others wait for this
+    const double dm = farthest_f64<G>(a, f, f + n, c0, c1, c2, sl, gm);
+    if (sl == 0) a.bmax64[c] = (unsigned long long)__double_as_longlong(dm);
 }
 
 // every cell of at most MOM_CH particles, and every leaf (a leaf holds more
@@ -1344,35 +1363,44 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
     const int lane = threadIdx.x & 31;
     const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
     const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (F64) {   // one warp per cell
-        for (uint32_t c = warp; c < total; c += nw) {
-            const uint32_t f = a.nfirst[c], n = a.nend[c] - f, up = a.nparent[c];
-            if (n <= MOM_CH || a.nchild[c] == NONE) {
-                const double o0 = a.x[f], o1 = a.y[f], o2 = a.z[f];
-                const MomSums r = mom_range(a, f, n, o0, o1, o2, lane);
-                if (lane == 0) mom_store(a, c, r, o0, o1, o2);
-                __syncwarp();
-                const double c0 = __shfl_sync(0xffffffffu, lane == 0 ? a.cx[c] : 0.0, 0);
-                const double c1 = __shfl_sync(0xffffffffu, lane == 0 ? a.cy[c] : 0.0, 0);
-                const double c2 = __shfl_sync(0xffffffffu, lane == 0 ? a.cz[c] : 0.0, 0);
-                mom_climb<true, 32>(a, up, lane, 0xffffffffu);   // others wait for this
-                const double dm = farthest_f64(a, f, f + n, c0, c1, c2, lane);
-                if (lane == 0) a.bmax64[c] = (unsigned long long)__double_as_longlong(dm);
-            } else if (lane == 0) {
-                const uint32_t nch = (n + BM_CH - 1) / BM_CH;
-                const unsigned long long base = atomicAdd(nitems, (unsigned long long)nch);
-                if (base + nch > cap_items) {
-                    fail(st, HYBRID_ECAPACITY, where);
-                    continue;
-                }
-                bigbase[c] = (uint32_t)base;
-                for (uint32_t k = 0; k < nch; ++k) items[base + k] = c;
+    const int sub = lane >> 3, sl = lane & 7;
+    const unsigned gm = 0xFFu << (8 * sub);
+    const uint32_t nq = (total + 3) / 4;
+    auto list_big = [&](uint32_t c, uint32_t n) {   // by the cell's 8 lanes
+        const uint32_t nch = a.search ? 1u : (n + BM_CH - 1) / BM_CH;
+        unsigned long long base = 0;
+        if (sl == 0) base = atomicAdd(nitems, (unsigned long long)nch);
+        base = __shfl_sync(gm, base, 0, 8);
+        if (base + nch > cap_items) {
+            if (sl == 0) fail(st, HYBRID_ECAPACITY, where);
+            return;
+        }
+        if (sl == 0) bigbase[c] = (uint32_t)base;
+        for (uint32_t k = sl; k < nch; k += 8) items[base + k] = c;
+    };
+    if (F64) {
+        // Four cells per warp: an FP64 instruction takes the pipe 16 clocks for a warp, however few of its lanes are
+        // on, and most cells hold fewer than 16 particles (moments of a build at N = 30011: one warp per cell
+        // 0.132 ms, so 0.098).
+        // Leaves of more than MOM_CH particles come after that, by the whole warp.
+        for (uint32_t q = warp; q < nq; q += nw) {
+            const uint32_t c = 4 * q + sub;
+            const bool valid = c < total;
+            const uint32_t f = valid ? a.nfirst[c] : 0u, n = valid ? a.nend[c] - f : 0u, up = valid ? a.nparent[c] : NONE;
+            const bool leaf = valid && a.nchild[c] == NONE;
+            if (valid && n <= MOM_CH) {
+                mom_cell_f64<8>(a, c, f, n, up, sl, gm);
+            } else if (valid && !leaf) {
+                list_big(c, n);
+            }
+            __syncwarp();
+            for (unsigned todo = __ballot_sync(0xffffffffu, leaf && n > MOM_CH && sl == 0); todo; todo &= todo - 1) {
+                const int from = __ffs(todo) - 1;
+                mom_cell_f64<32>(a, __shfl_sync(0xffffffffu, c, from), __shfl_sync(0xffffffffu, f, from),
+                                 __shfl_sync(0xffffffffu, n, from), __shfl_sync(0xffffffffu, up, from), lane, 0xffffffffu);
             }
         }
     } else {   // FP32 form: four cells per warp, eight lanes each (most cells are leaves of a few particles)
-        const int sub = lane >> 3, sl = lane & 7;
-        const unsigned gm = 0xFFu << (8 * sub);
-        const uint32_t nq = (total + 3) / 4;
         for (uint32_t q = warp; q < nq; q += nw) {
             const uint32_t c = 4 * q + sub;
             if (c >= total) continue;
@@ -1389,16 +1417,7 @@ __global__ void __launch_bounds__(256) k_mom_small(MomArgs a, unsigned long long
                 }
                 mom_climb<false, 8>(a, up, sl, gm);
             } else {
-                const uint32_t nch = a.search ? 1u : (n + BM_CH - 1) / BM_CH;
-                unsigned long long base = 0;
-                if (sl == 0) base = atomicAdd(nitems, (unsigned long long)nch);
-                base = __shfl_sync(gm, base, 0, 8);
-                if (base + nch > cap_items) {
-                    if (sl == 0) fail(st, HYBRID_ECAPACITY, where);
-                    continue;
-                }
-                if (sl == 0) bigbase[c] = (uint32_t)base;
-                for (uint32_t k = sl; k < nch; k += 8) items[base + k] = c;
+                list_big(c, n);
             }
         }
     }
@@ -1421,7 +1440,7 @@ __global__ void __launch_bounds__(256) k_bmax_big(MomArgs a, const unsigned long
         const uint32_t f0 = f + k * BM_CH, n0 = min(BM_CH, f + n - f0);
         if (F64) {
             const double c0 = a.cx[c], c1 = a.cy[c], c2 = a.cz[c];
-            const double dm = farthest_f64(a, f0, f0 + n0, c0, c1, c2, lane);
+            const double dm = farthest_f64<32>(a, f0, f0 + n0, c0, c1, c2, lane, 0xffffffffu);
             if (lane == 0) atomicMax(a.bmax64 + c, (unsigned long long)__double_as_longlong(dm));
         } else {
             const float4 A = a.nA[c], B = a.nB[c];

@@ -63,9 +63,10 @@ def test_fp64_forces_at_the_splits_edges(H, n, n_crit, same, eps):
 
 
 # the FP64 walk: every cell opened (more pending cells than the shared part of a warp's stack holds), none, leaves of
-# 1 particle and leaves of 32 and more (offsets by ballots and by scan)
+# 1 particle and leaves of 32 and more (offsets by ballots and by scan); leaves above 128 (moments by a whole warp)
 @pytest.mark.parametrize("n,theta,n_leaf,same", [(6000, 0.0, 1, 0), (3000, 1e-3, 16, 0), (2500, 0.6, 31, 0),
-                                                 (2500, 0.6, 64, 0), (2500, 5.0, 1, 0), (1500, 0.6, 16, 40)])
+                                                 (2500, 0.6, 64, 0), (2500, 5.0, 1, 0), (1500, 0.6, 16, 40),
+                                                 (2500, 0.6, 64, 129), (2500, 0.6, 300, 0)])
 def test_fp64_walk_at_its_edges(H, n, theta, n_leaf, same):
     st = state(n, same)
     kw = dict(eps=0.01, theta=theta, R1=0.04, R2=0.08, n_crit=64, n_leaf=n_leaf)
