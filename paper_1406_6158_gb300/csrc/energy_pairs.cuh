@@ -3,13 +3,13 @@
 // allocation-free call.
 //
 // The FP64 pipe bounds it (2 lanes per SM and clock), so each pair is taken
-// once (W = -G sum_{j < i} m_i m_j / sqrt(r^2 + eps^2)) with 13 FP64
-// instructions (seeded rsqrt, fp64_rsqrt.cuh). Work item = EN_ROW sinks (one
+// once (W = -G sum_{j < i} m_i m_j / sqrt(r^2 + eps^2)) with 7 FP64
+// instructions (rsqrt in fixed point, fp64_rsqrt.cuh). Work item = EN_ROW sinks (one
 // per thread) against EN_COL sources in shared memory, from the lower triangle
 // of the pair matrix; items go round robin to the blocks, which keep their
 // sums in registers and write one partial each, so the result does not depend
-// on timing. At n = 65536: 51.3 ms (44 ms at the full FP64 rate), against 239 ms
-// with every pair taken from both sides by sqrt and division.
+// on timing. At n = 65536: 27.0 ms (23.7 ms at the full FP64 rate), against 239
+// ms with every pair taken from both sides by sqrt and division.
 #pragma once
 
 #include <cstdint>

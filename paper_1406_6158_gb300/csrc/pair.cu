@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
 // (group, slice of at most F64_SINKS sinks), one block of F64_WARPS warps
 // each: a warp's lanes are lpc sinks (a power of two) times 32 / lpc copies,
 // and the unit's sources go round robin to the F64_WARPS x copies lanes of a
-// sink, straight from global memory (a source is 32 B against 4 sinks x 16
+// sink, straight from global memory (a source is 32 B against 4 sinks x 10
 // FP64 instructions of 16 clocks: loads are nowhere near the limit). The
 // partial sums are added in a fixed order (butterfly over the copies, then the
 // warps), and the split depends on the group alone, so a system's forces are
@@ -844,8 +844,10 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
 // kick-drift-kick step at N = 30011 from 30.3 to 4.8 ms (8 sinks a slice).
 // Slices of 4 sinks make twice the units, so the last ones leave fewer SMs
 // idle: far and near .374 + .244 -> .229 + .184 ms of that soft step, 2.51 +
-// .71 -> 2.36 + .68 ms at N = 30011. Slices of 2: .196 + .200 and 2.33 + .74;
-// 2 or 8 warps a unit: .302 + .220 and .208 + .204 (2.40 + .68, 2.36 + .74).
+// .71 -> 2.36 + .68 ms at N = 30011. With x^-3/2 and x^1/2 in fixed point
+// (fp64_rsqrt.cuh) .149 + .159 and 1.46 + .48 ms; slices of 2 then .128 + .173
+// and 1.44 + .55, of 8 .237 + .202 and 1.55 + .50, 8 warps a unit .134 + .182
+// and 1.45 + .56.
 // ---------------------------------------------------------------------------
 constexpr int F64_SINKS = 4, F64_WARPS = 4;
 

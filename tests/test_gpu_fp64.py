@@ -122,3 +122,24 @@ def test_energy_beyond_the_seeds_range(H):
         s = H.System(dict(st, x=st["x"] * f, y=st["y"] * f, z=st["z"] * f))
         W = H.Context(H.Params(eps=0.0)).hybrid_energy(s)[1]
         assert abs(W * f - W0) <= 1e-13 * abs(W0)
+
+
+# pairs alone, so that a force is one term: m / r^2 and the potential m / r, over binades, at both edges of [1, 4) and
+# beyond the fixed-point range. A term is rounded when r^2 is made (2 units of 2^-53: exact for one coordinate, r^2
+# itself 1), by x^-3/2 or x^-1/2 (2 units, by sqrt and division 9) and by products here and there (4): 2^-49 is 16
+@pytest.mark.parametrize("E", [-330, -321, -320, -319, -40, -1, 0, 1, 2, 33, 318, 319, 320, 330])
+def test_fp64_single_pairs(H, E):
+    rng = np.random.default_rng(E + 1000)
+    for r in list(2.0 ** rng.uniform(0, 1, 6)) + [1.0, np.nextafter(1.0, 2.0), np.nextafter(2.0, 1.0)]:
+        r = float(np.ldexp(r, E))
+        z = np.zeros(2)
+        st = dict(x=np.array([0.0, r]), y=z, z=z, vx=z, vy=z, vz=z, m=np.array([1.0, 1.5]))
+        ctx = H.Context(H.Params(eps=0.0, theta=0.5, R1=0.0, R2=0.0, precision=0))
+        s = H.System(st, precision=0)
+        T, W = ctx.hybrid_energy(s)
+        assert abs(W * r + 1.5) <= 1.5 * 2.0 ** -49
+        ctx.hybrid_build_tree(s)
+        ctx.hybrid_soft_force(s)
+        a = s.numpy()["ax_s"]
+        for v, m in ((a[np.argmin(s.numpy()["x"])], 1.5), (-a[np.argmax(s.numpy()["x"])], 1.0)):
+            assert abs(v * r * r - m) <= m * 2.0 ** -49
