@@ -1,4 +1,5 @@
-// fp64_rsqrt.cuh -- x^-1/2, x^-3/2 and x^1/2 of FP64 numbers in fixed point.
+// fp64_rsqrt.cuh -- r^2 + eps^2 and x^-1/2, x^-3/2 and x^1/2 of FP64 numbers in
+// fixed point.
 //
 // The FP64 pipe of this GPU retires 2 lanes per SM and clock (one warp
 // instruction per 16 clocks) against 64 and more of integer work, so a pair's
@@ -12,8 +13,9 @@
 // (against an exact root, over seeds off by 2 units either way), where the
 // FP64 step rounded 3 times.
 // Energy of 65536 particles: 51.3 ms with the FP64 step (13 instructions a
-// pair), 27.0 with this one (7). One kick-drift-kick step at N = 30011: far
-// forces 2.36 ms (16 instructions a pair), 1.46 (10).
+// pair), 27.0 with this one (7), 16.2 with r^2 + eps^2 in fixed point too (4).
+// One kick-drift-kick step at N = 30011: far forces 2.36 ms (16 instructions a
+// pair), 1.46 (10), 1.07 (7).
 #pragma once
 
 #include <cstdint>
@@ -28,23 +30,70 @@ struct RsqrtSeed {
     int k;
 };
 
-// For x between 2^-640 and 2^640, where none of the results leaves the range of normal numbers; false for the rest
-// (0, tiny, huge, negative, infinity, NaN), for which the callers below take sqrt and division.
-__device__ __forceinline__ bool rsqrt_seed(double x, RsqrtSeed &s)
+__device__ __forceinline__ RsqrtSeed seed_of(uint64_t A, int k)
 {
-    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    const int E = (int)hi >> 20;
-    if ((unsigned)(E - 383) > 1280u) return false;
-    const int p = (E + 1) & 1;
-    s.k = (E - 1023 - p) >> 1;
-    const float f = __uint_as_float(((127u + p) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29));
-    const uint32_t y = (uint32_t)(rsqrtf(f) * 16777216.0f);   // exact
-    s.A = ((uint64_t)((hi & 0xfffffu) | 0x100000u) << 32 | lo) << (10 + p);
+    RsqrtSeed s;
+    s.A = A;
+    s.k = k;
+    const uint32_t y = (uint32_t)(rsqrtf((float)(uint32_t)(A >> 32)) * 549755813888.0f);   // 2^39; exact
     s.Q = ((uint64_t)y * y) << 15;
     s.Y = y << 7;
     s.e = (int64_t)((1ull << 61) - __umul64hi(s.A, s.Q));
     const int e = (int)(s.e >> 20);
     s.e2 = (int64_t)e * e;
+    return s;
+}
+
+__device__ __forceinline__ uint64_t significand(double x)
+{
+    return (uint64_t)(((uint32_t)__double2hiint(x) & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x);
+}
+
+// Numbers between 2^-640 and 2^640 have a seed: none of their results leaves the range of normal numbers. For the rest
+// (0, tiny, huge, negative, infinity, NaN) the callers below take sqrt and division.
+__device__ __forceinline__ bool rsqrt_seed(double x, RsqrtSeed &s)
+{
+    const int E = __double2hiint(x) >> 20;
+    if ((unsigned)(E - 383) > 1280u) return false;
+    const int p = (E + 1) & 1;
+    s = seed_of(significand(x) << (10 + p), (E - 1023 - p) >> 1);
+    return true;
+}
+
+// eps^2 = S 2^-60 4^(E - 1023), S 2^-60 in [1, 4) (S = E = 0: none)
+struct Eps2Fixed {
+    uint64_t S;
+    int E;
+    double eps2;
+};
+
+__device__ __forceinline__ Eps2Fixed eps2_fixed(double eps2)
+{
+    const int E = __double2hiint(eps2) >> 20, p = (E + 1) & 1;
+    if (E == 0) return Eps2Fixed{0ull, 0, eps2};
+    return Eps2Fixed{significand(eps2) << (8 + p), ((E - 1023 - p) >> 1) + 1023, eps2};
+}
+
+// v^2 2^60 / 4^(Em - 1023), for v of exponent E <= Em (0, and what is below 2^-63 of the largest, give 0)
+__device__ __forceinline__ uint64_t square_fixed(double v, int E, int Em)
+{
+    const uint64_t m = (significand(v) << 11) >> min(Em - E, 63);
+    const uint32_t h = (uint32_t)(m >> 32), l = (uint32_t)m;
+    return ((uint64_t)h * h + (((uint64_t)h * l) >> 31)) >> 2;
+}
+
+// The seed of dx^2 + dy^2 + dz^2 + eps^2, summed in units of 2^-60 of the largest term's power of four (4 units of
+// truncation at most, 2^-58 of the sum, where three multiply-adds in FP64 round by up to 2^-53 each).
+__device__ __forceinline__ bool r2_seed(double dx, double dy, double dz, const Eps2Fixed &eps, RsqrtSeed &s)
+{
+    const int Ex = (__double2hiint(dx) >> 20) & 0x7ff, Ey = (__double2hiint(dy) >> 20) & 0x7ff,
+              Ez = (__double2hiint(dz) >> 20) & 0x7ff;
+    const int Em = max(max(Ex, Ey), max(Ez, eps.E));
+    if ((unsigned)(Em - 703) > 638u) return false;   // 2^-320 to 2^318
+    const uint64_t S = square_fixed(dx, Ex, Em) + square_fixed(dy, Ey, Em) + square_fixed(dz, Ez, Em) +
+                       (eps.S >> min(2 * (Em - eps.E), 63));   // in [2^60, 2^64)
+    const bool up = S >> 62;
+    s = seed_of(up ? S : S << 2, Em - (up ? 1022 : 1023));
     return true;
 }
 
@@ -66,11 +115,12 @@ __device__ __forceinline__ double from_fixed(uint64_t v, int E)
     return __longlong_as_double(((int64_t)(1023 + E) << 52) + (int64_t)((v - (1ull << 61) + 256) >> 9));
 }
 
-// m x^-3/2; 0 for x = 0 (a sink met by itself without softening)
-__device__ __forceinline__ double mass_over_r3(double m, double x)
+// m (r^2 + eps^2)^-3/2; 0 for r = eps = 0 (a sink met by itself without softening)
+__device__ __forceinline__ double mass_over_r3(double m, double dx, double dy, double dz, const Eps2Fixed &eps)
 {
     RsqrtSeed s;
-    if (!rsqrt_seed(x, s)) {
+    if (!r2_seed(dx, dy, dz, eps, s)) {
+        const double x = __fma_rn(dx, dx, __fma_rn(dy, dy, __fma_rn(dz, dz, eps.eps2)));
         const double ri = x > 0.0 ? 1.0 / sqrt(x) : 0.0;
         return m * ri * ri * ri;
     }
@@ -89,11 +139,13 @@ __device__ __forceinline__ double sqrt_seeded(double x)
     return from_fixed(__umul64hi(s.A, rsqrt_fixed(s) << 1), s.k);
 }
 
-// w + m x^-1/2
-__device__ __forceinline__ double add_mass_over_r(double w, double m, double x)
+// w + m (r^2 + eps^2)^-1/2
+__device__ __forceinline__ double add_mass_over_r(double w, double m, double dx, double dy, double dz,
+                                                  const Eps2Fixed &eps)
 {
     RsqrtSeed s;
-    if (!rsqrt_seed(x, s)) return w + m / sqrt(x);
+    if (!r2_seed(dx, dy, dz, eps, s))
+        return w + m / sqrt(__fma_rn(dx, dx, __fma_rn(dy, dy, __fma_rn(dz, dz, eps.eps2))));
     return __fma_rn(m, from_fixed(rsqrt_fixed(s), -1 - s.k), w);
 }
 

@@ -833,7 +833,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
 // (group, slice of at most F64_SINKS sinks), one block of F64_WARPS warps
 // each: a warp's lanes are lpc sinks (a power of two) times 32 / lpc copies,
 // and the unit's sources go round robin to the F64_WARPS x copies lanes of a
-// sink, straight from global memory (a source is 32 B against 4 sinks x 10
+// sink, straight from global memory (a source is 32 B against 4 sinks x 7
 // FP64 instructions of 16 clocks: loads are nowhere near the limit). The
 // partial sums are added in a fixed order (butterfly over the copies, then the
 // warps), and the split depends on the group alone, so a system's forces are
@@ -847,7 +847,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
 // .71 -> 2.36 + .68 ms at N = 30011. With x^-3/2 and x^1/2 in fixed point
 // (fp64_rsqrt.cuh) .149 + .159 and 1.46 + .48 ms; slices of 2 then .128 + .173
 // and 1.44 + .55, of 8 .237 + .202 and 1.55 + .50, 8 warps a unit .134 + .182
-// and 1.45 + .56.
+// and 1.45 + .56. With r^2 + eps^2 in fixed point too .123 + .155 and 1.07 + .46
+// ms; slices of 2 .096 + .171 and 1.05 + .53.
 // ---------------------------------------------------------------------------
 constexpr int F64_SINKS = 4, F64_WARPS = 4;
 
@@ -872,7 +873,8 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
         const int n = (int)(a.gfirst[g + 1] - first);
         if (slice * F64_SINKS >= n) continue;
         const SysParams &P = a.sp[a.gsys[g]];
-        const double eps2 = P.eps2, R2 = P.R2, R2sq = P.R2sq, invdR = P.invdR;
+        const Eps2Fixed eps = eps2_fixed(P.eps2);
+        const double R2 = P.R2, R2sq = P.R2sq, invdR = P.invdR;
         uint64_t c0 = 0, p0;
         int64_t Lc = 0, L;   // entries: cells [0, Lc), then particles [Lc, L)
         if (!NEAR) {
@@ -908,8 +910,7 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
                 i1 = index(e + 2 * step);
                 const double dx = __dsub_rn(q.x, s.x), dy = __dsub_rn(q.y, s.y), dz = __dsub_rn(q.z, s.z);
                 if (!NEAR) {
-                    const double r2 = __fma_rn(dx, dx, __fma_rn(dy, dy, __fma_rn(dz, dz, eps2)));
-                    const double f = mass_over_r3(q.w, r2);
+                    const double f = mass_over_r3(q.w, dx, dy, dz, eps);
                     ax = __fma_rn(f, dx, ax);
                     ay = __fma_rn(f, dy, ay);
                     az = __fma_rn(f, dz, az);
@@ -919,7 +920,7 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
                     const bool in = e < L && __double_as_longlong(r2u) < __double_as_longlong(R2sq);
                     const bool any_in = __any_sync(0xffffffffu, in);
                     if (!SOFT && !any_in) continue;
-                    const double f = mass_over_r3(q.w, __dadd_rn(r2u, eps2));
+                    const double f = mass_over_r3(q.w, dx, dy, dz, eps);
                     double K = 0.0;
                     if (any_in) {   // Eq. (10); 0 outside R2
                         const double r = sqrt_seeded(r2u);
