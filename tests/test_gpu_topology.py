@@ -63,3 +63,20 @@ def test_search_for_the_farthest_particle(H):  # noqa: F811
         st[d][402000:410000] = (np.arange(8000) // 20 ** k % 20) / 16.0 - 3.0
     st["x"][500000] = 60.0
     check_tree(*tree_of(H, st, n_leaf=16, n_crit=256, precision=1), 1)
+
+
+# group boxes: sub-warps of eight lanes, several groups after one another on large systems, and groups that take the
+# whole warp (more than 1024 particles: of one level-21 cell, or by n_crit). Exact: minimum and maximum of the members.
+@pytest.mark.parametrize("n,n_crit,same", [(1, 64, 0), (7, 1, 0), (1000, 5, 0), (5000, 64, 1024), (5000, 64, 1025),
+                                           (9000, 2000, 0), (400000, 1, 0)])
+def test_group_boxes_are_the_members_bounds(H, n, n_crit, same):  # noqa: F811
+    st = ics.plummer(n, 5)
+    for k in ("x", "y", "z"):
+        st[k][:same] = 0.125
+    ctx, s = H.Context(H.Params(n_crit=n_crit, n_leaf=min(16, n_crit))), H.System(st)
+    ctx.hybrid_build_tree(s)
+    t, o = ctx.tree(n), s.numpy()
+    first = t["first"][t["gnode"]]
+    for d, k in enumerate("xyz"):
+        assert np.array_equal(t["glo"][:, d], np.minimum.reduceat(o[k], first))
+        assert np.array_equal(t["ghi"][:, d], np.maximum.reduceat(o[k], first))
