@@ -596,7 +596,9 @@ void launch_walk(hybrid_ctx *c, int mode)
     // Near time per step with 64, 128, 256 entries: N = 2^12 0.071, 0.077, 0.083 ms; 2^17 0.292, 0.256, 0.266;
     // 2^20 1.51, 1.17, 1.09; with 512 and 1024: 2^24 35.6, 35.2.
     a.lch_near = c->N <= 1 << 15 ? 64 : (c->N <= 1 << 18 ? 128 : (c->N <= 1 << 20 ? 256 : 1024));
-    a.lch_far = small_job ? LCH_FAR_SMALL : LCH_FAR;
+    // Far time per step with 64, 128, 256 entries: N = 2^10 0.029, 0.033, 0.034 ms; 2^12 0.038, 0.045, 0.055; 2^14
+    // 0.061, 0.062, 0.065; 2^15 0.105, 0.099, 0.103; 2^17 0.391, 0.335, 0.319.
+    a.lch_far = c->N <= 1 << 14 ? 64 : (small_job ? LCH_FAR_SMALL : LCH_FAR);
     const int grid = c->walk_warps * 32 / WALK_THREADS;
     cudaEvent_t e0 = nullptr;
     prof_begin(c, PROF_WALK, &e0);
