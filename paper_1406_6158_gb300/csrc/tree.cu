@@ -1077,12 +1077,27 @@ __device__ __forceinline__ MomSums mom_range(const MomArgs &a, uint32_t f, uint3
     return r;
 }
 
-__device__ __forceinline__ void mom_store(const MomArgs &a, uint32_t c, const MomSums &r, double o0, double o1,
-                                          double o2)
+// (s0, s1, s2) / M, one quotient per lane: a division is some 8 dependent FP64 instructions, and they cost the same for
+// one lane as for all
+template <int G>
+__device__ __forceinline__ void div3(double s0, double s1, double s2, double M, int lane, unsigned gm, double &q0,
+                                     double &q1, double &q2)
 {
-    double c0, c1, c2, B2 = 0.0;
+    const double q = (lane == 1 ? s1 : (lane == 2 ? s2 : s0)) / M;
+    q0 = __shfl_sync(gm, q, 0, G);
+    q1 = __shfl_sync(gm, q, 1, G);
+    q2 = __shfl_sync(gm, q, 2, G);
+}
+
+// by all G lanes, which have the same sums; the centre to (c0, c1, c2)
+template <int G>
+__device__ __forceinline__ void mom_store(const MomArgs &a, uint32_t c, const MomSums &r, double o0, double o1,
+                                          double o2, int sl, unsigned gm, double &c0, double &c1, double &c2)
+{
+    double B2 = 0.0;
     if (r.M > 0.0) {
-        const double e0 = r.sx / r.M, e1 = r.sy / r.M, e2 = r.sz / r.M;
+        double e0, e1, e2;
+        div3<G>(r.sx, r.sy, r.sz, r.M, sl, gm, e0, e1, e2);
         c0 = o0 + e0;
         c1 = o1 + e1;
         c2 = o2 + e2;
@@ -1095,7 +1110,7 @@ __device__ __forceinline__ void mom_store(const MomArgs &a, uint32_t c, const Mo
         c1 = o[1] + 0.5 * sd;
         c2 = o[2] + 0.5 * sd;
     }
-    store_com(a, c, r.M, c0, c1, c2, B2);
+    if (sl == 0) store_com(a, c, r.M, c0, c1, c2, B2);
 }
 
 // sum over the first 8 of G lanes (the children of a cell), in all of them
@@ -1132,7 +1147,8 @@ __device__ void mom_combine_f64(const MomArgs &a, uint32_t c, uint32_t f, uint32
     const double Mt = sum8_d<G>(M, gm);   // the same in all lanes: the branch below has sums over them
     double c0, c1, c2, B2t = 0.0;
     if (Mt > 0.0) {
-        const double ex = sum8_d<G>(M * dx, gm) / Mt, ey = sum8_d<G>(M * dy, gm) / Mt, ez = sum8_d<G>(M * dz, gm) / Mt;
+        double ex, ey, ez;
+        div3<G>(sum8_d<G>(M * dx, gm), sum8_d<G>(M * dy, gm), sum8_d<G>(M * dz, gm), Mt, lane, gm, ex, ey, ez);
         c0 = rx + ex;
         c1 = ry + ey;
         c2 = rz + ez;
@@ -1335,16 +1351,8 @@ __device__ __forceinline__ void mom_cell_f64(const MomArgs &a, uint32_t c, uint3
 {
     const double o0 = a.x[f], o1 = a.y[f], o2 = a.z[f];
     const MomSums r = mom_range<G>(a, f, n, o0, o1, o2, sl, gm);
-    double c0 = 0.0, c1 = 0.0, c2 = 0.0;
-    if (sl == 0) {
-        mom_store(a, c, r, o0, o1, o2);
-        c0 = a.cx[c];
-        c1 = a.cy[c];
-        c2 = a.cz[c];
-    }
-    c0 = __shfl_sync(gm, c0, 0, G);
-    c1 = __shfl_sync(gm, c1, 0, G);
-    c2 = __shfl_sync(gm, c2, 0, G);
+    double c0, c1, c2;
+    mom_store<G>(a, c, r, o0, o1, o2, sl, gm, c0, c1, c2);
     mom_climb<true, G>(a, up, sl, gm);   // others wait for this
     const double dm = farthest_f64<G>(a, f, f + n, c0, c1, c2, sl, gm);
     if (sl == 0) a.bmax64[c] = (unsigned long long)__double_as_longlong(dm);
