@@ -152,11 +152,11 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
     uint32_t *sstk = sstk_all[threadIdx.x >> 5];  // top part of the stack
     const bool want_soft = a.mode & 1, want_hard = (a.mode >> 1) & 1;
 
-    for (;;) {
-        unsigned long long gg = 0;
-        if (lane == 0) gg = atomicAdd(a.counter, 1ull);
-        const int64_t g = (int64_t)__shfl_sync(0xffffffffu, gg, 0);
-        if (g >= ng) break;
+    // A warp's first group by its place in the grid, the later ones in turn. Taken in turn from the start, neighbouring
+    // groups, which are heavy together, go to the four warps of a block and their SM's FP64 pipe: walks of one step at
+    // N = 30011 0.497 -> 0.320 ms, of 5 at N = 4096 0.319 -> 0.288.
+    int64_t g = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+    while (g < ng) {
         const uint32_t s = a.gsys[g];
         const bool has_hard = a.sp[s].has_hard != 0;
         const bool wh0 = want_hard && has_hard;
@@ -288,6 +288,9 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
             a.cnt[ng + g] = np;
             a.cnt[2 * ng + g] = nh;
         }
+        unsigned long long gg = 0;
+        if (lane == 0) gg = atomicAdd(a.counter, 1ull);
+        g = (int64_t)__shfl_sync(0xffffffffu, gg, 0) + (int64_t)(WALK_THREADS / 32) * gridDim.x;
     }
 }
 
