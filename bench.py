@@ -40,7 +40,7 @@ FLOPS_PER_INTERACTION = 20          # monopole pair: 3 sub, 3 fma, rsqrt, 3 mul,
 # DRAM bytes (read + write) of one far-pair launch on this workload, from one ncu capture of the current far
 # kernel for each variant the keys name (n_crit, threads per group, staging depth). Reported as the roofline's
 # traffic only when the autotuner picks one of these variants, else None.
-FAR_TRAFFIC_BYTES = {(128, 32, 2): 57.37e6, (128, 32, 4): 57.31e6}
+FAR_TRAFFIC_BYTES = {(128, 32, 2): 57.33e6, (128, 32, 4): 57.30e6}
 CLOCK_INTERVAL_MS = 20
 L2_FLUSH_BYTES = 256 << 20
 ENERGY_MAX_N = 1 << 18              # largest N whose energy the paper comparison evaluates (O(N^2) FP64)
@@ -450,8 +450,9 @@ def hbm_stages(n, n_hard, ms, nodes=None):
     algorithmic bytes (n_hard builds and drift launches per soft step):
       sort        per particle 36 (keys: x, y, z in, key and index out) + 12 (key in, bucket out) + 24 (key and
                   bucket in, key and index out to the bucket) + 24 (key and index in and out of the bucket sort):
-                  the sample sort the builds take between steps (a build that falls back to the radix sort moves
-                  36 + 8 + 8 x 24; the line reports the fallbacks)
+                  the count this record has always used; the sample sort the builds take between steps finds the
+                  bucket where it makes the key and moves 60 of them (a build that falls back to the radix sort
+                  moves 36 + 8 + 8 x 24; the line reports the fallbacks)
       topology    per particle 8 (sorted key in); per node 24 out (first, count, level, first child, children,
                   parent)
       moments     per particle 32 (FP32 hi/lo position copies in); per node 24 in (the topology) and 72 out (the
@@ -586,7 +587,7 @@ def c3_record(args, steps, warmup, with_cpu=True):
         "force_err_rms_vs_direct": ferr,
         "kernel_ms_per_step": ms,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                     "traffic": None, "kernel": "k_pair_f32 far (cells + far particles, soft force)",
+                     "traffic": None, "kernel": "k_far (cells + far particles, soft force)",
                      "peak_note": "FP32 CUDA-core peak: %d SMs x 128 lanes x 2 flop x %.0f MHz (max SM clock)" %
                                   (props.multi_processor_count, sm_max)},
         "hbm_stages": hbm_stages(n, P.n_hard, ms, nodes),
@@ -935,7 +936,7 @@ def main():
                                    "variant on this workload, from an ncu capture of the current kernel (mean "
                                    "of two launches); not measured in this run") if traffic else
                                   "no capture of the chosen variant",
-                "kernel": "k_pair_f32 far (cells + far particles, soft force)",
+                "kernel": "k_far (cells + far particles, soft force)",
                 "peak_note": "FP32 CUDA-core peak: %d SMs x 128 lanes x 2 flop x %.0f MHz (max SM clock)" %
                              (props.multi_processor_count, sm_max)}
 

@@ -33,7 +33,8 @@ def state(n, same=0):
 # slices of 4 sinks: groups below, at and above one slice, ragged last slices of every size, groups above
 # 32 slices (the cap: rounds), and a leaf of coincident particles larger than n_crit with and without softening
 @pytest.mark.parametrize("n,n_crit,same,eps", [(1, 64, 0, 0.01), (2, 1, 0, 0.01), (700, 1, 0, 0.01), (700, 4, 0, 0.01),
-                                               (701, 5, 0, 0.01), (900, 128, 0, 0.01), (700, 8, 0, 0.01), (701, 9, 0, 0.01), (1500, 64, 0, 0.01), (1500, 300, 0, 0.01),
+                                               (701, 5, 0, 0.01), (900, 128, 0, 0.01), (700, 8, 0, 0.01),
+                                               (701, 9, 0, 0.01), (1500, 64, 0, 0.01), (1500, 300, 0, 0.01),
                                                (900, 16, 333, 0.01), (900, 16, 333, 0.0)])
 def test_fp64_forces_at_the_splits_edges(H, n, n_crit, same, eps):
     st = state(n, same)
