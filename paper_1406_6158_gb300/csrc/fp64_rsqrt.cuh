@@ -15,7 +15,8 @@
 // Energy of 65536 particles: 51.3 ms with the FP64 step (13 instructions a
 // pair), 27.0 with this one (7), 16.2 with r^2 + eps^2 in fixed point too (4).
 // One kick-drift-kick step at N = 30011: far forces 2.36 ms (16 instructions a
-// pair), 1.46 (10), 1.07 (7).
+// pair), 1.46 (10), 1.07 (7); near forces 0.68, 0.48, 0.46, and 0.37 ms with the
+// K argument's r^2 and its comparison with R2^2 in fixed point too.
 #pragma once
 
 #include <cstdint>
@@ -49,17 +50,6 @@ __device__ __forceinline__ uint64_t significand(double x)
     return (uint64_t)(((uint32_t)__double2hiint(x) & 0xfffffu) | 0x100000u) << 32 | (uint32_t)__double2loint(x);
 }
 
-// Numbers between 2^-640 and 2^640 have a seed: none of their results leaves the range of normal numbers. For the rest
-// (0, tiny, huge, negative, infinity, NaN) the callers below take sqrt and division.
-__device__ __forceinline__ bool rsqrt_seed(double x, RsqrtSeed &s)
-{
-    const int E = __double2hiint(x) >> 20;
-    if ((unsigned)(E - 383) > 1280u) return false;
-    const int p = (E + 1) & 1;
-    s = seed_of(significand(x) << (10 + p), (E - 1023 - p) >> 1);
-    return true;
-}
-
 // eps^2 = S 2^-60 4^(E - 1023), S 2^-60 in [1, 4) (S = E = 0: none)
 struct Eps2Fixed {
     uint64_t S;
@@ -82,18 +72,40 @@ __device__ __forceinline__ uint64_t square_fixed(double v, int E, int Em)
     return ((uint64_t)h * h + (((uint64_t)h * l) >> 31)) >> 2;
 }
 
-// The seed of dx^2 + dy^2 + dz^2 + eps^2, summed in units of 2^-60 of the largest term's power of four (4 units of
-// truncation at most, 2^-58 of the sum, where three multiply-adds in FP64 round by up to 2^-53 each).
-__device__ __forceinline__ bool r2_seed(double dx, double dy, double dz, const Eps2Fixed &eps, RsqrtSeed &s)
+// A number as A 2^-62 4^k, A 2^-62 in [1, 4); larger numbers have a larger k, or the same k and a larger A.
+struct Fixed {
+    uint64_t A;
+    int k;
+};
+
+// x >= 0, below everything for zero and subnormals, above everything for infinity
+__device__ __forceinline__ Fixed to_fixed(double x)
+{
+    const int E = __double2hiint(x) >> 20, p = (E + 1) & 1;
+    if (E == 0) return Fixed{0ull, -2000};
+    return Fixed{significand(x) << (10 + p), (E - 1023 - p) >> 1};
+}
+
+// dx^2 + dy^2 + dz^2 + eps^2, summed in units of 2^-60 of the largest term's power of four (4 units of truncation at
+// most, 2^-58 of the sum, where three multiply-adds in FP64 round by up to 2^-53 each). False outside 2^-640 to 2^640,
+// where a result could leave the range of normal numbers (and for NaN and all zero): the callers take sqrt and division.
+__device__ __forceinline__ bool r2_fixed(double dx, double dy, double dz, const Eps2Fixed &eps, Fixed &r2)
 {
     const int Ex = (__double2hiint(dx) >> 20) & 0x7ff, Ey = (__double2hiint(dy) >> 20) & 0x7ff,
               Ez = (__double2hiint(dz) >> 20) & 0x7ff;
     const int Em = max(max(Ex, Ey), max(Ez, eps.E));
-    if ((unsigned)(Em - 703) > 638u) return false;   // 2^-320 to 2^318
+    if ((unsigned)(Em - 703) > 638u) return false;   // the largest from 2^-320 to below 2^319
     const uint64_t S = square_fixed(dx, Ex, Em) + square_fixed(dy, Ey, Em) + square_fixed(dz, Ez, Em) +
                        (eps.S >> min(2 * (Em - eps.E), 63));   // in [2^60, 2^64)
     const bool up = S >> 62;
-    s = seed_of(up ? S : S << 2, Em - (up ? 1022 : 1023));
+    r2 = Fixed{up ? S : S << 2, Em - (up ? 1022 : 1023)};
+    return true;
+}
+__device__ __forceinline__ bool r2_seed(double dx, double dy, double dz, const Eps2Fixed &eps, RsqrtSeed &s)
+{
+    Fixed r2;
+    if (!r2_fixed(dx, dy, dz, eps, r2)) return false;
+    s = seed_of(r2.A, r2.k);
     return true;
 }
 
@@ -131,11 +143,10 @@ __device__ __forceinline__ double mass_over_r3(double m, double dx, double dy, d
     return __dmul_rn(m, __longlong_as_double(((int64_t)(1023 - z - 3 * s.k) << 52) + b));
 }
 
-// sqrt(x) = x x^-1/2 for x >= 0
-__device__ __forceinline__ double sqrt_seeded(double x)
+// sqrt(x) = x x^-1/2
+__device__ __forceinline__ double sqrt_fixed(const Fixed &x)
 {
-    RsqrtSeed s;
-    if (!rsqrt_seed(x, s)) return x == 0.0 ? 0.0 : sqrt(x);
+    const RsqrtSeed s = seed_of(x.A, x.k);
     return from_fixed(__umul64hi(s.A, rsqrt_fixed(s) << 1), s.k);
 }
 

@@ -848,7 +848,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
 // (fp64_rsqrt.cuh) .149 + .159 and 1.46 + .48 ms; slices of 2 then .128 + .173
 // and 1.44 + .55, of 8 .237 + .202 and 1.55 + .50, 8 warps a unit .134 + .182
 // and 1.45 + .56. With r^2 + eps^2 in fixed point too .123 + .155 and 1.07 + .46
-// ms; slices of 2 .096 + .171 and 1.05 + .53.
+// ms; slices of 2 .096 + .171 and 1.05 + .53. With the near pairs' r^2 too .121 +
+// .132 and 1.07 + .366.
 // ---------------------------------------------------------------------------
 constexpr int F64_SINKS = 4, F64_WARPS = 4;
 
@@ -875,6 +876,7 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
         const SysParams &P = a.sp[a.gsys[g]];
         const Eps2Fixed eps = eps2_fixed(P.eps2);
         const double R2 = P.R2, R2sq = P.R2sq, invdR = P.invdR;
+        const Fixed R2f = to_fixed(R2sq);
         uint64_t c0 = 0, p0;
         int64_t Lc = 0, L;   // entries: cells [0, Lc), then particles [Lc, L)
         if (!NEAR) {
@@ -915,15 +917,23 @@ __global__ void __launch_bounds__(32 * F64_WARPS) k_pair_f64(PairArgs a, int sli
                     ay = __fma_rn(f, dy, ay);
                     az = __fma_rn(f, dz, az);
                 } else {
-                    const double r2u = __fma_rn(dx, dx, __fma_rn(dy, dy, __dmul_rn(dz, dz)));
-                    // r2u < R2^2, compared as integers (both are >= 0; NaN compares above)
-                    const bool in = e < L && __double_as_longlong(r2u) < __double_as_longlong(R2sq);
+                    Fixed r2f;
+                    double r2u = 0.0;
+                    const bool fixed = r2_fixed(dx, dy, dz, Eps2Fixed{0ull, 0, 0.0}, r2f);
+                    bool in;   // r^2 < R2^2
+                    if (fixed) {
+                        in = r2f.k < R2f.k || (r2f.k == R2f.k && r2f.A < R2f.A);
+                    } else {   // compared as integers (both are >= 0; NaN compares above)
+                        r2u = __fma_rn(dx, dx, __fma_rn(dy, dy, __dmul_rn(dz, dz)));
+                        in = __double_as_longlong(r2u) < __double_as_longlong(R2sq);
+                    }
+                    in = in && e < L;
                     const bool any_in = __any_sync(0xffffffffu, in);
                     if (!SOFT && !any_in) continue;
                     const double f = mass_over_r3(q.w, dx, dy, dz, eps);
                     double K = 0.0;
                     if (any_in) {   // Eq. (10); 0 outside R2
-                        const double r = sqrt_seeded(r2u);
+                        const double r = fixed ? sqrt_fixed(r2f) : (r2u == 0.0 ? 0.0 : sqrt(r2u));
                         const double Y = __dmul_rn(__dsub_rn(R2, r), invdR);
                         const double Y2 = __dmul_rn(Y, Y);
                         K = __dmul_rn(__dmul_rn(Y2, __dmul_rn(Y2, Y2)),
