@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(256) k_kick_drift(int64_t N, StatePtrs w, cons
     if (!BOX && skip) return;
     Bounds bounds;
     if (BOX) begin_sort(box);
-    bool soft = false, hard = false;
+    bool soft = false, hard = false, tripped = false;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         soft = soft || (k < ks.n && ks.which[k] == 0);
@@ -204,13 +204,27 @@ __global__ void __launch_bounds__(256) k_kick_drift(int64_t N, StatePtrs w, cons
                 // rounded up by a few units in the last place: a bound, not an estimate
                 const float moved = w.disp[i] + sqrtf(d0 * d0 + d1 * d1 + d2 * d2) * 1.000001f + 1e-30f;
                 w.disp[i] = moved;
-                if (moved > P.half_skinf) fail(st, ST_SKIN, ks.where);
+                tripped = tripped || moved > P.half_skinf;
             }
         }
     }
     if (BOX) {
         bounds.reduce_block(box, 0);
         finish_boxes(box);
+    } else if (ks.resplit) {
+        // The sequence resumes after this drift, which therefore has to be whole: a block that started after the
+        // status was set would return at the top and lose its particles' kicks and drift. So the blocks only note
+        // that a particle went too far, and the last one to get here (a ticket, no waiting) records it.
+        const bool any = __syncthreads_or(tripped);
+        if (threadIdx.x == 0) {
+            if (any) atomicExch(box.trip, 1u);
+            __threadfence();   // this block's note is visible before its ticket
+            if (atomicAdd(box.ticket, 1u) == gridDim.x - 1) {
+                __threadfence();
+                if (atomicExch(box.trip, 0u)) fail(st, ST_SKIN, ks.where);
+                *box.ticket = 0u;
+            }
+        }
     }
 }
 

@@ -26,6 +26,7 @@ struct BoxArgs {
     const uint64_t *key;               // the last build's sorted keys
     uint32_t *cnt, *flag;
     unsigned *ticket;                  // 0 between launches
+    unsigned *trip;                    // 0 between launches: a particle of a list-reusing drift has moved too far
     SysBox *box;
 };
 
@@ -42,6 +43,7 @@ inline BoxArgs box_args(hybrid_ctx *c)
     b.cnt = (uint32_t *)c->ss_cnt.p;
     b.flag = (uint32_t *)c->ss_flag.p;
     b.ticket = (unsigned *)((unsigned long long *)c->counter.p + 14);
+    b.trip = b.ticket + 1;
     b.box = (SysBox *)c->box.p;
     return b;
 }
