@@ -1084,7 +1084,8 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
     if (c->p.precision == 0) {
         // a unit for each slice of F64_SINKS sinks a group of n_crit can have (32 slices at most: larger groups take
         // rounds); units past a group's size are passed over
-        const int slices = std::min(32, (c->p.n_crit + F64_SINKS - 1) / F64_SINKS);
+        // (no sum that overflows: n_crit may be anything up to 2^31 - 1, and 0 or fewer slices would never end)
+        const int slices = std::min(32, (c->p.n_crit - 1) / F64_SINKS + 1);
         const int grid = c->nsm * 16;
         if (!near) k_pair_f64<false, true, false><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
         else if (a.want_soft && a.want_hard) k_pair_f64<true, true, true><<<grid, 32 * F64_WARPS, 0, c->st>>>(a, slices);
