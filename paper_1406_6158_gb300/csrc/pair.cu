@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 0) k_far(PairArgs a)
 // 1.60 -> 1.09, 2^24 40.2 -> 35.2 ms.
 // ---------------------------------------------------------------------------
 constexpr int NEAR_TILE = PAIR_THREADS;
-constexpr float FAR_AWAY = 1e18f;   // padding sources: far beyond any R2, r^2 still finite
+constexpr float FAR_AWAY = 1e18f;   // padding sources: r^2 is finite; massless, so R2 may be larger (SI or cgs units)
 
 struct NearTile {
     float4 hi[NEAR_TILE];   // rebased hi parts and mass (differences with the sinks' hi parts are exact)
@@ -569,7 +569,7 @@ struct NearTile {
 
 // the sources a distance step runs over, two by two
 struct NearPacked {
-    float x[NEAR_TILE + 2], y[NEAR_TILE + 2], z[NEAR_TILE + 2];
+    float x[NEAR_TILE], y[NEAR_TILE], z[NEAR_TILE];
     uint8_t j[NEAR_TILE];   // their entries in the tile
 };
 
@@ -771,7 +771,6 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
                         nin += __popc(km);
                     }
                     if (nin == 0) continue;
-                    if (lane == 0) p.x[nin] = FAR_AWAY;   // the last pair's other half, if any
                     __syncwarp();
                     const int rounds = (nin + 1) / 2;
                     for (int m0 = 0; m0 < rounds; m0 += 16) {   // 16 source pairs: one mask word
@@ -787,6 +786,8 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
                             mark |= ra < H.R2sq ? bit : 0u;
                             mark |= rb < H.R2sq ? 2u * bit : 0u;
                         }
+                        // with an odd number of sources the last pair's other half is none of them
+                        if (2 * m1 > nin) mark &= ~(2u << 2 * (m1 - 1 - m0));
                         while (__any_sync(0xffffffffu, mark != 0u)) {
                             const bool on = mark != 0u;
                             const int j = on ? p.j[2 * m0 + __ffs(mark) - 1] : 0;
