@@ -240,9 +240,11 @@ struct hybrid_ctx {
     int64_t sort_fallbacks = 0;
     bool tree_valid = false, have_soft = false, have_hard = false;
     // reused neighbour lists (skin > 0): the lists of the last walk still hold for the working state of the
-    // batch with this signature (set at the end of a step, cleared by anything else that builds or walks)
+    // batch with this signature and in these buffers (set at the end of a step, cleared by anything else that builds
+    // or walks)
     bool lists_fresh = false;
     uint64_t lists_sig = 0;
+    int64_t lists_gen = 0;
 
     // capacities
     int64_t capN = 0, capS = 0, capChunks = 0, capNodes = 0, capGroups = 0, capList = 0, capStack = 0;

@@ -963,13 +963,15 @@ hybrid_status hybrid_step_batched(hybrid_ctx *c, hybrid_system *sys, int n_sys, 
         mixs((uint64_t)sys[s].n);
         mixs((uint64_t)(uintptr_t)sys[s].x);
     }
-    const bool lists_ok = valid && c->lists_fresh && c->lists_sig == sig;
+    // (and no buffer has been allocated anew since, as hybrid_energy of a larger system does)
+    const bool lists_ok = valid && c->lists_fresh && c->lists_sig == sig && c->lists_gen == c->gen;
     c->lists_fresh = false;
     launch_copy_in(c, (const SysIO *)c->io_dev.p, valid);
     r = run_ops(c, step_ops(c, n_soft_steps, valid, lists_ok), true);
     if (r != HYBRID_OK) return r;
     c->lists_fresh = c->p.skin > 0.0;
     c->lists_sig = sig;
+    c->lists_gen = c->gen;
     for (int k = 0; k < n_sys; ++k) sys[k].forces_valid = 1;
     c->tree_valid = (n_sys == 1);
     c->have_soft = c->have_hard = true;

@@ -41,3 +41,28 @@ def test_exceeded_skin_leaves_the_drift_whole(H, n, graphs):  # noqa: F811
     d = np.sqrt(sum((a[k] - b[k]) ** 2 for k in "xyz"))
     fast = v > 0.05
     assert np.all(d[fast] <= 0.01 * v[fast] * P.dt_soft / P.n_hard)
+
+
+@pytest.mark.parametrize("graphs", [False, True], ids=["eager", "graphs"])
+@pytest.mark.parametrize("other", [100, 3000, 250000])
+def test_energy_of_another_system_between_steps(H, graphs, other):  # noqa: F811
+    # the energy of a larger system makes the context's buffers anew: the lists of the last step are gone then, and the
+    # next step must not take them up. Positions follow the steps without it as far as lists in another order may
+    # differ (FP32 forces: 1e-8, as in the comparison of reused lists with the oracle)
+    n = 3000
+    st, big = ics.plummer(n, 9), ics.plummer(other, 10)
+    res = []
+    for between in (False, True):
+        P = H.Params(eps=1 / 64, theta=0.0, R1=4 / 64, R2=8 / 64, dt_soft=1 / 128, n_hard=4, skin=0.05)
+        ctx = H.Context(P, torch.cuda.Stream() if graphs else None)
+        s, o = H.System(st, precision=1), H.System(big, precision=1)
+        torch.cuda.synchronize()
+        for _ in range(3):
+            ctx.hybrid_step(s, 1)
+            if between:
+                ctx.hybrid_energy(o)
+        out = s.numpy()
+        res.append({k: out[k][np.argsort(out["id"])] for k in H.System.FIELDS})
+        ctx.close()
+    for k in "xyz":
+        assert np.max(np.abs(res[0][k] - res[1][k])) <= 1e-8, k
