@@ -137,13 +137,17 @@ constexpr int32_t ST_SORT = 101;
 // build's keys at every SS_BUCKET-th position; a bucket of at most SS_CAP keys
 // (over twice the target: only the particles that crossed a coarse cell boundary
 // since move between buckets) is sorted by one warp: 8 keys a lane for up to
-// 256 keys, which a bucket of 224 seldom outgrows, else 16.
+// 256 keys, which a bucket of 224 seldom outgrows, else 16. A bucket's region
+// holds SS_CAP entries, or as many as the system has particles (12 B each: a
+// region of SS_CAP for every system would be 6 KiB for one of a few particles).
 constexpr int SS_BUCKET = 224;
 constexpr int SS_CAP = 512;
 constexpr int SS_SUM_MAX = 4096;   // buckets up to which the sorting blocks add up the counts themselves
 struct SSys {
     int32_t nb;      // buckets of the system
     int32_t bbase;   // index of its first bucket
+    int64_t rbase;   // first entry of its buckets' regions
+    int32_t rcap;    // entries of a bucket's region
 };
 
 // Device status block: first failure wins (atomicCAS on code).
@@ -236,6 +240,7 @@ struct hybrid_ctx {
     // with the radix sort after a bucket overflowed
     std::vector<hy::SSys> h_ss;
     int nbk = 0;
+    int64_t nreg = 0;   // entries of all regions
     bool sort_fallback = false;
     int64_t sort_fallbacks = 0;
     bool tree_valid = false, have_soft = false, have_hard = false;
@@ -256,8 +261,8 @@ struct hybrid_ctx {
     hy::Buf phi, plo, pd;                  // float4 hi/lo (precision 1), double4_32a (precision 0)
     hy::Buf disp;                          // float: bound of the distance moved since the last build (skin > 0)
     hy::Buf keys[2], vals[2], hist, blocksum;
-    hy::Buf ss_sys, ss_cnt, ss_rk, ss_rv, ss_flag;   // sample sort: counts and regions of the buckets
-    int64_t capBk = 0;
+    hy::Buf ss_sys, ss_cnt, ss_bsys, ss_rk, ss_rv, ss_flag;   // sample sort: counts, systems and regions of the buckets
+    int64_t capBk = 0, capReg = 0;
     hy::Buf off_dev, sp_dev, chunks_dev, boxmin, boxmax, box, sysroot;
     hy::Buf status;
     // tree

@@ -231,9 +231,12 @@ bool reserve(hybrid_ctx *c)
     ok = ok && ensure(c, c->ss_sys, (size_t)S * sizeof(SSys)) && ensure(c, c->ss_flag, 256);
     if (c->nbk > c->capBk) {
         const size_t nb = (size_t)c->nbk;
-        ok = ok && ensure(c, c->ss_cnt, (nb + 1) * 4) && ensure(c, c->ss_rk, nb * SS_CAP * 8) &&
-             ensure(c, c->ss_rv, nb * SS_CAP * 4);
+        ok = ok && ensure(c, c->ss_cnt, (nb + 1) * 4) && ensure(c, c->ss_bsys, nb * 4);
         if (ok) c->capBk = c->nbk;
+    }
+    if (c->nreg > c->capReg) {
+        ok = ok && ensure(c, c->ss_rk, (size_t)c->nreg * 8) && ensure(c, c->ss_rv, (size_t)c->nreg * 4);
+        if (ok) c->capReg = c->nreg;
     }
     // radix sort scratch: 64 tickets, digit counts [S][8][256], look-back words [8][chunks][256]
     ok = ok && ensure(c, c->hist, ((size_t)64 + (size_t)2048 * (S + c->nchunks)) * 4);
@@ -328,12 +331,16 @@ hybrid_status setup_batch(hybrid_ctx *c, const hybrid_system *sys, int S, bool n
     // sample sort layout: about SS_BUCKET keys per bucket
     c->h_ss.resize(S);
     c->nbk = 0;
+    c->nreg = 0;
     for (int s = 0; s < S; ++s) {
         const int64_t n = c->h_off[s + 1] - c->h_off[s];
         SSys &y = c->h_ss[s];
         y.nb = (int32_t)((n + SS_BUCKET - 1) / SS_BUCKET);
         y.bbase = c->nbk;
+        y.rcap = (int32_t)std::min<int64_t>(SS_CAP, n);
+        y.rbase = c->nreg;
         c->nbk += y.nb;
+        c->nreg += (int64_t)y.nb * y.rcap;
     }
     if (!reserve(c)) return HYBRID_ENOMEM;
     c->h_io.resize(S);
@@ -846,7 +853,7 @@ hybrid_status hybrid_destroy(hybrid_ctx *c)
     else cudaDeviceSynchronize();
     Buf *all[] = {&c->id, &c->ida, &c->orig, &c->origa, &c->psys, &c->phi, &c->plo, &c->pd, &c->disp, &c->keys[0], &c->keys[1],
                   &c->vals[0], &c->vals[1], &c->hist, &c->blocksum, &c->off_dev, &c->sp_dev, &c->chunks_dev,
-                  &c->ss_sys, &c->ss_cnt, &c->ss_rk, &c->ss_rv, &c->ss_flag,
+                  &c->ss_sys, &c->ss_cnt, &c->ss_bsys, &c->ss_rk, &c->ss_rv, &c->ss_flag,
                   &c->boxmin, &c->boxmax, &c->box, &c->sysroot, &c->status, &c->lvl, &c->nfirst, &c->nend,
                   &c->nchild, &c->nchend, &c->nparent, &c->nlevel, &c->ndone, &c->cells, &c->ccnt, &c->nM, &c->ncx,
                   &c->ncy, &c->ncz, &c->nB2, &c->nbmax, &c->nA, &c->nB, &c->ncrit, &c->ntopo, &c->nD, &c->nrb,

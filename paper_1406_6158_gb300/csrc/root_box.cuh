@@ -24,7 +24,7 @@ struct BoxArgs {
     const int64_t *off;
     const SSys *ss;
     const uint64_t *key;               // the last build's sorted keys
-    uint32_t *cnt, *flag;
+    uint32_t *cnt, *bsys, *flag;
     unsigned *ticket;                  // 0 between launches
     unsigned *trip;                    // 0 between launches: a particle of a list-reusing drift has moved too far
     SysBox *box;
@@ -41,6 +41,7 @@ inline BoxArgs box_args(hybrid_ctx *c)
     b.ss = (const SSys *)c->ss_sys.p;
     b.key = (const uint64_t *)c->keys[0].p;
     b.cnt = (uint32_t *)c->ss_cnt.p;
+    b.bsys = (uint32_t *)c->ss_bsys.p;
     b.flag = (uint32_t *)c->ss_flag.p;
     b.ticket = (unsigned *)((unsigned long long *)c->counter.p + 14);
     b.trip = b.ticket + 1;
@@ -48,8 +49,8 @@ inline BoxArgs box_args(hybrid_ctx *c)
     return b;
 }
 
-// The sample sort's bucket counts cleared, its overflow flag reset, and whether its splitters (the last build's keys
-// at every SS_BUCKET-th position) are in order. Every thread of the grid.
+// The sample sort's bucket counts cleared, the buckets' systems (of a batch), its overflow flag reset, and whether its
+// splitters (the last build's keys at every SS_BUCKET-th position) are in order. Every thread of the grid.
 __device__ __forceinline__ void begin_sort(const BoxArgs &a)
 {
     const int gtid = blockIdx.x * blockDim.x + threadIdx.x;
@@ -67,6 +68,7 @@ __device__ __forceinline__ void begin_sort(const BoxArgs &a)
                 if (a.ss[mid].bbase <= b) s = mid;
                 else hi = mid;
             }
+            a.bsys[b] = (uint32_t)s;
         }
         const SSys y = a.ss[s];
         const int j = b - y.bbase;

@@ -315,7 +315,7 @@ __global__ void __launch_bounds__(256) k_onesweep(const uint64_t *__restrict__ k
 // the keys into nb buckets: particle i is tried in the bucket of its position
 // (most are still there: two comparisons against keys a whole warp shares),
 // then in buckets ever farther away, and its key and index are appended to the
-// bucket's region of SS_CAP entries. One warp then sorts each bucket in
+// bucket's region (SS_CAP entries, fewer for a small system). One warp then sorts each bucket in
 // registers (bitonic, by composite) and writes it to its place, the sum of the
 // earlier buckets' counts. Keys end sorted in keys[0] with their source
 // positions in vals[0], exactly as the radix sort leaves them. Splitters out
@@ -350,8 +350,9 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < N; i0 += stride) {
         const int64_t i = i0 + threadIdx.x;
-        uint32_t b = ~0u;
+        uint32_t b = ~0u, cap = 0u;
         uint64_t k = 0ull;
+        int64_t region = 0;
         if (i < N) {
             const int sy = S == 1 ? 0 : psys[i];
             const SysBox &bx = box[sy];
@@ -393,21 +394,23 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
                 else hi = mid;
             }
             b = (uint32_t)(yy.bbase + lo);
+            cap = (uint32_t)yy.rcap;
+            region = yy.rbase + (int64_t)lo * yy.rcap;
         }
         const unsigned peers = __match_any_sync(0xffffffffu, b);
         const int leader = __ffs(peers) - 1;
         uint32_t base = 0;
         if (b != ~0u && lane == leader) {
             base = atomicAdd(cnt + b, (uint32_t)__popc(peers));
-            if (base + (uint32_t)__popc(peers) > (uint32_t)SS_CAP) {
+            if (base + (uint32_t)__popc(peers) > cap) {
                 atomicExch(flag, 1u);
                 fail(st, ST_SORT, where);
             }
         }
         base = __shfl_sync(0xffffffffu, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
-        if (b != ~0u && base < (uint32_t)SS_CAP) {
-            rk[(size_t)b * SS_CAP + base] = k;
-            rv[(size_t)b * SS_CAP + base] = (uint32_t)i;
+        if (b != ~0u && base < cap) {
+            rk[region + base] = k;
+            rv[region + base] = (uint32_t)i;
         }
     }
 }
@@ -507,7 +510,9 @@ __device__ __forceinline__ void sort_bucket(const uint64_t *__restrict__ rk, con
 // One warp per bucket. SCANNED: cnt holds the exclusive sums of the counts (nbk + 1 entries), else the counts,
 // which each block adds up itself.
 template <bool SCANNED>
-__global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, const uint32_t *__restrict__ cnt,
+__global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, int S, const SSys *__restrict__ ss,
+                                                         const uint32_t *__restrict__ bsys,
+                                                         const uint32_t *__restrict__ cnt,
                                                          const uint64_t *__restrict__ rk,
                                                          const uint32_t *__restrict__ rv, uint64_t *__restrict__ k0,
                                                          uint32_t *__restrict__ v0, const uint32_t *flag)
@@ -536,8 +541,10 @@ __global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, const uint32_t
             __syncthreads();
         }
         if (n == 0u) continue;   // the whole warp
-        const uint64_t *kb = rk + (size_t)b * SS_CAP;
-        const uint32_t *vb = rv + (size_t)b * SS_CAP;
+        const SSys y = ss[S == 1 ? 0u : bsys[b]];
+        const int64_t region = y.rbase + (int64_t)(b - y.bbase) * y.rcap;
+        const uint64_t *kb = rk + region;
+        const uint32_t *vb = rv + region;
         if (n <= 256u) sort_bucket<8>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
         else sort_bucket<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
     }
@@ -1836,18 +1843,20 @@ void launch_keys_sort(hybrid_ctx *c)
         uint32_t *cnt = (uint32_t *)c->ss_cnt.p, *flag = (uint32_t *)c->ss_flag.p;
         uint64_t *rk = (uint64_t *)c->ss_rk.p;
         uint32_t *rv = (uint32_t *)c->ss_rv.p;
+        const SSys *ss = (const SSys *)c->ss_sys.p;
+        const uint32_t *bsys = (const uint32_t *)c->ss_bsys.p;
         k_keys_append<<<grid_for(c, N, 256), 256, 0, c->st>>>(
             N, (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p,
             (const int32_t *)c->psys.p, c->S, (const SysBox *)c->box.p, (const int64_t *)c->off_dev.p,
-            (const SSys *)c->ss_sys.p, k0, rk, rv, cnt, flag, st, c->op);
+            ss, k0, rk, rv, cnt, flag, st, c->op);
         const int grid = std::min((c->nbk + SSB_WARPS - 1) / SSB_WARPS, c->nsm * 16);
         // up to SS_SUM_MAX buckets every block of the sort adds up the counts before its buckets (at most 32 loads
         // a thread); above, a scan does it once
         if (c->nbk <= SS_SUM_MAX) {
-            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, cnt, rk, rv, k0, v0, flag);
+            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag);
         } else {
             scan_u32(c, cnt, c->nbk + 1, nullptr, c->nbk + 1, nullptr, true);
-            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, cnt, rk, rv, k0, v0, flag);
+            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag);
         }
         c->launches += 2;
         return;
