@@ -236,11 +236,12 @@ struct hybrid_ctx {
     std::vector<hy::SysIO> h_io;
     int nchunks = 0;
     int ipt = hy::RS_IPT_MAX, tile = hy::RS_TILE_MAX;   // radix tile: 8 warps x 32 lanes x ipt keys, sized to fill the GPU
-    // sample sort layout of the batch (buckets over all systems) and whether the current call repeats a build
-    // with the radix sort after a bucket overflowed
+    // sample sort layout of the batch (buckets over all systems); the op of the current sequence whose build is
+    // repeated with the radix sort after a bucket overflowed (-1: none), and whether that build is being enqueued
     std::vector<hy::SSys> h_ss;
     int nbk = 0;
     int64_t nreg = 0;   // entries of all regions
+    int radix_op = -1;
     bool sort_fallback = false;
     int64_t sort_fallbacks = 0;
     bool tree_valid = false, have_soft = false, have_hard = false;
