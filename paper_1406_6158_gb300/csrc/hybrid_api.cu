@@ -1181,10 +1181,15 @@ hybrid_status hybrid_lists_copy(hybrid_ctx *c, int64_t *counts, int64_t *entries
             return cuda_fail(c, cudaGetLastError(), "list copy");
         std::vector<WorkItem> itf, itn;
         std::vector<uint32_t> gf, L;
-        if (!d2h(c, itf, c->wmap, (size_t)ctr[11]) || !d2h(c, itn, c->wnear, (size_t)ctr[12]) ||
+        const size_t nnear = (uint32_t)ctr[12], ndense = (size_t)(ctr[12] >> 32);   // from the array's two ends
+        Buf dense;
+        dense.p = (WorkItem *)c->wnear.p + (c->capWork - (int64_t)ndense);
+        std::vector<WorkItem> itd;
+        if (!d2h(c, itf, c->wmap, (size_t)ctr[11]) || !d2h(c, itn, c->wnear, nnear) || !d2h(c, itd, dense, ndense) ||
             !d2h(c, gf, c->gfirst, (size_t)ng) || !d2h(c, L, c->list, (size_t)ctr[10]) ||
             cudaStreamSynchronize(c->st) != cudaSuccess)
             return cuda_fail(c, cudaGetLastError(), "list copy");
+        itn.insert(itn.end(), itd.begin(), itd.end());
         auto group_of = [&](uint32_t first) {
             return (int64_t)(std::lower_bound(gf.begin(), gf.end(), first) - gf.begin());
         };

@@ -56,6 +56,8 @@ struct PairArgs {
     // FP32 work items (see WorkItem) and their number
     const WorkItem *items;
     const uint64_t *nwork;
+    const WorkItem *dense_items;          // the end of the near items' array: the dense ones lie before it
+    unsigned long long *dense_counter;
     int want_soft, want_hard;
 };
 
@@ -546,6 +548,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 0) k_far(PairArgs a)
 //    together the sources within R2 of the box of its sinks (computed with the
 //    pair distance's roundings: none is missed).
 //  - SOFT: every pair adds F at weight 1 unless it is marked.
+// Groups with many pairs within R2 take the loop of near_dense instead.
 //
 // One block per work item: its warps take blocks of at most 32 consecutive
 // sinks (compact in key order), one sink per lane, and share the tiles of
@@ -613,17 +616,244 @@ __device__ __forceinline__ int ord_f(float v)
 }
 __device__ __forceinline__ float unord_f(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
 
+// ---- dense items ----------------------------------------------------------
+// Where many of the listed pairs lie within R2 (a clump inside one R2, an R2 of many leaves), marking them and walking
+// the marks costs more than it saves: the K step is bound by the issue rate (89 %), at some 95 instructions a pair, and
+// with one sink a lane half the lanes idle on groups of about 20. The walk tells such groups by their boxes (NEAR_DENSE),
+// and their items, at the other end of the near items' array, are worked on by the loop below: no distance step, two
+// sources per packed instruction, and the lanes that a block of sinks leaves over hold further copies of it, each with
+// its own source pairs (lanes busy on the groups of a Plummer sphere of 2^17: 86 % against 52 %).
+// Near time per step, marks alone -> with this: 2^17 with R2 = 32, 64, 128 eps 1.07 -> .81, 4.37 -> 2.78, 21.9 -> 12.2 ms
+// (R2 = 8 eps .178 -> .181, 10^6 1.028 -> 1.045: the registers of the two loops together); a tenth of 2^17 particles in a
+// clump of half an R2 4.70 -> 2.25; N = 30000 with 64 eps 1.27 -> .76. NEAR_DENSE = 0.7: with 0.4 .93 and 2.89 ms for 32
+// and 64 eps, with 1 as with 0.7. Counting the near leaves close to the group in the walk chose no better and cost it 4 %.
+// A kernel of its own for these items (80 registers, beside k_near on the second stream) was 2 to 4 % faster on them, but
+// its launch cost steps of 2^13 particles 2 %.
+
+struct NearSink2 {   // a sink's rebased hi parts and lo parts, twice over
+    uint64_t hx, hy, hz, lx, ly, lz;
+};
+
+// Two sources (rebased hi parts, masses, lo parts) against one sink, K evaluated if one of them is within R2 (it is 0
+// beyond): r^2 from the parts' differences, K term by term as dll_K_precise has it.
+template <bool SOFT, bool HARD>
+__device__ __forceinline__ void near_both(uint64_t HX, uint64_t HY, uint64_t HZ, uint64_t M, uint64_t LX, uint64_t LY,
+                                          uint64_t LZ, const NearSink2 &S, const HardC &H, uint64_t &AX, uint64_t &AY,
+                                          uint64_t &AZ, uint64_t &BX, uint64_t &BY, uint64_t &BZ)
+{
+    const uint64_t hx = sub2(HX, S.hx), hy = sub2(HY, S.hy), hz = sub2(HZ, S.hz);
+    const uint64_t lx = sub2(LX, S.lx), ly = sub2(LY, S.ly), lz = sub2(LZ, S.lz);
+    const uint64_t dx = add2(hx, lx), dy = add2(hy, ly), dz = add2(hz, lz);
+    const uint64_t r2u = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    float u0, u1, m0, m1;
+    upk2(r2u, u0, u1);
+    upk2(M, m0, m1);
+    const float r0 = u0 + H.eps2, r1 = u1 + H.eps2;
+    const float i0 = r0 > 0.0f ? rsqrtf(r0) : 0.0f, i1 = r1 > 0.0f ? rsqrtf(r1) : 0.0f;
+    uint64_t f = 0ull;
+    if (SOFT) f = mul2(mul2(M, pk2(i0, i1)), mul2(pk2(i0, i1), pk2(i0, i1)));
+    if (u0 < H.R2sq || u1 < H.R2sq) {
+        const uint64_t nx = mul2(hx, sub2(S.hx, HX)), ny = mul2(hy, sub2(S.hy, HY)), nz = mul2(hz, sub2(S.hz, HZ));   // -h^2
+        const uint64_t R = pk2(H.R2sq, H.R2sq);
+        const uint64_t d1 = add2(R, nx), d2 = add2(d1, ny), d3 = add2(d2, nz);
+        const uint64_t e = add2(add2(add2(sub2(R, d1), nx), add2(sub2(d1, d2), ny)), add2(sub2(d2, d3), nz));
+        const uint64_t q = add2(add2(fma2(hx, hx, nx), fma2(hy, hy, ny)), fma2(hz, hz, nz));
+        const uint64_t cross = fma2(add2(add2(hx, hx), lx), lx, fma2(add2(add2(hy, hy), ly), ly, mul2(add2(add2(hz, hz), lz), lz)));
+        const uint64_t D = add2(d3, sub2(add2(e, sub2(pk2(H.R2sqlo, H.R2sqlo), q)), cross));
+        float D0, D1;
+        upk2(D, D0, D1);
+        auto K_of = [&](float u, float Dk) -> float {
+            const float Y = __saturatef(__fdividef(Dk * H.invdR, H.R2 + sqrtf(u)));
+            const float Y2 = Y * Y;
+            return (Y2 * Y2 * Y2) * fmaf(Y2, fmaf(6.0f, Y2, -15.0f), 10.0f);
+        };
+        const uint64_t K = pk2(K_of(u0, D0), K_of(u1, D1));
+        if (!SOFT) f = mul2(mul2(M, pk2(i0, i1)), mul2(pk2(i0, i1), pk2(i0, i1)));
+        if (HARD) {
+            const uint64_t fh = mul2(f, K);
+            BX = fma2(dx, fh, BX);
+            BY = fma2(dy, fh, BY);
+            BZ = fma2(dz, fh, BZ);
+        }
+        if (SOFT) f = mul2(f, sub2(pk2(1.0f, 1.0f), K));
+    }
+    if (SOFT) {
+        AX = fma2(dx, f, AX);
+        AY = fma2(dy, f, AY);
+        AZ = fma2(dz, f, AZ);
+    }
+}
+
+// A dense item's tile, its sources two by two: {hx hx' hy hy'} {hz hz' m m'} {lx lx' ly ly'} {lz lz'}.
+struct NearPairs {
+    float4 a[NEAR_TILE / 2], b[NEAR_TILE / 2], c[NEAR_TILE / 2];
+    float2 d[NEAR_TILE / 2];
+};
+static_assert(sizeof(NearPairs) <= sizeof(NearTile), "either form of a tile");
+
+// Blocks of sinks that a group of up to 64 is cut into: the fewest that keep the most lanes busy, a warp holding 32 / per
+// copies of a block of per sinks.
+constexpr int near_cut(int n)
+{
+    int best = n <= 32 ? 1 : 2;
+    for (int nb = 2 * best; nb <= 4; nb *= 2) {
+        const int c0 = 32 / ((n + best - 1) / best), c1 = 32 / ((n + nb - 1) / nb);   // slots per sink: 32 nb / copies
+        if (nb * c0 < best * c1) best = nb;
+    }
+    return best;
+}
+constexpr uint64_t near_cuts(int nb)   // bit n - 1: groups of n are cut into nb blocks
+{
+    uint64_t m = 0;
+    for (int n = 1; n <= 64; ++n) m |= near_cut(n) == nb ? 1ull << (n - 1) : 0ull;
+    return m;
+}
+constexpr uint64_t NEAR_CUT2 = near_cuts(2), NEAR_CUT4 = near_cuts(4);
+
+// The dense items, W of them, by the blocks in turn. Returns the number of pairs of this block's.
+template <bool SOFT, bool HARD>
+__device__ __forceinline__ unsigned long long near_dense(const PairArgs &a, uint32_t W, NearTile *tiles, uint32_t &sh_item)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    unsigned long long inter = 0;
+    uint32_t next = 0;
+    for (uint32_t it = blockIdx.x; it < W;) {   // a block's first item by its place in the grid
+        if (threadIdx.x == 0) next = gridDim.x + (uint32_t)atomicAdd(a.dense_counter, 1ull);   // arrives while this one runs
+        const WorkItem d = a.dense_items[-1 - (int64_t)it];   // from the end of the array down
+        const SysParams &P = a.sp[d.sys];
+        const HardC H = {P.eps2f, P.R2f, P.R2sqf, P.R2sqlo, P.invdRf};
+        const uint32_t *list = a.list + d.pbase + d.e0;
+        const int ne = (int)(d.e1 - d.e0), n = (int)(d.n & ~MULTI);
+        inter += (unsigned long long)n * (unsigned long long)ne;
+        const bool multi = (d.n & MULTI) != 0;
+        const float4 cref = a.phi[d.first];
+        const int nblk = n > 64 ? (n + 31) / 32 : (((NEAR_CUT4 >> (n - 1)) & 1ull) ? 4 : (((NEAR_CUT2 >> (n - 1)) & 1ull) ? 2 : 1));
+        const int per = (n + nblk - 1) / nblk, ntile = (ne + NEAR_TILE - 1) / NEAR_TILE;
+        for (int b0 = 0; b0 < nblk; b0 += PAIR_WARPS) {
+            const int here = min(nblk - b0, PAIR_WARPS);
+            const int splits = here == 1 ? 4 : (here == 2 ? 2 : 1);   // warps per block of sinks, each a part of every tile
+            const int blk = b0 + w / splits, part = w - (w / splits) * splits;
+            const int s0 = blk * per, sn = blk < nblk ? min(per, n - s0) : 0;
+            const bool busy = sn > 0;
+            // a lane is sink `slot` of copy `copy`, which takes every copies-th pair of sources (the lanes left over: none)
+            const uint32_t inv = busy ? (65536u + sn - 1) / sn : 0u;   // lane / sn = (lane inv) >> 16
+            const int copies = (int)((32u * inv) >> 16), own = (int)((lane * inv) >> 16), slot = lane - own * sn;
+            const int copy = own < copies ? own : NEAR_TILE;
+            NearSink2 S = {0, 0, 0, 0, 0, 0};
+            if (busy) {
+                const float4 h = a.phi[d.first + s0 + slot], l = a.plo[d.first + s0 + slot];
+                const float x = h.x - cref.x, y = h.y - cref.y, z = h.z - cref.z;
+                S = NearSink2{pk2(x, x), pk2(y, y), pk2(z, z), pk2(l.x, l.x), pk2(l.y, l.y), pk2(l.z, l.z)};
+            }
+            uint64_t AX = 0ull, AY = 0ull, AZ = 0ull, BX = 0ull, BY = 0ull, BZ = 0ull;
+            auto index = [&](int t) -> uint32_t {
+                const int e = t * NEAR_TILE + (int)threadIdx.x;
+                return e < ne ? list[e] : NONE;
+            };
+            float4 gh = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.0f), gl = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            auto gather = [&](uint32_t i) {
+                if (i != NONE) {
+                    gh = a.phi[i];
+                    gl = a.plo[i];
+                } else {
+                    gh = make_float4(FAR_AWAY, FAR_AWAY, FAR_AWAY, 0.0f);
+                }
+            };
+            uint32_t i1 = index(0);
+            gather(i1);
+            i1 = ntile > 1 ? index(1) : NONE;
+            for (int t = 0; t < ntile; ++t) {
+                NearPairs &T = *(NearPairs *)&tiles[t & 1];
+                {
+                    const int k = threadIdx.x >> 1, b = threadIdx.x & 1;
+                    float *u = (float *)&T.a[k] + b;
+                    u[0] = gh.x - cref.x;
+                    u[2] = gh.y - cref.y;
+                    u = (float *)&T.b[k] + b;
+                    u[0] = gh.z - cref.z;
+                    u[2] = gh.w;
+                    u = (float *)&T.c[k] + b;
+                    u[0] = gl.x;
+                    u[2] = gl.y;
+                    ((float *)&T.d[k])[b] = gl.z;
+                }
+                if (t + 1 < ntile) {
+                    gather(i1);
+                    i1 = t + 2 < ntile ? index(t + 2) : NONE;
+                }
+                __syncthreads();
+                if (!busy) continue;
+                const int nt = min(NEAR_TILE, ne - t * NEAR_TILE);
+                const int q0 = part * (NEAR_TILE / 2 / splits), q1 = min((nt + 1) / 2, q0 + NEAR_TILE / 2 / splits);
+#pragma unroll 1
+                for (int q = q0 + copy; q < q1; q += copies) {
+                    const uint32_t u = (uint32_t)__cvta_generic_to_shared(&T) + 16u * (uint32_t)q;
+                    uint64_t HX, HY, HZ, M, LX, LY, LZ;
+                    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(HX), "=l"(HY) : "r"(u));
+                    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(HZ), "=l"(M) : "r"(u + 8u * NEAR_TILE));
+                    asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(LX), "=l"(LY) : "r"(u + 16u * NEAR_TILE));
+                    asm volatile("ld.shared.b64 %0, [%1];" : "=l"(LZ) : "r"(u - 8u * (uint32_t)q + 24u * NEAR_TILE));
+                    near_both<SOFT, HARD>(HX, HY, HZ, M, LX, LY, LZ, S, H, AX, AY, AZ, BX, BY, BZ);
+                }
+            }
+            if (busy) {   // the copies' sums into the first
+                float v[6], t0, t1;
+                upk2(SOFT ? AX : BX, t0, t1);
+                v[0] = t0 + t1;
+                upk2(SOFT ? AY : BY, t0, t1);
+                v[1] = t0 + t1;
+                upk2(SOFT ? AZ : BZ, t0, t1);
+                v[2] = t0 + t1;
+                if (SOFT && HARD) {
+                    upk2(BX, t0, t1);
+                    v[3] = t0 + t1;
+                    upk2(BY, t0, t1);
+                    v[4] = t0 + t1;
+                    upk2(BZ, t0, t1);
+                    v[5] = t0 + t1;
+                }
+                constexpr int NV = SOFT && HARD ? 6 : 3;
+                for (int k = 1; k < copies; ++k) {
+                    const int src = min(lane + k * sn, 31);
+#pragma unroll
+                    for (int j = 0; j < NV; ++j) {
+                        const float y = __shfl_sync(0xffffffffu, v[j], src);
+                        if (copy == 0) v[j] += y;
+                    }
+                }
+                if (copy == 0) {
+                    const uint32_t i = d.first + s0 + slot;
+#pragma unroll
+                    for (int j = 0; j < NV; ++j) {
+                        float *o = (float *)(SOFT && j < 3 ? a.as[j] : a.ah[j % 3]) + i;
+                        if (!(SOFT && j < 3) && !multi && splits == 1) *o = P.Gf * v[j];
+                        else atomicAdd(o, P.Gf * v[j]);   // the near part of the soft force is added to the far part
+                    }
+                }
+            }
+            if (b0 + PAIR_WARPS < nblk) __syncthreads();   // the next blocks of sinks write tile 0 again
+        }
+        if (threadIdx.x == 0) sh_item = next;
+        __syncthreads();   // and this item's tiles are used
+        it = sh_item;
+    }
+    return inter;
+}
+
 template <bool SOFT, bool HARD>
 __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs a)
 {
-    __shared__ NearTile tiles[2];
+    __shared__ __align__(16) NearTile tiles[2];
     __shared__ __align__(16) float packed_mem[SOFT ? 2 * 4 * NEAR_TILE : PAIR_WARPS * (sizeof(NearPacked) + 3) / 4];
     __shared__ int64_t sh_item;
+    __shared__ uint32_t sh_dense;
     if (a.st->code) return;
+    unsigned long long inter = 0;
+    const uint32_t ndense = (uint32_t)(*a.nwork >> 32);   // these first: they take longer
+    if (blockIdx.x < ndense) inter = near_dense<SOFT, HARD>(a, ndense, tiles, sh_dense);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned ltm = (1u << lane) - 1u;
-    const int64_t W = (int64_t)*a.nwork;
-    unsigned long long inter = 0;
+    const int64_t W = (uint32_t)*a.nwork;
     unsigned long long next = 0;
     if (threadIdx.x == 0) next = atomicAdd(a.counter, 1ull);
     for (;;) {
@@ -1026,6 +1256,8 @@ void fill_args(hybrid_ctx *c, PairArgs &a)
     a.st = status_dev(c);
     a.items = nullptr;
     a.nwork = nullptr;
+    a.dense_items = nullptr;
+    a.dense_counter = nullptr;
     a.want_soft = a.want_hard = 0;
 }
 
@@ -1052,6 +1284,7 @@ __global__ void __launch_bounds__(256) k_clear_pairs(PairArgs a, bool near, int 
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         *a.counter = 0ull;
+        if (near) a.counter[5] = 0ull;   // the dense near kernel's
         *(near ? a.inter_hard : a.inter_soft) = 0ull;
     }
     void *const *acc = near ? a.ah : a.as;
@@ -1104,6 +1337,8 @@ void launch_pairs(hybrid_ctx *c, bool near, int mode)
             else if (ks == 4) go_far<4>(c, a);
             else go_far<8>(c, a);
         } else {
+            a.dense_counter = a.counter + 5;
+            a.dense_items = a.items + c->capWork;
             const int grid = c->nsm * NEAR_MIN_BLOCKS;
             if (a.want_soft && a.want_hard) k_near<true, true><<<grid, PAIR_THREADS, 0, c->st>>>(a);
             else if (a.want_soft) k_near<true, false><<<grid, PAIR_THREADS, 0, c->st>>>(a);

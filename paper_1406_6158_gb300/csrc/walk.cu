@@ -55,19 +55,24 @@ struct WalkArgs {
     int mode;
     Status *st;
     int where;
-    unsigned long long *queue;   // [0], [1]: next far / near item or unit of the pair kernels, zeroed here with
+    unsigned long long *queue;   // [0], [1]: next far / near item or unit of the pair kernels, [6]: next dense near item;
+                                 // zeroed here with
     unsigned long long *pairs;   // [0], [1]: the pair counts
     float *acc_s[3], *acc_h[3];  // FP32 form: the accelerations this walk's pair kernels add to, zeroed here
     // one-pass form
     const uint32_t *gfirst;
     unsigned long long *list_cursor;     // next free list entry
-    unsigned long long *item_count;      // [0] far items, [1] near items
+    unsigned long long *item_count;      // [0] far items, [1] near items (low half) and dense near items (high half)
     WorkItem *items_far, *items_near;
     int64_t cap_items;
     int lch_far, lch_near;               // base lengths of far and near work items
 };
 
 constexpr uint32_t WALK_REGION = 2048;
+// A group is dense (near_dense in pair.cu) when its box fits in a sphere of sqrt(NEAR_DENSE) R2: its near leaves, which are
+// no larger, then lie within about twice R2, and a good part of them within R2. Marked in its size (see gd).
+constexpr float NEAR_DENSE = 0.7f;
+constexpr uint32_t GROUP_DENSE = 0x80000000u;
 constexpr int WALK_SSTK = 1024;   // entries of a warp's stack kept in shared memory (one walk iteration pushes <= 256)
 
 __device__ __forceinline__ void fail(Status *st, int code, int where)
@@ -117,7 +122,7 @@ __device__ __forceinline__ int reaches(float d2, float r2)
 __device__ __forceinline__ void clear_pair_counters(const WalkArgs &a)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.queue[0] = a.queue[1] = 0ull;
+        a.queue[0] = a.queue[1] = a.queue[6] = 0ull;
         if (a.mode & 1) a.pairs[0] = 0ull;
         a.pairs[1] = 0ull;
     }
@@ -296,17 +301,21 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs a)
 
 // Work items, of at most per entries, of one contiguous run [start, start +
 // len) of a group's entries of kind t (0 cells, 1 far particles, 2 near
-// particles); all lanes call it.
+// particles; those of a dense group fill the near items' array from its end);
+// all lanes call it.
 __device__ __forceinline__ bool emit_items(const WalkArgs &a, int t, uint64_t start, uint32_t len, uint32_t per,
                                            uint32_t first, uint32_t n, uint32_t sys, bool multi, int lane)
 {
     const int cls = t == 2 ? 1 : 0;
+    const bool dense = t == 2 && (n & GROUP_DENSE);
+    n &= ~GROUP_DENSE;
     const uint32_t m = (len + per - 1) / per;
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(a.item_count + cls, (unsigned long long)m);
+    if (lane == 0) base = atomicAdd(a.item_count + cls, (unsigned long long)m << (dense ? 32 : 0));
     base = __shfl_sync(0xffffffffu, base, 0);
-    if ((int64_t)(base + m) > a.cap_items) return false;
-    WorkItem *dst = (cls ? a.items_near : a.items_far) + base;
+    const int64_t lo = (uint32_t)base, hi = (int64_t)(base >> 32);
+    if (lo + hi + m > a.cap_items) return false;
+    WorkItem *dst = (cls ? a.items_near : a.items_far) + (dense ? a.cap_items - hi - m : lo);
     for (uint32_t j = lane; j < m; j += 32) {
         WorkItem d;
         d.cbase = t == 0 ? start : 0;
@@ -380,6 +389,7 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
             }
         run[0].len = run[1].len = run[2].len = 0;
         const uint32_t per_far = item_len(gn, a.lch_far), per_near = item_len(gn, a.lch_near);
+        const uint32_t gd = gn | (hx * hx + hy * hy + hz * hz < NEAR_DENSE * a.sp[s].R2sqf ? GROUP_DENSE : 0u);
         uint32_t early_far = 0, early_near = 0;   // items already emitted for this group
         int sp = 0;        // entries in the shared-memory part
         int64_t gp = 0;    // entries in the global part
@@ -394,7 +404,7 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
             if (tot <= r.left) return true;
             if (r.len > 0) {
                 const uint32_t per = t == 2 ? per_near : per_far;
-                if (!emit_items(a, t, r.pos - r.len, r.len, per, gfirst, gn, s, true, lane)) {
+                if (!emit_items(a, t, r.pos - r.len, r.len, per, gfirst, gd, s, true, lane)) {
                     fail_items = true;
                     return false;
                 }
@@ -526,7 +536,7 @@ __global__ void __launch_bounds__(WALK_THREADS, MINB) k_walk1(WalkArgs a)
 #pragma unroll
         for (int t = 0; t < 3; ++t)
             if (run[t].len > 0 && !fail_items)
-                if (!emit_items(a, t, run[t].pos - run[t].len, run[t].len, t == 2 ? per_near : per_far, gfirst, gn, s,
+                if (!emit_items(a, t, run[t].pos - run[t].len, run[t].len, t == 2 ? per_near : per_far, gfirst, gd, s,
                                 (t == 2 ? fin_near : fin_far) > 1, lane))
                     fail_items = true;
         if (fail_items) break;
