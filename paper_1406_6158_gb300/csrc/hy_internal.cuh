@@ -127,9 +127,8 @@ __device__ __forceinline__ void grid_split(double x, double lo0, const SysBox &b
 // Internal status code (never returned to the caller): a particle moved more
 // than skin / 2 since the last build; the step resumes with a rebuild.
 constexpr int32_t ST_SKIN = 100;
-// Internal status code: a bucket of the sample sort held more keys than a
-// block sorts in shared memory; the build left the order unchanged and is
-// repeated with the radix sort.
+// Internal status code: a bucket of the sample sort held more than SS_CAP keys;
+// the build left the order unchanged and is repeated with the radix sort.
 constexpr int32_t ST_SORT = 101;
 
 // Sample sort of the keys (the usual path once the state is close to key
@@ -142,6 +141,7 @@ constexpr int32_t ST_SORT = 101;
 // region of SS_CAP for every system would be 6 KiB for one of a few particles).
 constexpr int SS_BUCKET = 224;
 constexpr int SS_CAP = 512;
+constexpr int SS_SMALL = 19;       // buckets (4256 particles) up to which a system with an overflow takes other splitters
 constexpr int SS_SUM_MAX = 4096;   // buckets up to which the sorting blocks add up the counts themselves
 struct SSys {
     int32_t nb;      // buckets of the system

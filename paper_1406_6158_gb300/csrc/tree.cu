@@ -324,7 +324,11 @@ __global__ void __launch_bounds__(256) k_onesweep(const uint64_t *__restrict__ k
 // and keeps buckets in order whatever the splitters are. A bucket of more than
 // SS_CAP keys (a state far from key order) makes the build leave the order
 // unchanged and record ST_SORT; the build is then repeated with the radix
-// sort.
+// sort. A system of at most SS_SMALL buckets takes splitters of its own instead
+// (sort_small): a first build of it, or one after another system's, nearly
+// always overflows, and the repetition cost more than the rest of the build
+// (hybrid_build_tree of a new state: N = 600 203 -> 111 us, 4096 228 -> 151; with
+// buckets of 4096 keys, which held any such system, 143 and 189).
 // Three launches, each key written and read twice. Before: buckets of 1024 or
 // 2048 keys, a splitter, a counting, a scan and a scatter launch, and a radix
 // sort of each bucket in shared memory. Root box and key sort per soft step of
@@ -351,6 +355,7 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
     for (int64_t i0 = (int64_t)blockIdx.x * blockDim.x; i0 < N; i0 += stride) {
         const int64_t i = i0 + threadIdx.x;
         uint32_t b = ~0u, cap = 0u;
+        bool small = false;
         uint64_t k = 0ull;
         int64_t region = 0;
         if (i < N) {
@@ -395,6 +400,7 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
             }
             b = (uint32_t)(yy.bbase + lo);
             cap = (uint32_t)yy.rcap;
+            small = yy.nb <= SS_SMALL;
             region = yy.rbase + (int64_t)lo * yy.rcap;
         }
         const unsigned peers = __match_any_sync(0xffffffffu, b);
@@ -403,8 +409,8 @@ __global__ void __launch_bounds__(256) k_keys_append(int64_t N, const double *__
         if (b != ~0u && lane == leader) {
             base = atomicAdd(cnt + b, (uint32_t)__popc(peers));
             if (base + (uint32_t)__popc(peers) > cap) {
-                atomicExch(flag, 1u);
-                fail(st, ST_SORT, where);
+                atomicOr(flag, small ? 2u : 1u);
+                if (!small) fail(st, ST_SORT, where);
             }
         }
         base = __shfl_sync(0xffffffffu, base, leader) + (uint32_t)__popc(peers & ((1u << lane) - 1u));
@@ -476,15 +482,16 @@ __device__ __forceinline__ void warp_sort(uint64_t (&k)[R], uint32_t (&v)[R], in
 constexpr int SSB_THREADS = 128, SSB_WARPS = SSB_THREADS / 32;
 constexpr int SS_PAD = SS_CAP + SS_CAP / 8;   // a bucket in shared memory, one entry of padding after every R
 
+// n <= 32 R composites sorted by one warp (from global or shared memory). Not inlined: its code is fetched once, whoever
+// calls it (inlined three times more for sort_small, a build of 600 new particles took 160 us, not 111).
 template <int R>
-__device__ __forceinline__ void sort_bucket(const uint64_t *__restrict__ rk, const uint32_t *__restrict__ rv, int n,
-                                            uint64_t *__restrict__ k0, uint32_t *__restrict__ v0, uint64_t *sk,
-                                            uint32_t *sv, int lane)
+__device__ __noinline__ void sort_run(const uint64_t *rk, const uint32_t *rv, int n, uint64_t *k0, uint32_t *v0, uint64_t *sk,
+                                      uint32_t *sv, int lane)
 {
     uint64_t k[R];
     uint32_t v[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {   // any order will do; slots past the bucket sort to the end
+    for (int r = 0; r < R; ++r) {   // any order will do; slots past the run sort to the end
         const int e = r * 32 + lane;
         k[r] = e < n ? rk[e] : ~0ull;
         v[r] = e < n ? rv[e] : ~0u;
@@ -507,21 +514,110 @@ __device__ __forceinline__ void sort_bucket(const uint64_t *__restrict__ rk, con
     }
 }
 
+// A small system with an overflowed bucket, by the blocks that its buckets belong to, each by itself: keys made anew,
+// splitters from the sorted keys of up to SS_SAMPLE of its particles, the block's buckets gathered from all of them, and
+// their place from the number of keys before them. A bucket that overflows again sends the build to the radix sort.
+constexpr int SS_SAMPLE = 256;
+struct SmallArgs {
+    const double *x, *y, *z;
+    const SysBox *box;
+    const int64_t *off;
+    Status *st;
+    int where;
+};
+struct SortMem {
+    uint64_t k[SSB_WARPS][SS_PAD];   // a bucket per warp
+    uint32_t v[SSB_WARPS][SS_PAD];
+    uint64_t sk[SS_SAMPLE];          // the sample of a small system
+    uint32_t sv[SS_SAMPLE];
+    uint32_t cnt[SSB_WARPS + 1];     // keys of the block's buckets; before them
+};
+
+__device__ __noinline__ void sort_small(const SmallArgs &a, int s, const SSys &y, int b0, uint32_t *flag,
+                                        uint64_t *__restrict__ k0, uint32_t *__restrict__ v0, SortMem &m)
+{
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t o = a.off[s];
+    const int n = (int)(a.off[s + 1] - o), M = min(n, SS_SAMPLE);
+    const SysBox b = a.box[s];
+    const int es = pow2_exponent(b.scale);
+    auto composite = [&](int i, uint64_t &k, uint32_t &v) {
+        k = (spread3(cell_coord(a.x[o + i], b.lo[0], es)) << 2) | (spread3(cell_coord(a.y[o + i], b.lo[1], es)) << 1) |
+            spread3(cell_coord(a.z[o + i], b.lo[2], es));
+        v = (uint32_t)(o + i);
+    };
+    if (threadIdx.x <= SSB_WARPS) m.cnt[threadIdx.x] = 0u;
+    for (int e = threadIdx.x; e < M; e += SSB_THREADS) composite(e * n / M, m.k[0][e], m.v[0][e]);
+    __syncthreads();
+    if (w == 0) sort_run<SS_SAMPLE / 32>(m.k[0], m.v[0], M, m.sk, m.sv, m.k[0], m.v[0], lane);
+    __syncthreads();
+    const int j0 = max(0, b0 - y.bbase), J = min(y.nb, b0 + SSB_WARPS - y.bbase) - j0;   // this block's buckets
+    uint64_t ck[SSB_WARPS + 1];   // bucket q: composites from splitter q up to splitter q + 1
+    uint32_t cv[SSB_WARPS + 1];
+#pragma unroll
+    for (int q = 0; q <= SSB_WARPS; ++q) {
+        const int j = j0 + q;
+        ck[q] = j == 0 ? 0ull : (j < y.nb ? m.sk[j * M / y.nb] : ~0ull);
+        cv[q] = j == 0 ? 0u : (j < y.nb ? m.sv[j * M / y.nb] : ~0u);
+    }
+    for (int i = threadIdx.x; i < n; i += SSB_THREADS) {
+        uint64_t k;
+        uint32_t v;
+        composite(i, k, v);
+        int q = -1;
+#pragma unroll
+        for (int u = 0; u <= SSB_WARPS; ++u) q += comp_less(k, v, ck[u], cv[u]) ? 0 : 1;
+        if (q < 0) {
+            atomicAdd(m.cnt + SSB_WARPS, 1u);
+        } else if (q < J) {
+            const uint32_t at = atomicAdd(m.cnt + q, 1u);
+            if (at < (uint32_t)SS_CAP) {
+                m.k[q][at] = k;
+                m.v[q][at] = v;
+            }
+        }
+    }
+    __syncthreads();
+    if (w < J) {
+        const int c = (int)m.cnt[w];
+        uint32_t s0 = (uint32_t)o + m.cnt[SSB_WARPS];
+        for (int q = 0; q < w; ++q) s0 += m.cnt[q];
+        if (c > SS_CAP) {
+            if (lane == 0) {
+                atomicOr(flag, 1u);
+                fail(a.st, ST_SORT, a.where);
+            }
+        } else if (c > 256) {
+            sort_run<SS_CAP / 32>(m.k[w], m.v[w], c, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+        } else {
+            sort_run<8>(m.k[w], m.v[w], c, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+        }
+    }
+    __syncthreads();   // the buckets and counts are used
+}
+
 // One warp per bucket. SCANNED: cnt holds the exclusive sums of the counts (nbk + 1 entries), else the counts,
 // which each block adds up itself.
 template <bool SCANNED>
-__global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, int S, const SSys *__restrict__ ss,
-                                                         const uint32_t *__restrict__ bsys,
-                                                         const uint32_t *__restrict__ cnt,
-                                                         const uint64_t *__restrict__ rk,
-                                                         const uint32_t *__restrict__ rv, uint64_t *__restrict__ k0,
-                                                         uint32_t *__restrict__ v0, const uint32_t *flag)
+__global__ void __launch_bounds__(SSB_THREADS, 4) k_ss_sort(int nbk, int S, const SSys *__restrict__ ss,
+                                                            const uint32_t *__restrict__ bsys,
+                                                            const uint32_t *__restrict__ cnt,
+                                                            const uint64_t *__restrict__ rk,
+                                                            const uint32_t *__restrict__ rv, uint64_t *__restrict__ k0,
+                                                            uint32_t *__restrict__ v0, uint32_t *flag,
+                                                            const __grid_constant__ SmallArgs small)
 {
-    __shared__ uint64_t sk[SSB_WARPS][SS_PAD];
-    __shared__ uint32_t sv[SSB_WARPS][SS_PAD];
+    __shared__ SortMem m;
     __shared__ uint32_t wsum[SSB_WARPS];
-    if (*flag) return;
+    const uint32_t fl = *flag;
+    if (fl & 1u) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    // whether a small system has an overflowed bucket, by a whole warp
+    auto overflowed = [&](const SSys &y) -> bool {
+        const int b = y.bbase + lane;
+        const bool on = y.nb <= SS_SMALL && lane < y.nb;
+        return __any_sync(0xffffffffu, on && (SCANNED ? cnt[b + 1] - cnt[b] : cnt[b]) > (uint32_t)y.rcap);
+    };
     for (int b0 = blockIdx.x * SSB_WARPS; b0 < nbk; b0 += gridDim.x * SSB_WARPS) {
         const int b = b0 + w;
         uint32_t s0, n;
@@ -540,13 +636,27 @@ __global__ void __launch_bounds__(SSB_THREADS) k_ss_sort(int nbk, int S, const S
             n = b < nbk ? cnt[b] : 0u;
             __syncthreads();
         }
-        if (n == 0u) continue;   // the whole warp
-        const SSys y = ss[S == 1 ? 0u : bsys[b]];
-        const int64_t region = y.rbase + (int64_t)(b - y.bbase) * y.rcap;
-        const uint64_t *kb = rk + region;
-        const uint32_t *vb = rv + region;
-        if (n <= 256u) sort_bucket<8>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
-        else sort_bucket<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, sk[w], sv[w], lane);
+        if (n > 0u) {   // the whole warp
+            const SSys y = ss[S == 1 ? 0u : bsys[b]];
+            const int64_t region = y.rbase + (int64_t)(b - y.bbase) * y.rcap;
+            const uint64_t *kb = rk + region;
+            const uint32_t *vb = rv + region;
+            if ((fl & 2u) && overflowed(y)) {
+                // below
+            } else if (n <= 256u) {
+                sort_run<8>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+            } else {
+                sort_run<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+            }
+        }
+        if (fl & 2u) {
+            __syncthreads();
+            const int last = min(b0 + SSB_WARPS, nbk) - 1;
+            for (int s = S == 1 ? 0 : (int)bsys[b0]; s <= (S == 1 ? 0 : (int)bsys[last]); ++s) {
+                const SSys y = ss[s];
+                if (overflowed(y)) sort_small(small, s, y, b0, flag, k0, v0, m);
+            }
+        }
     }
 }
 
@@ -568,7 +678,7 @@ struct PermArgs {
     int64_t N;
     unsigned long long *bmin, *bmax;   // reset for the next build (the root cubes are made)
     int S;
-    uint32_t *flag;       // [0] an overflowed sample sort: the order stays; [1] reset for the next build
+    uint32_t *flag;       // [0] bit 0: an overflowed sample sort: the order stays; [1] reset for the next build
 };
 
 // MINB blocks per SM: 8 (32 registers) for batches above 2^18 particles, where the gathers' bandwidth counts (2^24:
@@ -578,7 +688,7 @@ template <int MINB>
 __global__ void __launch_bounds__(256, MINB) k_permute(PermArgs a)
 {
     // whatever the status: later kernels rely on a consistent permutation
-    const bool keep = a.flag[0] != 0u;
+    const bool keep = (a.flag[0] & 1u) != 0u;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < 3 * a.S; k += gridDim.x * blockDim.x) {
         a.bmin[k] = ~0ull;
         a.bmax[k] = 0ull;
@@ -1849,14 +1959,16 @@ void launch_keys_sort(hybrid_ctx *c)
             N, (const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p,
             (const int32_t *)c->psys.p, c->S, (const SysBox *)c->box.p, (const int64_t *)c->off_dev.p,
             ss, k0, rk, rv, cnt, flag, st, c->op);
+        const SmallArgs small = {(const double *)c->x[0].p, (const double *)c->x[1].p, (const double *)c->x[2].p,
+                                 (const SysBox *)c->box.p,  (const int64_t *)c->off_dev.p, st, c->op};
         const int grid = std::min((c->nbk + SSB_WARPS - 1) / SSB_WARPS, c->nsm * 16);
         // up to SS_SUM_MAX buckets every block of the sort adds up the counts before its buckets (at most 32 loads
         // a thread); above, a scan does it once
         if (c->nbk <= SS_SUM_MAX) {
-            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag);
+            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag, small);
         } else {
             scan_u32(c, cnt, c->nbk + 1, nullptr, c->nbk + 1, nullptr, true);
-            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag);
+            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag, small);
         }
         c->launches += 2;
         return;
