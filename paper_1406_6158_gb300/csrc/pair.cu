@@ -847,13 +847,14 @@ __global__ void __launch_bounds__(PAIR_THREADS, NEAR_MIN_BLOCKS) k_near(PairArgs
     __shared__ __align__(16) float packed_mem[SOFT ? 2 * 4 * NEAR_TILE : PAIR_WARPS * (sizeof(NearPacked) + 3) / 4];
     __shared__ int64_t sh_item;
     __shared__ uint32_t sh_dense;
+    const uint64_t nwork = *a.nwork;   // on its way with the status
     if (a.st->code) return;
     unsigned long long inter = 0;
-    const uint32_t ndense = (uint32_t)(*a.nwork >> 32);   // these first: they take longer
+    const uint32_t ndense = (uint32_t)(nwork >> 32);   // these first: they take longer
     if (blockIdx.x < ndense) inter = near_dense<SOFT, HARD>(a, ndense, tiles, sh_dense);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned ltm = (1u << lane) - 1u;
-    const int64_t W = (uint32_t)*a.nwork;
+    const int64_t W = (uint32_t)nwork;
     unsigned long long next = 0;
     if (threadIdx.x == 0) next = atomicAdd(a.counter, 1ull);
     for (;;) {
