@@ -445,14 +445,17 @@ def run_c5(args):
     return 0
 
 
-def hbm_stages(n, n_hard, ms, nodes=None):
+# bytes per particle of the sample sort that the builds take between steps: 36 (x, y, z in, key and index out) where the
+# key is made and appended to its bucket, 24 (key and index in and out) in the buckets' sort
+SORT_BYTES = 36 + 24
+
+
+def hbm_stages(n, n_hard, ms, nodes=None, sort_bytes=36 + 12 + 24 + 24):
     """Achieved HBM bandwidth of the memory-bound stages from their live times per soft step and their
     algorithmic bytes (n_hard builds and drift launches per soft step):
-      sort        per particle 36 (keys: x, y, z in, key and index out) + 12 (key in, bucket out) + 24 (key and
-                  bucket in, key and index out to the bucket) + 24 (key and index in and out of the bucket sort):
-                  the count this record has always used; the sample sort the builds take between steps finds the
-                  bucket where it makes the key and moves 60 of them (a build that falls back to the radix sort
-                  moves 36 + 8 + 8 x 24; the line reports the fallbacks)
+      sort        per particle sort_bytes: what the sort moves is SORT_BYTES, which the benchmark's lines are made with
+                  (the default counts a sort that finds each key's bucket in a pass of its own; a build that falls
+                  back to the radix sort moves 36 + 8 + 8 x 24: the line reports the fallbacks)
       topology    per particle 8 (sorted key in); per node 24 out (first, count, level, first child, children,
                   parent)
       moments     per particle 32 (FP32 hi/lo position copies in); per node 24 in (the topology) and 72 out (the
@@ -461,7 +464,7 @@ def hbm_stages(n, n_hard, ms, nodes=None):
       kick_drift  per particle 108 (v 24, a 12, x 24 in; v 24, x 24 out)
     nodes: tree nodes of one build (topology and moments are reported only when it is given)."""
     peak = float(measured_peaks().get("hbm_gbs", 6655.6))
-    per = {"sort": (36 + 12 + 24 + 24, 0), "kick_drift": (108, 0)}
+    per = {"sort": (sort_bytes, 0), "kick_drift": (108, 0)}
     if nodes:
         per["topology"] = (8, 24)
         per["moments"] = (32, 24 + 72)
@@ -590,7 +593,7 @@ def c3_record(args, steps, warmup, with_cpu=True):
                      "traffic": None, "kernel": "k_far (cells + far particles, soft force)",
                      "peak_note": "FP32 CUDA-core peak: %d SMs x 128 lanes x 2 flop x %.0f MHz (max SM clock)" %
                                   (props.multi_processor_count, sm_max)},
-        "hbm_stages": hbm_stages(n, P.n_hard, ms, nodes),
+        "hbm_stages": hbm_stages(n, P.n_hard, ms, nodes, SORT_BYTES),
         "gpu_launches": launches, "sort_fallbacks": fallbacks, "clocks": clk, "cpu_baseline": cpu,
     }
 
@@ -994,7 +997,8 @@ def main():
             "clocks": clk,
             "tree": {"nodes": nodes, "groups": groups},
             "hbm_stages": hbm_stages(w["n"], w["n_hard"], {"sort": stage[5], "topology": stage[6],
-                                                           "moments": stage[7], "kick_drift": stage[4]}, nodes),
+                                                           "moments": stage[7], "kick_drift": stage[4]}, nodes,
+                                     SORT_BYTES),
         }
         line.update(subs)
         print(json.dumps(line), flush=True)
