@@ -482,10 +482,9 @@ __device__ __forceinline__ void warp_sort(uint64_t (&k)[R], uint32_t (&v)[R], in
 constexpr int SSB_THREADS = 128, SSB_WARPS = SSB_THREADS / 32;
 constexpr int SS_PAD = SS_CAP + SS_CAP / 8;   // a bucket in shared memory, one entry of padding after every R
 
-// n <= 32 R composites sorted by one warp (from global or shared memory). Not inlined: its code is fetched once, whoever
-// calls it (inlined three times more for sort_small, a build of 600 new particles took 160 us, not 111).
+// n <= 32 R composites sorted by one warp (from global or shared memory).
 template <int R>
-__device__ __noinline__ void sort_run(const uint64_t *rk, const uint32_t *rv, int n, uint64_t *k0, uint32_t *v0, uint64_t *sk,
+__device__ __forceinline__ void sort_bucket(const uint64_t *rk, const uint32_t *rv, int n, uint64_t *k0, uint32_t *v0, uint64_t *sk,
                                       uint32_t *sv, int lane)
 {
     uint64_t k[R];
@@ -512,6 +511,15 @@ __device__ __noinline__ void sort_run(const uint64_t *rk, const uint32_t *rv, in
             v0[e] = sv[e + e / R];
         }
     }
+}
+
+// The same, its code fetched once for all its callers: inlined three times in sort_small, a build of 600 new particles
+// took 160 us, not 111. (The buckets' own sort is inlined: 2 us of a step of 2^17.)
+template <int R>
+__device__ __noinline__ void sort_run(const uint64_t *rk, const uint32_t *rv, int n, uint64_t *k0, uint32_t *v0, uint64_t *sk,
+                                      uint32_t *sv, int lane)
+{
+    sort_bucket<R>(rk, rv, n, k0, v0, sk, sv, lane);
 }
 
 // A small system with an overflowed bucket, by the blocks that its buckets belong to, each by itself: keys made anew,
@@ -597,9 +605,9 @@ __device__ __noinline__ void sort_small(const SmallArgs &a, int s, const SSys &y
 }
 
 // One warp per bucket. SCANNED: cnt holds the exclusive sums of the counts (nbk + 1 entries), else the counts,
-// which each block adds up itself.
+// which each block adds up itself. rcap: entries of a region of a single system.
 template <bool SCANNED>
-__global__ void __launch_bounds__(SSB_THREADS, 4) k_ss_sort(int nbk, int S, const SSys *__restrict__ ss,
+__global__ void __launch_bounds__(SSB_THREADS, 4) k_ss_sort(int nbk, int S, int rcap, const SSys *__restrict__ ss,
                                                             const uint32_t *__restrict__ bsys,
                                                             const uint32_t *__restrict__ cnt,
                                                             const uint64_t *__restrict__ rk,
@@ -637,16 +645,19 @@ __global__ void __launch_bounds__(SSB_THREADS, 4) k_ss_sort(int nbk, int S, cons
             __syncthreads();
         }
         if (n > 0u) {   // the whole warp
-            const SSys y = ss[S == 1 ? 0u : bsys[b]];
-            const int64_t region = y.rbase + (int64_t)(b - y.bbase) * y.rcap;
+            int64_t region = (int64_t)b * rcap;   // a single system's regions are known without a load
+            if (S > 1) {
+                const SSys y = ss[bsys[b]];
+                region = y.rbase + (int64_t)(b - y.bbase) * y.rcap;
+            }
             const uint64_t *kb = rk + region;
             const uint32_t *vb = rv + region;
-            if ((fl & 2u) && overflowed(y)) {
+            if ((fl & 2u) && overflowed(ss[S == 1 ? 0u : bsys[b]])) {
                 // below
             } else if (n <= 256u) {
-                sort_run<8>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+                sort_bucket<8>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
             } else {
-                sort_run<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
+                sort_bucket<SS_CAP / 32>(kb, vb, (int)n, k0 + s0, v0 + s0, m.k[w], m.v[w], lane);
             }
         }
         if (fl & 2u) {
@@ -1965,10 +1976,12 @@ void launch_keys_sort(hybrid_ctx *c)
         // up to SS_SUM_MAX buckets every block of the sort adds up the counts before its buckets (at most 32 loads
         // a thread); above, a scan does it once
         if (c->nbk <= SS_SUM_MAX) {
-            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag, small);
+            k_ss_sort<false><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, c->h_ss[0].rcap, ss, bsys, cnt, rk,
+                                                              rv, k0, v0, flag, small);
         } else {
             scan_u32(c, cnt, c->nbk + 1, nullptr, c->nbk + 1, nullptr, true);
-            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, ss, bsys, cnt, rk, rv, k0, v0, flag, small);
+            k_ss_sort<true><<<grid, SSB_THREADS, 0, c->st>>>(c->nbk, c->S, c->h_ss[0].rcap, ss, bsys, cnt, rk,
+                                                              rv, k0, v0, flag, small);
         }
         c->launches += 2;
         return;
