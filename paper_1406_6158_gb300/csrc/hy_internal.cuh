@@ -269,7 +269,7 @@ struct hybrid_ctx {
     // tree
     hy::Buf lvl, nfirst, nend, nchild, nchend, nparent, nlevel, ndone;   // nodes: particles and children [first, end)
     hy::Buf cells, ccnt;                          // topology scratch: packed levels per particle, counts per tile
-    hy::Buf nbig, mitems;                         // b_max of large cells: the cells (FP64 form: their chunks)
+    hy::Buf nbig, mitems;                         // b_max of large cells: their chunks (FP32 form above 2^20: the cells)
     hy::Buf nbmax32;                              // b_max as FP32 bits (FP32 form)
     int64_t capItems = 0;
     hy::Buf nM, ncx, ncy, ncz, nB2, nbmax;     // FP64 moments

@@ -9,7 +9,8 @@
 //
 // FP32 form. Work item = (group, run of at most item_len consecutive entries
 // of one of the group's lists), written by the walk and pulled from a global
-// counter. Near kernel: one block per work item, see k_near. Far kernel: one
+// counter. Near kernel: one block per work item, see k_near and, for the items
+// of groups well inside R2, near_dense. Far kernel: one
 // warp per work item; sources are staged, 64 at a time, into the
 // warp's shared-memory tile relative to the group's reference point (the hi
 // part of its first sink: on the hi grid, so hi - c is exact), as {x, y, z, m}
@@ -624,8 +625,9 @@ __device__ __forceinline__ float unord_f(int i) { return __int_as_float(i ^ ((i 
 // sources per packed instruction, and the lanes that a block of sinks leaves over hold further copies of it, each with
 // its own source pairs (lanes busy on the groups of a Plummer sphere of 2^17: 86 % against 52 %).
 // Near time per step, marks alone -> with this: 2^17 with R2 = 32, 64, 128 eps 1.07 -> .81, 4.37 -> 2.78, 21.9 -> 12.2 ms
-// (R2 = 8 eps .178 -> .181, 10^6 1.028 -> 1.045: the registers of the two loops together); a tenth of 2^17 particles in a
-// clump of half an R2 4.70 -> 2.25; N = 30000 with 64 eps 1.27 -> .76. NEAR_DENSE = 0.7: with 0.4 .93 and 2.89 ms for 32
+// (R2 = 8 eps .176 -> .178, 10^6 1.019 -> 1.034: the registers of the two loops together); a tenth of 2^17 particles in a
+// clump of half an R2 4.70 -> 2.25 (bound by the FMA pipe then: its throttle is the top stall; the form before the marks
+// took 2.31); N = 30000 with 64 eps 1.27 -> .76. NEAR_DENSE = 0.7: with 0.4 .93 and 2.89 ms for 32
 // and 64 eps, with 1 as with 0.7. Counting the near leaves close to the group in the walk chose no better and cost it 4 %.
 // A kernel of its own for these items (80 registers, beside k_near on the second stream) was 2 to 4 % faster on them, but
 // its launch cost steps of 2^13 particles 2 %.

@@ -1,12 +1,13 @@
 // tree.cu -- octree construction on the device (Sec. III-A1 of the paper,
-// done on the GPU instead of the host): root cube, Morton keys, a stable LSD
-// radix sort of the keys with the particle data gathered into key order, a
-// level-wise split (a cell with more than n_leaf particles splits into its
-// non-empty octants), cell moments (Sec. II-B: mass, centre of mass; Eq. 5-6:
-// b_max, B2, MAC radius) and the sink groups.
+// done on the GPU instead of the host): root cube, Morton keys, their stable
+// order (a sample sort with the last build's keys as splitters, or an LSD radix
+// sort) with the particle data gathered into it, the octree of all levels at
+// once (a cell with more than n_leaf particles splits into its non-empty
+// octants) with the sink groups, and cell moments (Sec. II-B: mass, centre of
+// mass; Eq. 5-6: b_max, B2, MAC radius).
 //
 // All systems of a batch are processed by the same launches; every node,
-// particle range and radix tile stays inside one system.
+// particle range, bucket and radix tile stays inside one system.
 #include "hy_internal.cuh"
 #include "root_box.cuh"
 
@@ -315,21 +316,22 @@ __global__ void __launch_bounds__(256) k_onesweep(const uint64_t *__restrict__ k
 // the keys into nb buckets: particle i is tried in the bucket of its position
 // (most are still there: two comparisons against keys a whole warp shares),
 // then in buckets ever farther away, and its key and index are appended to the
-// bucket's region (SS_CAP entries, fewer for a small system). One warp then sorts each bucket in
-// registers (bitonic, by composite) and writes it to its place, the sum of the
-// earlier buckets' counts. Keys end sorted in keys[0] with their source
+// bucket's region (SS_CAP entries, fewer for a small system). One warp then
+// sorts each bucket in registers (bitonic, by composite) and writes it to its
+// place, the sum of the earlier buckets' counts. Keys end sorted in keys[0] with their source
 // positions in vals[0], exactly as the radix sort leaves them. Splitters out
 // of order (another batch's keys, a first build) only send every particle
 // through one binary search, which gives the same bucket to equal composites
 // and keeps buckets in order whatever the splitters are. A bucket of more than
 // SS_CAP keys (a state far from key order) makes the build leave the order
-// unchanged and record ST_SORT; the build is then repeated with the radix
-// sort. A system of at most SS_SMALL buckets takes splitters of its own instead
+// unchanged and record ST_SORT; that one build is then repeated with the radix
+// sort, which leaves the splitters of the next. A system of at most SS_SMALL buckets takes splitters of its own instead
 // (sort_small): a first build of it, or one after another system's, nearly
 // always overflows, and the repetition cost more than the rest of the build
 // (hybrid_build_tree of a new state: N = 600 203 -> 111 us, 4096 228 -> 151; with
 // buckets of 4096 keys, which held any such system, 143 and 189).
-// Three launches, each key written and read twice. Before: buckets of 1024 or
+// Two launches (four with the scan of many counts), each key written and read
+// twice. Before: buckets of 1024 or
 // 2048 keys, a splitter, a counting, a scan and a scatter launch, and a radix
 // sort of each bucket in shared memory. Root box and key sort per soft step of
 // 4 hard sub-steps (8 at 2^24): N = 4096 0.190 -> 0.079 ms, 2^17 0.222 ->
@@ -694,7 +696,8 @@ struct PermArgs {
 
 // MINB blocks per SM: 8 (32 registers) for batches above 2^18 particles, where the gathers' bandwidth counts (2^24:
 // tree build 30.1 -> 28.7 ms per soft step against 64 registers, 2^20 1.172 -> 1.138); below, a thread's loads all go
-// out at once with 64 (2^12 and 2^17 2 and 1 % of the step faster).
+// out at once with 64 (2^12 and 2^17 2 and 1 % of the step faster). At 32 a thread spills about 270 bytes, out and in, in the
+// grid-stride loop's body; they stay in L1: DRAM moves 153 + 184 MB for 2^21 particles (336 algorithmic) in 75 us.
 template <int MINB>
 __global__ void __launch_bounds__(256, MINB) k_permute(PermArgs a)
 {

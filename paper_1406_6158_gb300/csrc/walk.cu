@@ -20,7 +20,8 @@
 // WALK_REGION entries per kind at a time), so a group's entries of one kind
 // are contiguous until a region runs out; every contiguous run becomes pair
 // work items of at most item_len entries, appended to the far (cells, far
-// particles) or near item array, which the pair kernels consume directly.
+// particles) or near item array, which the pair kernels consume directly (the
+// near items of groups well inside R2 from the array's other end).
 // FP64 form (two passes): the count pass sizes every list, a scan turns
 // counts into offsets, and the fill pass writes them (one list per group and
 // kind, for the deterministic FP64 pair kernel).
